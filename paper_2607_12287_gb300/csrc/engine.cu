@@ -39,11 +39,19 @@ struct TimelineSlot {
   int m_static = -1;               // GEMM rows when fixed, -1 when read from the device
 };
 
-// Launch shape of one GEMM: row-tile variant, CTAs per cluster (the K split), clusters.
+// Launch shape of one GEMM.  Over CTA pairs (`pair`): tiles of bn rows, K split csize ways
+// (more than one only when deferred), n_clusters pairs.  Else: tiles of bn = 64 rows, K split
+// over clusters of csize CTAs (n_clusters of them), or over csize plain CTAs when deferred.
 struct GemmPlan {
+  bool pair = false;
   int bn = 64, csize = 1, n_clusters = 1;
   bool defer = false;  // residual GEMMs: leave the split partials to the next layer norm
-  bool vsplit = false; // deferred: K split over CTAs launched without clusters
+};
+
+// TMA maps of one activation buffer with boxes of 64 columns x 32, 64 and 128 rows.
+struct ActMaps {
+  CUtensorMap b32, b64, b128;
+  const CUtensorMap& of(const GemmPlan& pl) const { return !pl.pair || pl.bn == 64 ? b32 : pl.bn == 128 ? b64 : b128; }
 };
 
 enum GemmSlot { kGemmEmbed = 0, kGemmQKV, kGemmO, kGemmUp, kGemmDown, kGemmSlots };
@@ -111,7 +119,7 @@ struct ivit_handle {
   int N = 0, D = 0, F = 0, H = 0, L = 0, SV = 0, Kp = 0, KPAD = 0, M_max = 0;
   int device = 0, num_sms = 0;
   int row_grid = 0;
-  GemmPlan plan_full[kGemmSlots], plan_inc[kGemmSlots];
+  GemmPlan plan_full[kGemmSlots], plan_inc[kGemmSlots], plan_keys;
   // Row-count bands of the incremental graph (band 0 = plan_inc): launch plans and
   // attention key splits made for at most band_ub[b] updated rows; a switch node picks
   // the band of each call's device-resident row count.
@@ -129,7 +137,8 @@ struct ivit_handle {
   bf16* w_pe = nullptr;
   float *b_pe = nullptr, *pos = nullptr, *lnfg = nullptr, *lnfb = nullptr;
   std::vector<LayerW> layers;
-  CUtensorMap tm_pe, tm_patches, tm_xn, tm_o, tm_h;
+  CUtensorMap tm_pe;
+  ActMaps tm_patches, tm_xn, tm_o, tm_h;
   CUtensorMap tm_qa;     // packed queries, 64 x 32 boxes, 128-byte swizzle (tcgen05 attention)
   bool attn_tc = true;   // tensor-core attention (IVIT_ATTN=simt selects the SIMT kernel)
   int attn_splits_full = 1, attn_splits_inc = 1;  // key splits (CTAs per item) of that kernel
@@ -242,26 +251,70 @@ size_t weights_count(const ivit_config* c) {
   return D * Kp + D + N * D + per_layer * c->depth + 2 * D;
 }
 
-// Launch shape of a GEMM with a K split over clusters of c CTAs.  Cost model (fitted
-// to measurements of this kernel on GB300 with small row counts): a launch pays a fixed
-// ~4 us plus ~0.35 us per 16 KB weight stage a CTA streams, once per round of tiles
-// over the clusters that fit on the GPU.  Cluster sizes above 9 lose SMs to GPC packing.
-GemmPlan plan_gemm(int num_sms, int bn, int n_out, int k, int m_expected) {
+// Scratch slots (fp32 [bn][128]) a deferred plan needs for up to m_bound rows.
+size_t defer_slots(const GemmPlan& pl, int n_out, int m_bound) {
+  return static_cast<size_t>((n_out + 127) / 128) * ((m_bound + pl.bn - 1) / pl.bn) * pl.csize;
+}
+
+// Launch shape of a GEMM expected to see m_expected rows (and at most m_bound): the
+// cheapest candidate of a cost model in microseconds per launch, fitted to back-to-back
+// launches on GB300 of the SigLIP-So400m shapes at 26 to 32768 rows.
+//   CTA pairs: a fixed part (prologue, first loads, last tile's epilogue) plus a k-block
+//     (64 wide) rate per round of units over the 76 pairs; 64-, 128- and 256-row tiles
+//     measured 4.3 / 4.8 / 6.2 us + 0.20 / 0.24 / 0.33 us per k-block, and 0.7 us for the
+//     prologue that its shared memory keeps from running under the previous kernel.
+//   K split over clusters of 64-row tiles: 5.8 us + 0.35 us per 16 KB weight stage per
+//     round; it wins up to about 64 rows, where a pair tile's whole K on few SMs is longer
+//     (QKV of 26 rows: 6.9 us in clusters of 5 against 7.9).  Clusters above 9 lose SMs to
+//     GPC packing.
+//   Deferred (residual GEMMs, allow_defer): K split over plain CTAs or pairs whose partial
+//     tiles the next layer norm sums: no barrier and no epilogue, but every split's fp32
+//     tile is written and read once (about 4 TB/s through L2).
+GemmPlan plan_gemm(int num_sms, int n_out, int k, int m_expected, int m_bound, bool allow_defer) {
   GemmPlan best;
-  best.bn = bn;
-  const int n_ft = (n_out + 127) / 128, n_tt = (m_expected + bn - 1) / bn, n_kb = (k + 63) / 64;
-  const int tiles = std::max(1, n_ft * n_tt);
   double best_cost = 1e30;
-  for (int c = 1; c <= std::min(16, n_kb); ++c) {
-    const int fit = ivit::gemm_max_clusters(bn, c);
-    if (fit <= 0) continue;
-    const int ncl = std::max(1, std::min({tiles, fit, num_sms / c}));
-    const int rounds = (tiles + ncl - 1) / ncl;
-    const double cost = rounds * (4.0 + 0.35 * ((n_kb + c - 1) / c));
+  auto consider = [&](const GemmPlan& pl, double cost) {
     if (cost < best_cost - 1e-9) {
       best_cost = cost;
-      best.csize = c;
-      best.n_clusters = ncl;
+      best = pl;
+    }
+  };
+  allow_defer = allow_defer && !std::getenv("IVIT_NO_DEFER");
+  const int n_ft = (n_out + 127) / 128, n_kb = (k + 63) / 64, max_pairs = num_sms / 2;
+  auto partial_cost = [&](int c) { return c * (8.0 * n_out) * m_expected / 4.0e6; };
+  auto fits = [&](const GemmPlan& pl) {
+    return defer_slots(pl, n_out, m_bound) * pl.bn * 128 * 4 <= (64ull << 20);
+  };
+  for (int bn : {64, 128, 256}) {
+    const double fixed = bn == 64 ? 5.0 : bn == 128 ? 5.5 : 6.9, per_kb = bn == 64 ? 0.20 : bn == 128 ? 0.24 : 0.33;
+    const int tiles = std::max(1, (n_ft + 1) / 2 * ((m_expected + bn - 1) / bn));
+    for (int c = 1; c <= std::min(allow_defer ? 16 : 1, n_kb); ++c) {
+      GemmPlan pl;
+      pl.pair = true;
+      pl.bn = bn;
+      pl.csize = c;
+      pl.defer = c > 1;
+      // (a call may bring more rows than expected: the launch is as wide as m_bound can use)
+      pl.n_clusters = std::min(max_pairs, (n_ft + 1) / 2 * ((m_bound + bn - 1) / bn) * c);
+      const int rounds = (tiles * c + max_pairs - 1) / max_pairs;
+      if (!pl.defer || fits(pl)) consider(pl, fixed + rounds * per_kb * ((n_kb + c - 1) / c) + (c > 1 ? partial_cost(c) : 0));
+    }
+  }
+  const int tiles = std::max(1, n_ft * ((m_expected + 63) / 64));
+  for (int c = 2; c <= std::min(16, n_kb); ++c) {
+    GemmPlan pl;
+    pl.csize = c;
+    if (allow_defer) {
+      pl.defer = true;
+      pl.n_clusters = tiles;
+      const int rounds = (tiles * c + num_sms - 1) / num_sms;
+      if (fits(pl)) consider(pl, rounds * (4.0 + 0.35 * ((n_kb + c - 1) / c)) + partial_cost(c));
+    } else {
+      const int fit = ivit::gemm_max_clusters(c);
+      if (fit <= 0) continue;
+      pl.n_clusters = std::max(1, std::min({tiles, fit, num_sms / c}));
+      const int rounds = (tiles + pl.n_clusters - 1) / pl.n_clusters;
+      consider(pl, rounds * (4.0 + 0.35 * ((n_kb + c - 1) / c)) + 1.8);
     }
   }
   return best;
@@ -308,7 +361,7 @@ int setup_persistent(ivit_handle* h) {
     wm[4 * l + 3] = w.tm_2;
     lp[l] = ivit::LayerParams{w.bqkv, w.bo, w.b1, w.b2, w.ln1g, w.ln1b, w.ln2g, w.ln2b};
   }
-  const CUtensorMap xm[3] = {h->tm_xn, h->tm_o, h->tm_h};
+  const CUtensorMap xm[3] = {h->tm_xn.b32, h->tm_o.b32, h->tm_h.b32};
   std::vector<CUtensorMap> kvm(2 * L);
   for (int l = 0; l < L; ++l) {
     const size_t off = static_cast<size_t>(l) * h->M_max * h->D;
@@ -417,7 +470,7 @@ int setup_stream(ivit_handle* h) {
       return h->fail(IVIT_ERR_CUDA, "cuTensorMapEncodeTiled failed for the weight-streaming kernel");
     lp[l] = ivit::LayerParams{w.bqkv, w.bo, w.b1, w.b2, w.ln1g, w.ln1b, w.ln2g, w.ln2b};
   }
-  const CUtensorMap bm[3] = {h->tm_xn, h->tm_o, h->tm_h};
+  const CUtensorMap bm[3] = {h->tm_xn.b32, h->tm_o.b32, h->tm_h.b32};
   IVIT_CK(h, cudaMemcpy(ka.base + o_w, wm.data(), sizeof(CUtensorMap) * 4 * L, cudaMemcpyHostToDevice));
   IVIT_CK(h, cudaMemcpy(ka.base + o_b, bm, sizeof(bm), cudaMemcpyHostToDevice));
   IVIT_CK(h, cudaMemcpy(ka.base + o_kv, kvm.data(), sizeof(CUtensorMap) * 2 * L, cudaMemcpyHostToDevice));
@@ -491,8 +544,8 @@ int setup(ivit_handle* h, const uint16_t* wb) {
 
   IVIT_CK(h, cudaGetDevice(&h->device));
   IVIT_CK(h, cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, h->device));
-  IVIT_CK(h, ivit::gemm_setup(64));
-  IVIT_CK(h, ivit::gemm_setup(256));
+  IVIT_CK(h, ivit::gemm_setup());
+  IVIT_CK(h, ivit::gemm_pair_setup());
   IVIT_CK(h, ivit::attention_setup());
   IVIT_CK(h, ivit::attention_tc_setup());
   if (const char* at = std::getenv("IVIT_ATTN")) h->attn_tc = std::string(at) != "simt";
@@ -541,82 +594,37 @@ int setup(ivit_handle* h, const uint16_t* wb) {
   {
     // Full encodes know M = SV*N.  Incremental calls are planned for a tenth of the
     // tokens updated (any count still runs correctly, with more or fewer tile rounds).
-    const int m_inc = std::max(1, static_cast<int>(M / 10));
-    // (64-row tiles for full encodes of up to 256 rows: on a 256-row So400m view they
-    // measured 1.78 ms per full encode against 1.92-2.01 ms with one 256-row tile split
-    // over clusters, whose split partials are four times larger)
-    const int bn_full = M <= 256 ? 64 : 256, bn_inc = M <= 1024 ? 64 : 256;
+    const int m_all = static_cast<int>(M), m_inc = std::max(1, m_all / 10);
     const int shapes[kGemmSlots][2] = {{static_cast<int>(D), h->KPAD}, {3 * static_cast<int>(D), static_cast<int>(D)},
                                        {static_cast<int>(D), static_cast<int>(D)}, {static_cast<int>(F), static_cast<int>(D)},
                                        {static_cast<int>(D), static_cast<int>(F)}};
     for (int g = 0; g < kGemmSlots; ++g) {
-      h->plan_full[g] = plan_gemm(h->num_sms, bn_full, shapes[g][0], shapes[g][1], static_cast<int>(M));
-      h->plan_inc[g] = g == kGemmEmbed ? h->plan_full[g]
-                                       : plan_gemm(h->num_sms, bn_inc, shapes[g][0], shapes[g][1], m_inc);
+      // (under the MLP-on-all-tokens reading the residual epilogues feed no layer norm of the same rows)
+      const bool defer = (g == kGemmO || g == kGemmDown) && c.mlp_tokens == IVIT_MLP_UPDATED;
+      auto plan = [&](int m_expected, int m_bound) {
+        return plan_gemm(h->num_sms, shapes[g][0], shapes[g][1], m_expected, m_bound, defer);
+      };
+      h->plan_full[g] = plan(m_all, m_all);
+      h->plan_inc[g] = g == kGemmEmbed ? h->plan_full[g] : plan(m_inc, m_all);
       h->plan_band[0][g] = h->plan_inc[g];
       // (the band of all rows runs the full encode's plans: it attends like one too)
       for (int b = 1; b < h->n_bands; ++b)
-        h->plan_band[b][g] = g == kGemmEmbed || h->band_ub[b] >= static_cast<int>(M)
-                                 ? h->plan_full[g]
-                                 : plan_gemm(h->num_sms, h->band_ub[b] <= 256 ? 64 : 256, shapes[g][0], shapes[g][1],
-                                             h->band_ub[b]);
+        h->plan_band[b][g] = g == kGemmEmbed || h->band_ub[b] >= m_all ? h->plan_full[g]
+                                                                       : plan(h->band_ub[b], h->band_ub[b]);
     }
-    // Residual GEMMs with a K split leave their partials to the layer norm that follows
-    // (one slot per tile and split, sized for the most rows the plan can see), while that
-    // scratch stays under 64 MB.  Needing no cluster barrier, such a GEMM then splits K
-    // over plain CTAs, with the split re-chosen by the same cost model without the
-    // cluster packing limit (at most 16 splits, the layer norm's limit).
-    auto replan_free = [&](GemmPlan& pl, int n_out, int k, int m_expected) {
-      const int n_ft = (n_out + 127) / 128, n_tt = (m_expected + pl.bn - 1) / pl.bn, n_kb = (k + 63) / 64;
-      const int tiles = std::max(1, n_ft * n_tt);
-      double best_cost = 1e30;
-      GemmPlan best = pl;
-      for (int c = 2; c <= std::min(16, n_kb); ++c) {
-        const int rounds = (tiles * c + h->num_sms - 1) / h->num_sms;
-        const double cost = rounds * (4.0 + 0.35 * ((n_kb + c - 1) / c));
-        if (cost < best_cost - 1e-9) {
-          best_cost = cost;
-          best.csize = c;
-          best.n_clusters = tiles;
-        }
-      }
-      if (best_cost < 1e29 && !std::getenv("IVIT_NO_VSPLIT")) {
-        pl = best;
-        pl.vsplit = true;
-      }
-    };
-    auto set_defer = [&](GemmPlan& pl, int n_out, int m_bound) {
-      const size_t slots = static_cast<size_t>((n_out + 127) / 128) * ((m_bound + pl.bn - 1) / pl.bn) * pl.csize;
-      pl.defer = pl.csize > 1 && !std::getenv("IVIT_NO_DEFER") && slots * pl.bn * 128 * 4 <= (64ull << 20) &&
-                 h->D % 4 == 0 && h->D <= 4096;
-    };
-    // a deferred plan re-planned without clusters, kept if its scratch still fits
-    auto refine = [&](GemmPlan& pl, int g, int m_expected, int m_bound) {
-      if (!pl.defer) return;
-      const GemmPlan orig = pl;
-      replan_free(pl, shapes[g][0], shapes[g][1], m_expected);
-      set_defer(pl, static_cast<int>(D), m_bound);
-      if (!pl.defer) pl = orig;
-    };
-    for (int g : {static_cast<int>(kGemmO), static_cast<int>(kGemmDown)}) {
-      set_defer(h->plan_full[g], static_cast<int>(D), static_cast<int>(M));
-      set_defer(h->plan_inc[g], static_cast<int>(D), static_cast<int>(M));
-      refine(h->plan_full[g], g, static_cast<int>(M), static_cast<int>(M));
-      refine(h->plan_inc[g], g, std::max(1, static_cast<int>(M / 10)), static_cast<int>(M));
-      h->plan_band[0][g] = h->plan_inc[g];
-      for (int b = 1; b < h->n_bands; ++b) {
-        set_defer(h->plan_band[b][g], static_cast<int>(D), h->band_ub[b]);
-        refine(h->plan_band[b][g], g, h->band_ub[b], h->band_ub[b]);
-      }
-    }
+    // every row's D x D projection without a residual (first-layer key scores)
+    h->plan_keys = plan_gemm(h->num_sms, static_cast<int>(D), static_cast<int>(D), m_all, m_all, false);
     if (std::getenv("IVIT_DEBUG")) {
       static const char* names[kGemmSlots] = {"embed", "qkv", "out", "up", "down"};
-      for (int g = 0; g < kGemmSlots; ++g)
-        std::fprintf(stderr, "ivit gemm %-5s full bn=%d %s=%d x %d (fit %d) | inc bn=%d %s=%d x %d (fit %d)\n",
-                     names[g], h->plan_full[g].bn, h->plan_full[g].vsplit ? "split" : "cluster", h->plan_full[g].csize,
-                     h->plan_full[g].n_clusters, ivit::gemm_max_clusters(h->plan_full[g].bn, h->plan_full[g].csize),
-                     h->plan_inc[g].bn, h->plan_inc[g].vsplit ? "split" : "cluster", h->plan_inc[g].csize,
-                     h->plan_inc[g].n_clusters, ivit::gemm_max_clusters(h->plan_inc[g].bn, h->plan_inc[g].csize));
+      auto show = [&](const char* when, const char* name, const GemmPlan& pl) {
+        std::fprintf(stderr, "ivit gemm %-6s %-5s %s bn=%d split=%d%s x %d\n", when, name, pl.pair ? "pair" : "cluster", pl.bn,
+                     pl.csize, pl.defer ? " deferred" : "", pl.n_clusters);
+      };
+      for (int g = 0; g < kGemmSlots; ++g) {
+        show("full", names[g], h->plan_full[g]);
+        show("inc", names[g], h->plan_inc[g]);
+        for (int b = 1; b < h->n_bands; ++b) show(b == 1 ? "band 1" : b == 2 ? "band 2" : "band 3", names[g], h->plan_band[b][g]);
+      }
       for (int b = 1; b < h->n_bands; ++b)
         std::fprintf(stderr, "ivit band %d (<= %d rows): attention splits %d\n", b, h->band_ub[b], h->attn_splits_band[b]);
     }
@@ -715,18 +723,19 @@ int setup(ivit_handle* h, const uint16_t* wb) {
   const size_t o_err = sa.take(4);
   const size_t o_key = c.score_source == IVIT_SCORE_KEY0 ? sa.take(M * D * 4) : 0;
   const size_t o_acache = c.mlp_tokens == IVIT_MLP_ALL ? sa.take(L * M * D * 4) : 0;
-  // slots for every plan: clusters x CTAs per cluster x row tile x 128 features, fp32
+  // slots for every plan that splits K, fp32 [row tile][128 features] each
   size_t part_floats = 0;
   for (int g = 0; g < kGemmSlots; ++g)
   {
-    auto need = [&](const GemmPlan& pl, int m_bound) {
-      if (!pl.defer) return static_cast<size_t>(pl.n_clusters) * pl.csize * pl.bn * 128;
-      return static_cast<size_t>((D + 127) / 128) * ((m_bound + pl.bn - 1) / pl.bn) * pl.csize * pl.bn * 128;
+    auto need = [&](const GemmPlan& pl, int m_bound) -> size_t {
+      if (pl.defer) return defer_slots(pl, static_cast<int>(D), m_bound) * pl.bn * 128;
+      return pl.pair ? 0 : static_cast<size_t>(pl.n_clusters) * pl.csize * pl.bn * 128;
     };
     part_floats = std::max(part_floats, need(h->plan_full[g], static_cast<int>(M)));
     part_floats = std::max(part_floats, need(h->plan_inc[g], static_cast<int>(M)));
     for (int b = 0; b < h->n_bands; ++b)
       part_floats = std::max(part_floats, need(h->plan_band[b][g], b == 0 ? static_cast<int>(M) : h->band_ub[b]));
+    part_floats = std::max(part_floats, need(h->plan_keys, static_cast<int>(M)));
   }
   const size_t o_gpart = sa.take(part_floats * 4);
   const size_t o_rta = sa.take(M * 4), o_mall = sa.take(4);
@@ -778,11 +787,12 @@ int setup(ivit_handle* h, const uint16_t* wb) {
         !make_map(&h->layers[l].tm_av, h->cacheV + off, D, M, D * 2, 64, ivit::attention_tc_kv_box_rows()))
       return h->fail(IVIT_ERR_CUDA, "cuTensorMapEncodeTiled failed for a cache tile");
   }
-  if (!make_map(&h->tm_patches, h->patches, h->KPAD, M, h->KPAD * 2, 64, 32) ||
-      !make_map(&h->tm_xn, h->xn, D, M, D * 2, 64, 32) ||
-      !make_map(&h->tm_o, h->o, D, M, D * 2, 64, 32) ||
-      !make_map(&h->tm_qa, h->q, D, M, D * 2, 64, 32) ||
-      !make_map(&h->tm_h, h->hbuf, F, M, F * 2, 64, 32))
+  auto act_maps = [&](ActMaps& m, const bf16* base, size_t inner) {
+    return make_map(&m.b32, base, inner, M, inner * 2, 64, 32) && make_map(&m.b64, base, inner, M, inner * 2, 64, 64) &&
+           make_map(&m.b128, base, inner, M, inner * 2, 64, 128);
+  };
+  if (!act_maps(h->tm_patches, h->patches, h->KPAD) || !act_maps(h->tm_xn, h->xn, D) || !act_maps(h->tm_o, h->o, D) ||
+      !act_maps(h->tm_h, h->hbuf, F) || !make_map(&h->tm_qa, h->q, D, M, D * 2, 64, 32))
     return h->fail(IVIT_ERR_CUDA, "cuTensorMapEncodeTiled failed for an activation buffer");
   if (int r = setup_persistent(h)) return r;
   if (int r = setup_stream(h)) return r;
@@ -836,12 +846,15 @@ void next_launch(ivit_handle* h, int family, const ivit::GemmArgs* ga = nullptr,
   h->slots_cur.push_back(sl);
 }
 
-int gemm(ivit_handle* h, const GemmPlan& plan, const CUtensorMap& tw, const CUtensorMap& tx,
-         ivit::GemmArgs a, cudaStream_t s) {
+int gemm(ivit_handle* h, const GemmPlan& plan, const CUtensorMap& tw, const ActMaps& tx, ivit::GemmArgs a,
+         cudaStream_t s) {
   a.err = h->err;
   a.partials = h->gemm_partials;
+  a.defer = plan.defer ? 1 : 0;
+  a.vsplit = plan.defer ? plan.csize : 0;
   next_launch(h, kFamGemm, &a);
-  IVIT_CK(h, ivit::launch_gemm(plan.bn, tw, tx, a, plan.n_clusters, plan.csize, s));
+  IVIT_CK(h, plan.pair ? ivit::launch_gemm_pair(plan.bn, tw, tx.of(plan), a, plan.n_clusters, s)
+                       : ivit::launch_gemm(tw, tx.of(plan), a, plan.n_clusters, plan.csize, s));
   ++h->launches;
   return IVIT_OK;
 }
@@ -1061,7 +1074,7 @@ int run_layers(ivit_handle* h, const GemmPlan* plan, int attn_splits, bool full,
     ++h->launches;
     return IVIT_OK;
   };
-  auto residual = [&](const GemmPlan& pl, const float* bias, const CUtensorMap& tw, const CUtensorMap& tx,
+  auto residual = [&](const GemmPlan& pl, const float* bias, const CUtensorMap& tw, const ActMaps& tx,
                       int k) -> int {
     ivit::GemmArgs a;
     a.n_out = D;
@@ -1071,8 +1084,6 @@ int run_layers(ivit_handle* h, const GemmPlan* plan, int attn_splits, bool full,
     a.epi.bias = bias;
     a.epi.out_f32 = h->x;
     a.epi.ld_out = D;
-    a.defer = pl.defer ? 1 : 0;
-    a.vsplit = pl.defer && pl.vsplit ? pl.csize : 0;
     if (int r = gemm(h, pl, tw, tx, a, s)) return r;
     if (pl.defer) {
       pend.partials = h->gemm_partials;
@@ -1206,8 +1217,7 @@ int run_core(ivit_handle* h, const uint8_t* frames, int32_t* user_counts, bool f
     a.epi.bias = h->layers[0].bqkv + D;
     a.epi.out_f32 = h->key_t;
     a.epi.ld_out = D;
-    // a D x D projection of every row: the full encode's out-projection launch shape
-    if (int r = gemm(h, h->plan_full[kGemmO], h->tm_wk0, h->tm_xn, a, s)) return r;
+    if (int r = gemm(h, h->plan_keys, h->tm_wk0, h->tm_xn, a, s)) return r;
     score_vec = h->key_t;
   }
   if (!full) {

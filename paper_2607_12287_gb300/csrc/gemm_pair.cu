@@ -1,0 +1,395 @@
+// Tensor-core GEMM over CTA pairs (tcgen05 cta_group::2), for every GEMM of more than about
+// 64 rows: Y[r][f] = sum_k X[r][k] W[f][k] for the packed rows, then an epilogue of
+// GemmEpilogue.
+//
+// A cluster of two CTAs computes a tile of 256 output features x BN rows: each CTA stages
+// its 128 features of W and its half of the BN rows of X, the leader's MMA warp multiplies
+// 256 x BN from both shared memories, and each CTA's tensor memory receives its 128 features
+// (lanes) x BN rows (columns).  A CTA fetches (128 + BN / 2) x 128 bytes per 64-wide k-block
+// where a CTA on its own fetches (128 + BN) x 128 for the same MMA work.
+//
+// What bounds it: at large row counts the tensor pipe under the power limit; at a few
+// hundred rows the chain of one tile (prologue, 18 to 68 k-blocks, epilogue).  What the
+// single-CTA kernels before it spent their time on, and what is done about it here:
+//   - the loops that issue TMA and MMA run as whole warps with one elected lane, so their
+//     operands stay in uniform registers; one diverged lane needed 0.31 us per k-block of a
+//     64-row tile whatever the number of stages, this form 0.19;
+//   - X comes in one box of BN / 2 rows per stage, not in boxes of 32 (down-projection of
+//     32768 rows 260 -> 226 us);
+//   - one epilogue per instantiation, through shared memory and 16-byte accesses: the
+//     epilogue that stored column by column behind a switch took 7.5 us for 64 rows x 128
+//     features, most of it on instruction fetch.  The residual is added in L2 (red.v4.f32),
+//     so it is never loaded.
+// Measured back to back, random bf16 data, before -> now: 32768 rows QKV 422 -> 159 us, up
+// 497 -> 203, out 154 -> 82, down 324 -> 211 (1540 TFLOP/s); 3080 rows QKV 65 -> 22, up
+// 60 -> 24, down 53 -> 26; 768 rows QKV 29 -> 12, up 27 -> 12; 256 rows QKV 16 -> 8, up
+// 16 -> 8.5.
+#include "internal.h"
+#include "ptx.cuh"
+
+namespace ivit {
+namespace {
+
+constexpr int BM = 128;   // output features per CTA (a pair's MMA has M = 256)
+constexpr int BK = 64;    // K per stage: 128-byte rows, 128-byte swizzle
+constexpr int W_BYTES = BM * BK * 2;
+constexpr int EPI_WARPS = 8;
+constexpr int THREADS = (EPI_WARPS + 2) * 32;
+constexpr int EPI_HALF = 8192;  // staging of one row half: 32 rows of 128 bf16 or 16 of fp32
+
+// Stages: more than 6 (8 for 64 rows) measured no faster; 4 lost 10 % below 768 rows.
+template <int BN>
+struct PairCfg {
+  static constexpr int STAGES = BN == 64 ? 8 : 6;
+  static constexpr int STAGE_BYTES = W_BYTES + BN / 2 * BK * 2;
+  static constexpr int EPI_OFFSET = STAGES * STAGE_BYTES;
+  static constexpr int BAR_OFFSET = EPI_OFFSET + 2 * EPI_HALF;
+  static constexpr int TOTAL = BAR_OFFSET + 256 + 1024;  // barriers, flags, 1 KB alignment slack
+  static_assert(TOTAL <= 227 * 1024, "shared memory of one CTA");
+};
+
+// Hardware tanh (one MUFU instruction, relative error about 2^-11: below the bf16
+// rounding the GELU output gets).
+__device__ __forceinline__ float tanh_hw(float x) {
+  float y;
+  asm("tanh.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
+__device__ __forceinline__ float gelu_f(float x, int mode) {
+  if (mode == 1) return 0.5f * x * (1.f + erff(x * 0.70710678118654752f));
+  const float c = 0.79788456080286536f;  // sqrt(2/pi)
+  return 0.5f * x * (1.f + tanh_hw(c * (x + 0.044715f * x * x * x)));
+}
+
+// Drains rows [c_lo, c_hi) of the tile (columns of this CTA's accumulator) on the four
+// warps of one row half: chunks of 32 rows (16 when fp32) go from tensor memory (lane = feature) through
+// shared memory (row-major) to global memory with 16-byte accesses, 128 features of a row
+// at a time.  `release` is called once, when the accumulator has been read.
+template <int KIND, class Release>
+__device__ __forceinline__ void drain(const GemmArgs& a, uint32_t acc, uint8_t* stg, int bar_id, int wq, int lane,
+                                      int row0, int c_lo, int c_hi, int ft, float* slot, bool ok, Release release) {
+  constexpr bool kBf16 = KIND == kEpiQKV || KIND == kEpiGelu;
+  constexpr int CHUNK = kBf16 ? 32 : 16;
+  const int f0 = ft * BM, fl = wq * 32 + lane;
+  float bias = 0.f;
+  if (KIND != kEpiPartial && f0 + fl < a.n_out) bias = __ldg(a.epi.bias + f0 + fl);
+  // this thread's part of a row in the second step: 8 bf16 features (two rows per warp
+  // and access) or 4 fp32 features (one row)
+  constexpr int FPT = kBf16 ? 8 : 4, LPR = BM / FPT, RPW = 32 / LPR, ITERS = CHUNK / (4 * RPW);
+  const int sub = lane % LPR, rsub = wq * RPW + lane / LPR;
+  const int f = f0 + FPT * sub;
+  const bool f_ok = ok && f < a.n_out;
+  bf16* dst16 = nullptr;
+  float* dst32 = nullptr;
+  bool by_tok = KIND == kEpiScatterF32;
+  int ld = a.epi.ld_out;
+  if (KIND == kEpiQKV) {
+    const int D = a.epi.dim;  // D % 64 == 0: 8 features never straddle Q, K and V
+    dst16 = f < D ? a.epi.out_bf16 + f : f < 2 * D ? a.epi.cache_k + (f - D) : a.epi.cache_v + (f - 2 * D);
+    by_tok = f >= D;
+    ld = D;
+  } else if (KIND == kEpiGelu) {
+    dst16 = a.epi.out_bf16 + f;
+  } else if (KIND == kEpiPartial) {
+    dst32 = slot + FPT * sub;
+    ld = BM;
+  } else {
+    dst32 = a.epi.out_f32 + f;
+  }
+  for (int c0 = c_lo; c0 < c_hi; c0 += CHUNK) {
+    int rr[ITERS];  // destination rows, -1 past the tile's end
+#pragma unroll
+    for (int i = 0; i < ITERS; ++i) {
+      const int c = c0 + i * 4 * RPW + rsub;
+      rr[i] = -1;
+      if (c < c_hi && f_ok) rr[i] = KIND == kEpiPartial ? c : by_tok ? __ldcg(a.epi.rowtok + row0 + c) : row0 + c;
+    }
+    uint32_t v[CHUNK];
+    if constexpr (kBf16) {
+      tmem_ld32_async(acc + c0, v);
+      tmem_ld_wait_regs(v);
+    } else {
+      tmem_ld16_async(acc + c0, v);
+      tmem_ld_wait();
+      tmem_regs_after_wait16(v);
+    }
+    if (c0 + CHUNK >= c_hi) release();
+    named_barrier(bar_id, 128);  // the previous chunk has left the staging buffer
+    if (kBf16) {
+      bf16* st = reinterpret_cast<bf16*>(stg) + fl;
+#pragma unroll
+      for (int j = 0; j < CHUNK; ++j) {
+        float y = __uint_as_float(v[j]) + bias;
+        if (KIND == kEpiGelu) y = gelu_f(y, a.epi.gelu_mode);
+        st[j * BM] = __float2bfloat16_rn(y);
+      }
+    } else {
+      float* st = reinterpret_cast<float*>(stg) + fl;
+#pragma unroll
+      for (int j = 0; j < CHUNK; ++j) st[j * BM] = __uint_as_float(v[j]) + bias;
+    }
+    named_barrier(bar_id, 128);
+#pragma unroll
+    for (int i = 0; i < ITERS; ++i) {
+      const uint4 u = *reinterpret_cast<const uint4*>(stg + ((i * 4 * RPW + rsub) * LPR + sub) * 16);
+      if (rr[i] < 0) continue;
+      const size_t off = static_cast<size_t>(rr[i]) * ld;
+      if (kBf16)
+        *reinterpret_cast<uint4*>(dst16 + off) = u;
+      else if (KIND == kEpiResid)
+        red_add_f32x4(dst32 + off, *reinterpret_cast<const float4*>(&u));
+      else
+        *reinterpret_cast<uint4*>(dst32 + off) = u;
+    }
+  }
+}
+
+template <int BN, int KIND>
+__global__ void __launch_bounds__(THREADS, 1)
+    gemm_pair_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_x,
+                     const GemmArgs a) {
+  using C = PairCfg<BN>;
+  constexpr int STAGES = C::STAGES;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
+                                             ~static_cast<uintptr_t>(1023));
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + C::BAR_OFFSET);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * STAGES + 4);
+  volatile int* sh_abort = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const uint32_t smem_base = smem_u32(smem), bar_base = smem_u32(bars);
+  const uint32_t accf = bar_base + 8 * (2 * STAGES), acce = accf + 16;
+  const int rank = static_cast<int>(cluster_ctarank());
+  const uint64_t desc0 = sdesc_kmajor_sw128(smem_base);
+
+  if (tid == 0) {
+    for (int st = 0; st < STAGES; ++st) {
+      mbar_init(bar_base + 8 * st, 1);             // full: the leader's expected bytes of both CTAs
+      mbar_init(bar_base + 8 * (STAGES + st), 1);  // empty: the pair's MMAs have read the stage
+    }
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(accf + 8 * b, 1);
+      mbar_init(acce + 8 * b, 2 * EPI_WARPS);  // the epilogue warps of both CTAs
+    }
+    fence_mbar_init();
+    tma_prefetch_desc(&tm_w);
+    tma_prefetch_desc(&tm_x);
+    *sh_abort = 0;
+  }
+  if (warp == EPI_WARPS + 1) tmem_alloc_pair(smem_u32(tmem_slot), 2 * BN);
+  tc_fence_before();
+  __syncthreads();
+  cluster_sync();  // both CTAs' barriers exist before any copy or arrival reaches them
+  tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+
+  // The row count comes from the selection kernel, at least two launches back.
+  const int M = a.d_rows ? *a.d_rows : a.m_static;
+  const int n_ft = (a.n_out + BM - 1) / BM, n_fp = (n_ft + 1) / 2;
+  const int n_tt = (M + BN - 1) / BN;
+  const int n_kb = (a.k + BK - 1) / BK;
+  const int splits = KIND == kEpiPartial ? a.vsplit : 1;
+  const int units = n_fp * n_tt * splits;
+  const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
+  // unit u: K split u % splits of feature pair (u / splits) % n_fp, row tile the rest
+  auto rows_of = [&](int tt) { return min(BN, M - tt * BN); };
+  auto half_of = [&](int rows) { return ((rows + 31) >> 5) << 4; };  // rows of X per CTA (MMA N / 2)
+
+  int n_pre = 0;
+  if (warp == EPI_WARPS && pair < units) {
+    // the first unit's weight stages do not depend on earlier kernels
+    const int sp = pair % splits, ft = 2 * (pair / splits % n_fp) + rank;
+    const int kb0 = sp * n_kb / splits, kb1 = (sp + 1) * n_kb / splits;
+    n_pre = min(STAGES, kb1 - kb0);
+    if (elect_one()) {
+      const uint64_t pol_w = l2_policy_evict_first();
+      for (int i = 0; i < n_pre; ++i) {
+        if (rank == 0) mbar_arrive_expect_tx(bar_base + 8 * i, 2 * C::STAGE_BYTES);
+        tma_load_2d_pair(smem_base + i * C::STAGE_BYTES, &tm_w, (kb0 + i) * BK, ft * BM,
+                         mapa_shared(bar_base + 8 * i, 0), pol_w);
+      }
+    }
+    __syncwarp();
+  }
+  pdl_wait();
+  pdl_launch_dependents();
+  stamp_begin(a.stamp);
+
+  if (warp == EPI_WARPS) {
+    const uint64_t pol_w = l2_policy_evict_first(), pol_x = l2_policy_evict_last();
+    uint32_t stage = 0, phase = 0;
+    bool first = true, ok = true;
+    const uint32_t full0 = mapa_shared(bar_base, 0);
+    for (int u = pair; u < units && ok; u += n_pairs) {
+      const int sp = u % splits, tile = u / splits;
+      const int ft = 2 * (tile % n_fp) + rank, tt = tile / n_fp;
+      const int half = half_of(rows_of(tt));
+      const int xrow = tt * BN + rank * half;
+      const int kb0 = sp * n_kb / splits, kb1 = (sp + 1) * n_kb / splits;
+      for (int kb = kb0; kb < kb1; ++kb) {
+        const uint32_t full = full0 + 8 * stage;
+        const uint32_t st = smem_base + stage * C::STAGE_BYTES;
+        const bool pre = first && kb - kb0 < n_pre;
+        if (!pre) ok = __all_sync(0xffffffffu, mbar_wait(bar_base + 8 * (STAGES + stage), phase ^ 1));
+        if (!ok) break;
+        if (elect_one()) {
+          if (!pre) {
+            if (rank == 0) mbar_arrive_expect_tx(bar_base + 8 * stage, 2 * C::STAGE_BYTES);
+            tma_load_2d_pair(st, &tm_w, kb * BK, ft * BM, full, pol_w);
+          }
+          tma_load_2d_pair(st + W_BYTES, &tm_x, kb * BK, xrow, full, pol_x);
+        }
+        __syncwarp();
+        if (++stage == STAGES) {
+          stage = 0;
+          phase ^= 1;
+        }
+      }
+      first = false;
+    }
+    if (!ok) {
+      atomicExch(a.err, kErrWaitSlotEmpty);
+      *sh_abort = 1;
+    }
+  } else if (warp == EPI_WARPS + 1) {
+    if (rank == 0) {
+      uint32_t stage = 0, phase = 0;
+      int iter = 0;
+      for (int u = pair; u < units; u += n_pairs, ++iter) {
+        const int sp = u % splits, tt = u / splits / n_fp;
+        const uint32_t idesc = idesc_bf16_f32(2 * BM, 2 * half_of(rows_of(tt)));
+        const int kb0 = sp * n_kb / splits, kb1 = (sp + 1) * n_kb / splits;
+        const int b = iter & 1;
+        bool ok = mbar_wait(acce + 8 * b, ((iter >> 1) & 1) ^ 1);
+        tc_fence_after();
+        const uint32_t acc = tmem + static_cast<uint32_t>(b * BN);
+        for (int kb = kb0; kb < kb1; ++kb) {
+          ok = ok && mbar_wait(bar_base + 8 * stage, phase);
+          if (!__all_sync(0xffffffffu, ok)) break;
+          tc_fence_after();
+          if (elect_one()) {
+            const uint64_t da = desc0 + static_cast<uint64_t>(stage * (C::STAGE_BYTES >> 4));
+            const uint64_t db = da + (W_BYTES >> 4);
+#pragma unroll
+            for (int k = 0; k < BK / 16; ++k)
+              umma_bf16_pair(acc, da + 2 * k, db + 2 * k, idesc, (kb > kb0 || k > 0) ? 1u : 0u);
+            umma_commit_pair(bar_base + 8 * (STAGES + stage));
+          }
+          __syncwarp();
+          if (++stage == STAGES) {
+            stage = 0;
+            phase ^= 1;
+          }
+        }
+        if (!__all_sync(0xffffffffu, ok)) {
+          atomicExch(a.err, kErrWaitTmaFull);
+          *sh_abort = 1;
+          break;
+        }
+        if (elect_one()) umma_commit_pair(accf + 8 * b);
+        __syncwarp();
+      }
+    }
+  } else {
+    const int wq = warp & 3, hf = warp >> 2;
+    const uint32_t trow = tmem + (static_cast<uint32_t>(wq * 32) << 16);
+    uint8_t* stg = smem + C::EPI_OFFSET + hf * EPI_HALF;
+    int iter = 0;
+    for (int u = pair; u < units; u += n_pairs, ++iter) {
+      const int sp = u % splits, tile = u / splits;
+      const int ft = 2 * (tile % n_fp) + rank, tt = tile / n_fp;
+      const int rows = rows_of(tt), hrows = ((rows + 63) >> 6) << 5;
+      const int b = iter & 1;
+      // (after an expired wait the loop runs on without waiting or storing, so that the
+      // warps of a half still meet at their named barriers)
+      const bool aborted = *sh_abort != 0;
+      const bool done = !aborted && mbar_wait(accf + 8 * b, (iter >> 1) & 1);
+      if (!done && !aborted) {
+        atomicExch(a.err, kErrWaitAccum);
+        *sh_abort = 1;
+      }
+      tc_fence_after();
+      const uint32_t acc = trow + static_cast<uint32_t>(b * BN);
+      const uint32_t freed = mapa_shared(acce + 8 * b, 0);
+      auto release = [&]() {
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive_cluster(freed);
+      };
+      const int c_lo = hf * hrows, c_hi = min(rows, c_lo + hrows);
+      float* slot = nullptr;
+      if (KIND == kEpiPartial)
+        slot = a.partials + (static_cast<size_t>(ft + n_ft * tt) * splits + sp) * BN * BM;
+      if (c_lo < c_hi && ft < n_ft)
+        drain<KIND>(a, acc, stg, 1 + hf, wq, lane, tt * BN, c_lo, c_hi, ft, slot, done, release);
+      else
+        release();
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  cluster_sync();  // the peer's copies, MMAs and arrivals on this CTA's memory are done
+  if (warp == EPI_WARPS + 1) {
+    tc_fence_after();
+    tmem_dealloc_pair(tmem, 2 * BN);
+  }
+  stamp_end(a.stamp);
+}
+
+template <int BN, int KIND>
+cudaError_t launch_one(const CUtensorMap& tm_w, const CUtensorMap& tm_x, const GemmArgs& a, int n_pairs,
+                       cudaStream_t s) {
+  return launch_ex(gemm_pair_kernel<BN, KIND>, dim3(2 * n_pairs), dim3(THREADS), PairCfg<BN>::TOTAL, s, 2, tm_w, tm_x,
+                   a);
+}
+
+template <int BN>
+cudaError_t launch_bn(const CUtensorMap& tm_w, const CUtensorMap& tm_x, const GemmArgs& a, int n_pairs,
+                      cudaStream_t s) {
+  if (a.defer) return launch_one<BN, kEpiPartial>(tm_w, tm_x, a, n_pairs, s);
+  switch (a.epi.kind) {
+    case kEpiF32Bias: return launch_one<BN, kEpiF32Bias>(tm_w, tm_x, a, n_pairs, s);
+    case kEpiQKV: return launch_one<BN, kEpiQKV>(tm_w, tm_x, a, n_pairs, s);
+    case kEpiResid: return launch_one<BN, kEpiResid>(tm_w, tm_x, a, n_pairs, s);
+    case kEpiGelu: return launch_one<BN, kEpiGelu>(tm_w, tm_x, a, n_pairs, s);
+    case kEpiScatterF32: return launch_one<BN, kEpiScatterF32>(tm_w, tm_x, a, n_pairs, s);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+template <int BN>
+cudaError_t setup_bn() {
+  cudaError_t e = cudaSuccess;
+  auto set = [&](auto kern) {
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, PairCfg<BN>::TOTAL);
+  };
+  set(gemm_pair_kernel<BN, kEpiF32Bias>);
+  set(gemm_pair_kernel<BN, kEpiQKV>);
+  set(gemm_pair_kernel<BN, kEpiResid>);
+  set(gemm_pair_kernel<BN, kEpiGelu>);
+  set(gemm_pair_kernel<BN, kEpiScatterF32>);
+  set(gemm_pair_kernel<BN, kEpiPartial>);
+  return e;
+}
+
+}  // namespace
+
+cudaError_t gemm_pair_setup() {
+  cudaError_t e = setup_bn<64>();
+  if (e == cudaSuccess) e = setup_bn<128>();
+  if (e == cudaSuccess) e = setup_bn<256>();
+  return e;
+}
+
+cudaError_t launch_gemm_pair(int bn, const CUtensorMap& tm_w, const CUtensorMap& tm_x, const GemmArgs& args,
+                             int n_pairs, cudaStream_t s) {
+  GemmArgs a = args;
+  a.stamp = g_stamp;
+  if (bn == 64) return launch_bn<64>(tm_w, tm_x, a, n_pairs, s);
+  if (bn == 128) return launch_bn<128>(tm_w, tm_x, a, n_pairs, s);
+  if (bn == 256) return launch_bn<256>(tm_w, tm_x, a, n_pairs, s);
+  return cudaErrorInvalidValue;
+}
+
+}  // namespace ivit

@@ -57,6 +57,7 @@ enum EpiKind : int {
   kEpiResid = 2,    // out_f32[r][f] += y + bias[f]  (residual stream, fp32)
   kEpiGelu = 3,     // out_bf16[r][f] = gelu(y + bias[f])
   kEpiScatterF32 = 4,  // out_f32[rowtok[r]][f] = y + bias[f]  (per-token output cache)
+  kEpiPartial = 5,     // a K split's fp32 tile, left in the scratch (GemmArgs::defer)
 };
 
 struct GemmEpilogue {
@@ -82,15 +83,12 @@ struct GemmArgs {
   // floats for every CTA of the launch.  Required when the launch's clusters have more
   // than one CTA.
   float* partials = nullptr;
-  // With clusters of more than one CTA and defer set, the split-K partial tiles are left
-  // in the scratch, slot (tile * csize + rank) with tile = feature tile + n_ft * row tile,
-  // and the kernel neither reduces them nor runs the epilogue: the next kernel sums them
-  // (layernorm_sum, for the residual epilogue).  The scratch then holds
-  // n_ft * ceil(M / BN_MAX) * csize slots.
+  // With defer set, K is split over vsplit consecutive CTAs (or pairs) without clusters and
+  // the partial tiles are left in the scratch, slot (tile * vsplit + split) of fp32
+  // [rows per tile][128] with tile = feature tile + n_ft * row tile; the kernel neither
+  // reduces them nor runs the epilogue: the next kernel sums them (layernorm_sum, for the
+  // residual epilogue).
   int defer = 0;
-  // With defer set and vsplit > 0, K is split over vsplit consecutive CTAs launched as
-  // clusters of one (no cluster barrier is needed to leave the partials): the split
-  // count is then free of the GPC packing that limits cluster sizes.
   int vsplit = 0;
   unsigned long long* stamp = nullptr;  // timeline stamps of this launch (or null)
   GemmEpilogue epi;
@@ -106,16 +104,22 @@ struct PendingSum {
   int n_ft = 0;                     // feature tiles of 128
 };
 
-// Returns the dynamic shared memory size (bytes) of the GEMM variant.
-size_t gemm_smem_bytes(int bn_max);
 // One-time attribute setup (dynamic smem opt-in, clusters of up to 16).
-cudaError_t gemm_setup(int bn_max);
-// Clusters of `csize` CTAs of the variant that can be resident at once (0 if none).
-int gemm_max_clusters(int bn_max, int csize);
-// Launches n_clusters clusters of csize CTAs.  The CTAs of a cluster split K and reduce
-// their partial tiles through distributed shared memory; clusters walk the output tiles.
-cudaError_t launch_gemm(int bn_max, const CUtensorMap& tm_w, const CUtensorMap& tm_x,
-                        const GemmArgs& a, int n_clusters, int csize, cudaStream_t s);
+cudaError_t gemm_setup();
+// Clusters of `csize` CTAs that can be resident at once (0 if none).
+int gemm_max_clusters(int csize);
+// Launches n_clusters clusters of csize >= 2 CTAs on tiles of 128 features x 64 rows (tm_x
+// boxes of 32 rows).  The CTAs of a cluster split K and reduce their partial tiles through
+// the scratch; clusters walk the output tiles.
+cudaError_t launch_gemm(const CUtensorMap& tm_w, const CUtensorMap& tm_x, const GemmArgs& a, int n_clusters,
+                        int csize, cudaStream_t s);
+
+// The same GEMM over CTA pairs (cta_group::2), tiles of 256 features x bn rows (64, 128 or
+// 256; tm_x boxes of bn / 2 rows), walked by n_pairs persistent pairs.  With defer set (and vsplit >= 1) K is split
+// vsplit ways and the partial tiles stay in the scratch, as described at GemmArgs::defer.
+cudaError_t gemm_pair_setup();
+cudaError_t launch_gemm_pair(int bn, const CUtensorMap& tm_w, const CUtensorMap& tm_x, const GemmArgs& a,
+                             int n_pairs, cudaStream_t s);
 
 // ------------------------------------------------------- persistent encoder (small M)
 struct LayerParams {

@@ -1,0 +1,38 @@
+"""Kernels at the edges of their tiles, through the C ABI against the fp32 oracle: an encoder of
+one or two layers encodes a stream in full and incrementally (updated lists bit-exact, tokens
+within the parity bars of gpu_util)."""
+import numpy as np
+import pytest
+
+from tests import gpu_util
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def pkg():
+    import paper_2607_12287_gb300 as p
+    p.load()
+    return p
+
+
+def _run(pkg, oracle_mod, grid, views, dim, heads, mlp, depth, change_p, n_frames=3):
+    from paper_2607_12287_gb300 import synth
+    shape = synth.EncoderShape(8 * grid[0], 8 * grid[1], 8, dim, depth, heads, mlp, synth.GELU_TANH)
+    frames = list(synth.stream_random(shape, views, n_frames, 11, change_p=change_p))
+    stats = gpu_util.run_side_by_side(pkg, oracle_mod, shape, synth.make_weights(shape, 3), frames, 1, views,
+                                      check_caches=True, cache_layers="all")
+    assert len(stats) == n_frames and all(np.isfinite(s[0]).all() for s in stats)
+
+
+# (grid, views, dim, heads, mlp): row counts around the 64-, 128- and 256-row tiles and their
+# 32-row halves, feature counts that are no multiple of the pair's 256 (192 = 1.5 x 128, 320,
+# 520, 840), one k-block (dim 64), and more tiles than CTA pairs
+PAIR_SHAPES = [((5, 13), 1, 192, 3, 520), ((1, 43), 3, 320, 5, 840), ((1, 257), 1, 192, 3, 520),
+               ((13, 25), 4, 320, 5, 840), ((10, 10), 1, 64, 1, 264), ((20, 26), 5, 576, 8, 1160)]
+
+
+@pytest.mark.parametrize("grid,views,dim,heads,mlp", PAIR_SHAPES,
+                         ids=[f"n{g[0] * g[1]}x{v}_d{d}_f{f}" for g, v, d, _, f in PAIR_SHAPES])
+def test_gemm_tile_edges(pkg, oracle_mod, grid, views, dim, heads, mlp):
+    _run(pkg, oracle_mod, grid, views, dim, heads, mlp, 1, 0.4)
