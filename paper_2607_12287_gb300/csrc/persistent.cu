@@ -378,6 +378,12 @@ __device__ __forceinline__ uint8_t* attention_smem(const Ctx& c) {
   return c.smem + PT_RING_BYTES + PT_MISC_BYTES;
 }
 
+// Bytes from the key tile to the value tile, and from there to the queries: a TMA tile's
+// shared-memory address must be a multiple of 128 bytes.
+__host__ __device__ __forceinline__ size_t kv_tile_stride(int n_tok, int head_dim) {
+  return (static_cast<size_t>(n_tok) * head_dim * 2 + 127) & ~static_cast<size_t>(127);
+}
+
 // Warp 0 lane 0: TMA of the cached keys and values of (view, head) of layer l, [N][dh]
 // each, into the attention region.  Reused tokens' rows are final before the layer
 // runs; the rows of this call's updated tokens are read again after the QKV reduce.
@@ -391,7 +397,7 @@ __device__ void prefetch_kv(Ctx& c, int l, int item) {
   const uint32_t tile = static_cast<uint32_t>(a.N) * a.dh * 2;
   mbar_arrive_expect_tx(kv_bar(c), 2 * tile);
   tma_load_2d(smem_u32(base), a.kvmaps + 2 * l, h * a.dh, v * a.N, kv_bar(c), l2_policy_evict_first());
-  tma_load_2d(smem_u32(base + tile), a.kvmaps + 2 * l + 1, h * a.dh, v * a.N, kv_bar(c),
+  tma_load_2d(smem_u32(base + kv_tile_stride(a.N, a.dh)), a.kvmaps + 2 * l + 1, h * a.dh, v * a.N, kv_bar(c),
               l2_policy_evict_first());
   c.kv_item = item;
 }
@@ -404,9 +410,10 @@ __device__ void attention_phase(Ctx& c, int l) {
   const int N = a.N, D = a.D, dh = a.dh;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   uint8_t* base = attention_smem(c);
-  bf16* sk = reinterpret_cast<bf16*>(base);                              // [N][dh]
-  bf16* sv = sk + static_cast<size_t>(N) * dh;                           // [N][dh]
-  float* sq = reinterpret_cast<float*>(sv + static_cast<size_t>(N) * dh);  // [QPI][dh]
+  const size_t tile = kv_tile_stride(N, dh);
+  bf16* sk = reinterpret_cast<bf16*>(base);               // [N][dh]
+  bf16* sv = reinterpret_cast<bf16*>(base + tile);        // [N][dh]
+  float* sq = reinterpret_cast<float*>(base + 2 * tile);  // [QPI][dh]
   float* sp = sq + PT_QPI * dh;                                          // [QPI][N]
   const bf16* ck = a.cacheK + static_cast<size_t>(l) * a.M_max * D;
   const bf16* cv = a.cacheV + static_cast<size_t>(l) * a.M_max * D;
@@ -699,7 +706,7 @@ __global__ void __launch_bounds__(PT_THREADS, 1)
 size_t persistent_smem_bytes(int n_tok, int head_dim) {
   // attention region: key and value tiles [N][dh] bf16, queries [QPI][dh] fp32,
   // probabilities [QPI][N] fp32
-  const size_t attn = 2 * static_cast<size_t>(n_tok) * head_dim * sizeof(bf16) +
+  const size_t attn = 2 * kv_tile_stride(n_tok, head_dim) +
                       static_cast<size_t>(PT_QPI) * head_dim * sizeof(float) +
                       static_cast<size_t>(PT_QPI) * n_tok * sizeof(float);
   return 1024 + PT_RING_BYTES + PT_MISC_BYTES + attn;

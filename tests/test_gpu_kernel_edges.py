@@ -36,3 +36,12 @@ PAIR_SHAPES = [((5, 13), 1, 192, 3, 520), ((1, 43), 3, 320, 5, 840), ((1, 257), 
                          ids=[f"n{g[0] * g[1]}x{v}_d{d}_f{f}" for g, v, d, _, f in PAIR_SHAPES])
 def test_gemm_tile_edges(pkg, oracle_mod, grid, views, dim, heads, mlp):
     _run(pkg, oracle_mod, grid, views, dim, heads, mlp, 1, 0.4)
+
+
+# head tiles (tokens x head width x 2 bytes) that are no multiple of the 128 bytes a TMA
+# destination needs
+@pytest.mark.parametrize("grid,views,dim,heads", [((5, 19), 2, 64, 4), ((1, 1), 2, 64, 8), ((5, 13), 2, 128, 4)],
+                         ids=["n95_dh16", "n1_dh8", "n65_dh32"])
+def test_persistent_kernel_odd_key_tiles(pkg, oracle_mod, monkeypatch, grid, views, dim, heads):
+    monkeypatch.setenv("IVIT_PATH", "persistent")
+    _run(pkg, oracle_mod, grid, views, dim, heads, 2 * dim, 2, 0.5)
