@@ -4,619 +4,432 @@
 //
 //   O = softmax(Q K^T / sqrt(dh)) V          per (view, head).
 //
-// Work item = (query tile of up to 128 packed updated rows of view v, head h).  Each
-// item is handled by a thread-block cluster of `ns` CTAs that split the view's keys:
-// CTA rank s takes keys [s*kpc, (s+1)*kpc), kpc = ceil(N / ns), in groups of up to 256
-// keys with an online softmax across the groups.  The clusters
-// walk the items with a stride; items past a view's row count (device-resident, written
-// by the selection kernel) are skipped, so one launch shape serves every row count and
-// the launch can sit in a CUDA graph.  Shared memory and TMEM are sized by kpc, so that
-// with 64 keys per CTA an attention CTA fits on an SM beside a GEMM CTA and starts (and
-// prefetches) while the QKV GEMM is still running.
+// Work item = (view v, head h, query tile of up to 128 packed updated rows).  Every CTA
+// derives the list of items from the device-resident row offsets (written by the selection
+// kernel) and walks it with a stride, so one launch shape serves every row count and the
+// launch can sit in a CUDA graph.  Per item the keys are walked in blocks of KB (128, 96 or
+// 64 by head width, so that S, P and O of a block fit in 256 tensor-memory columns) with an
+// online softmax.  Two CTAs share an SM: while one's warps take exponentials the other's
+// MMAs run.
 //
-// Per item and CTA, 128 threads (thread i <-> query row i <-> TMEM lane i) or, for key
-// groups of 128 keys and more, 256: threads i and i + 128 share row i, each taking every
-// other 32-key chunk of S (their partial row maxima and sums meet in shared memory) and
-// every other 16-column chunk of the output, so that two warps per TMEM lane quadrant
-// hide each other's latencies:
-//   Q tile [128 rows][dh] by TMA (128-byte swizzle, 64-column slices; the padding columns
-//   dh..round16(dh) are zeroed in shared memory); K, V of the CTA's keys by TMA into
-//   [kpc keys][64 columns] slices;
-//   per key group (its K/V tile fetched as soon as the previous group's one is consumed):
-//   S = Q K^T   tcgen05.mma M = 128, N = the group's keys, K = round16(dh), fp32 in TMEM;
-//   softmax     each thread reads its row of S from TMEM; running max m, P = 2^((S - m) c)
-//               (c = log2(e) / sqrt(dh)) rounded to bf16 into shared memory as the next
-//               MMA's A operand (K-major, 128-byte swizzle), l = the running sum of those
-//               values;
-//   O_g = P V   V is the B operand in MN-major form (its rows are the keys = the MMA's
-//               K, its columns the head's dims = the MMA's N): one MMA for dims 0..63
-//               and one for the rest, each inside one 64-column swizzle atom; the thread
-//               folds O_g into its running output (registers), rescaled when m grows;
-//   merge       every CTA stores the partial (m, l, O_s) of each row into the shared
-//               memory of the row's owner CTA (distributed shared memory stores); after
-//               a cluster barrier the owner combines them in rank order (deterministic):
-//               M = max m_s,  O = sum_s 2^((m_s - M) c) O_s / sum_s 2^((m_s - M) c) l_s.
-// Incremental calls fetch the cached K/V of the item's view before waiting on the QKV
-// kernel (programmatic dependent launch: reused tokens' keys are final) and afterwards
-// copy only the rows of this call's updated tokens into the swizzled tiles.
+// Bound: the exponentials and the softmax's other arithmetic (one row per thread) at large
+// row counts, the chain K -> S -> softmax -> P V of an item at small ones.  Measured with 16
+// heads of 72 against the kernel before it (one CTA per SM or a cluster splitting the keys,
+// softmax and MMAs in turn, P through shared memory): 32 views x 1024 queries x 1024 keys
+// 690 -> 218 us (709 TFLOP/s), 32 x 96 queries 158 -> 38 us.  Of that, the order of the items
+// (query tiles of a head together, K/V from L2 instead of DRAM) and the narrow second slice
+// took 327 to 218 us.
+//
+// Warps of a CTA:
+//   4      TMA: Q tile of 128 rows, then K and V blocks through a ring of 4 to 7 tiles.  The
+//          maps are [rows][heads][dh]: the columns past a head's dh are out of bounds, zero
+//          in shared memory and not fetched.  Columns 0..63 form one slice with 128-byte
+//          swizzle, the rest (8 of a 72-wide head) a second one as narrow as a swizzle
+//          allows, which leaves room for two more tiles.
+//   5      MMA: S = Q K^T (fp32, tensor memory) of block i+1 is issued before O += P V of
+//          block i, so it runs while block i's softmax finishes; P is read from tensor
+//          memory, V is the B operand in MN-major form.
+//   0 - 3  softmax, thread = query row = tensor-memory lane: S into registers, P = 2^((S - m) c)
+//          (c = log2(e) / sqrt(dh)) rounded to bf16 into tensor memory, l = the sum of those
+//          values.  The reference m is the row's running maximum, moved (and O, l rescaled)
+//          only when a block exceeds it by more than 2^8, which keeps P in bf16's and the
+//          sums in fp32's range; the result does not depend on the reference.  At the end
+//          O / l goes to global memory.
 #include "internal.h"
 #include "ptx.cuh"
 
 namespace ivit {
 namespace {
 
-constexpr int AQ = 128;            // queries per item (MMA M)
-constexpr int AKMAX = 256;         // max keys per CTA (MMA N of S)
-constexpr int KROWS = 64;          // rows of one K/V TMA box
-constexpr int SLICE_Q = AQ * 128;  // [128 rows][128 B]: 16 KB (a Q slice or a 64-key P slice)
-constexpr int QBOX = 32;           // rows of one query TMA box
-constexpr int MAX_SPLITS = 8;
+constexpr int AQ = 128;             // queries per item (MMA M)
+constexpr int THREADS = 192;
+constexpr int MAX_VIEWS = 4096;
+constexpr int SMEM_HALF = 113 * 1024;  // two CTAs share an SM
+constexpr float RESCALE = 8.f;      // log2 of the growth that moves the reference maximum
 
-// Shared-memory and TMEM layout of one CTA for kpc keys and head width dhp (padded to
-// 16), identical on host and device.
-struct AttnLayout {
-  int nt;        // threads per CTA (128 or 256)
-  int nsl;       // 64-column slices per row
-  int kgrp;      // keys per group: the CTA's keys, at most AKMAX (more run in several groups)
-  int kpad;      // keys per group rounded up to 64 (K/V slice rows)
-  int kslice;    // bytes of one K or V slice
-  int rp, pst;   // merge: row slots per owner, row stride of a partial output (floats)
-  int off_q, off_p, off_k, off_v, off_part, off_red, off_bar, bytes;
-  int tm_o, tm_cols;
+template <int DHP>
+struct AttnCfg {
+  static constexpr int KB = attention_key_block(DHP);
+  // A row's columns past 64 form a second slice, as narrow as a swizzle allows.
+  static constexpr int W2 = attention_slice2(DHP);
+  static constexpr int Q1 = AQ * 128, Q2 = AQ * W2 * 2;                // bytes of the slices of Q
+  static constexpr int T1 = KB * 128, TILE = (T1 + KB * W2 * 2 + 1023) / 1024 * 1024;  // of a K or V block
+  static constexpr int T_BYTES = T1 + KB * W2 * 2;
+  static constexpr int TM_O = KB, TM_P = KB + DHP, TM_COLS = 256;      // S at column 0
+  static_assert(TM_P + KB / 2 <= TM_COLS, "tensor memory of one CTA");
+  static constexpr int OFF_RING = Q1 + Q2;
+  static constexpr int RING = (SMEM_HALF - OFF_RING - 1024 - 512) / TILE < 8 ? (SMEM_HALF - OFF_RING - 1024 - 512) / TILE : 8;
+  static constexpr int OFF_BAR = OFF_RING + RING * TILE;
+  static constexpr int OFF_CUM = OFF_BAR + 256;  // [sv + 1] items before each view
+  static constexpr int BYTES = OFF_CUM + 1024;   // alignment slack
 };
-
-// Threads per CTA for kpc keys per CTA: two per query row once a key group holds 128 keys.
-__host__ __device__ inline int attn_threads(int kpc) { return kpc >= 128 ? 2 * AQ : AQ; }
-
-__host__ __device__ inline AttnLayout attn_layout(int kpc, int dhp, int ns) {
-  AttnLayout L;
-  L.nt = attn_threads(kpc);
-  L.nsl = dhp > 64 ? 2 : 1;
-  L.kgrp = kpc < AKMAX ? kpc : AKMAX;
-  L.kpad = (L.kgrp + 63) / 64 * 64;
-  L.kslice = L.kpad * 128;
-  L.rp = (AQ + ns - 1) / ns;
-  L.pst = dhp + 4;
-  L.off_q = 0;
-  L.off_p = L.off_q + L.nsl * SLICE_Q;
-  L.off_k = L.off_p + (L.kpad / 64) * SLICE_Q;
-  L.off_v = L.off_k + L.nsl * L.kslice;
-  L.off_part = L.off_v + L.nsl * L.kslice;
-  const int part = ns > 1 ? ns * L.rp * (L.pst + 2) * 4 : 0;  // O_s, m, l of every slot
-  L.off_red = L.off_part + (part + 1023) / 1024 * 1024;
-  L.off_bar = L.off_red + (L.nt > AQ ? 2 * AQ * 4 : 0);  // row max / sum exchange [2][AQ]
-  L.bytes = L.off_bar + 64 + 1024;  // barriers + TMEM slot, alignment slack
-  L.tm_o = L.kpad;
-  int need = L.kpad + dhp, cols = 32;
-  while (cols < need) cols *= 2;
-  L.tm_cols = cols;
-  return L;
-}
-
-// Byte offset of 16-byte chunk `chunk` (0..7) of row `row` in a slice of 128-byte rows
-// written by TMA with 128-byte swizzle (slice base 1024-byte aligned).
-__device__ __forceinline__ uint32_t swz(int row, int chunk) {
-  return static_cast<uint32_t>(row * 128 + ((chunk ^ (row & 7)) << 4));
-}
 
 struct Item {
   int v, h, r0, nq;
 };
 
-// Item s = (query tile, view, head) with the query tile slowest, so that the first
-// tiles of every (view, head) are spread over the grid first.
-__device__ __forceinline__ bool item_at(int s, const AttnTcArgs& a, Item& it) {
-  const int vh = a.sv * a.heads;
-  const int qt = s / vh, rem = s - qt * vh;
-  it.v = rem / a.heads;
-  it.h = rem - it.v * a.heads;
-  const int rb = a.cu_rows[it.v], m = a.cu_rows[it.v + 1] - rb;
+// Item g of the call: views in order, in a view the heads, in a head the query tiles, so that
+// the tiles that share keys and values run at the same time (their K and V come from L2).
+// cum[v] = items before view v.
+__device__ __forceinline__ Item item_at(int g, const int* cum, const AttnTcArgs& a) {
+  int lo = 0, hi = a.sv - 1;  // last view with cum[view] <= g
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (cum[mid] <= g) lo = mid; else hi = mid - 1;
+  }
+  Item it;
+  it.v = lo;
+  const int rb = a.cu_rows[lo], m = a.cu_rows[lo + 1] - rb;
+  const int tiles = (m + AQ - 1) / AQ, rem = g - cum[lo];
+  it.h = rem / tiles;
+  const int qt = rem - it.h * tiles;
   it.r0 = rb + qt * AQ;
   it.nq = min(AQ, m - qt * AQ);
-  return it.nq > 0;
+  return it;
 }
 
-// 2^x (the softmax's exponentials on logits pre-scaled by log2(e) / sqrt(dh)).
 __device__ __forceinline__ float ex2(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
 
-// Running maximum of the valid entries (index < lim) of a 32-column chunk of S, in four
-// independent accumulators.
-__device__ __forceinline__ void chunk_max(const uint32_t (&r)[32], int lim, float (&mx)[4]) {
-  if (lim >= 32) {
-#pragma unroll
-    for (int u = 0; u < 32; ++u) mx[u & 3] = fmaxf(mx[u & 3], __uint_as_float(r[u]));
-  } else {
-#pragma unroll
-    for (int u = 0; u < 32; ++u)
-      if (u < lim) mx[u & 3] = fmaxf(mx[u & 3], __uint_as_float(r[u]));
-  }
-}
-
-// P = 2^(S c - mo) of a 32-column chunk (0 past lim), rounded to bf16 and stored as the
-// row's 16-byte chunks kc0.. of the P operand (those below gns); lsum gets the rounded
-// values.
-__device__ __forceinline__ void chunk_exp(const uint32_t (&r)[32], int lim, float sc, float mo, uint8_t* sp,
-                                          int row, int kc0, int gns, float (&lsum)[4]) {
-  uint32_t pk[16];
+// 32 columns of S (bits) -> 16 packed bf16 pairs of P; l gets the rounded values.
+__device__ __forceinline__ void exp_chunk(const uint32_t* s, float sc, float mo, uint32_t* pk, float2 (&l)[2]) {
+  const float2 c2 = make_float2(sc, sc), m2 = make_float2(-mo, -mo);
 #pragma unroll
   for (int u = 0; u < 16; ++u) {
-    const int j = 2 * u;
-    const float p0 = j < lim ? ex2(fmaf(__uint_as_float(r[j]), sc, -mo)) : 0.f;
-    const float p1 = j + 1 < lim ? ex2(fmaf(__uint_as_float(r[j + 1]), sc, -mo)) : 0.f;
-    const __nv_bfloat162 b = __floats2bfloat162_rn(p0, p1);
-    const float2 f = __bfloat1622float2(b);
-    lsum[u & 3] += f.x + f.y;  // the normaliser sums the values the MMA multiplies
-    pk[u] = *reinterpret_cast<const uint32_t*>(&b);
-  }
-#pragma unroll
-  for (int q4 = 0; q4 < 4; ++q4) {
-    const int kc = kc0 + q4;  // 16-byte chunk (8 keys) of this row of P
-    if (kc * 8 < gns)
-      *reinterpret_cast<uint4*>(sp + (kc >> 3) * SLICE_Q + swz(row, kc & 7)) =
-          make_uint4(pk[4 * q4], pk[4 * q4 + 1], pk[4 * q4 + 2], pk[4 * q4 + 3]);
+    const float2 t = fma_f32x2(make_float2(__uint_as_float(s[2 * u]), __uint_as_float(s[2 * u + 1])), c2, m2);
+    const __nv_bfloat162 b = __floats2bfloat162_rn(ex2(t.x), ex2(t.y));
+    const uint32_t w = *reinterpret_cast<const uint32_t*>(&b);
+    // (bf16 widens to fp32 by its bits; the normaliser sums the values the MMA multiplies)
+    l[u & 1] = add_f32x2(l[u & 1], make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u)));
+    pk[u] = w;
   }
 }
 
-template <int DHP, int NT>
-__global__ void __launch_bounds__(NT, 1)
+// Shared-memory descriptor of a slice whose rows are W2 columns (and one swizzle span) wide:
+// groups of 8 rows follow each other.  For a K-major operand the rows are its M or N index,
+// for an MN-major one (V) its K index.
+template <int W2>
+__device__ __forceinline__ uint64_t sdesc_rows(uint32_t saddr) {
+  constexpr uint32_t group = 8 * W2 * 2;
+  uint64_t d = sdesc_sw128(saddr, group, group) & ~(static_cast<uint64_t>(7) << 61);
+  return d | (static_cast<uint64_t>(W2 == 16 ? 6 : W2 == 32 ? 4 : 2) << 61);  // 32-, 64-, 128-byte swizzle
+}
+
+template <int DHP>
+__global__ void __launch_bounds__(THREADS, 2)
     attention_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
-                        const __grid_constant__ CUtensorMap tm_v, const AttnTcArgs a) {
-  constexpr int NH = NT / AQ;                       // threads per query row
-  constexpr int OCH = (DHP / 16 + NH - 1) / NH;     // 16-column output chunks per thread
+                        const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_q2,
+                        const __grid_constant__ CUtensorMap tm_k2, const __grid_constant__ CUtensorMap tm_v2,
+                        const AttnTcArgs a) {
+  using C = AttnCfg<DHP>;
+  constexpr int KB = C::KB, RING = C::RING, W2 = C::W2;
   extern __shared__ uint8_t at_raw[];
   uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(at_raw) + 1023) &
                                            ~static_cast<uintptr_t>(1023));
-  const int tid = threadIdx.x, warp = tid >> 5;
-  const int row = tid & (AQ - 1), hf = tid / AQ;  // query row (TMEM lane) and column half
-  const int N = a.n_tok, D = a.dim, dh = a.dh;
-  const int n_items = a.sv * a.heads * a.qtiles;
-  const int ns = static_cast<int>(cluster_nctarank()), rank = static_cast<int>(cluster_ctarank());
-  const int cl = blockIdx.x / ns, ncl = gridDim.x / ns;
-  const int kpc = (N + ns - 1) / ns;
-  const int k0 = rank * kpc, nk = max(0, min(kpc, N - k0));  // this CTA's keys
-  const AttnLayout L = attn_layout(kpc, DHP, ns);
-  const int G = L.kgrp;                                      // keys per group
-  const int ngroups = (nk + G - 1) / G;
-  const int NSL = L.nsl;
-  const uint32_t sb = smem_u32(sm);
-  const uint32_t bq = sb + L.off_bar, bk = bq + 8, bv = bq + 16, bs = bq + 24, bo = bq + 32;
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(sm + L.off_bar + 40);
-  // merge slots of the rows this CTA owns: O_s [ns][rp][pst], then m [ns][rp], l [ns][rp]
-  float* po = reinterpret_cast<float*>(sm + L.off_part);
-  float* pm = po + ns * L.rp * L.pst;
-  float* pl = pm + ns * L.rp;
-  float* red = reinterpret_cast<float*>(sm + L.off_red);  // [NH][AQ] partial row max / sum
-
-  // The row offsets come from the selection kernel, at least two launches back (every
-  // kernel of the library triggers its dependents only after its own wait).  Every CTA
-  // of a cluster walks the same items, so a cluster leaves as a whole.
-  int s = cl;
-  Item it;
-  while (s < n_items && !item_at(s, a, it)) s += ncl;
-  if (s >= n_items) return;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int N = a.n_tok;
+  const int nb = (N + KB - 1) / KB;  // key blocks of an item
+  const uint32_t sb = smem_u32(sm), bar = sb + C::OFF_BAR;
+  const uint32_t q_full = bar, q_empty = bar + 8, s_full = bar + 16, s_free = bar + 24, p_ready = bar + 32,
+                 o_done = bar + 40, o_free = bar + 48, t_full = bar + 56, t_empty = t_full + 8 * RING;
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(sm + C::OFF_BAR + 56 + 16 * RING);
+  volatile int* sh_abort = reinterpret_cast<volatile int*>(tslot + 1);
+  int* cum = reinterpret_cast<int*>(sm + C::OFF_CUM);
 
   if (tid == 0) {
-    mbar_init(bq, 1);
-    mbar_init(bk, 1);
-    mbar_init(bv, 1);
-    mbar_init(bs, 1);
-    mbar_init(bo, 1);
+    mbar_init(q_full, 1);
+    mbar_init(q_empty, 1);
+    mbar_init(s_full, 1);
+    mbar_init(s_free, 4);
+    mbar_init(p_ready, 4);
+    mbar_init(o_done, 1);
+    mbar_init(o_free, 4);
+    for (int i = 0; i < RING; ++i) {
+      mbar_init(t_full + 8 * i, 1);
+      mbar_init(t_empty + 8 * i, 1);
+    }
     fence_mbar_init();
     tma_prefetch_desc(&tm_q);
     tma_prefetch_desc(&tm_k);
     tma_prefetch_desc(&tm_v);
+    if (W2 > 0) {
+      tma_prefetch_desc(&tm_q2);
+      tma_prefetch_desc(&tm_k2);
+      tma_prefetch_desc(&tm_v2);
+    }
+    *sh_abort = 0;
   }
+  // The row offsets come from the selection kernel, at least two launches back (every kernel
+  // of the library triggers its dependents only after its own wait).
   if (warp == 0) {
-    tmem_alloc(smem_u32(tslot), static_cast<uint32_t>(L.tm_cols));
+    int before = 0;
+    for (int v0 = 0; v0 < a.sv; v0 += 32) {
+      const int v = v0 + lane;
+      int n = v < a.sv ? (a.cu_rows[v + 1] - a.cu_rows[v] + AQ - 1) / AQ * a.heads : 0;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int up = __shfl_up_sync(0xffffffffu, n, o);
+        if (lane >= o) n += up;
+      }
+      if (v < a.sv) cum[v + 1] = before + n;
+      before += __shfl_sync(0xffffffffu, n, 31);
+    }
+    if (lane == 0) cum[0] = 0;
+  }
+  if (warp == 5) {
+    tmem_alloc(smem_u32(tslot), C::TM_COLS);
     tmem_relinquish();
   }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tslot;
-  const uint32_t trow = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16);
-  const uint32_t tm_s = tmem, tm_o = tmem + static_cast<uint32_t>(L.tm_o);
-  const uint64_t pol_q = l2_policy_evict_first(), pol_kv = l2_policy_evict_last();
 
-  // K or V of key group g of this CTA's keys of item (v, h): boxes of 64 keys x 64 dims
-  // per slice.
-  auto load_kv = [&](uint32_t bar, int off, const CUtensorMap* map, int v, int h, int g) {
-    const int gk0 = k0 + g * G, gn = min(G, nk - g * G);
-    const int nbox = (gn + KROWS - 1) / KROWS;
-    mbar_arrive_expect_tx(bar, static_cast<uint32_t>(nbox * NSL * KROWS * 128));
-    for (int sl = 0; sl < NSL; ++sl)
-      for (int b = 0; b < nbox; ++b)
-        tma_load_2d(sb + off + sl * L.kslice + b * KROWS * 128, map, h * dh + sl * 64, v * N + gk0 + b * KROWS,
-                    bar, pol_kv);
-  };
-
-  // Incremental calls whose keys fit one group fetch the cached K/V before the wait.
-  const bool pre = a.prefetch && ngroups == 1;
-  if (pre && tid == 0) {
-    load_kv(bk, L.off_k, &tm_k, it.v, it.h, 0);
-    load_kv(bv, L.off_v, &tm_v, it.v, it.h, 0);
-  }
   pdl_wait();  // queries and this call's K/V rows (QKV kernel) are visible from here
   pdl_launch_dependents();
   stamp_begin(a.stamp);
 
-  uint32_t ph_q = 0, ph_g = 0;  // completed phases: bq once per item, the others once per group
-  bool ok = true;
-  const float sc = rsqrtf(static_cast<float>(dh)) * 1.4426950408889634f;  // log2(e) / sqrt(dh)
-  bool first = true;
-  while (true) {
-    const bool patch = first && pre;
-    first = false;
-    if (tid == 0) {
-      // only the 32-row boxes that hold the item's queries (rows past them are never stored)
-      const int nqb = (it.nq + QBOX - 1) / QBOX;
-      mbar_arrive_expect_tx(bq, static_cast<uint32_t>(NSL * nqb * QBOX * 128));
-      for (int sl = 0; sl < NSL; ++sl)
-        for (int b = 0; b < nqb; ++b)
-          tma_load_2d(sb + L.off_q + sl * SLICE_Q + b * QBOX * 128, &tm_q, it.h * dh + sl * 64, it.r0 + b * QBOX, bq,
-                      pol_q);
-      if (!patch && ngroups > 0) {
-        load_kv(bk, L.off_k, &tm_k, it.v, it.h, 0);
-        load_kv(bv, L.off_v, &tm_v, it.v, it.h, 0);
-      }
-    }
-    if (patch) {
-      // the prefetched tiles hold the cache as it was before the QKV kernel: overwrite
-      // the rows of the tokens it updated that fall in this CTA's key range
-      if (!mbar_wait(bk, ph_g & 1) || !mbar_wait(bv, ph_g & 1)) ok = false;
-      const int rb = a.cu_rows[it.v], m = a.cu_rows[it.v + 1] - rb;
-      const int dh8 = dh >> 3;
-      for (int e = tid; e < m * dh8; e += blockDim.x) {
-        const int r = e / dh8, c = e - r * dh8;
-        const int j = a.rowtok[rb + r] - it.v * N - k0;
-        if (j < 0 || j >= nk) continue;
-        const size_t g = (static_cast<size_t>(it.v) * N + k0 + j) * D + it.h * dh + c * 8;
-        const uint32_t off = (c >> 3) * L.kslice + swz(j, c & 7);
-        *reinterpret_cast<uint4*>(sm + L.off_k + off) = __ldcg(reinterpret_cast<const uint4*>(a.cache_k + g));
-        *reinterpret_cast<uint4*>(sm + L.off_v + off) = __ldcg(reinterpret_cast<const uint4*>(a.cache_v + g));
-      }
-    }
-    if (!mbar_wait(bq, ph_q & 1)) ok = false;
-    ++ph_q;
-    if (DHP != dh && tid < AQ) {  // columns dh..dh+7 of the Q tile hold the next head: zero them
-      const int c = dh >> 3;
-      *reinterpret_cast<uint4*>(sm + L.off_q + (c >> 3) * SLICE_Q + swz(tid, c & 7)) = make_uint4(0, 0, 0, 0);
-    }
-    fence_proxy_async_shared();
-    tc_fence_before();
-    __syncthreads();
+  // Every wait is bounded; after one has expired no role waits again and all leave.
+  auto wait = [&](uint32_t b, uint32_t parity) {
+    if (*sh_abort) return false;
+    if (mbar_wait(b, parity)) return true;
+    atomicExch(a.err, kErrWaitTmaFull);
+    *sh_abort = 1;
+    return false;
+  };
 
-    // Online softmax over the key groups (running max m, running sum l, output in
-    // registers rescaled by 2^((m_old - m_new) c) when the max grows).
-    const bool wrow = (warp & 3) * 32 < it.nq;  // warp-uniform: padding warps skip the math
-    float m_run = -INFINITY, l_run = 0.f;       // l_run: this thread's columns only
-    float o_run[OCH * 16];                      // chunks hf, hf + NH, ... of the output row
-#pragma unroll
-    for (int d = 0; d < OCH * 16; ++d) o_run[d] = 0.f;
-    for (int g = 0; g < ngroups; ++g) {
-      const int gn = min(G, nk - g * G), gns = (gn + 15) & ~15;
-      // ---- S = Q K^T
-      if (tid == 0) {
-        tc_fence_after();
-        if (!mbar_wait(bk, ph_g & 1)) ok = false;
-        tc_fence_after();
-        if (ok) {
-          const uint32_t id = idesc_bf16_f32(AQ, gns);
-#pragma unroll
-          for (int t = 0; t < DHP / 16; ++t) {
-            const uint32_t qo = sb + L.off_q + (t >> 2) * SLICE_Q + (t & 3) * 32;
-            const uint32_t ko = sb + L.off_k + (t >> 2) * L.kslice + (t & 3) * 32;
-            umma_bf16(tm_s, sdesc_kmajor_sw128(qo), sdesc_kmajor_sw128(ko), id, t > 0);
-          }
-        }
-        umma_commit(bs);
+  const int n_items = cum[a.sv];
+  int s = blockIdx.x;
+  if (warp == 4) {
+    const uint64_t pol_q = l2_policy_evict_first(), pol_kv = l2_policy_evict_last();
+    uint32_t t = 0;  // K / V tiles so far
+    for (uint32_t n = 0; s < n_items; ++n, s += gridDim.x) {
+      const Item it = item_at(s, cum, a);
+      if (!__all_sync(0xffffffffu, wait(q_empty, (n & 1) ^ 1))) break;
+      if (elect_one()) {
+        mbar_arrive_expect_tx(q_full, C::Q1 + C::Q2);
+        tma_load_3d(sb, &tm_q, 0, it.h, it.r0, q_full, pol_q);
+        if (W2 > 0) tma_load_3d(sb + C::Q1, &tm_q2, 64, it.h, it.r0, q_full, pol_q);
       }
       __syncwarp();
-      if (!mbar_wait(bs, ph_g & 1)) ok = false;
-      tc_fence_after();
-      if (tid == 0 && g + 1 < ngroups) load_kv(bk, L.off_k, &tm_k, it.v, it.h, g + 1);  // K tile consumed
-
-      // ---- softmax of the group, P to shared memory.  This thread's 32-column chunks of
-      // S are cb = 32 hf, 32 (hf + NH), ...; two TMEM loads are in flight at a time.
-      float alpha = 1.f;
-      float mpart = -INFINITY;
-      if (wrow) {
-        float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-        for (int cb = 32 * hf; cb < gns; cb += 64 * NH) {
-          const int cb1 = cb + 32 * NH;
-          uint32_t r0[32], r1[32];
-          tmem_ld32_async(trow + cb, r0);
-          if (cb1 < gns) tmem_ld32_async(trow + cb1, r1);
-          tmem_ld_wait_regs(r0);
-          chunk_max(r0, gn - cb, mx);
-          if (cb1 < gns) {
-            tmem_ld_wait_regs(r1);
-            chunk_max(r1, gn - cb1, mx);
-          }
+      bool ok = true;
+      for (int i = 0; i < 2 * nb && ok; ++i, ++t) {  // K and V of block i / 2
+        const uint32_t slot = t % RING;
+        ok = __all_sync(0xffffffffu, wait(t_empty + 8 * slot, ((t / RING) & 1) ^ 1));
+        if (ok && elect_one()) {
+          const uint32_t dst = sb + C::OFF_RING + slot * C::TILE, full = t_full + 8 * slot;
+          const int row = it.v * N + (i >> 1) * KB;
+          mbar_arrive_expect_tx(full, C::T_BYTES);
+          tma_load_3d(dst, (i & 1) ? &tm_v : &tm_k, 0, it.h, row, full, pol_kv);
+          if (W2 > 0) tma_load_3d(dst + C::T1, (i & 1) ? &tm_v2 : &tm_k2, 64, it.h, row, full, pol_kv);
         }
-        mpart = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
+        __syncwarp();
       }
-      if (NH > 1) {  // the row's maximum over both halves' columns
-        red[hf * AQ + row] = mpart;
-        __syncthreads();
-        mpart = fmaxf(mpart, red[(hf ^ 1) * AQ + row]);
-      }
-      if (wrow) {
-        const float m_new = fmaxf(m_run, mpart);
-        alpha = ex2((m_run - m_new) * sc);  // 0 on the first group (m_run = -inf)
-        const float mo = m_new * sc;
-        float lsum[4] = {0.f, 0.f, 0.f, 0.f};
-        if constexpr (NH > 1) {
-          uint32_t ra[32], rb[32];
-          int cb = 32 * hf;
-          if (cb < gns) {
-            tmem_ld32_async(trow + cb, ra);
-            tmem_ld_wait_regs(ra);
+      if (!ok) break;
+    }
+  } else if (warp == 5) {
+    uint32_t j0 = 0;  // key blocks of the earlier items
+    bool ok = true;
+    for (uint32_t n = 0; ok && s < n_items; ++n, s += gridDim.x, j0 += nb) {
+      ok = __all_sync(0xffffffffu, wait(q_full, n & 1));
+      for (int i = 0; i <= nb && ok; ++i) {
+        if (i < nb) {  // S of block i
+          const uint32_t j = j0 + i, t = 2 * j, slot = t % RING;
+          ok = __all_sync(0xffffffffu, wait(t_full + 8 * slot, (t / RING) & 1) && wait(s_free, (j & 1) ^ 1));
+          if (!ok) break;
+          tc_fence_after();
+          const uint32_t id = idesc_bf16_f32(AQ, (min(KB, N - i * KB) + 15) & ~15);
+          if (elect_one()) {
+            const uint32_t kt = sb + C::OFF_RING + slot * C::TILE;
+#pragma unroll
+            for (int u = 0; u < DHP / 16; ++u)
+              umma_bf16(tmem,
+                        u < 4 ? sdesc_kmajor_sw128(sb + u * 32) : sdesc_rows<W2>(sb + C::Q1 + (u - 4) * 32),
+                        u < 4 ? sdesc_kmajor_sw128(kt + u * 32) : sdesc_rows<W2>(kt + C::T1 + (u - 4) * 32), id, u > 0);
+            umma_commit(t_empty + 8 * slot);
+            umma_commit(s_full);
+            if (i == nb - 1) umma_commit(q_empty);
           }
-          while (cb < gns) {  // chunk cb is in ra; the next one loads while it is used
-            const int cn = cb + 32 * NH;
-            if (cn < gns) tmem_ld32_async(trow + cn, rb);
-            chunk_exp(ra, gn - cb, sc, mo, sm + L.off_p, row, cb >> 3, gns, lsum);
-            if (cn >= gns) break;
-            tmem_ld_wait_regs(rb);
-            const int cn2 = cn + 32 * NH;
-            if (cn2 < gns) tmem_ld32_async(trow + cn2, ra);
-            chunk_exp(rb, gn - cn, sc, mo, sm + L.off_p, row, cn >> 3, gns, lsum);
-            if (cn2 >= gns) break;
-            tmem_ld_wait_regs(ra);
-            cb = cn2;
-          }
-        } else {  // one thread per row holds the whole output row: one chunk at a time
-          for (int cb = 0; cb < gns; cb += 32) {
-            uint32_t r[32];
-            tmem_ld32_async(trow + cb, r);
-            tmem_ld_wait_regs(r);
-            chunk_exp(r, gn - cb, sc, mo, sm + L.off_p, row, cb >> 3, gns, lsum);
-          }
+          __syncwarp();
         }
-        l_run = l_run * alpha + ((lsum[0] + lsum[1]) + (lsum[2] + lsum[3]));
-        m_run = m_new;
-      }
-      fence_proxy_async_shared();
-      tc_fence_before();
-      __syncthreads();
-
-      // ---- O_g = P V, folded into the running output
-      if (tid == 0) {
-        tc_fence_after();
-        if (!mbar_wait(bv, ph_g & 1)) ok = false;
-        tc_fence_after();
-        if (ok) {
-          const uint32_t id0 = idesc_bf16_f32_bmn(AQ, DHP > 64 ? 64 : DHP);
-          const uint32_t id1 = idesc_bf16_f32_bmn(AQ, DHP > 64 ? DHP - 64 : 16);
-          for (int t = 0; t < gns / 16; ++t) {
-            const uint64_t ad = sdesc_kmajor_sw128(sb + L.off_p + (t >> 2) * SLICE_Q + (t & 3) * 32);
-            umma_bf16(tm_o, ad, sdesc_sw128(sb + L.off_v + t * 2048, 1024, 1024), id0, t > 0);
-            if (DHP > 64)
-              umma_bf16(tm_o + 64, ad, sdesc_sw128(sb + L.off_v + L.kslice + t * 2048, 1024, 1024), id1, t > 0);
-          }
-        }
-        umma_commit(bo);
-      }
-      __syncwarp();
-      if (!mbar_wait(bo, ph_g & 1)) ok = false;
-      tc_fence_after();
-      ++ph_g;
-      if (tid == 0 && g + 1 < ngroups) load_kv(bv, L.off_v, &tm_v, it.v, it.h, g + 1);  // V tile consumed
-      if (wrow) {  // warp-uniform: tcgen05.ld is a warp-collective instruction
-        // two chunks' loads in flight per wait (one for the widest heads with two threads
-        // per row, whose registers are otherwise spent)
-        constexpr int OB = (DHP >= 112 && NH > 1) ? 1 : 2;
-#pragma unroll
-        for (int q = 0; q < OCH; q += OB) {
-          uint32_t ov[OB][16];
-#pragma unroll
-          for (int t = 0; t < OB; ++t)
-            if (q + t < OCH && (hf + (q + t) * NH) * 16 < DHP)
-              tmem_ld16_async(trow + L.tm_o + (hf + (q + t) * NH) * 16, ov[t]);
-          tmem_ld_wait();
-#pragma unroll
-          for (int t = 0; t < OB; ++t) {
-            tmem_regs_after_wait16(ov[t]);
-            if (q + t < OCH && (hf + (q + t) * NH) * 16 < DHP) {
-#pragma unroll
-              for (int u = 0; u < 16; ++u)
-                o_run[(q + t) * 16 + u] = o_run[(q + t) * 16 + u] * alpha + __uint_as_float(ov[t][u]);
+        if (i > 0) {  // O += P V of block i - 1
+          const uint32_t j = j0 + i - 1, t = 2 * j + 1, slot = t % RING;
+          ok = __all_sync(0xffffffffu, wait(t_full + 8 * slot, (t / RING) & 1) && wait(p_ready, j & 1) &&
+                                           (i > 1 || wait(o_free, (n & 1) ^ 1)));
+          if (!ok) break;
+          tc_fence_after();
+          const int steps = (min(KB, N - (i - 1) * KB) + 15) >> 4;
+          if (elect_one()) {
+            const uint32_t vt = sb + C::OFF_RING + slot * C::TILE;
+            const uint32_t id0 = idesc_bf16_f32_bmn(AQ, DHP > 64 ? 64 : DHP);
+            const uint32_t id1 = idesc_bf16_f32_bmn(AQ, DHP > 64 ? DHP - 64 : 16);
+            for (int u = 0; u < steps; ++u) {
+              const uint32_t acc = (i > 1 || u > 0) ? 1u : 0u;
+              umma_bf16_ts(tmem + C::TM_O, tmem + C::TM_P + u * 8, sdesc_sw128(vt + u * 2048, 1024, 1024), id0, acc);
+              if (DHP > 64)
+                umma_bf16_ts(tmem + C::TM_O + 64, tmem + C::TM_P + u * 8,
+                             sdesc_rows<W2>(vt + C::T1 + u * 32 * W2), id1, acc);
             }
+            umma_commit(t_empty + 8 * slot);
+            umma_commit(o_done);
           }
+          __syncwarp();
         }
       }
     }
-
-    // next item of this cluster (the same for every rank)
-    int s_next = s + ncl;
-    Item nxt;
-    while (s_next < n_items && !item_at(s_next, a, nxt)) s_next += ncl;
-
-    if (NH > 1) {  // the row's sum over both halves' columns (the same order on both)
-      red[hf * AQ + row] = l_run;
-      __syncthreads();
-      const float lo_ = red[row], hi_ = red[AQ + row];
-      l_run = lo_ + hi_;
-    }
-    if (ns == 1) {
-      if (wrow && row < it.nq) {
-        const float inv = 1.f / l_run;
-        bf16* orow = a.o + static_cast<size_t>(it.r0 + row) * D + it.h * dh;
+  } else {
+    const uint32_t trow = tmem + (static_cast<uint32_t>(warp * 32) << 16);
+    const float sc = rsqrtf(static_cast<float>(a.dh)) * 1.4426950408889634f;  // log2(e) / sqrt(dh)
+    uint32_t j = 0;  // key blocks so far
+    bool ok = true;
+    auto arrive = [&](uint32_t b) {
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(b);
+    };
+    for (; ok && s < n_items; s += gridDim.x) {
+      const Item it = item_at(s, cum, a);
+      const bool wrow = warp * 32 < it.nq;  // warp-uniform: a warp of padding rows only keeps step
+      float m_ref = -INFINITY;
+      float2 l[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+      for (int i = 0; i < nb; ++i, ++j) {
+        if (!(ok = __all_sync(0xffffffffu, wait(s_full, j & 1)))) break;
+        tc_fence_after();
+        if (!wrow) {
+          arrive(s_free);
+          if (!(ok = __all_sync(0xffffffffu, j == 0 || wait(o_done, (j & 1) ^ 1)))) break;
+          arrive(p_ready);
+          continue;
+        }
+        uint32_t r[KB];
 #pragma unroll
-        for (int q = 0; q < OCH; ++q) {
+        for (int c = 0; c < KB; c += 32) tmem_ld32_async(trow + c, *reinterpret_cast<uint32_t(*)[32]>(r + c));
+#pragma unroll
+        for (int c = 0; c < KB; c += 32) tmem_ld_wait_regs(*reinterpret_cast<uint32_t(*)[32]>(r + c));
+        arrive(s_free);
+        const int gn = N - i * KB;
+        if (gn < KB) {
+#pragma unroll
+          for (int c = 0; c < KB; ++c)
+            if (c >= gn) r[c] = 0xff800000u;  // -inf: P = 0
+        }
+        float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+        for (int c = 0; c < KB; ++c) mx[c & 3] = fmaxf(mx[c & 3], __uint_as_float(r[c]));
+        const float m_blk = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
+        float alpha = 1.f;
+        const bool grow = i > 0 && (m_blk - m_ref) * sc > RESCALE;
+        if (i == 0 || grow) {
+          alpha = ex2((m_ref - m_blk) * sc);
+          m_ref = m_blk;
+        }
+        const float mo = m_ref * sc;
+        const bool rescale = __any_sync(0xffffffffu, grow);
+        if (rescale) {
+#pragma unroll
+          for (int e = 0; e < 2; ++e) {
+            l[e].x *= alpha;
+            l[e].y *= alpha;
+          }
+        }
+        uint32_t pk[KB / 2];
+#pragma unroll
+        for (int c = 0; c < KB; c += 32) exp_chunk(r + c, sc, mo, pk + c / 2, l);
+        // P and O are free once the previous block's (or item's) P V has run
+        if (!(ok = __all_sync(0xffffffffu, j == 0 || wait(o_done, (j & 1) ^ 1)))) break;
+        tc_fence_after();
+        if (rescale) {
+#pragma unroll
+          for (int d = 0; d < DHP; d += 16) {
+            uint32_t o[16];
+            tmem_ld16_async(trow + C::TM_O + d, o);
+            tmem_ld_wait();
+            tmem_regs_after_wait16(o);
+#pragma unroll
+            for (int e = 0; e < 16; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
+            tmem_st16(trow + C::TM_O + d, o);
+          }
+        }
+#pragma unroll
+        for (int c = 0; c < KB / 2; c += 16) tmem_st16(trow + C::TM_P + c, pk + c);
+        tmem_st_wait();
+        arrive(p_ready);
+      }
+      if (!ok || !(ok = __all_sync(0xffffffffu, wait(o_done, (j & 1) ^ 1)))) break;
+      tc_fence_after();
+      if (wrow) {
+        const float inv = 1.f / ((l[0].x + l[0].y) + (l[1].x + l[1].y));
+        const int row = warp * 32 + lane;
+        bf16* orow = a.o + static_cast<size_t>(it.r0 + row) * a.dim + it.h * a.dh;
+#pragma unroll
+        for (int d = 0; d < DHP; d += 16) {
+          uint32_t o[16];
+          tmem_ld16_async(trow + C::TM_O + d, o);
+          tmem_ld_wait();
+          tmem_regs_after_wait16(o);
 #pragma unroll
           for (int h8 = 0; h8 < 16; h8 += 8) {
-            const int c = (hf + q * NH) * 16 + h8;
-            if (c < dh) {
-              uint4 u;
-              uint32_t* w = reinterpret_cast<uint32_t*>(&u);
+            uint4 u;
+            uint32_t* w = reinterpret_cast<uint32_t*>(&u);
 #pragma unroll
-              for (int e = 0; e < 4; ++e) {
-                const __nv_bfloat162 b = __floats2bfloat162_rn(o_run[q * 16 + h8 + 2 * e] * inv,
-                                                               o_run[q * 16 + h8 + 2 * e + 1] * inv);
-                w[e] = *reinterpret_cast<const uint32_t*>(&b);
-              }
-              *reinterpret_cast<uint4*>(orow + c) = u;
+            for (int e = 0; e < 4; ++e) {
+              const __nv_bfloat162 b = __floats2bfloat162_rn(__uint_as_float(o[h8 + 2 * e]) * inv,
+                                                             __uint_as_float(o[h8 + 2 * e + 1]) * inv);
+              w[e] = *reinterpret_cast<const uint32_t*>(&b);
             }
+            if (row < it.nq && d + h8 < a.dh) *reinterpret_cast<uint4*>(orow + d + h8) = u;
           }
         }
       }
-    } else {
-      // push this CTA's partial (m, l, O_s) of row i to slot [rank][i - owner * rpi] of
-      // the owner CTA i / rpi; a CTA without keys pushes m = -inf, l = 0, O = 0
-      const int rpi = (it.nq + ns - 1) / ns;  // rows per owner in this item (<= rp)
-      if (row < it.nq) {
-        const int owner = row / rpi, slot = row - owner * rpi;
-        const uint32_t obase =
-            mapa_shared(smem_u32(po + (rank * L.rp + slot) * L.pst), static_cast<uint32_t>(owner));
-#pragma unroll
-        for (int q = 0; q < OCH; ++q) {
-          const int c0 = (hf + q * NH) * 16;
-          if (c0 < DHP) {
-#pragma unroll
-            for (int c = 0; c < 16; c += 4)
-              st_dsmem_f32x4(obase + 4 * (c0 + c), make_float4(o_run[q * 16 + c], o_run[q * 16 + c + 1],
-                                                               o_run[q * 16 + c + 2], o_run[q * 16 + c + 3]));
-          }
-        }
-        if (hf == 0) {
-          st_dsmem_f32(mapa_shared(smem_u32(pm + rank * L.rp + slot), static_cast<uint32_t>(owner)), m_run);
-          st_dsmem_f32(mapa_shared(smem_u32(pl + rank * L.rp + slot), static_cast<uint32_t>(owner)), l_run);
-        }
-      }
-      cluster_sync();  // every rank's partials of this CTA's rows are in its shared memory
-      const int lo = rank * rpi, nmine = max(0, min(it.nq, lo + rpi) - lo);
-      constexpr int C8 = DHP / 8;
-      for (int e = tid; e < nmine * C8; e += blockDim.x) {
-        const int sl = e / C8, c = e - sl * C8;
-        if (c * 8 >= dh) continue;
-        float M = -INFINITY;
-#pragma unroll
-        for (int q = 0; q < MAX_SPLITS; ++q)
-          if (q < ns) M = fmaxf(M, pm[q * L.rp + sl]);
-        float Lsum = 0.f, acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-        for (int q = 0; q < MAX_SPLITS; ++q) {
-          if (q < ns) {
-            const float w = ex2((pm[q * L.rp + sl] - M) * sc);  // m = -inf (no keys): w = 0
-            Lsum += w * pl[q * L.rp + sl];
-            const float4 x0 = *reinterpret_cast<const float4*>(po + (q * L.rp + sl) * L.pst + c * 8);
-            const float4 x1 = *reinterpret_cast<const float4*>(po + (q * L.rp + sl) * L.pst + c * 8 + 4);
-            acc[0] += w * x0.x;
-            acc[1] += w * x0.y;
-            acc[2] += w * x0.z;
-            acc[3] += w * x0.w;
-            acc[4] += w * x1.x;
-            acc[5] += w * x1.y;
-            acc[6] += w * x1.z;
-            acc[7] += w * x1.w;
-          }
-        }
-        const float inv = 1.f / Lsum;
-        uint4 u;
-        uint32_t* w = reinterpret_cast<uint32_t*>(&u);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const __nv_bfloat162 b = __floats2bfloat162_rn(acc[2 * q] * inv, acc[2 * q + 1] * inv);
-          w[q] = *reinterpret_cast<const uint32_t*>(&b);
-        }
-        *reinterpret_cast<uint4*>(a.o + static_cast<size_t>(it.r0 + lo + sl) * D + it.h * dh + c * 8) = u;
-      }
-      if (s_next < n_items) cluster_sync();  // slots are read before the next item's pushes
+      arrive(o_free);
     }
-    tc_fence_before();
-    __syncthreads();  // Q, P and TMEM are reused by the next item
-
-    if (s_next >= n_items) break;
-    s = s_next;
-    it = nxt;
   }
-
-  if (!ok) atomicExch(a.err, kErrWaitTmaFull);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  if (warp == 0) tmem_dealloc(tmem, static_cast<uint32_t>(L.tm_cols));
+  if (warp == 5) tmem_dealloc(tmem, C::TM_COLS);
   stamp_end(a.stamp);
-}
-
-template <int DHP>
-cudaError_t launch_dhp(const CUtensorMap& tm_q, const CUtensorMap& tm_k, const CUtensorMap& tm_v,
-                       const AttnTcArgs& a, int grid, int smem, int nt, cudaStream_t s) {
-  if (nt > AQ)
-    return launch_ex(attention_tc_kernel<DHP, 2 * AQ>, dim3(grid), dim3(nt), static_cast<size_t>(smem), s,
-                     static_cast<unsigned>(a.key_splits), tm_q, tm_k, tm_v, a);
-  return launch_ex(attention_tc_kernel<DHP, AQ>, dim3(grid), dim3(nt), static_cast<size_t>(smem), s,
-                   static_cast<unsigned>(a.key_splits), tm_q, tm_k, tm_v, a);
-}
-
-// The device's opt-in limit of dynamic shared memory per block (0 when unknown).
-int smem_optin() {
-  int dev = 0, v = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
-  if (cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) return 0;
-  return v;
 }
 
 }  // namespace
 
-int attention_tc_kv_box_rows() { return KROWS; }
-
-size_t attention_tc_smem(int n_tok, int dh, int key_splits) {
-  const int kpc = (n_tok + key_splits - 1) / key_splits;
-  return static_cast<size_t>(attn_layout(kpc, (dh + 15) & ~15, key_splits).bytes);
-}
-
 cudaError_t attention_tc_setup() {
-  const int max_bytes = smem_optin();
-  if (max_bytes <= 0) return cudaErrorInvalidDevice;
   cudaError_t e = cudaSuccess;
-  auto set = [&](auto kern) {
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, max_bytes);
+  auto set = [&](auto kern, int bytes) {
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes + 4 * (MAX_VIEWS + 1));
   };
-  set(attention_tc_kernel<16, AQ>);
-  set(attention_tc_kernel<16, 2 * AQ>);
-  set(attention_tc_kernel<32, AQ>);
-  set(attention_tc_kernel<32, 2 * AQ>);
-  set(attention_tc_kernel<48, AQ>);
-  set(attention_tc_kernel<48, 2 * AQ>);
-  set(attention_tc_kernel<64, AQ>);
-  set(attention_tc_kernel<64, 2 * AQ>);
-  set(attention_tc_kernel<80, AQ>);
-  set(attention_tc_kernel<80, 2 * AQ>);
-  set(attention_tc_kernel<96, AQ>);
-  set(attention_tc_kernel<96, 2 * AQ>);
-  set(attention_tc_kernel<112, AQ>);
-  set(attention_tc_kernel<112, 2 * AQ>);
-  set(attention_tc_kernel<128, AQ>);
-  set(attention_tc_kernel<128, 2 * AQ>);
+  set(attention_tc_kernel<16>, AttnCfg<16>::BYTES);
+  set(attention_tc_kernel<32>, AttnCfg<32>::BYTES);
+  set(attention_tc_kernel<48>, AttnCfg<48>::BYTES);
+  set(attention_tc_kernel<64>, AttnCfg<64>::BYTES);
+  set(attention_tc_kernel<80>, AttnCfg<80>::BYTES);
+  set(attention_tc_kernel<96>, AttnCfg<96>::BYTES);
+  set(attention_tc_kernel<112>, AttnCfg<112>::BYTES);
+  set(attention_tc_kernel<128>, AttnCfg<128>::BYTES);
   return e;
 }
 
-cudaError_t launch_attention_tc(const CUtensorMap& tm_q, const CUtensorMap& tm_k, const CUtensorMap& tm_v,
-                                const AttnTcArgs& a, int max_ctas, cudaStream_t s) {
-  const int ns = a.key_splits;
-  if (ns < 1 || ns > MAX_SPLITS) return cudaErrorInvalidValue;
-  const int items = a.sv * a.heads * a.qtiles;
-  const int clusters = max(1, min(items, max_ctas / ns));
-  const int grid = clusters * ns;
-  const int smem = static_cast<int>(attention_tc_smem(a.n_tok, a.dh, ns));
-  if (smem > smem_optin()) return cudaErrorInvalidValue;
-  const int nt = attn_threads((a.n_tok + ns - 1) / ns);
+cudaError_t launch_attention_tc(const AttnMaps& q, const AttnMaps& k, const AttnMaps& v, const AttnTcArgs& a,
+                                int num_sms, cudaStream_t s) {
+  if (a.sv > MAX_VIEWS) return cudaErrorInvalidValue;
+  const int grid = max(1, min(a.sv * a.heads * ((a.n_tok + AQ - 1) / AQ), 2 * num_sms));
+  auto launch = [&](auto kern, size_t bytes) {
+    return launch_ex(kern, dim3(grid), dim3(THREADS), bytes + 4 * (a.sv + 1), s, 1, q.lo, k.lo, v.lo, q.hi, k.hi, v.hi,
+                     a);
+  };
   switch ((a.dh + 15) & ~15) {
-    case 16: return launch_dhp<16>(tm_q, tm_k, tm_v, a, grid, smem, nt, s);
-    case 32: return launch_dhp<32>(tm_q, tm_k, tm_v, a, grid, smem, nt, s);
-    case 48: return launch_dhp<48>(tm_q, tm_k, tm_v, a, grid, smem, nt, s);
-    case 64: return launch_dhp<64>(tm_q, tm_k, tm_v, a, grid, smem, nt, s);
-    case 80: return launch_dhp<80>(tm_q, tm_k, tm_v, a, grid, smem, nt, s);
-    case 96: return launch_dhp<96>(tm_q, tm_k, tm_v, a, grid, smem, nt, s);
-    case 112: return launch_dhp<112>(tm_q, tm_k, tm_v, a, grid, smem, nt, s);
-    case 128: return launch_dhp<128>(tm_q, tm_k, tm_v, a, grid, smem, nt, s);
+    case 16: return launch(attention_tc_kernel<16>, AttnCfg<16>::BYTES);
+    case 32: return launch(attention_tc_kernel<32>, AttnCfg<32>::BYTES);
+    case 48: return launch(attention_tc_kernel<48>, AttnCfg<48>::BYTES);
+    case 64: return launch(attention_tc_kernel<64>, AttnCfg<64>::BYTES);
+    case 80: return launch(attention_tc_kernel<80>, AttnCfg<80>::BYTES);
+    case 96: return launch(attention_tc_kernel<96>, AttnCfg<96>::BYTES);
+    case 112: return launch(attention_tc_kernel<112>, AttnCfg<112>::BYTES);
+    case 128: return launch(attention_tc_kernel<128>, AttnCfg<128>::BYTES);
     default: return cudaErrorInvalidValue;
   }
 }

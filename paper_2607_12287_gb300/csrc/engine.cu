@@ -27,7 +27,7 @@ struct LayerW {
   float *bqkv, *bo, *b1, *b2, *ln1g, *ln1b, *ln2g, *ln2b;
   CUtensorMap tm_qkv, tm_o, tm_1, tm_2;
   CUtensorMap tm_ck, tm_cv;  // this layer's key / value cache, SIMT attention key-split tiles
-  CUtensorMap tm_ak, tm_av;  // the same caches, 64 x 128 boxes, 128-byte swizzle (tcgen05)
+  ivit::AttnMaps tm_ak, tm_av;  // the same caches for the tcgen05 attention
 };
 
 // Kernel families of the timeline.
@@ -86,6 +86,29 @@ bool make_map(CUtensorMap* m, const void* base, uint64_t inner, uint64_t rows, u
              CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// The attention's maps of a [rows][heads][dh] array, boxes of box_rows rows.
+bool make_attn_maps(ivit::AttnMaps* m, const void* base, uint64_t dh, uint64_t heads, uint64_t rows,
+                    uint32_t box_rows) {
+  auto enc = tensor_map_encoder();
+  if (!enc) return false;
+  auto make = [&](CUtensorMap* map, uint32_t cols) {
+    cuuint64_t dims[3] = {dh, heads, rows};
+    cuuint64_t strides[2] = {dh * 2, dh * heads * 2};
+    cuuint32_t box[3] = {cols, 1, box_rows};
+    cuuint32_t estr[3] = {1, 1, 1};
+    const auto swizzle = cols == 64   ? CU_TENSOR_MAP_SWIZZLE_128B
+                         : cols == 32 ? CU_TENSOR_MAP_SWIZZLE_64B
+                                      : CU_TENSOR_MAP_SWIZZLE_32B;
+    return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+  };
+  const int hi = ivit::attention_slice2(static_cast<int>((dh + 15) & ~15ull));
+  if (!make(&m->lo, 64)) return false;
+  m->hi = m->lo;
+  return hi == 0 || make(&m->hi, static_cast<uint32_t>(hi));
+}
+
 // Bump allocator over one device allocation; every sub-buffer 256-byte aligned.
 struct Arena {
   size_t size = 0;
@@ -120,13 +143,12 @@ struct ivit_handle {
   int device = 0, num_sms = 0;
   int row_grid = 0;
   GemmPlan plan_full[kGemmSlots], plan_inc[kGemmSlots], plan_keys;
-  // Row-count bands of the incremental graph (band 0 = plan_inc): launch plans and
-  // attention key splits made for at most band_ub[b] updated rows; a switch node picks
-  // the band of each call's device-resident row count.
+  // Row-count bands of the incremental graph (band 0 = plan_inc): launch plans made for at
+  // most band_ub[b] updated rows; a switch node picks the band of each call's device-resident
+  // row count.
   int n_bands = 1;
   int band_ub[4] = {0, 0, 0, 0};
   GemmPlan plan_band[4][kGemmSlots];
-  int attn_splits_band[4] = {1, 1, 1, 1};
   bool capture_bands = false;  // set while the incremental graph is captured with bands
   int known_band = -1;         // set while it is captured for a row count known in advance
   ivit::RowBands bands;        // the switch node's handle and the bands' row bounds
@@ -139,9 +161,8 @@ struct ivit_handle {
   std::vector<LayerW> layers;
   CUtensorMap tm_pe;
   ActMaps tm_patches, tm_xn, tm_o, tm_h;
-  CUtensorMap tm_qa;     // packed queries, 64 x 32 boxes, 128-byte swizzle (tcgen05 attention)
+  ivit::AttnMaps tm_qa;  // packed queries (tcgen05 attention)
   bool attn_tc = true;   // tensor-core attention (IVIT_ATTN=simt selects the SIMT kernel)
-  int attn_splits_full = 1, attn_splits_inc = 1;  // key splits (CTAs per item) of that kernel
 
   bf16* patches = nullptr;
   float *e_t = nullptr, *e_ref = nullptr, *sims = nullptr, *x = nullptr;
@@ -562,30 +583,6 @@ int setup(ivit_handle* h, const uint16_t* wb) {
     }
     if (std::getenv("IVIT_NO_BANDS")) h->n_bands = 1;
   }
-  {
-    // Key splits of the tensor-core attention: as many as fill the SMs once for the
-    // expected items (query tiles x heads x views: all tokens when full, a tenth when
-    // incremental), at least 64 keys per CTA, one (online softmax over key groups) when
-    // the items alone fill the GPU; more while one CTA's shared memory exceeds the limit.
-    int optin = 0;
-    IVIT_CK(h, cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device));
-    const int dh = h->D / h->H;
-    auto splits = [&](int m_exp) {
-      const int ns_cap = std::max(1, std::min(8, (h->N + 63) / 64));  // at least 64 keys per CTA
-      const int items = h->SV * h->H * ((m_exp + 127) / 128);
-      int ns = std::max(1, std::min(ns_cap, h->num_sms / std::max(1, items)));
-      if (const char* e = std::getenv("IVIT_ATTN_SPLITS")) ns = std::max(1, std::min(8, std::atoi(e)));
-      while (ns < 8 && ivit::attention_tc_smem(h->N, dh, ns) > static_cast<size_t>(optin)) ++ns;
-      return ns;
-    };
-    h->attn_splits_full = splits(h->N);
-    h->attn_splits_inc = splits(std::max(1, h->N / 10));
-    h->attn_splits_band[0] = h->attn_splits_inc;
-    for (int b = 1; b < h->n_bands; ++b) h->attn_splits_band[b] = splits(std::max(1, h->band_ub[b] / h->SV));
-    if (ivit::attention_tc_smem(h->N, dh, h->attn_splits_full) > static_cast<size_t>(optin) ||
-        ivit::attention_tc_smem(h->N, dh, h->attn_splits_inc) > static_cast<size_t>(optin))
-      h->attn_tc = false;  // not reachable for N <= 1024, dh <= 128
-  }
   if (std::getenv("IVIT_NO_PDL")) ivit::g_use_pdl = false;
   if (std::getenv("IVIT_NO_GRAPH")) h->use_graphs = false;
   IVIT_CK(h, cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking));
@@ -607,7 +604,7 @@ int setup(ivit_handle* h, const uint16_t* wb) {
       h->plan_full[g] = plan(m_all, m_all);
       h->plan_inc[g] = g == kGemmEmbed ? h->plan_full[g] : plan(m_inc, m_all);
       h->plan_band[0][g] = h->plan_inc[g];
-      // (the band of all rows runs the full encode's plans: it attends like one too)
+      // (the band of all rows runs the full encode's plans)
       for (int b = 1; b < h->n_bands; ++b)
         h->plan_band[b][g] = g == kGemmEmbed || h->band_ub[b] >= m_all ? h->plan_full[g]
                                                                        : plan(h->band_ub[b], h->band_ub[b]);
@@ -625,8 +622,6 @@ int setup(ivit_handle* h, const uint16_t* wb) {
         show("inc", names[g], h->plan_inc[g]);
         for (int b = 1; b < h->n_bands; ++b) show(b == 1 ? "band 1" : b == 2 ? "band 2" : "band 3", names[g], h->plan_band[b][g]);
       }
-      for (int b = 1; b < h->n_bands; ++b)
-        std::fprintf(stderr, "ivit band %d (<= %d rows): attention splits %d\n", b, h->band_ub[b], h->attn_splits_band[b]);
     }
   }
 
@@ -779,12 +774,13 @@ int setup(ivit_handle* h, const uint16_t* wb) {
   h->frames_buf = sa.at<uint8_t>(o_fb);
   h->counts_buf = sa.at<int>(o_cb);
   const int kps = ivit::attention_keys_per_split(h->N);
+  const int dh = h->D / h->H, kb = ivit::attention_key_block((dh + 15) & ~15);
   for (size_t l = 0; l < L; ++l) {
     const size_t off = l * M * D;
     if (!make_map(&h->layers[l].tm_ck, h->cacheK + off, D, M, D * 2, D / h->H, kps, false) ||
         !make_map(&h->layers[l].tm_cv, h->cacheV + off, D, M, D * 2, D / h->H, kps, false) ||
-        !make_map(&h->layers[l].tm_ak, h->cacheK + off, D, M, D * 2, 64, ivit::attention_tc_kv_box_rows()) ||
-        !make_map(&h->layers[l].tm_av, h->cacheV + off, D, M, D * 2, 64, ivit::attention_tc_kv_box_rows()))
+        !make_attn_maps(&h->layers[l].tm_ak, h->cacheK + off, dh, h->H, M, kb) ||
+        !make_attn_maps(&h->layers[l].tm_av, h->cacheV + off, dh, h->H, M, kb))
       return h->fail(IVIT_ERR_CUDA, "cuTensorMapEncodeTiled failed for a cache tile");
   }
   auto act_maps = [&](ActMaps& m, const bf16* base, size_t inner) {
@@ -792,7 +788,7 @@ int setup(ivit_handle* h, const uint16_t* wb) {
            make_map(&m.b128, base, inner, M, inner * 2, 64, 128);
   };
   if (!act_maps(h->tm_patches, h->patches, h->KPAD) || !act_maps(h->tm_xn, h->xn, D) || !act_maps(h->tm_o, h->o, D) ||
-      !act_maps(h->tm_h, h->hbuf, F) || !make_map(&h->tm_qa, h->q, D, M, D * 2, 64, 32))
+      !act_maps(h->tm_h, h->hbuf, F) || !make_attn_maps(&h->tm_qa, h->q, dh, h->H, M, 128))
     return h->fail(IVIT_ERR_CUDA, "cuTensorMapEncodeTiled failed for an activation buffer");
   if (int r = setup_persistent(h)) return r;
   if (int r = setup_stream(h)) return r;
@@ -939,15 +935,11 @@ void print_stream_trace(ivit_handle* h, cudaStream_t s) {
 }
 
 // Attention of the updated queries over all tokens of their view for one layer.
-int attention(ivit_handle* h, const LayerW& w, const bf16* ck, const bf16* cv, bool full, cudaStream_t s,
-              int key_splits = 0) {
+int attention(ivit_handle* h, const LayerW& w, const bf16* ck, const bf16* cv, bool full, cudaStream_t s) {
   const int N = h->N, D = h->D, SV = h->SV;
   if (h->attn_tc) {
     ivit::AttnTcArgs at;
-    at.cache_k = ck;
-    at.cache_v = cv;
     at.cu_rows = h->cu_rows;
-    at.rowtok = h->rowtok;
     at.o = h->o;
     at.err = h->err;
     at.n_tok = N;
@@ -955,9 +947,6 @@ int attention(ivit_handle* h, const LayerW& w, const bf16* ck, const bf16* cv, b
     at.dh = D / h->H;
     at.heads = h->H;
     at.sv = SV;
-    at.qtiles = (N + 127) / 128;
-    at.prefetch = full ? 0 : 1;
-    at.key_splits = key_splits > 0 ? key_splits : (full ? h->attn_splits_full : h->attn_splits_inc);
     next_launch(h, kFamAttn);
     at.stamp = ivit::g_stamp;
     IVIT_CK(h, ivit::launch_attention_tc(h->tm_qa, w.tm_ak, w.tm_av, at, h->num_sms, s));
@@ -1055,8 +1044,8 @@ int run_layers_mlp_all(ivit_handle* h, const GemmPlan* plan, bool full, cudaStre
 
 // Per layer {LN1, QKV + K/V cache scatter (Eq. 4-5), attention, out-proj + residual,
 // LN2, MLP up + GELU, MLP down + residual}, then the final LN scattered into the
-// final-token cache, with the given launch plans and attention key splits.
-int run_layers(ivit_handle* h, const GemmPlan* plan, int attn_splits, bool full, cudaStream_t s) {
+// final-token cache, with the given launch plans.
+int run_layers(ivit_handle* h, const GemmPlan* plan, bool full, cudaStream_t s) {
   const ivit_config& c = h->cfg;
   const int D = h->D, F = h->F, SV = h->SV, M = h->M_max;
   const int* total = h->cu_rows + SV;
@@ -1114,7 +1103,7 @@ int run_layers(ivit_handle* h, const GemmPlan* plan, int attn_splits, bool full,
       a.epi.dim = D;
       if (int r = gemm(h, plan[kGemmQKV], w.tm_qkv, h->tm_xn, a, s)) return r;
     }
-    if (int r = attention(h, w, ck, cv, full, s, attn_splits)) return r;
+    if (int r = attention(h, w, ck, cv, full, s)) return r;
     if (int r = residual(plan[kGemmO], w.bo, w.tm_o, h->tm_o, D)) return r;
     if (int r = layernorm(w.ln2g, w.ln2b, h->xn, nullptr)) return r;
     {
@@ -1157,8 +1146,7 @@ int capture_band_bodies(ivit_handle* h, cudaStream_t s) {
     h->launches = pre;
     IVIT_CK(h, cudaStreamBeginCaptureToGraph(h->cap_stream2, np.conditional.phGraph_out[b], nullptr, nullptr, 0,
                                              cudaStreamCaptureModeThreadLocal));
-    // (the band of every row attends like a full encode: no cached-K/V prefetch to patch)
-    const int r = run_layers(h, h->plan_band[b], h->attn_splits_band[b], h->band_ub[b] >= h->M_max, h->cap_stream2);
+    const int r = run_layers(h, h->plan_band[b], h->band_ub[b] >= h->M_max, h->cap_stream2);
     cudaGraph_t body = nullptr;
     const cudaError_t e = cudaStreamEndCapture(h->cap_stream2, &body);
     if (r) return r;
@@ -1285,9 +1273,8 @@ int run_core(ivit_handle* h, const uint8_t* frames, int32_t* user_counts, bool f
   }
   if (h->capture_bands) return capture_band_bodies(h, s);
   if (!full && h->known_band >= 0)  // top-k: the row count is fixed, so is its band
-    return run_layers(h, h->plan_band[h->known_band], h->attn_splits_band[h->known_band],
-                      h->band_ub[h->known_band] >= h->M_max, s);
-  return run_layers(h, plan, full ? h->attn_splits_full : h->attn_splits_inc, full, s);
+    return run_layers(h, h->plan_band[h->known_band], h->band_ub[h->known_band] >= h->M_max, s);
+  return run_layers(h, plan, full, s);
 }
 
 int capture_once(ivit_handle* h, bool full, cudaGraphExec_t* exec, int64_t* launches);

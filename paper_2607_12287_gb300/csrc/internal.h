@@ -267,38 +267,34 @@ cudaError_t launch_attention(const CUtensorMap& tm_k, const CUtensorMap& tm_v, c
 
 // ----------------------------------------------------------- attention (tcgen05)
 struct AttnTcArgs {
-  const bf16* cache_k = nullptr;  // this layer's key cache, bf16 [SV*N][D] (token-major)
-  const bf16* cache_v = nullptr;  // this layer's value cache, same layout
-  const int* cu_rows = nullptr;   // [SV+1] packed-row offsets of the views' updated rows
-  const int* rowtok = nullptr;    // packed row -> token v*N + i
-  bf16* o = nullptr;              // [rows][D] attention output, packed rows
-  int* err = nullptr;             // device error word
+  const int* cu_rows = nullptr;  // [SV+1] packed-row offsets of the views' updated rows
+  bf16* o = nullptr;             // [rows][D] attention output, packed rows
+  int* err = nullptr;            // device error word
   int n_tok = 0, dim = 0, dh = 0, heads = 0, sv = 0;
-  int qtiles = 0;                 // query tiles of 128 rows per (view, head): ceil(N / 128)
-  int key_splits = 1;             // CTAs per cluster splitting the keys (1..8, N/splits <= 256)
-  int prefetch = 0;               // 1: cached K/V loaded before the wait, then the updated
-                                  //    rows re-read (incremental calls)
   unsigned long long* stamp = nullptr;  // timeline stamps of this launch (or null)
 };
 
 // One-time function attributes of the tensor-core attention kernel.
 cudaError_t attention_tc_setup();
 
-// Rows of the K/V TMA box the tensor-core attention kernel expects (the tensor maps of
-// the caches use box 64 columns x this many rows).
-int attention_tc_kv_box_rows();
+// Keys per block for a head width padded to 16: the widest whose S (a column per key), P (half
+// a column) and O (dhp columns) fit in 256 tensor-memory columns.
+constexpr int attention_key_block(int dhp) { return dhp <= 64 ? 128 : dhp <= 80 ? 96 : 64; }
+// Columns of the second slice of a row, past the first 64 (0: none): one swizzle span wide.
+constexpr int attention_slice2(int dhp) { return dhp <= 64 ? 0 : dhp <= 80 ? 16 : dhp <= 96 ? 32 : 64; }
 
-// Dynamic shared memory of one tensor-core attention CTA for N keys split key_splits ways.
-size_t attention_tc_smem(int n_tok, int dh, int key_splits);
+// TMA maps of a [rows][H][dh] array for the attention: boxes of 1 head x 128 rows (queries) or
+// attention_key_block rows (caches), `lo` of 64 columns with 128-byte swizzle, `hi` (when
+// attention_slice2 > 0) of that many columns with a swizzle span of their size.
+struct AttnMaps {
+  CUtensorMap lo, hi;
+};
 
 // O[r] = softmax(Q[r] K_v^T / sqrt(dh)) V_v per head on the tensor cores, for the packed
-// query rows r of each view v, over the N cached keys/values of that view.  tm_q: the
-// packed queries bf16 [rows][D] with box 64 columns x 32 rows; tm_k / tm_v: this
-// layer's caches bf16 [SV*N][D] with box 64 columns x attention_tc_kv_box_rows(); all
-// three with 128-byte swizzle.  Grid: clusters of
-// key_splits CTAs (128 threads each), at most max_ctas CTAs, walking the (query tile,
-// view, head) items.
-cudaError_t launch_attention_tc(const CUtensorMap& tm_q, const CUtensorMap& tm_k, const CUtensorMap& tm_v,
-                                const AttnTcArgs& a, int max_ctas, cudaStream_t s);
+// query rows r of each view v, over the N cached keys/values of that view (q, k, v: the packed
+// queries, this layer's caches [SV*N]).  Two CTAs per SM walk the (view, head, query tile)
+// items.  At most 4096 views.
+cudaError_t launch_attention_tc(const AttnMaps& q, const AttnMaps& k, const AttnMaps& v, const AttnTcArgs& a,
+                                int num_sms, cudaStream_t s);
 
 }  // namespace ivit
