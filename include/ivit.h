@@ -163,13 +163,11 @@ int ivit_timeline_read(ivit_handle* h, void* stream, double* family_ms, int64_t*
  * wait expired, the kernel skipped its work and returned).  Synchronises `stream`. */
 int ivit_device_status(ivit_handle* h, void* stream);
 
-/* Execution paths (chosen at create; the environment variable IVIT_PATH=kernels,
- * IVIT_PATH=persistent or IVIT_PATH=stream selects one): one kernel per operation,
- * chained with programmatic dependent launch and replayed as a CUDA graph (every
- * incremental call, and the full encodes for dim > 384); every transformer block of a
- * call in one persistent cooperative kernel with grid barriers (the full encodes for
- * dim <= 384, where per-operation launches dominate); or, on request only
- * (IVIT_PATH=stream), the incremental calls without cold views in one cooperative
+/* Execution paths: one kernel per operation, chained with programmatic dependent launch
+ * and replayed as a CUDA graph, is what every call runs.  On request (environment
+ * variable IVIT_PATH read at create): IVIT_PATH=persistent, every transformer block of a
+ * call in one persistent cooperative kernel with grid barriers (at most 256 tokens per
+ * view); IVIT_PATH=stream, the incremental calls without cold views in one cooperative
  * weight-streaming kernel that keeps each SM's share of the next weights in flight
  * through a shared-memory ring.  All give the same result within the bf16 rounding. */
 

@@ -181,12 +181,8 @@ struct ivit_handle {
   std::vector<uint8_t> cold;
   int64_t launches = 0;
 
-  // Persistent encoder (all blocks in one cooperative launch) for small encoders: it runs
-  // the full encodes; incremental calls run it only when forced (persistent_inc), since
-  // the kernel chain is faster for a few updated rows (its tensor-core attention against
-  // the persistent kernel's SIMT attention phase).
+  // Persistent encoder (all blocks in one cooperative launch), on request.
   bool persistent = false;
-  bool persistent_inc = false;
   size_t pt_smem = 0;
   int pt_grid = 0;
   void* pt_mem = nullptr;  // device: tensor maps, layer parameters, partials, barrier words
@@ -291,7 +287,9 @@ size_t defer_slots(const GemmPlan& pl, int n_out, int m_bound) {
 //   Deferred (residual GEMMs, allow_defer): K split over plain CTAs or pairs whose partial
 //     tiles the next layer norm sums: no barrier and no epilogue, but every split's fp32
 //     tile is written and read once (about 4 TB/s through L2).
-GemmPlan plan_gemm(int num_sms, int n_out, int k, int m_expected, int m_bound, bool allow_defer) {
+// fit_clusters[c]: clusters of c CTAs of the split kernel that fit on the GPU at once.
+GemmPlan plan_gemm(int num_sms, const int* fit_clusters, int n_out, int k, int m_expected, int m_bound,
+                   bool allow_defer) {
   GemmPlan best;
   double best_cost = 1e30;
   auto consider = [&](const GemmPlan& pl, double cost) {
@@ -331,7 +329,7 @@ GemmPlan plan_gemm(int num_sms, int n_out, int k, int m_expected, int m_bound, b
       const int rounds = (tiles * c + num_sms - 1) / num_sms;
       if (fits(pl)) consider(pl, rounds * (4.0 + 0.35 * ((n_kb + c - 1) / c)) + partial_cost(c));
     } else {
-      const int fit = ivit::gemm_max_clusters(c);
+      const int fit = fit_clusters[c];
       if (fit <= 0) continue;
       pl.n_clusters = std::max(1, std::min({tiles, fit, num_sms / c}));
       const int rounds = (tiles + pl.n_clusters - 1) / pl.n_clusters;
@@ -341,17 +339,15 @@ GemmPlan plan_gemm(int num_sms, int n_out, int k, int m_expected, int m_bound, b
   return best;
 }
 
-// Prepares the persistent encoder when its shared memory fits (attention keeps a whole
-// view's keys and values of one head resident, so N * head_dim is bounded).
+// Prepares the persistent encoder (IVIT_PATH=persistent: every call runs it) when its shared
+// memory fits (attention keeps a whole view's keys and values of one head resident, so
+// N * head_dim is bounded).  It is not the default anywhere: its SIMT attention phase and
+// 64-row GEMM tiles lose to the kernel chain also on the full encodes of small encoders
+// (six 196-token views of ViT-Tiny 1.40 ms against 0.43 ms for the chain).
 int setup_persistent(ivit_handle* h) {
-  // IVIT_PATH=kernels / IVIT_PATH=persistent (every call) override the choice made from
-  // the shape.  Default: the full encodes of small encoders (dim <= 384), whose
-  // per-layer kernels are launch-bound at every row of every view.
   const char* path = std::getenv("IVIT_PATH");
-  if (path && std::strcmp(path, "kernels") == 0) return IVIT_OK;
+  if (!path || std::strcmp(path, "persistent") != 0) return IVIT_OK;
   if (h->cfg.mlp_tokens == IVIT_MLP_ALL) return IVIT_OK;  // the kernel chain runs that reading
-  const bool forced = path && std::strcmp(path, "persistent") == 0;
-  if (!forced && h->D > 384) return IVIT_OK;
   const int dh = h->D / h->H;
   const size_t smem = ivit::persistent_smem_bytes(h->N, dh);
   if (smem > 227 * 1024 || h->D > 2048 || h->N > 256) return IVIT_OK;
@@ -432,7 +428,6 @@ int setup_persistent(ivit_handle* h) {
   h->pt_smem = smem;
   h->pt_grid = grid;
   h->persistent = true;
-  h->persistent_inc = forced;
   return IVIT_OK;
 }
 
@@ -592,6 +587,8 @@ int setup(ivit_handle* h, const uint16_t* wb) {
     // Full encodes know M = SV*N.  Incremental calls are planned for a tenth of the
     // tokens updated (any count still runs correctly, with more or fewer tile rounds).
     const int m_all = static_cast<int>(M), m_inc = std::max(1, m_all / 10);
+    int fit[17] = {};
+    for (int c = 2; c <= 16; ++c) fit[c] = ivit::gemm_max_clusters(c);
     const int shapes[kGemmSlots][2] = {{static_cast<int>(D), h->KPAD}, {3 * static_cast<int>(D), static_cast<int>(D)},
                                        {static_cast<int>(D), static_cast<int>(D)}, {static_cast<int>(F), static_cast<int>(D)},
                                        {static_cast<int>(D), static_cast<int>(F)}};
@@ -599,7 +596,7 @@ int setup(ivit_handle* h, const uint16_t* wb) {
       // (under the MLP-on-all-tokens reading the residual epilogues feed no layer norm of the same rows)
       const bool defer = (g == kGemmO || g == kGemmDown) && c.mlp_tokens == IVIT_MLP_UPDATED;
       auto plan = [&](int m_expected, int m_bound) {
-        return plan_gemm(h->num_sms, shapes[g][0], shapes[g][1], m_expected, m_bound, defer);
+        return plan_gemm(h->num_sms, fit, shapes[g][0], shapes[g][1], m_expected, m_bound, defer);
       };
       h->plan_full[g] = plan(m_all, m_all);
       h->plan_inc[g] = g == kGemmEmbed ? h->plan_full[g] : plan(m_inc, m_all);
@@ -610,7 +607,7 @@ int setup(ivit_handle* h, const uint16_t* wb) {
                                                                        : plan(h->band_ub[b], h->band_ub[b]);
     }
     // every row's D x D projection without a residual (first-layer key scores)
-    h->plan_keys = plan_gemm(h->num_sms, static_cast<int>(D), static_cast<int>(D), m_all, m_all, false);
+    h->plan_keys = plan_gemm(h->num_sms, fit, static_cast<int>(D), static_cast<int>(D), m_all, m_all, false);
     if (std::getenv("IVIT_DEBUG")) {
       static const char* names[kGemmSlots] = {"embed", "qkv", "out", "up", "down"};
       auto show = [&](const char* when, const char* name, const GemmPlan& pl) {
@@ -1260,7 +1257,7 @@ int run_core(ivit_handle* h, const uint8_t* frames, int32_t* user_counts, bool f
     }
     return IVIT_OK;
   }
-  if (h->persistent && (full || h->persistent_inc)) {
+  if (h->persistent) {
     IVIT_CK(h, cudaMemsetAsync(h->pt_args.gbar, 0, 4 * sizeof(unsigned), s));
     IVIT_CK(h, ivit::launch_persistent(h->pt_args, h->pt_grid, h->pt_smem, s));
     ++h->launches;
@@ -1283,7 +1280,7 @@ int capture_once(ivit_handle* h, bool full, cudaGraphExec_t* exec, int64_t* laun
 // bands when there are several; if that capture fails the plain graph (band 0's plans
 // for every row count) is captured instead.
 int capture(ivit_handle* h, bool full, cudaGraphExec_t* exec, int64_t* launches) {
-  const bool chain = h->cfg.mlp_tokens == IVIT_MLP_UPDATED && !h->stream_ok && !h->persistent_inc;
+  const bool chain = h->cfg.mlp_tokens == IVIT_MLP_UPDATED && !h->stream_ok && !h->persistent;
   if (!full && chain && h->n_bands > 1 && h->cfg.select_mode == IVIT_SEL_TOPK) {
     // top-k (no cold view in a captured call): exactly k rows per view, so the band is
     // known when the graph is captured and no switch is needed
