@@ -39,19 +39,19 @@ struct TimelineSlot {
   int m_static = -1;               // GEMM rows when fixed, -1 when read from the device
 };
 
-// Launch shape of one GEMM.  Over CTA pairs (`pair`): tiles of bn rows, K split csize ways
-// (more than one only when deferred), n_clusters pairs.  Else: tiles of bn = 64 rows, K split
-// over clusters of csize CTAs (n_clusters of them), or over csize plain CTAs when deferred.
+// Launch shape of one GEMM.  Over CTA pairs (nt = 0): tiles of bn rows, walked by n_pairs
+// pairs.  Else the few-row kernel: CTAs of 8 nt features, passes of bn = 32 rows.  K is split
+// `splits` ways, more than one only when deferred.
 struct GemmPlan {
-  bool pair = false;
-  int bn = 64, csize = 1, n_clusters = 1;
+  int nt = 0, bn = 64, splits = 1, n_pairs = 1;
   bool defer = false;  // residual GEMMs: leave the split partials to the next layer norm
 };
 
-// TMA maps of one activation buffer with boxes of 64 columns x 32, 64 and 128 rows.
+// One activation buffer: its TMA maps with boxes of 64 columns x 32, 64 and 128 rows.
 struct ActMaps {
+  const bf16* base = nullptr;
   CUtensorMap b32, b64, b128;
-  const CUtensorMap& of(const GemmPlan& pl) const { return !pl.pair || pl.bn == 64 ? b32 : pl.bn == 128 ? b64 : b128; }
+  const CUtensorMap& of(const GemmPlan& pl) const { return pl.bn <= 64 ? b32 : pl.bn == 128 ? b64 : b128; }
 };
 
 enum GemmSlot { kGemmEmbed = 0, kGemmQKV, kGemmO, kGemmUp, kGemmDown, kGemmSlots };
@@ -168,7 +168,7 @@ struct ivit_handle {
   float *e_t = nullptr, *e_ref = nullptr, *sims = nullptr, *x = nullptr;
   float* key_t = nullptr;          // first-layer keys of every token (score_source KEY0)
   float* acache = nullptr;         // [L][M_max][D] attention-block outputs (mlp_tokens ALL)
-  float* gemm_partials = nullptr;  // split-K exchange slots of the GEMMs (global scratch)
+  float* gemm_partials = nullptr;  // split-K partial tiles of the deferred GEMMs (global scratch)
   int* rowtok_all = nullptr;       // identity row -> token map, all SV*N rows
   int* m_all = nullptr;            // device copy of SV*N
   CUtensorMap tm_wk0;              // layer 0's key projection (rows D..2D-1 of W_qkv)
@@ -270,70 +270,64 @@ size_t weights_count(const ivit_config* c) {
 
 // Scratch slots (fp32 [bn][128]) a deferred plan needs for up to m_bound rows.
 size_t defer_slots(const GemmPlan& pl, int n_out, int m_bound) {
-  return static_cast<size_t>((n_out + 127) / 128) * ((m_bound + pl.bn - 1) / pl.bn) * pl.csize;
+  return static_cast<size_t>((n_out + 127) / 128) * ((m_bound + pl.bn - 1) / pl.bn) * pl.splits;
 }
 
 // Launch shape of a GEMM expected to see m_expected rows (and at most m_bound): the
 // cheapest candidate of a cost model in microseconds per launch, fitted to back-to-back
-// launches on GB300 of the SigLIP-So400m shapes at 26 to 32768 rows.
+// launches on GB300 of the SigLIP-So400m and ViT-Tiny shapes at 16 to 32768 rows.
 //   CTA pairs: a fixed part (prologue, first loads, last tile's epilogue) plus a k-block
 //     (64 wide) rate per round of units over the 76 pairs; 64-, 128- and 256-row tiles
 //     measured 4.3 / 4.8 / 6.2 us + 0.20 / 0.24 / 0.33 us per k-block, and 0.7 us for the
 //     prologue that its shared memory keeps from running under the previous kernel.
-//   K split over clusters of 64-row tiles: 5.8 us + 0.35 us per 16 KB weight stage per
-//     round; it wins up to about 64 rows, where a pair tile's whole K on few SMs is longer
-//     (QKV of 26 rows: 6.9 us in clusters of 5 against 7.9).  Clusters above 9 lose SMs to
-//     GPC packing.
-//   Deferred (residual GEMMs, allow_defer): K split over plain CTAs or pairs whose partial
-//     tiles the next layer norm sums: no barrier and no epilogue, but every split's fp32
-//     tile is written and read once (about 4 TB/s through L2).
-// fit_clusters[c]: clusters of c CTAs of the split kernel that fit on the GPU at once.
-GemmPlan plan_gemm(int num_sms, const int* fit_clusters, int n_out, int k, int m_expected, int m_bound,
-                   bool allow_defer) {
+//   Few rows (`few`: the epilogues that kernel has): 1.1 us, then per pass of 32 rows and
+//     round of CTAs over the SMs 0.9 us and 0.15 to 0.36 us per chunk (32 wide) of a warp for 8
+//     to 32 features per CTA.  QKV of 26 rows 4.0 us against 7.9 in pairs, of 64 rows 6.6
+//     against 7.9, of 128 rows 11.1 against 7.9.
+//   Deferred (residual GEMMs, `defer`): the next layer norm sums the partial tiles: no
+//     epilogue, but every split's fp32 tile is written and read once (about 4 TB/s through L2).
+GemmPlan plan_gemm(int num_sms, int n_out, int k, int m_expected, int m_bound, bool few, bool defer) {
   GemmPlan best;
   double best_cost = 1e30;
+  defer = defer && !std::getenv("IVIT_NO_DEFER");
   auto consider = [&](const GemmPlan& pl, double cost) {
+    if (pl.defer) {
+      if (defer_slots(pl, n_out, m_bound) * pl.bn * 128 * 4 > (64ull << 20)) return;
+      cost += pl.splits * (8.0 * n_out) * m_expected / 4.0e6;
+    }
     if (cost < best_cost - 1e-9) {
       best_cost = cost;
       best = pl;
     }
   };
-  allow_defer = allow_defer && !std::getenv("IVIT_NO_DEFER");
   const int n_ft = (n_out + 127) / 128, n_kb = (k + 63) / 64, max_pairs = num_sms / 2;
-  auto partial_cost = [&](int c) { return c * (8.0 * n_out) * m_expected / 4.0e6; };
-  auto fits = [&](const GemmPlan& pl) {
-    return defer_slots(pl, n_out, m_bound) * pl.bn * 128 * 4 <= (64ull << 20);
-  };
   for (int bn : {64, 128, 256}) {
     const double fixed = bn == 64 ? 5.0 : bn == 128 ? 5.5 : 6.9, per_kb = bn == 64 ? 0.20 : bn == 128 ? 0.24 : 0.33;
     const int tiles = std::max(1, (n_ft + 1) / 2 * ((m_expected + bn - 1) / bn));
-    for (int c = 1; c <= std::min(allow_defer ? 16 : 1, n_kb); ++c) {
+    for (int c = 1; c <= std::min(defer ? 16 : 1, n_kb); ++c) {
       GemmPlan pl;
-      pl.pair = true;
       pl.bn = bn;
-      pl.csize = c;
+      pl.splits = c;
       pl.defer = c > 1;
       // (a call may bring more rows than expected: the launch is as wide as m_bound can use)
-      pl.n_clusters = std::min(max_pairs, (n_ft + 1) / 2 * ((m_bound + bn - 1) / bn) * c);
+      pl.n_pairs = std::min(max_pairs, (n_ft + 1) / 2 * ((m_bound + bn - 1) / bn) * c);
       const int rounds = (tiles * c + max_pairs - 1) / max_pairs;
-      if (!pl.defer || fits(pl)) consider(pl, fixed + rounds * per_kb * ((n_kb + c - 1) / c) + (c > 1 ? partial_cost(c) : 0));
+      consider(pl, fixed + rounds * per_kb * ((n_kb + c - 1) / c));
     }
   }
-  const int tiles = std::max(1, n_ft * ((m_expected + 63) / 64));
-  for (int c = 2; c <= std::min(16, n_kb); ++c) {
-    GemmPlan pl;
-    pl.csize = c;
-    if (allow_defer) {
-      pl.defer = true;
-      pl.n_clusters = tiles;
-      const int rounds = (tiles * c + num_sms - 1) / num_sms;
-      if (fits(pl)) consider(pl, rounds * (4.0 + 0.35 * ((n_kb + c - 1) / c)) + partial_cost(c));
-    } else {
-      const int fit = fit_clusters[c];
-      if (fit <= 0) continue;
-      pl.n_clusters = std::max(1, std::min({tiles, fit, num_sms / c}));
-      const int rounds = (tiles + pl.n_clusters - 1) / pl.n_clusters;
-      consider(pl, rounds * (4.0 + 0.35 * ((n_kb + c - 1) / c)) + 1.8);
+  if (!few) return best;
+  const int n_ck = (k + 31) / 32, passes = std::max(1, (m_expected + 31) / 32);
+  for (int nt = 1; nt <= 4; ++nt) {
+    for (int c = 1; c <= std::min(defer ? 16 : 1, n_ck); ++c) {
+      GemmPlan pl;
+      pl.nt = nt;
+      pl.bn = 32;
+      pl.splits = c;
+      pl.defer = c > 1;
+      if (ivit::gemm_rows_smem(nt, k, c) > ivit::GEMM_ROWS_SMEM_MAX) continue;
+      const int ctas = (n_out + 8 * nt - 1) / (8 * nt) * c, rounds = (ctas + num_sms - 1) / num_sms;
+      const int per_warp = ((n_ck + c - 1) / c + 7) / 8;
+      consider(pl, 1.1 + passes * rounds * (0.9 + per_warp * (0.08 + 0.07 * nt)));
     }
   }
   return best;
@@ -560,7 +554,7 @@ int setup(ivit_handle* h, const uint16_t* wb) {
 
   IVIT_CK(h, cudaGetDevice(&h->device));
   IVIT_CK(h, cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, h->device));
-  IVIT_CK(h, ivit::gemm_setup());
+  IVIT_CK(h, ivit::gemm_rows_setup());
   IVIT_CK(h, ivit::gemm_pair_setup());
   IVIT_CK(h, ivit::attention_setup());
   IVIT_CK(h, ivit::attention_tc_setup());
@@ -587,16 +581,14 @@ int setup(ivit_handle* h, const uint16_t* wb) {
     // Full encodes know M = SV*N.  Incremental calls are planned for a tenth of the
     // tokens updated (any count still runs correctly, with more or fewer tile rounds).
     const int m_all = static_cast<int>(M), m_inc = std::max(1, m_all / 10);
-    int fit[17] = {};
-    for (int c = 2; c <= 16; ++c) fit[c] = ivit::gemm_max_clusters(c);
     const int shapes[kGemmSlots][2] = {{static_cast<int>(D), h->KPAD}, {3 * static_cast<int>(D), static_cast<int>(D)},
                                        {static_cast<int>(D), static_cast<int>(D)}, {static_cast<int>(F), static_cast<int>(D)},
                                        {static_cast<int>(D), static_cast<int>(F)}};
     for (int g = 0; g < kGemmSlots; ++g) {
-      // (under the MLP-on-all-tokens reading the residual epilogues feed no layer norm of the same rows)
-      const bool defer = (g == kGemmO || g == kGemmDown) && c.mlp_tokens == IVIT_MLP_UPDATED;
+      // (under the MLP-on-all-tokens reading the out-projection goes to a cache, not to a layer norm)
+      const bool defer = g == kGemmDown || (g == kGemmO && c.mlp_tokens == IVIT_MLP_UPDATED);
       auto plan = [&](int m_expected, int m_bound) {
-        return plan_gemm(h->num_sms, fit, shapes[g][0], shapes[g][1], m_expected, m_bound, defer);
+        return plan_gemm(h->num_sms, shapes[g][0], shapes[g][1], m_expected, m_bound, g != kGemmEmbed, defer);
       };
       h->plan_full[g] = plan(m_all, m_all);
       h->plan_inc[g] = g == kGemmEmbed ? h->plan_full[g] : plan(m_inc, m_all);
@@ -607,12 +599,12 @@ int setup(ivit_handle* h, const uint16_t* wb) {
                                                                        : plan(h->band_ub[b], h->band_ub[b]);
     }
     // every row's D x D projection without a residual (first-layer key scores)
-    h->plan_keys = plan_gemm(h->num_sms, fit, static_cast<int>(D), static_cast<int>(D), m_all, m_all, false);
+    h->plan_keys = plan_gemm(h->num_sms, static_cast<int>(D), static_cast<int>(D), m_all, m_all, false, false);
     if (std::getenv("IVIT_DEBUG")) {
       static const char* names[kGemmSlots] = {"embed", "qkv", "out", "up", "down"};
       auto show = [&](const char* when, const char* name, const GemmPlan& pl) {
-        std::fprintf(stderr, "ivit gemm %-6s %-5s %s bn=%d split=%d%s x %d\n", when, name, pl.pair ? "pair" : "cluster", pl.bn,
-                     pl.csize, pl.defer ? " deferred" : "", pl.n_clusters);
+        std::fprintf(stderr, "ivit gemm %-6s %-5s %s bn=%d nt=%d splits=%d\n", when, name, pl.nt ? "rows" : "pair", pl.bn,
+                     pl.nt, pl.splits);
       };
       for (int g = 0; g < kGemmSlots; ++g) {
         show("full", names[g], h->plan_full[g]);
@@ -716,18 +708,16 @@ int setup(ivit_handle* h, const uint16_t* wb) {
   const size_t o_key = c.score_source == IVIT_SCORE_KEY0 ? sa.take(M * D * 4) : 0;
   const size_t o_acache = c.mlp_tokens == IVIT_MLP_ALL ? sa.take(L * M * D * 4) : 0;
   // slots for every plan that splits K, fp32 [row tile][128 features] each
-  size_t part_floats = 0;
+  size_t part_floats = 64;
   for (int g = 0; g < kGemmSlots; ++g)
   {
     auto need = [&](const GemmPlan& pl, int m_bound) -> size_t {
-      if (pl.defer) return defer_slots(pl, static_cast<int>(D), m_bound) * pl.bn * 128;
-      return pl.pair ? 0 : static_cast<size_t>(pl.n_clusters) * pl.csize * pl.bn * 128;
+      return pl.defer ? defer_slots(pl, static_cast<int>(D), m_bound) * pl.bn * 128 : 0;
     };
     part_floats = std::max(part_floats, need(h->plan_full[g], static_cast<int>(M)));
     part_floats = std::max(part_floats, need(h->plan_inc[g], static_cast<int>(M)));
     for (int b = 0; b < h->n_bands; ++b)
       part_floats = std::max(part_floats, need(h->plan_band[b][g], b == 0 ? static_cast<int>(M) : h->band_ub[b]));
-    part_floats = std::max(part_floats, need(h->plan_keys, static_cast<int>(M)));
   }
   const size_t o_gpart = sa.take(part_floats * 4);
   const size_t o_rta = sa.take(M * 4), o_mall = sa.take(4);
@@ -781,6 +771,7 @@ int setup(ivit_handle* h, const uint16_t* wb) {
       return h->fail(IVIT_ERR_CUDA, "cuTensorMapEncodeTiled failed for a cache tile");
   }
   auto act_maps = [&](ActMaps& m, const bf16* base, size_t inner) {
+    m.base = base;
     return make_map(&m.b32, base, inner, M, inner * 2, 64, 32) && make_map(&m.b64, base, inner, M, inner * 2, 64, 64) &&
            make_map(&m.b128, base, inner, M, inner * 2, 64, 128);
   };
@@ -839,15 +830,17 @@ void next_launch(ivit_handle* h, int family, const ivit::GemmArgs* ga = nullptr,
   h->slots_cur.push_back(sl);
 }
 
-int gemm(ivit_handle* h, const GemmPlan& plan, const CUtensorMap& tw, const ActMaps& tx, ivit::GemmArgs a,
-         cudaStream_t s) {
+int gemm(ivit_handle* h, const GemmPlan& plan, const CUtensorMap& tw, const bf16* w, const ActMaps& x,
+         ivit::GemmArgs a, cudaStream_t s) {
   a.err = h->err;
   a.partials = h->gemm_partials;
   a.defer = plan.defer ? 1 : 0;
-  a.vsplit = plan.defer ? plan.csize : 0;
+  a.vsplit = plan.defer ? plan.splits : 0;
+  a.w = w;
+  a.x = x.base;
   next_launch(h, kFamGemm, &a);
-  IVIT_CK(h, plan.pair ? ivit::launch_gemm_pair(plan.bn, tw, tx.of(plan), a, plan.n_clusters, s)
-                       : ivit::launch_gemm(tw, tx.of(plan), a, plan.n_clusters, plan.csize, s));
+  IVIT_CK(h, plan.nt ? ivit::launch_gemm_rows(plan.nt, a, s)
+                     : ivit::launch_gemm_pair(plan.bn, tw, x.of(plan), a, plan.n_pairs, s));
   ++h->launches;
   return IVIT_OK;
 }
@@ -956,6 +949,18 @@ int attention(ivit_handle* h, const LayerW& w, const bf16* ck, const bf16* cv, b
   return IVIT_OK;
 }
 
+// What a residual GEMM launched with plan pl left for the next layer norm to add.
+ivit::PendingSum pending_sum(ivit_handle* h, const GemmPlan& pl, const float* bias) {
+  ivit::PendingSum p;
+  if (!pl.defer) return p;
+  p.partials = h->gemm_partials;
+  p.bias = bias;
+  p.csize = pl.splits;
+  p.bn = pl.bn;
+  p.n_ft = (h->D + 127) / 128;
+  return p;
+}
+
 // The blocks under the MLP-on-all-tokens reading (Sec. III-B, after Eq. 5): x holds
 // every token's residual stream (row = token v*N + i).  Per layer, the updated tokens
 // (packed rows, rowtok) run LN1, QKV with the K/V scatter (Eq. 5), attention over all
@@ -966,14 +971,21 @@ int run_layers_mlp_all(ivit_handle* h, const GemmPlan* plan, bool full, cudaStre
   const ivit_config& c = h->cfg;
   const int N = h->N, D = h->D, F = h->F, SV = h->SV, M = h->M_max;
   const int* total = h->cu_rows + SV;
+  // The down-projection's residual update of every token may still be split over the GEMM
+  // scratch: the next layer's LN1 reads it for the updated tokens, its LN2 adds it to x.
+  ivit::PendingSum pend;
   for (int l = 0; l < h->L; ++l) {
     const LayerW& w = h->layers[l];
     bf16* ck = h->cacheK + static_cast<size_t>(l) * M * D;
     bf16* cv = h->cacheV + static_cast<size_t>(l) * M * D;
     float* al = h->acache + static_cast<size_t>(l) * M * D;
     next_launch(h, kFamLN);
-    IVIT_CK(h, ivit::launch_layernorm_ex(total, h->x, nullptr, h->rowtok, w.ln1g, w.ln1b, h->xn, nullptr, D,
-                                         c.ln_eps, M, h->row_grid, s));
+    if (pend.partials)
+      IVIT_CK(h, ivit::launch_layernorm_sum(total, h->x, pend, nullptr, h->rowtok, w.ln1g, w.ln1b, h->xn, nullptr, D,
+                                            c.ln_eps, M, h->row_grid, s));
+    else
+      IVIT_CK(h, ivit::launch_layernorm_ex(total, h->x, nullptr, h->rowtok, w.ln1g, w.ln1b, h->xn, nullptr, D,
+                                           c.ln_eps, M, h->row_grid, s));
     ++h->launches;
     {
       ivit::GemmArgs a;
@@ -988,7 +1000,7 @@ int run_layers_mlp_all(ivit_handle* h, const GemmPlan* plan, bool full, cudaStre
       a.epi.cache_v = cv;
       a.epi.rowtok = h->rowtok;
       a.epi.dim = D;
-      if (int r = gemm(h, plan[kGemmQKV], w.tm_qkv, h->tm_xn, a, s)) return r;
+      if (int r = gemm(h, plan[kGemmQKV], w.tm_qkv, w.wqkv, h->tm_xn, a, s)) return r;
     }
     if (int r = attention(h, w, ck, cv, full, s)) return r;
     {
@@ -1001,11 +1013,15 @@ int run_layers_mlp_all(ivit_handle* h, const GemmPlan* plan, bool full, cudaStre
       a.epi.out_f32 = al;
       a.epi.ld_out = D;
       a.epi.rowtok = h->rowtok;
-      if (int r = gemm(h, plan[kGemmO], w.tm_o, h->tm_o, a, s)) return r;
+      if (int r = gemm(h, plan[kGemmO], w.tm_o, w.wo, h->tm_o, a, s)) return r;
     }
     next_launch(h, kFamLN);
-    IVIT_CK(h, ivit::launch_layernorm_ex(h->m_all, h->x, al, nullptr, w.ln2g, w.ln2b, h->xn, nullptr, D, c.ln_eps,
-                                         M, h->row_grid, s));
+    if (pend.partials)
+      IVIT_CK(h, ivit::launch_layernorm_sum(h->m_all, h->x, pend, al, nullptr, w.ln2g, w.ln2b, h->xn, nullptr, D,
+                                            c.ln_eps, M, h->row_grid, s));
+    else
+      IVIT_CK(h, ivit::launch_layernorm_ex(h->m_all, h->x, al, nullptr, w.ln2g, w.ln2b, h->xn, nullptr, D, c.ln_eps,
+                                           M, h->row_grid, s));
     ++h->launches;
     {
       ivit::GemmArgs a;
@@ -1017,7 +1033,7 @@ int run_layers_mlp_all(ivit_handle* h, const GemmPlan* plan, bool full, cudaStre
       a.epi.out_bf16 = h->hbuf;
       a.epi.ld_out = F;
       a.epi.gelu_mode = c.gelu;
-      if (int r = gemm(h, h->plan_full[kGemmUp], w.tm_1, h->tm_xn, a, s)) return r;
+      if (int r = gemm(h, h->plan_full[kGemmUp], w.tm_1, w.w1, h->tm_xn, a, s)) return r;
     }
     {
       ivit::GemmArgs a;
@@ -1028,12 +1044,17 @@ int run_layers_mlp_all(ivit_handle* h, const GemmPlan* plan, bool full, cudaStre
       a.epi.bias = w.b2;
       a.epi.out_f32 = h->x;
       a.epi.ld_out = D;
-      if (int r = gemm(h, h->plan_full[kGemmDown], w.tm_2, h->tm_h, a, s)) return r;
+      if (int r = gemm(h, h->plan_full[kGemmDown], w.tm_2, w.w2, h->tm_h, a, s)) return r;
+      pend = pending_sum(h, h->plan_full[kGemmDown], w.b2);
     }
   }
   next_launch(h, kFamLN);
-  IVIT_CK(h, ivit::launch_layernorm(h->m_all, h->x, h->lnfg, h->lnfb, h->tok_out, nullptr, D, c.ln_eps, M,
-                                    h->row_grid, s));
+  if (pend.partials)
+    IVIT_CK(h, ivit::launch_layernorm_sum(h->m_all, h->x, pend, nullptr, nullptr, h->lnfg, h->lnfb, h->tok_out, nullptr,
+                                          D, c.ln_eps, M, h->row_grid, s));
+  else
+    IVIT_CK(h, ivit::launch_layernorm(h->m_all, h->x, h->lnfg, h->lnfb, h->tok_out, nullptr, D, c.ln_eps, M,
+                                      h->row_grid, s));
   ++h->launches;
   (void)N;
   return IVIT_OK;
@@ -1052,7 +1073,8 @@ int run_layers(ivit_handle* h, const GemmPlan* plan, bool full, cudaStream_t s) 
   auto layernorm = [&](const float* g, const float* b, bf16* y, const int* dst) -> int {
     next_launch(h, kFamLN);
     if (pend.partials) {
-      IVIT_CK(h, ivit::launch_layernorm_sum(total, h->x, pend, g, b, y, dst, D, c.ln_eps, M, h->row_grid, s));
+      IVIT_CK(h, ivit::launch_layernorm_sum(total, h->x, pend, nullptr, nullptr, g, b, y, dst, D, c.ln_eps, M,
+                                            h->row_grid, s));
       pend = ivit::PendingSum();
     } else {
       IVIT_CK(h, ivit::launch_layernorm(total, h->x, g, b, y, dst, D, c.ln_eps, M, h->row_grid, s));
@@ -1060,8 +1082,8 @@ int run_layers(ivit_handle* h, const GemmPlan* plan, bool full, cudaStream_t s) 
     ++h->launches;
     return IVIT_OK;
   };
-  auto residual = [&](const GemmPlan& pl, const float* bias, const CUtensorMap& tw, const ActMaps& tx,
-                      int k) -> int {
+  auto residual = [&](const GemmPlan& pl, const float* bias, const CUtensorMap& tw, const bf16* wp,
+                      const ActMaps& tx, int k) -> int {
     ivit::GemmArgs a;
     a.n_out = D;
     a.k = k;
@@ -1070,14 +1092,8 @@ int run_layers(ivit_handle* h, const GemmPlan* plan, bool full, cudaStream_t s) 
     a.epi.bias = bias;
     a.epi.out_f32 = h->x;
     a.epi.ld_out = D;
-    if (int r = gemm(h, pl, tw, tx, a, s)) return r;
-    if (pl.defer) {
-      pend.partials = h->gemm_partials;
-      pend.bias = bias;
-      pend.csize = pl.csize;
-      pend.bn = pl.bn;
-      pend.n_ft = (D + 127) / 128;
-    }
+    if (int r = gemm(h, pl, tw, wp, tx, a, s)) return r;
+    pend = pending_sum(h, pl, bias);
     return IVIT_OK;
   };
   for (int l = 0; l < h->L; ++l) {
@@ -1098,10 +1114,10 @@ int run_layers(ivit_handle* h, const GemmPlan* plan, bool full, cudaStream_t s) 
       a.epi.cache_v = cv;
       a.epi.rowtok = h->rowtok;
       a.epi.dim = D;
-      if (int r = gemm(h, plan[kGemmQKV], w.tm_qkv, h->tm_xn, a, s)) return r;
+      if (int r = gemm(h, plan[kGemmQKV], w.tm_qkv, w.wqkv, h->tm_xn, a, s)) return r;
     }
     if (int r = attention(h, w, ck, cv, full, s)) return r;
-    if (int r = residual(plan[kGemmO], w.bo, w.tm_o, h->tm_o, D)) return r;
+    if (int r = residual(plan[kGemmO], w.bo, w.tm_o, w.wo, h->tm_o, D)) return r;
     if (int r = layernorm(w.ln2g, w.ln2b, h->xn, nullptr)) return r;
     {
       ivit::GemmArgs a;
@@ -1113,9 +1129,9 @@ int run_layers(ivit_handle* h, const GemmPlan* plan, bool full, cudaStream_t s) 
       a.epi.out_bf16 = h->hbuf;
       a.epi.ld_out = F;
       a.epi.gelu_mode = c.gelu;
-      if (int r = gemm(h, plan[kGemmUp], w.tm_1, h->tm_xn, a, s)) return r;
+      if (int r = gemm(h, plan[kGemmUp], w.tm_1, w.w1, h->tm_xn, a, s)) return r;
     }
-    if (int r = residual(plan[kGemmDown], w.b2, w.tm_2, h->tm_h, F)) return r;
+    if (int r = residual(plan[kGemmDown], w.b2, w.tm_2, w.w2, h->tm_h, F)) return r;
   }
   return layernorm(h->lnfg, h->lnfb, h->tok_out, h->rowtok);
 }
@@ -1181,7 +1197,7 @@ int run_core(ivit_handle* h, const uint8_t* frames, int32_t* user_counts, bool f
     a.epi.bias = h->b_pe;
     a.epi.out_f32 = h->e_t;
     a.epi.ld_out = D;
-    if (int r = gemm(h, plan[kGemmEmbed], h->tm_pe, h->tm_patches, a, s)) return r;
+    if (int r = gemm(h, plan[kGemmEmbed], h->tm_pe, h->w_pe, h->tm_patches, a, s)) return r;
   }
   const float* score_vec = h->e_t;
   if (c.score_source == IVIT_SCORE_KEY0) {
@@ -1202,7 +1218,7 @@ int run_core(ivit_handle* h, const uint8_t* frames, int32_t* user_counts, bool f
     a.epi.bias = h->layers[0].bqkv + D;
     a.epi.out_f32 = h->key_t;
     a.epi.ld_out = D;
-    if (int r = gemm(h, h->plan_keys, h->tm_wk0, h->tm_xn, a, s)) return r;
+    if (int r = gemm(h, h->plan_keys, h->tm_wk0, nullptr, h->tm_xn, a, s)) return r;
     score_vec = h->key_t;
   }
   if (!full) {

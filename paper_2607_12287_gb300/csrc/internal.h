@@ -79,11 +79,8 @@ struct GemmArgs {
   const int* d_rows = nullptr;   // device row count M (nullptr: use m_static)
   int m_static = 0;
   int* err = nullptr;            // device error word
-  // Split-K exchange scratch (global memory, stays in L2): slot [cluster][rank][BN_MAX][128]
-  // floats for every CTA of the launch.  Required when the launch's clusters have more
-  // than one CTA.
-  float* partials = nullptr;
-  // With defer set, K is split over vsplit consecutive CTAs (or pairs) without clusters and
+  float* partials = nullptr;     // scratch of a deferred launch (global memory, stays in L2)
+  // With defer set, K is split over vsplit consecutive CTAs (or pairs) and
   // the partial tiles are left in the scratch, slot (tile * vsplit + split) of fp32
   // [rows per tile][128] with tile = feature tile + n_ft * row tile; the kernel neither
   // reduces them nor runs the epilogue: the next kernel sums them (layernorm_sum, for the
@@ -91,6 +88,8 @@ struct GemmArgs {
   int defer = 0;
   int vsplit = 0;
   unsigned long long* stamp = nullptr;  // timeline stamps of this launch (or null)
+  const bf16* w = nullptr;       // W and X themselves, for the kernel that uses no TMA maps
+  const bf16* x = nullptr;       // (gemm_rows)
   GemmEpilogue epi;
 };
 
@@ -99,27 +98,25 @@ struct GemmArgs {
 struct PendingSum {
   const float* partials = nullptr;  // the GEMM's scratch
   const float* bias = nullptr;      // [dim]
-  int csize = 0;                    // splits (CTAs per cluster), 2..16
-  int bn = 0;                       // rows per row tile (the GEMM's BN_MAX)
+  int csize = 0;                    // splits, 2..16
+  int bn = 0;                       // rows per row tile
   int n_ft = 0;                     // feature tiles of 128
 };
 
-// One-time attribute setup (dynamic smem opt-in, clusters of up to 16).
-cudaError_t gemm_setup();
-// Clusters of `csize` CTAs that can be resident at once (0 if none).
-int gemm_max_clusters(int csize);
-// Launches n_clusters clusters of csize >= 2 CTAs on tiles of 128 features x 64 rows (tm_x
-// boxes of 32 rows).  The CTAs of a cluster split K and reduce their partial tiles through
-// the scratch; clusters walk the output tiles.
-cudaError_t launch_gemm(const CUtensorMap& tm_w, const CUtensorMap& tm_x, const GemmArgs& a, int n_clusters,
-                        int csize, cudaStream_t s);
-
-// The same GEMM over CTA pairs (cta_group::2), tiles of 256 features x bn rows (64, 128 or
+// The GEMM over CTA pairs (cta_group::2), tiles of 256 features x bn rows (64, 128 or
 // 256; tm_x boxes of bn / 2 rows), walked by n_pairs persistent pairs.  With defer set (and vsplit >= 1) K is split
 // vsplit ways and the partial tiles stay in the scratch, as described at GemmArgs::defer.
 cudaError_t gemm_pair_setup();
 cudaError_t launch_gemm_pair(int bn, const CUtensorMap& tm_w, const CUtensorMap& tm_x, const GemmArgs& a,
                              int n_pairs, cudaStream_t s);
+
+// The same GEMM for a few rows: CTAs of 8 nt features (nt 1..4), rows in passes of 32, every
+// epilogue but kEpiF32Bias.  With defer set, K is split vsplit ways and the slots have 32 rows.
+// k a multiple of 8.
+constexpr int GEMM_ROWS_SMEM_MAX = 160 * 1024;
+size_t gemm_rows_smem(int nt, int k, int splits);
+cudaError_t gemm_rows_setup();
+cudaError_t launch_gemm_rows(int nt, const GemmArgs& a, cudaStream_t s);
 
 // ------------------------------------------------------- persistent encoder (small M)
 struct LayerParams {
@@ -241,12 +238,13 @@ cudaError_t launch_layernorm_ex(const int* rows, float* x, const float* add, con
                                 const float* gamma, const float* beta, bf16* y, const int* dst_rowtok, int dim,
                                 float eps, int max_rows, int grid, cudaStream_t s);
 
-// x[r] += bias + sum_s partial_s[r] (splits in order, as the GEMM's own reduction sums
-// them), written back to x, then y = LN(x[r]) (row dst_rowtok[r] of y when set), for
-// r < *rows.  dim a multiple of 4, at most 4096.
-cudaError_t launch_layernorm_sum(const int* rows, float* x, const PendingSum& ps, const float* gamma,
-                                 const float* beta, bf16* y, const int* dst_rowtok, int dim, float eps,
-                                 int max_rows, int grid, cudaStream_t s);
+// x[r] += bias + sum_s partial_s[r] (splits in order), written back to x, then y = LN(x[r])
+// (row dst_rowtok[r] of y when set), for r < *rows.  With src_rowtok, row r is row
+// src_rowtok[r] of x and of the partials, and x is left as it is; with add (not both), row r
+// of add is added to x too.  dim a multiple of 4, at most 4096.
+cudaError_t launch_layernorm_sum(const int* rows, float* x, const PendingSum& ps, const float* add,
+                                 const int* src_rowtok, const float* gamma, const float* beta, bf16* y,
+                                 const int* dst_rowtok, int dim, float eps, int max_rows, int grid, cudaStream_t s);
 
 // One-time function attributes of the attention kernel (dynamic shared memory opt-in).
 cudaError_t attention_setup();

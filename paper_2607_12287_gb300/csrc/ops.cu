@@ -386,8 +386,11 @@ __global__ void layernorm_kernel(const int* __restrict__ nrows, float* __restric
 // bias + sum_s partial_s (the splits in order, the same fp32 sum the GEMM's own
 // reduction forms), x written back, then y = LN(x).  One CTA per row and one float4 of
 // the row per thread, so every split's partial of every element is in flight at once
-// (a row's partials are spread over the csize slots of its feature tiles).
+// (a row's partials are spread over the csize slots of its feature tiles).  kGather: the row
+// is src_rowtok[r], and x is not written; kAdd: a row of `add` is added as well.
+template <bool kGather, bool kAdd>
 __global__ void layernorm_sum_kernel(const int* __restrict__ nrows, float* __restrict__ x, const PendingSum ps,
+                                     const float* __restrict__ add, const int* __restrict__ src_rowtok,
                                      const float* __restrict__ gamma, const float* __restrict__ beta,
                                      bf16* __restrict__ y, const int* __restrict__ dst_rowtok, int dim, float eps,
                                      unsigned long long* stamp) {
@@ -410,15 +413,18 @@ __global__ void layernorm_sum_kernel(const int* __restrict__ nrows, float* __res
   const size_t sstride = static_cast<size_t>(ps.bn) * 128;
   for (int r = blockIdx.x; r < rows; r += gridDim.x) {
     float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    const int irow = kGather ? src_rowtok[r] : r;
     if (act) {
-      const int tt = r / ps.bn, rr = r - tt * ps.bn;
+      const int tt = irow / ps.bn, rr = irow - tt * ps.bn;
       const float* p = ps.partials + (static_cast<size_t>(ft + ps.n_ft * tt) * ps.csize * ps.bn + rr) * 128 + fl;
       float4 q[MAXS];
 #pragma unroll
       for (int sp = 0; sp < MAXS; ++sp)
         if (sp < ps.csize) q[sp] = __ldcg(reinterpret_cast<const float4*>(p + sp * sstride));
-      float4* xr = reinterpret_cast<float4*>(x + static_cast<size_t>(r) * dim) + c;
+      float4* xr = reinterpret_cast<float4*>(x + static_cast<size_t>(irow) * dim) + c;
       const float4 x0 = *xr;
+      float4 w = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (kAdd) w = reinterpret_cast<const float4*>(add + static_cast<size_t>(irow) * dim)[c];
       float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
       for (int sp = 0; sp < MAXS; ++sp)
@@ -430,7 +436,8 @@ __global__ void layernorm_sum_kernel(const int* __restrict__ nrows, float* __res
         }
       v = make_float4(x0.x + (acc.x + bias.x), x0.y + (acc.y + bias.y), x0.z + (acc.z + bias.z),
                       x0.w + (acc.w + bias.w));
-      *xr = v;
+      if (kAdd) v = make_float4(v.x + w.x, v.y + w.y, v.z + w.z, v.w + w.w);
+      if (!kGather) *xr = v;
     }
     float sum = warp_sum((v.x + v.y) + (v.z + v.w));
     if (lane == 0) red[0][warp] = sum;
@@ -734,15 +741,18 @@ cudaError_t launch_layernorm(const int* rows, const float* x, const float* gamma
                              max_rows, grid, s);
 }
 
-cudaError_t launch_layernorm_sum(const int* rows, float* x, const PendingSum& ps, const float* gamma,
-                                 const float* beta, bf16* y, const int* dst_rowtok, int dim, float eps,
-                                 int max_rows, int grid, cudaStream_t s) {
-  if (dim % 4 != 0 || dim > 4096 || ps.csize < 2 || ps.csize > 16 || ps.bn < 1 || !ps.partials || !ps.bias)
+cudaError_t launch_layernorm_sum(const int* rows, float* x, const PendingSum& ps, const float* add,
+                                 const int* src_rowtok, const float* gamma, const float* beta, bf16* y,
+                                 const int* dst_rowtok, int dim, float eps, int max_rows, int grid, cudaStream_t s) {
+  if (dim % 4 != 0 || dim > 4096 || ps.csize < 2 || ps.csize > 16 || ps.bn < 1 || !ps.partials || !ps.bias ||
+      (add && src_rowtok))
     return cudaErrorInvalidValue;
   const int threads = (dim / 4 + 31) / 32 * 32;
   grid = max(1, min(grid, max_rows));
-  return launch_ex(layernorm_sum_kernel, dim3(grid), dim3(threads), 0, s, 1, rows, x, ps, gamma, beta, y,
-                   dst_rowtok, dim, eps, g_stamp);
+  auto kern = add ? layernorm_sum_kernel<false, true>
+                  : (src_rowtok ? layernorm_sum_kernel<true, false> : layernorm_sum_kernel<false, false>);
+  return launch_ex(kern, dim3(grid), dim3(threads), 0, s, 1, rows, x, ps, add, src_rowtok, gamma, beta, y, dst_rowtok,
+                   dim, eps, g_stamp);
 }
 
 cudaError_t launch_layernorm_ex(const int* rows, float* x, const float* add, const int* src_rowtok,

@@ -16,12 +16,13 @@ def pkg():
     return p
 
 
-def _run(pkg, oracle_mod, grid, views, dim, heads, mlp, depth, change_p, n_frames=3):
+def _run(pkg, oracle_mod, grid, views, dim, heads, mlp, depth, change_p, n_frames=3, mlp_tokens=0):
     from paper_2607_12287_gb300 import synth
     shape = synth.EncoderShape(8 * grid[0], 8 * grid[1], 8, dim, depth, heads, mlp, synth.GELU_TANH)
     frames = list(synth.stream_random(shape, views, n_frames, 11, change_p=change_p))
     stats = gpu_util.run_side_by_side(pkg, oracle_mod, shape, synth.make_weights(shape, 3), frames, 1, views,
-                                      check_caches=True, cache_layers="all")
+                                      check_caches=True, cache_layers="all",
+                                      mlp_tokens=mlp_tokens)
     assert len(stats) == n_frames and all(np.isfinite(s[0]).all() for s in stats)
 
 
@@ -45,6 +46,20 @@ def test_gemm_tile_edges(pkg, oracle_mod, grid, views, dim, heads, mlp):
 def test_persistent_kernel_odd_key_tiles(pkg, oracle_mod, monkeypatch, grid, views, dim, heads):
     monkeypatch.setenv("IVIT_PATH", "persistent")
     _run(pkg, oracle_mod, grid, views, dim, heads, 2 * dim, 2, 0.5)
+
+
+# (grid, dim, heads, mlp, change): a few updated rows in one to three passes of 32 and in one or
+# two 16-row tiles, K of a ragged last chunk (mlp 520, 840), one chunk per two warps (dim 64),
+# feature counts that are no multiple of a CTA's
+ROW_SHAPES = [((6, 10), 64, 1, 264, 0.05), ((6, 10), 320, 5, 840, 0.25), ((6, 10), 320, 5, 520, 0.5),
+              ((8, 12), 576, 8, 1160, 0.95)]
+
+
+@pytest.mark.parametrize("mlp_tokens", [0, 1], ids=["updated", "all"])
+@pytest.mark.parametrize("grid,dim,heads,mlp,change", ROW_SHAPES,
+                         ids=[f"d{d}_f{f}_p{int(100 * c)}" for _, d, _, f, c in ROW_SHAPES])
+def test_few_row_gemm_edges(pkg, oracle_mod, grid, dim, heads, mlp, change, mlp_tokens):
+    _run(pkg, oracle_mod, grid, 1, dim, heads, mlp, 2, change, n_frames=4, mlp_tokens=mlp_tokens)
 
 
 # (grid, views, dim, heads): head widths of every padded width (8 -> 16 ... 128), token counts
