@@ -1204,7 +1204,7 @@ int run_core(ivit_handle* h, const uint8_t* frames, int32_t* user_counts, bool f
     // Eq. 3 on first-layer keys of every token: W_K LN1(e + pos) + b_K (x, xn are free
     // until the updated rows are gathered below)
     next_launch(h, kFamOther, nullptr, 3);  // gather
-    IVIT_CK(h, ivit::launch_gather(h->m_all, h->rowtok_all, h->e_t, h->pos, h->x, nullptr, h->e_ref, N, D, 0,
+    IVIT_CK(h, ivit::launch_gather(h->m_all, h->rowtok_all, ivit::RowLists(), h->e_t, h->pos, h->x, nullptr, h->e_ref, N, D, 0,
                                    cm, M, h->row_grid, s));
     next_launch(h, kFamLN);
     IVIT_CK(h, ivit::launch_layernorm(h->m_all, h->x, h->layers[0].ln1g, h->layers[0].ln1b, h->xn, nullptr, D,
@@ -1226,19 +1226,19 @@ int run_core(ivit_handle* h, const uint8_t* frames, int32_t* user_counts, bool f
     IVIT_CK(h, ivit::launch_score(score_vec, h->e_ref, h->sims, M, D, c.ref_mode == IVIT_REF_PREV_FRAME, s));
     ++h->launches;
   }
+  const ivit::RowLists lists{h->idx, h->cu_rows, SV, N};
   next_launch(h, kFamOther, nullptr, 2);  // select
   IVIT_CK(h, ivit::launch_select(h->sims, N, SV, full ? IVIT_SEL_THRESHOLD : c.select_mode, c.threshold,
-                                 c.topk, cm, h->idx, h->counts, h->cu_rows, h->rowtok, h->done_ctr,
-                                 user_counts, s));
+                                 c.topk, cm, h->idx, h->counts, h->cu_rows, h->done_ctr, user_counts, s));
   ++h->launches;
   if (c.mlp_tokens == IVIT_MLP_ALL) {
     // every token's residual stream (token-indexed), then the references of the updated
     // tokens (last-refresh mode, cold views) without touching x
     next_launch(h, kFamOther, nullptr, 3);  // gather
-    IVIT_CK(h, ivit::launch_gather(h->m_all, h->rowtok_all, h->e_t, h->pos, h->x, nullptr, h->e_ref, N, D, 0,
+    IVIT_CK(h, ivit::launch_gather(h->m_all, h->rowtok_all, ivit::RowLists(), h->e_t, h->pos, h->x, nullptr, h->e_ref, N, D, 0,
                                    cm, M, h->row_grid, s));
     next_launch(h, kFamOther, nullptr, 3);  // gather
-    IVIT_CK(h, ivit::launch_gather(total, h->rowtok, h->e_t, h->pos, nullptr, score_vec, h->e_ref, N, D,
+    IVIT_CK(h, ivit::launch_gather(total, h->rowtok, lists, h->e_t, h->pos, nullptr, score_vec, h->e_ref, N, D,
                                    c.ref_mode == IVIT_REF_LAST_REFRESH, cm, M, h->row_grid, s));
     h->launches += 2;
     return run_layers_mlp_all(h, plan, full, s);
@@ -1256,7 +1256,7 @@ int run_core(ivit_handle* h, const uint8_t* frames, int32_t* user_counts, bool f
     h->bands = bands;
   }
   next_launch(h, kFamOther, nullptr, 3);  // gather
-  IVIT_CK(h, ivit::launch_gather(total, h->rowtok, h->e_t, h->pos, h->x, score_vec, h->e_ref, N, D,
+  IVIT_CK(h, ivit::launch_gather(total, h->rowtok, lists, h->e_t, h->pos, h->x, score_vec, h->e_ref, N, D,
                                  c.ref_mode == IVIT_REF_LAST_REFRESH, cm, M, h->row_grid, s, bands));
   ++h->launches;
 

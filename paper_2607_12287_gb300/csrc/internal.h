@@ -207,8 +207,16 @@ cudaError_t launch_score(const float* e_t, float* e_ref, float* sims, int rows, 
                          int copy_ref, cudaStream_t s);
 
 cudaError_t launch_select(const float* sims, int n_tok, int sv, int mode, float tau, int topk,
-                          const ColdMask& cold, int* idx, int* counts, int* cu_rows, int* rowtok,
-                          int* done_ctr, int* user_counts, cudaStream_t s);
+                          const ColdMask& cold, int* idx, int* counts, int* cu_rows, int* done_ctr,
+                          int* user_counts, cudaStream_t s);
+
+// The selection's ascending token lists idx [sv][n_tok] and the views' packed-row offsets
+// cu_rows [sv + 1]; idx null: none.
+struct RowLists {
+  const int* idx = nullptr;
+  const int* cu_rows = nullptr;
+  int sv = 0, n_tok = 0;
+};
 
 // Row-count bands of an incremental call's CUDA graph: the launch plans of band b are
 // made for at most ub[b] updated rows; the graph's switch node runs the body of the
@@ -219,10 +227,11 @@ struct RowBands {
   int ub[4] = {0, 0, 0, 0};
 };
 
-// x[r] = e_t[tok] + pos[tok % N] for the packed rows; refreshes e_ref[tok] from
+// x[r] = e_t[tok] + pos[tok % N] for the packed rows r, tok = rowtok[r] or, with lists, looked
+// up there and written to rowtok; refreshes e_ref[tok] from
 // ref_src[tok] for refreshed tokens (last-refresh reference or cold view).  With
 // bands.handle set, thread 0 of CTA 0 also selects the band of the row count.
-cudaError_t launch_gather(const int* cu_rows_total, const int* rowtok, const float* e_t,
+cudaError_t launch_gather(const int* cu_rows_total, int* rowtok, const RowLists& lists, const float* e_t,
                           const float* pos, float* x, const float* ref_src, float* e_ref, int n_tok,
                           int dim, int ref_last_refresh, const ColdMask& cold, int max_rows, int grid,
                           cudaStream_t s, const RowBands& bands = RowBands());

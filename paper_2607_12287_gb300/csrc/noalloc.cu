@@ -13,6 +13,7 @@
 #include "../../include/ivit.h"
 #include "internal.h"
 #include "ptx.cuh"
+#include "select.cuh"
 
 namespace ivit {
 void set_create_error(const char* msg);  // engine.cu: message for ivit_last_error(NULL)
@@ -63,10 +64,12 @@ __global__ void noalloc_score_kernel(const float* __restrict__ e_cur, const floa
                                      float* __restrict__ scores, int rows, int dim) {
   const int warps = blockDim.x >> 5;
   const int lane = threadIdx.x & 31;
+  ivit::pdl_launch_dependents();  // the selection waits for this grid's end, not for this
   for (int r = blockIdx.x * warps + (threadIdx.x >> 5); r < rows; r += gridDim.x * warps) {
     const float4* a = reinterpret_cast<const float4*>(e_cur + static_cast<size_t>(r) * dim);
     const float4* b = reinterpret_cast<const float4*>(e_ref + static_cast<size_t>(r) * dim);
     float dot = 0.f, na = 0.f, nb = 0.f;
+#pragma unroll 3
     for (int c = lane; c < dim / 4; c += 32) {
       const float4 x = a[c], y = b[c];
       dot += x.x * y.x + x.y * y.y + x.z * y.z + x.w * y.w;
@@ -80,49 +83,19 @@ __global__ void noalloc_score_kernel(const float* __restrict__ e_cur, const floa
   }
 }
 
-// One CTA per view: threshold or top-k flags compacted in index order (warp ballots and
-// a block prefix sum) into idx[v][0..count), the rest of the row set to -1.
+// One CTA per view: threshold or top-k flags compacted in index order into
+// idx[v][0..count), the rest of the row set to -1.
 __global__ void noalloc_select_kernel(const float* __restrict__ scores, int N, int mode, float tau,
                                       int topk, int* __restrict__ idx, int* __restrict__ counts) {
-  extern __shared__ float s_scores[];
-  __shared__ int s_warp[32];
-  __shared__ int s_total;
+  __shared__ int hist[256], scratch[33];
   const int v = blockIdx.x, i = threadIdx.x;
-  const int lane = i & 31, warp = i >> 5, nwarps = blockDim.x >> 5;
+  ivit::pdl_wait();  // the scores
   const float s = (i < N) ? scores[static_cast<size_t>(v) * N + i] : 0.f;
-  bool flag = false;
-  if (mode == IVIT_SEL_TOPK) {
-    if (i < N) s_scores[i] = s;
-    __syncthreads();
-    if (i < N) {
-      int rank = 0;
-      for (int j = 0; j < N; ++j) {
-        const float sj = s_scores[j];
-        rank += (sj < s || (sj == s && j < i)) ? 1 : 0;
-      }
-      flag = rank < topk;
-    }
-  } else if (i < N) {
-    flag = s < tau;
-  }
-  const unsigned ballot = __ballot_sync(0xffffffffu, flag);
-  if (lane == 0) s_warp[warp] = __popc(ballot);
-  __syncthreads();
-  if (warp == 0) {
-    const int x = lane < nwarps ? s_warp[lane] : 0;
-    int incl = x;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int y = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += y;
-    }
-    if (lane < nwarps) s_warp[lane] = incl - x;
-    if (lane == 31) s_total = incl;
-  }
-  __syncthreads();
-  const int total = s_total;
+  const bool flag = mode == IVIT_SEL_TOPK ? ivit::among_lowest(s, i < N, topk, hist, scratch) : i < N && s < tau;
+  int total;
+  const int pos = ivit::block_rank(flag, scratch, total);
   int* row = idx + static_cast<size_t>(v) * N;
-  if (flag) row[s_warp[warp] + __popc(ballot & ((1u << lane) - 1u))] = i;
+  if (flag) row[pos] = i;
   for (int k = total + i; k < N; k += blockDim.x) row[k] = -1;
   if (i == 0) counts[v] = total;
 }
@@ -169,10 +142,10 @@ extern "C" int ivit_select_noalloc(const float* e_cur_dev, const float* e_ref_de
   noalloc_score_kernel<<<grid, 256, 0, s>>>(e_cur_dev, e_ref_dev, scores, rows, dim);
   const int threads = (n_tok + 31) / 32 * 32;
   const int k = topk < 0 ? 0 : topk;
-  noalloc_select_kernel<<<n_views, threads, n_tok * sizeof(float), s>>>(scores, n_tok, select_mode,
-                                                                        threshold, k, idx_out_dev,
-                                                                        counts_out_dev);
-  const cudaError_t e = cudaGetLastError();
+  cudaError_t e = cudaGetLastError();
+  if (e == cudaSuccess)
+    e = ivit::launch_ex(noalloc_select_kernel, dim3(n_views), dim3(threads), 0, s, 1, scores, n_tok, select_mode,
+                        threshold, k, idx_out_dev, counts_out_dev);
   if (e != cudaSuccess) {
     ivit::set_create_error(cudaGetErrorString(e));
     return IVIT_ERR_CUDA;

@@ -6,6 +6,7 @@
 
 #include "internal.h"
 #include "ptx.cuh"
+#include "select.cuh"
 
 namespace ivit {
 
@@ -110,103 +111,83 @@ __global__ void score_kernel(const float* __restrict__ e_t, float* __restrict__ 
 }
 
 // ----------------------------------------------------------------------- select
-// One CTA per view (blockDim >= N).  flag(i) = cold || sim < tau (threshold mode) or
-// rank(i) < k with rank in (sim ascending, index ascending) order (top-k mode).  Flags
-// are compacted in index order with warp ballots and a block prefix sum into idx[v][.]
-// and counts[v].  The last CTA to finish turns the counts into cu_rows (exclusive
-// prefix, cu_rows[sv] = total rows) and writes rowtok[r] = v*N + idx[v][r - cu_rows[v]].
+// One CTA per view (blockDim >= N).  flag(i) = cold || sim < tau (threshold mode) or sim(i)
+// among the k lowest in (sim ascending, index ascending) order (top-k mode).  Flags are
+// compacted in index order into idx[v][.] and counts[v]; the last CTA to finish turns the
+// counts into cu_rows (exclusive prefix, cu_rows[sv] = total rows).
 __global__ void select_kernel(const float* __restrict__ sims, int N, int sv, int mode, float tau,
                               int topk, const ColdMask cold, int* __restrict__ idx,
-                              int* __restrict__ counts, int* __restrict__ cu_rows,
-                              int* __restrict__ rowtok, int* __restrict__ done_ctr,
+                              int* __restrict__ counts, int* __restrict__ cu_rows, int* __restrict__ done_ctr,
                               int* __restrict__ user_counts, unsigned long long* stamp) {
   pdl_wait();
   pdl_launch_dependents();
   stamp_begin(stamp);
-  extern __shared__ float s_sims[];  // [N]
-  __shared__ int s_warp[32];
+  __shared__ int hist[256], scratch[33];
   __shared__ int s_last;
   const int v = blockIdx.x, i = threadIdx.x;
-  const int lane = i & 31, warp = i >> 5, nwarps = blockDim.x >> 5;
   const bool c = is_cold(cold, v);
   const float s = (i < N) ? sims[static_cast<size_t>(v) * N + i] : 0.f;
-  bool flag = false;
-  if (mode == 1 && !c) {
-    if (i < N) s_sims[i] = s;
-    __syncthreads();
-    if (i < N) {
-      int rank = 0;
-      for (int j = 0; j < N; ++j) {
-        const float sj = s_sims[j];
-        rank += (sj < s || (sj == s && j < i)) ? 1 : 0;
-      }
-      flag = rank < topk;
-    }
-  } else if (i < N) {
-    flag = c || (s < tau);
-  }
-  const unsigned ballot = __ballot_sync(0xffffffffu, flag);
-  if (lane == 0) s_warp[warp] = __popc(ballot);
-  __syncthreads();
-  if (warp == 0) {
-    int x = lane < nwarps ? s_warp[lane] : 0;
-    int incl = x;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int y = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += y;
-    }
-    if (lane < nwarps) s_warp[lane] = incl - x;  // exclusive warp offsets
-    if (lane == 31) s_last = incl;               // view total
-  }
-  __syncthreads();
-  const int total = s_last;
-  if (flag) {
-    const int pos = s_warp[warp] + __popc(ballot & ((1u << lane) - 1u));
-    idx[static_cast<size_t>(v) * N + pos] = i;
-  }
+  const bool flag = mode == 1 && !c ? among_lowest(s, i < N, topk, hist, scratch) : i < N && (c || s < tau);
+  int total;
+  const int pos = block_rank(flag, scratch, total);
+  if (flag) idx[static_cast<size_t>(v) * N + pos] = i;
   if (i == 0) {
     counts[v] = total;
     if (user_counts) user_counts[v] = total;
+    __threadfence();
+    s_last = (atomicAdd(done_ctr, 1) == sv - 1) ? 1 : 0;
   }
-  __threadfence();
-  __syncthreads();
-  if (i == 0) s_last = (atomicAdd(done_ctr, 1) == sv - 1) ? 1 : 0;
   __syncthreads();
   if (!s_last) {
     stamp_end(stamp);
     return;
   }
   __threadfence();
-  if (i == 0) {
-    int acc = 0;
-    for (int u = 0; u < sv; ++u) {
-      cu_rows[u] = acc;
-      acc += __ldcg(counts + u);
+  if (i < 32) {
+    int before = 0;
+    for (int u0 = 0; u0 < sv; u0 += 32) {
+      const int n = u0 + i < sv ? __ldcg(counts + u0 + i) : 0;
+      int incl = n;
+#pragma unroll
+      for (int d = 1; d < 32; d <<= 1) {
+        const int up = __shfl_up_sync(0xffffffffu, incl, d);
+        if (i >= d) incl += up;
+      }
+      if (u0 + i < sv) cu_rows[u0 + i] = before + incl - n;
+      before += __shfl_sync(0xffffffffu, incl, 31);
     }
-    cu_rows[sv] = acc;
-    *done_ctr = 0;
-  }
-  __syncthreads();
-  const int rows = __ldcg(cu_rows + sv);
-  for (int r = i; r < rows; r += blockDim.x) {
-    int lo = 0, hi = sv - 1;  // last view u with cu_rows[u] <= r
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (__ldcg(cu_rows + mid) <= r) lo = mid; else hi = mid - 1;
+    if (i == 0) {
+      cu_rows[sv] = before;
+      *done_ctr = 0;
     }
-    const int k = r - __ldcg(cu_rows + lo);
-    rowtok[r] = lo * N + __ldcg(idx + static_cast<size_t>(lo) * N + k);
   }
   stamp_end(stamp);
+}
+
+// Token of packed row r from the selection's lists, by a whole warp: the last view u with
+// cu_rows[u] <= r (a 32-way search), then its list.
+__device__ __forceinline__ int token_of_row(const RowLists& ls, int r, int lane) {
+  if (ls.sv == 1) return ls.idx[r];
+  int lo = 0, n = ls.sv;
+  while (n > 1) {
+    const int step = (n + 31) >> 5;
+    const bool le = lane * step < n && ls.cu_rows[lo + lane * step] <= r;
+    const int m = __popc(__ballot_sync(0xffffffffu, le)) - 1;  // (true on a prefix of the lanes)
+    lo += m * step;
+    n = min(step, n - m * step);
+  }
+  return lo * ls.n_tok + ls.idx[static_cast<size_t>(lo) * ls.n_tok + (r - ls.cu_rows[lo])];
 }
 
 // ----------------------------------------------------------------------- gather
 // x[r] = e_t[tok] + pos[tok % N] for the packed updated rows (fp32 residual stream).
 // The reference row of an updated token (e_ref[tok] <- ref_src[tok], the score vector:
 // patch embedding or first-layer key) is refreshed here when the reference is the last
-// refresh, or when the view was cold.  ref_src may be null (no refresh).
-__global__ void gather_kernel(const int* __restrict__ total_rows, const int* __restrict__ rowtok,
+// refresh, or when the view was cold.  ref_src may be null (no refresh).  With ls.idx set the
+// rows' tokens are looked up in the selection's lists and written to rowtok (every row's
+// warp looks up its own: one CTA that did it for all rows took 40 us for 32768 of them);
+// else they are read from rowtok.
+__global__ void gather_kernel(const int* __restrict__ total_rows, int* __restrict__ rowtok, const RowLists ls,
                               const float* __restrict__ e_t, const float* __restrict__ pos,
                               float* __restrict__ x, const float* __restrict__ ref_src,
                               float* __restrict__ e_ref, int N, int dim, int ref_last_refresh,
@@ -223,7 +204,8 @@ __global__ void gather_kernel(const int* __restrict__ total_rows, const int* __r
   const int warps = blockDim.x >> 5;
   const int lane = threadIdx.x & 31;
   for (int r = blockIdx.x * warps + (threadIdx.x >> 5); r < rows; r += gridDim.x * warps) {
-    const int tok = rowtok[r];
+    const int tok = ls.idx ? token_of_row(ls, r, lane) : rowtok[r];
+    if (ls.idx && lane == 0) rowtok[r] = tok;
     const int ti = tok % N;
     const bool refresh = ref_src && (ref_last_refresh || is_cold(cold, tok / N));
     const float4* a = reinterpret_cast<const float4*>(e_t + static_cast<size_t>(tok) * dim);
@@ -250,7 +232,7 @@ __global__ void gather_kernel(const int* __restrict__ total_rows, const int* __r
 // group's mbarrier, then sums from shared memory into x with 128-bit stores.
 constexpr int GATHER_RPC = 4;
 
-__global__ void gather_bulk_kernel(const int* __restrict__ total_rows, const int* __restrict__ rowtok,
+__global__ void gather_bulk_kernel(const int* __restrict__ total_rows, int* __restrict__ rowtok, const RowLists ls,
                                    const float* __restrict__ e_t, const float* __restrict__ pos,
                                    float* __restrict__ x, const float* __restrict__ ref_src,
                                    float* __restrict__ e_ref, int N, int dim, int ref_last_refresh,
@@ -279,6 +261,12 @@ __global__ void gather_bulk_kernel(const int* __restrict__ total_rows, const int
   uint32_t phase = 0;
   for (int r0 = blockIdx.x * GATHER_RPC; r0 < rows; r0 += gridDim.x * GATHER_RPC, phase ^= 1u) {
     const int nr = min(GATHER_RPC, rows - r0);
+    if (ls.idx && threadIdx.x < 32) {
+      for (int i = 0; i < nr; ++i) {
+        const int tok = token_of_row(ls, r0 + i, threadIdx.x);
+        if (threadIdx.x == 0) rowtok[r0 + i] = tok;
+      }
+    }
     if (threadIdx.x == 0) {
       mbar_arrive_expect_tx(smem_u32(&bar), 2u * nr * row_bytes);
       for (int i = 0; i < nr; ++i) {
@@ -704,14 +692,14 @@ cudaError_t launch_score(const float* e_t, float* e_ref, float* sims, int rows, 
 }
 
 cudaError_t launch_select(const float* sims, int n_tok, int sv, int mode, float tau, int topk,
-                          const ColdMask& cold, int* idx, int* counts, int* cu_rows, int* rowtok,
-                          int* done_ctr, int* user_counts, cudaStream_t s) {
+                          const ColdMask& cold, int* idx, int* counts, int* cu_rows, int* done_ctr,
+                          int* user_counts, cudaStream_t s) {
   const int threads = (n_tok + 31) / 32 * 32;
-  return launch_ex(select_kernel, dim3(sv), dim3(threads), n_tok * sizeof(float), s, 1, sims, n_tok, sv,
-                   mode, tau, topk, cold, idx, counts, cu_rows, rowtok, done_ctr, user_counts, g_stamp);
+  return launch_ex(select_kernel, dim3(sv), dim3(threads), 0, s, 1, sims, n_tok, sv, mode, tau, topk, cold, idx,
+                   counts, cu_rows, done_ctr, user_counts, g_stamp);
 }
 
-cudaError_t launch_gather(const int* cu_rows_total, const int* rowtok, const float* e_t,
+cudaError_t launch_gather(const int* cu_rows_total, int* rowtok, const RowLists& lists, const float* e_t,
                           const float* pos, float* x, const float* ref_src, float* e_ref, int n_tok,
                           int dim, int ref_last_refresh, const ColdMask& cold, int max_rows, int grid,
                           cudaStream_t s, const RowBands& bands) {
@@ -727,11 +715,11 @@ cudaError_t launch_gather(const int* cu_rows_total, const int* rowtok, const flo
       attr = true;
     }
     grid = max(1, min(grid, (max_rows + GATHER_RPC - 1) / GATHER_RPC));
-    return launch_ex(gather_bulk_kernel, dim3(grid), dim3(256), smem, s, 1, cu_rows_total, rowtok, e_t, pos, x,
+    return launch_ex(gather_bulk_kernel, dim3(grid), dim3(256), smem, s, 1, cu_rows_total, rowtok, lists, e_t, pos, x,
                      ref_src, e_ref, n_tok, dim, ref_last_refresh, cold, bands, g_stamp);
   }
   grid = max(1, min(grid, (max_rows + 7) / 8));
-  return launch_ex(gather_kernel, dim3(grid), dim3(256), 0, s, 1, cu_rows_total, rowtok, e_t, pos, x,
+  return launch_ex(gather_kernel, dim3(grid), dim3(256), 0, s, 1, cu_rows_total, rowtok, lists, e_t, pos, x,
                    ref_src, e_ref, n_tok, dim, ref_last_refresh, cold, bands, g_stamp);
 }
 

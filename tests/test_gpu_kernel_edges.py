@@ -73,3 +73,37 @@ ATTN_SHAPES = [((1, 1), 2, 64, 8), ((5, 19), 2, 64, 4), ((3, 33), 1, 128, 4), ((
                          ids=[f"n{g[0] * g[1]}x{v}_dh{d // h}" for g, v, d, h in ATTN_SHAPES])
 def test_attention_block_edges(pkg, oracle_mod, grid, views, dim, heads):
     _run(pkg, oracle_mod, grid, views, dim, heads, 2 * dim, 2, 0.5)
+
+
+@pytest.mark.parametrize("with_nan", [False, True], ids=["finite", "nan"])
+@pytest.mark.parametrize("n_tok", [1, 31, 33, 200, 1024])
+def test_topk_selection_ties(pkg, n_tok, with_nan):
+    """Scores from a handful of values (-1 ... 1, zero vectors, NaN), so that every k falls into a
+    run of equal ones: exactly the order (score, index), a NaN beside the k lowest of the rest."""
+    import torch
+    from paper_2607_12287_gb300 import synth
+
+    rng = np.random.default_rng(n_tok)
+    views, dim = 2, 64
+    cos = rng.choice([-1.0, -0.5, 0.0, 0.25, 0.5, 1.0], size=(views, n_tok))
+    cur = np.zeros((views, n_tok, dim), np.float32)
+    cur[..., 0], cur[..., 1] = cos, np.sqrt(1 - cos ** 2)
+    zero = rng.random((views, n_tok)) < 0.1  # a zero vector's score is 0
+    cur[zero], cos[zero] = 0, 0.0
+    if with_nan:
+        nan = rng.random((views, n_tok)) < 0.05
+        cur[nan], cos[nan] = np.nan, np.nan
+    ref = np.zeros_like(cur)
+    ref[..., 0] = 1
+    d_cur, d_ref = torch.from_numpy(cur).cuda(), torch.from_numpy(ref).cuda()
+    idx = torch.empty(views, n_tok, dtype=torch.int32, device="cuda")
+    cnt = torch.empty(views, dtype=torch.int32, device="cuda")
+    for k in sorted({0, 1, n_tok // 3, n_tok - 1, n_tok, n_tok + 5}):
+        pkg.ivit_select_noalloc(d_cur, d_ref, views, n_tok, dim, synth.SEL_TOPK, 0.0, k, idx, cnt)
+        for v in range(views):
+            c = cos[v]
+            order = [i for i in np.argsort(np.where(np.isnan(c), np.inf, c), kind="stable") if not np.isnan(c[i])]
+            want = sorted(order[:k] + [i for i in range(n_tok) if np.isnan(c[i]) and k > 0])
+            got = idx[v].cpu().numpy()
+            assert int(cnt[v]) == len(want), (k, v)
+            assert got[: len(want)].tolist() == want and (got[len(want):] == -1).all(), (k, v)
