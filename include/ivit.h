@@ -219,8 +219,8 @@ int ivit_select_noalloc(const float* e_cur_dev, const float* e_ref_dev, int32_t 
  * prediction, all computed by the caller: this library holds neither network.  Needs no
  * handle; enqueued on `stream`, no allocation.  IVIT_ERR_ARG for negative sizes, a
  * NULL required pointer or a pointer that is not 4-byte aligned (checked before any
- * device work); batch * dim == 0 does nothing.  128-bit accesses are used when dim is a
- * multiple of 4 and the arrays are 16-byte aligned, scalar ones otherwise. */
+ * device work); batch * dim == 0 does nothing.  128-bit accesses are used when the arrays
+ * are 16-byte aligned, scalar ones otherwise. */
 int ivit_action_combine(const float* x0_dev, const float* v0_dev, const float* v7_dev,
                         const float* alpha_dev, const float* beta_dev, const float* b_dev,
                         int32_t batch, int32_t dim, float* xT_dev, void* stream);

@@ -107,3 +107,24 @@ def test_topk_selection_ties(pkg, n_tok, with_nan):
             got = idx[v].cpu().numpy()
             assert int(cnt[v]) == len(want), (k, v)
             assert got[: len(want)].tolist() == want and (got[len(want):] == -1).all(), (k, v)
+
+
+@pytest.mark.parametrize("bias", [False, True], ids=["nobias", "bias"])
+@pytest.mark.parametrize("batch,width", [(1, 1), (1, 3), (5, 1), (7, 2), (9, 3), (33, 5), (11, 7), (4096, 350), (257, 1023)])
+def test_action_combine_rows_of_any_width(pkg, batch, width, bias):
+    """128-bit accesses over rows that are no multiple of four values: every value is the same two
+    fused multiply-adds (and addition) in fp32, whichever loop it takes."""
+    import torch
+
+    g = torch.Generator().manual_seed(batch)
+    x0, v0, v7, b = (torch.randn(batch, width, generator=g) for _ in range(4))
+    al, be = (torch.rand(batch, generator=g) for _ in range(2))
+    out = torch.full((batch, width), float("nan"), device="cuda")
+    dev = [t.cuda() for t in (x0, v0, v7, al, be, b)]
+    pkg.ivit_action_combine(*dev[:5], dev[5] if bias else None, out)
+    d = [t.double() for t in (x0, v0, v7, al, be, b)]
+    inner = (d[3][:, None] * d[1] + d[0]).float().double()  # fp64 holds the product exactly: fmaf's rounding
+    want = (d[4][:, None] * d[2] + inner).float()
+    want = (want.double() + (d[5] if bias else 0.0)).float()
+    # (an fp64 sum rounds once before the rounding to fp32: at most the last bit in a tie)
+    assert torch.allclose(out.cpu(), want, rtol=2 ** -23, atol=2 ** -23)
