@@ -92,11 +92,26 @@ def load(path: str = LIB_PATH) -> C.CDLL:
 def _ptr(t) -> Optional[int]:
     if t is None:
         return None
+    if type(t) is _dtypes.get("tensor"):
+        return t.data_ptr()
     if isinstance(t, int):
         return t
     if isinstance(t, np.ndarray):
         return t.ctypes.data
     return t.data_ptr()
+
+
+_dtypes = {}  # torch dtypes by name, and torch.Tensor: filled on the first check (torch is imported late)
+
+
+def _tensor_type():
+    t = _dtypes.get("tensor")
+    if t is None:
+        import torch
+        for name in ("uint8", "int32", "float32", "bfloat16"):
+            _dtypes[name] = getattr(torch, name)
+        t = _dtypes["tensor"] = torch.Tensor
+    return t
 
 
 def _require(t, name: str, dtype_name: str, numel: int) -> None:
@@ -105,6 +120,10 @@ def _require(t, name: str, dtype_name: str, numel: int) -> None:
     non-contiguous view, or one with fewer than ``numel`` elements.  ``None`` (an optional
     output) and raw integer pointers pass unchecked: the caller vouches for those."""
     if t is None or isinstance(t, int):
+        return
+    # the common case: the checks below without formatting names
+    if (type(t) is _tensor_type() and t.is_cuda and t.dtype is _dtypes[dtype_name] and t.is_contiguous()
+            and t.numel() >= numel):
         return
     if isinstance(t, np.ndarray):
         raise TypeError(f"{name}: a numpy array (host memory); a CUDA tensor is required")
@@ -126,7 +145,8 @@ _dims = {}
 def _stream(stream) -> Optional[int]:
     if stream is None:
         import torch
-        return torch.cuda.current_stream().cuda_stream
+        raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)  # (without building a Stream object)
+        return raw(torch.cuda.current_device()) if raw else torch.cuda.current_stream().cuda_stream
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
@@ -252,14 +272,17 @@ def ivit_action_combine(x0, v0, v7, alpha, beta, b, xT, stream=None) -> None:
     alpha, beta fp32 [B]."""
     if x0.dim() != 2:
         raise ValueError(f"x0: shape {tuple(x0.shape)}, expected [batch, action width]")
-    B, A = int(x0.shape[0]), int(x0.shape[1])
-    for t, name in ((x0, "x0"), (v0, "v0"), (v7, "v7"), (b, "b"), (xT, "xT")):
-        _require(t, name, "float32", B * A)
+    B, A = x0.shape
+    n = B * A
+    _require(x0, "x0", "float32", n)
+    _require(v0, "v0", "float32", n)
+    _require(v7, "v7", "float32", n)
+    _require(b, "b", "float32", n)
+    _require(xT, "xT", "float32", n)
     _require(alpha, "alpha", "float32", B)
     _require(beta, "beta", "float32", B)
-    _check(load().ivit_action_combine(_ptr(x0), _ptr(v0), _ptr(v7), _ptr(alpha), _ptr(beta),
-                                      _ptr(b) if b is not None else None, B, A, _ptr(xT),
-                                      _stream(stream)), None)
+    _check(load().ivit_action_combine(_ptr(x0), _ptr(v0), _ptr(v7), _ptr(alpha), _ptr(beta), _ptr(b), B, A,
+                                      _ptr(xT), _stream(stream)), None)
 
 
 # ------------------------------------------------------------ convenience
