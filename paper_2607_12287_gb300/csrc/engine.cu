@@ -278,12 +278,12 @@ size_t defer_slots(const GemmPlan& pl, int n_out, int m_bound) {
 // launches on GB300 of the SigLIP-So400m and ViT-Tiny shapes at 16 to 32768 rows.
 //   CTA pairs: a fixed part (prologue, first loads, last tile's epilogue) plus a k-block
 //     (64 wide) rate per round of units over the 76 pairs; 64-, 128- and 256-row tiles
-//     measured 4.3 / 4.8 / 6.2 us + 0.20 / 0.24 / 0.33 us per k-block, and 0.7 us for the
+//     measured 4.3 / 4.8 / 6.2 us + 0.165 / 0.24 / 0.33 us per k-block, and 0.7 us for the
 //     prologue that its shared memory keeps from running under the previous kernel.
 //   Few rows (`few`: the epilogues that kernel has): 1.1 us, then per pass of 32 rows and
 //     round of CTAs over the SMs 0.9 us and 0.15 to 0.36 us per chunk (32 wide) of a warp for 8
-//     to 32 features per CTA.  QKV of 26 rows 4.0 us against 7.9 in pairs, of 64 rows 6.6
-//     against 7.9, of 128 rows 11.1 against 7.9.
+//     to 32 features per CTA.  QKV of 26 rows 4.0 us against 7.2 in pairs, of 64 rows 6.6
+//     against 7.2, of 128 rows 11.1 against 7.2.
 //   Deferred (residual GEMMs, `defer`): the next layer norm sums the partial tiles: no
 //     epilogue, but every split's fp32 tile is written and read once (about 4 TB/s through L2).
 GemmPlan plan_gemm(int num_sms, int n_out, int k, int m_expected, int m_bound, bool few, bool defer) {
@@ -302,7 +302,7 @@ GemmPlan plan_gemm(int num_sms, int n_out, int k, int m_expected, int m_bound, b
   };
   const int n_ft = (n_out + 127) / 128, n_kb = (k + 63) / 64, max_pairs = num_sms / 2;
   for (int bn : {64, 128, 256}) {
-    const double fixed = bn == 64 ? 5.0 : bn == 128 ? 5.5 : 6.9, per_kb = bn == 64 ? 0.20 : bn == 128 ? 0.24 : 0.33;
+    const double fixed = bn == 64 ? 5.0 : bn == 128 ? 5.5 : 6.9, per_kb = bn == 64 ? 0.165 : bn == 128 ? 0.24 : 0.33;
     const int tiles = std::max(1, (n_ft + 1) / 2 * ((m_expected + bn - 1) / bn));
     for (int c = 1; c <= std::min(defer ? 16 : 1, n_kb); ++c) {
       GemmPlan pl;
@@ -598,6 +598,14 @@ int setup(ivit_handle* h, const uint16_t* wb) {
         h->plan_band[b][g] = g == kGemmEmbed || h->band_ub[b] >= m_all ? h->plan_full[g]
                                                                        : plan(h->band_ub[b], h->band_ub[b]);
     }
+    // (a switch between equal plans would only cost its dispatch, about 10 us)
+    auto same = [](const GemmPlan& a, const GemmPlan& b) {
+      return a.nt == b.nt && a.bn == b.bn && a.splits == b.splits && a.n_pairs == b.n_pairs;
+    };
+    bool differ = false;
+    for (int b = 1; b < h->n_bands; ++b)
+      for (int g = 0; g < kGemmSlots; ++g) differ = differ || !same(h->plan_band[b][g], h->plan_band[0][g]);
+    if (!differ) h->n_bands = 1;
     // every row's D x D projection without a residual (first-layer key scores)
     h->plan_keys = plan_gemm(h->num_sms, static_cast<int>(D), static_cast<int>(D), m_all, m_all, false, false);
     if (std::getenv("IVIT_DEBUG")) {

@@ -22,8 +22,8 @@
 //     so it is never loaded.
 // Measured back to back, random bf16 data, before -> now: 32768 rows QKV 422 -> 159 us, up
 // 497 -> 203, out 154 -> 82, down 324 -> 211 (1540 TFLOP/s); 3080 rows QKV 65 -> 22, up
-// 60 -> 24, down 53 -> 26; 768 rows QKV 29 -> 12, up 27 -> 12; 256 rows QKV 16 -> 8, up
-// 16 -> 8.5.
+// 60 -> 24, down 53 -> 26; 768 rows QKV 29 -> 12, up 27 -> 12; 256 rows QKV 16 -> 7.6,
+// up 16 -> 7.8.
 #include "internal.h"
 #include "ptx.cuh"
 
@@ -37,11 +37,18 @@ constexpr int EPI_WARPS = 8;
 constexpr int THREADS = (EPI_WARPS + 2) * 32;
 constexpr int EPI_HALF = 8192;  // staging of one row half: 32 rows of 128 bf16 or 16 of fp32
 
-// Stages: more than 6 (8 for 64 rows) measured no faster; 4 lost 10 % below 768 rows.
+// Six stages of one k-block, or four of two: more measured no faster, four of one lost 10 %
+// below 768 rows.
 template <int BN>
 struct PairCfg {
-  static constexpr int STAGES = BN == 64 ? 8 : 6;
-  static constexpr int STAGE_BYTES = W_BYTES + BN / 2 * BK * 2;
+  // k-blocks per stage: 64-row tiles are bound by the issuing warps, not by the MMAs, so they
+  // take two per barrier (0.20 -> 0.16 us per k-block; up of 256 rows 8.5 -> 7.8 us)
+  static constexpr int KS = BN == 64 ? 2 : 1;
+  static constexpr int STAGES = BN == 64 ? 4 : 6;
+  static constexpr int X_BYTES = BN / 2 * BK * 2;
+  static constexpr int X_OFFSET = KS * W_BYTES;
+  static constexpr int KB_BYTES = W_BYTES + X_BYTES;
+  static constexpr int STAGE_BYTES = KS * KB_BYTES;
   static constexpr int EPI_OFFSET = STAGES * STAGE_BYTES;
   static constexpr int BAR_OFFSET = EPI_OFFSET + 2 * EPI_HALF;
   static constexpr int TOTAL = BAR_OFFSET + 256 + 1024;  // barriers, flags, 1 KB alignment slack
@@ -150,7 +157,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     gemm_pair_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_x,
                      const GemmArgs a) {
   using C = PairCfg<BN>;
-  constexpr int STAGES = C::STAGES;
+  constexpr int STAGES = C::STAGES, KS = C::KS;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~static_cast<uintptr_t>(1023));
@@ -201,13 +208,14 @@ __global__ void __launch_bounds__(THREADS, 1)
     // the first unit's weight stages do not depend on earlier kernels
     const int sp = pair % splits, ft = 2 * (pair / splits % n_fp) + rank;
     const int kb0 = sp * n_kb / splits, kb1 = (sp + 1) * n_kb / splits;
-    n_pre = min(STAGES, kb1 - kb0);
+    n_pre = min(STAGES * KS, kb1 - kb0);
     if (elect_one()) {
       const uint64_t pol_w = l2_policy_evict_first();
       for (int i = 0; i < n_pre; ++i) {
-        if (rank == 0) mbar_arrive_expect_tx(bar_base + 8 * i, 2 * C::STAGE_BYTES);
-        tma_load_2d_pair(smem_base + i * C::STAGE_BYTES, &tm_w, (kb0 + i) * BK, ft * BM,
-                         mapa_shared(bar_base + 8 * i, 0), pol_w);
+        const int st = i / KS, j = i - st * KS;
+        if (rank == 0 && j == 0) mbar_arrive_expect_tx(bar_base + 8 * st, 2 * min(KS, n_pre - i) * C::KB_BYTES);
+        tma_load_2d_pair(smem_base + st * C::STAGE_BYTES + j * W_BYTES, &tm_w, (kb0 + i) * BK, ft * BM,
+                         mapa_shared(bar_base + 8 * st, 0), pol_w);
       }
     }
     __syncwarp();
@@ -227,7 +235,8 @@ __global__ void __launch_bounds__(THREADS, 1)
       const int half = half_of(rows_of(tt));
       const int xrow = tt * BN + rank * half;
       const int kb0 = sp * n_kb / splits, kb1 = (sp + 1) * n_kb / splits;
-      for (int kb = kb0; kb < kb1; ++kb) {
+      for (int kb = kb0; kb < kb1; kb += KS) {
+        const int nk = min(KS, kb1 - kb);
         const uint32_t full = full0 + 8 * stage;
         const uint32_t st = smem_base + stage * C::STAGE_BYTES;
         const bool pre = first && kb - kb0 < n_pre;
@@ -235,10 +244,15 @@ __global__ void __launch_bounds__(THREADS, 1)
         if (!ok) break;
         if (elect_one()) {
           if (!pre) {
-            if (rank == 0) mbar_arrive_expect_tx(bar_base + 8 * stage, 2 * C::STAGE_BYTES);
-            tma_load_2d_pair(st, &tm_w, kb * BK, ft * BM, full, pol_w);
+            if (rank == 0) mbar_arrive_expect_tx(bar_base + 8 * stage, 2 * nk * C::KB_BYTES);
+#pragma unroll
+            for (int j = 0; j < KS; ++j)
+              if (j < nk) tma_load_2d_pair(st + j * W_BYTES, &tm_w, (kb + j) * BK, ft * BM, full, pol_w);
           }
-          tma_load_2d_pair(st + W_BYTES, &tm_x, kb * BK, xrow, full, pol_x);
+#pragma unroll
+          for (int j = 0; j < KS; ++j)
+            if (j < nk)
+              tma_load_2d_pair(st + C::X_OFFSET + j * C::X_BYTES, &tm_x, (kb + j) * BK, xrow, full, pol_x);
         }
         __syncwarp();
         if (++stage == STAGES) {
@@ -264,16 +278,21 @@ __global__ void __launch_bounds__(THREADS, 1)
         bool ok = mbar_wait(acce + 8 * b, ((iter >> 1) & 1) ^ 1);
         tc_fence_after();
         const uint32_t acc = tmem + static_cast<uint32_t>(b * BN);
-        for (int kb = kb0; kb < kb1; ++kb) {
+        for (int kb = kb0; kb < kb1; kb += KS) {
           ok = ok && mbar_wait(bar_base + 8 * stage, phase);
           if (!__all_sync(0xffffffffu, ok)) break;
           tc_fence_after();
           if (elect_one()) {
             const uint64_t da = desc0 + static_cast<uint64_t>(stage * (C::STAGE_BYTES >> 4));
-            const uint64_t db = da + (W_BYTES >> 4);
+            const uint64_t db = da + (C::X_OFFSET >> 4);
 #pragma unroll
-            for (int k = 0; k < BK / 16; ++k)
-              umma_bf16_pair(acc, da + 2 * k, db + 2 * k, idesc, (kb > kb0 || k > 0) ? 1u : 0u);
+            for (int j = 0; j < KS; ++j) {
+              if (kb + j >= kb1) break;
+#pragma unroll
+              for (int k = 0; k < BK / 16; ++k)
+                umma_bf16_pair(acc, da + j * (W_BYTES >> 4) + 2 * k, db + j * (C::X_BYTES >> 4) + 2 * k, idesc,
+                               (kb > kb0 || j > 0 || k > 0) ? 1u : 0u);
+            }
             umma_commit_pair(bar_base + 8 * (STAGES + stage));
           }
           __syncwarp();
