@@ -285,7 +285,7 @@ size_t defer_slots(const GemmPlan& pl, int n_out, int m_bound) {
 //     to 32 features per CTA.  QKV of 26 rows 4.0 us against 7.2 in pairs, of 64 rows 6.6
 //     against 7.2, of 128 rows 11.1 against 7.2.
 //   Deferred (residual GEMMs, `defer`): the next layer norm sums the partial tiles: no
-//     epilogue, but every split's fp32 tile is written and read once (about 4 TB/s through L2).
+//     epilogue, but every split's fp32 tile is written and read once (about 10 TB/s, in L2).
 GemmPlan plan_gemm(int num_sms, int n_out, int k, int m_expected, int m_bound, bool few, bool defer) {
   GemmPlan best;
   double best_cost = 1e30;
@@ -293,7 +293,7 @@ GemmPlan plan_gemm(int num_sms, int n_out, int k, int m_expected, int m_bound, b
   auto consider = [&](const GemmPlan& pl, double cost) {
     if (pl.defer) {
       if (defer_slots(pl, n_out, m_bound) * pl.bn * 128 * 4 > (64ull << 20)) return;
-      cost += pl.splits * (8.0 * n_out) * m_expected / 4.0e6;
+      cost += pl.splits * (8.0 * n_out) * m_expected / 1.0e7;
     }
     if (cost < best_cost - 1e-9) {
       best_cost = cost;

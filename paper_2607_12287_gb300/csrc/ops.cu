@@ -376,7 +376,7 @@ __global__ void layernorm_kernel(const int* __restrict__ nrows, float* __restric
 // the row per thread, so every split's partial of every element is in flight at once
 // (a row's partials are spread over the csize slots of its feature tiles).  kGather: the row
 // is src_rowtok[r], and x is not written; kAdd: a row of `add` is added as well.  MAXS: the
-// most splits, 4 or 16, whose partials a thread holds: with room for 16 (135 registers) one CTA
+// most splits, 4, 8 or 16, whose partials a thread holds: with room for 16 (135 registers) one CTA
 // fits on an SM, and 256 rows of the So400m width ran in two waves, 4.1 us against 2.0.
 template <int MAXS, bool kGather, bool kAdd>
 __global__ void layernorm_sum_kernel(const int* __restrict__ nrows, float* __restrict__ x, const PendingSum ps,
@@ -738,13 +738,18 @@ cudaError_t launch_layernorm_sum(const int* rows, float* x, const PendingSum& ps
     return cudaErrorInvalidValue;
   const int threads = (dim / 4 + 31) / 32 * 32;
   grid = max(1, min(grid, max_rows));
-  const bool few = ps.csize <= 4;
-  auto kern = add ? (few ? layernorm_sum_kernel<4, false, true> : layernorm_sum_kernel<16, false, true>)
-              : src_rowtok
-                  ? (few ? layernorm_sum_kernel<4, true, false> : layernorm_sum_kernel<16, true, false>)
-                  : (few ? layernorm_sum_kernel<4, false, false> : layernorm_sum_kernel<16, false, false>);
-  return launch_ex(kern, dim3(grid), dim3(threads), 0, s, 1, rows, x, ps, add, src_rowtok, gamma, beta, y, dst_rowtok,
-                   dim, eps, g_stamp);
+  auto launch = [&](auto plain, auto gather, auto with_add) {
+    return launch_ex(add ? with_add : (src_rowtok ? gather : plain), dim3(grid), dim3(threads), 0, s, 1, rows, x, ps, add,
+                     src_rowtok, gamma, beta, y, dst_rowtok, dim, eps, g_stamp);
+  };
+  if (ps.csize <= 4)
+    return launch(layernorm_sum_kernel<4, false, false>, layernorm_sum_kernel<4, true, false>,
+                  layernorm_sum_kernel<4, false, true>);
+  if (ps.csize <= 8)
+    return launch(layernorm_sum_kernel<8, false, false>, layernorm_sum_kernel<8, true, false>,
+                  layernorm_sum_kernel<8, false, true>);
+  return launch(layernorm_sum_kernel<16, false, false>, layernorm_sum_kernel<16, true, false>,
+                layernorm_sum_kernel<16, false, true>);
 }
 
 cudaError_t launch_layernorm_ex(const int* rows, float* x, const float* add, const int* src_rowtok,
