@@ -37,14 +37,15 @@ constexpr int EPI_WARPS = 8;
 constexpr int THREADS = (EPI_WARPS + 2) * 32;
 constexpr int EPI_HALF = 8192;  // staging of one row half: 32 rows of 128 bf16 or 16 of fp32
 
-// Six stages of one k-block, or four of two: more measured no faster, four of one lost 10 %
-// below 768 rows.
+// As many stages as fit for the two smaller tiles: the first ones hold weights requested before
+// the wait on the previous kernel.  64-row tiles with 2 / 3 / 4 / 5 stages: four-layer 224 px
+// full encode 221 / 200 / 192 / 189 us.
 template <int BN>
 struct PairCfg {
   // k-blocks per stage: 64-row tiles are bound by the issuing warps, not by the MMAs, so they
   // take two per barrier (0.20 -> 0.16 us per k-block; up of 256 rows 8.5 -> 7.8 us)
   static constexpr int KS = BN == 64 ? 2 : 1;
-  static constexpr int STAGES = BN == 64 ? 4 : 6;
+  static constexpr int STAGES = BN == 64 ? 5 : BN == 128 ? 8 : 6;
   static constexpr int X_BYTES = BN / 2 * BK * 2;
   static constexpr int X_OFFSET = KS * W_BYTES;
   static constexpr int KB_BYTES = W_BYTES + X_BYTES;
