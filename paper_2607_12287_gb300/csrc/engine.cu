@@ -197,15 +197,13 @@ struct ivit_handle {
   size_t sk_sync_bytes = 0;
   ivit::StreamArgs sk_args{};
 
-  // CUDA graphs of the full and the steady-state incremental chain.  Inputs and outputs
-  // are staged through handle-owned buffers (copies outside the graph), so the graph's
-  // kernel parameters never change.
+  // CUDA graphs of the full and the steady-state incremental chain.  The kernels that see the
+  // caller's pointers (patchify before it, the output copy after it) are launched outside the
+  // graph, so its kernel parameters never change.
   bool use_graphs = true;
   cudaStream_t cap_stream = nullptr;
   cudaGraphExec_t graph_full = nullptr, graph_inc = nullptr;
   int64_t graph_full_launches = 0, graph_inc_launches = 0;
-  uint8_t* frames_buf = nullptr;
-  int* counts_buf = nullptr;
 
   // Timeline mode (ivit_timeline): every launch of a call writes per-CTA start/end
   // stamps into its slot of `stamps`; `slots_*` record each slot's kernel family and,
@@ -729,8 +727,6 @@ int setup(ivit_handle* h, const uint16_t* wb) {
   }
   const size_t o_gpart = sa.take(part_floats * 4);
   const size_t o_rta = sa.take(M * 4), o_mall = sa.take(4);
-  const size_t o_fb = sa.take(static_cast<size_t>(h->SV) * c.img_h * c.img_w * 3);
-  const size_t o_cb = sa.take(h->SV * 4);
   IVIT_CK(h, cudaMalloc(&h->smem, sa.size));
   IVIT_CK(h, cudaMemset(h->smem, 0, sa.size));
   sa.base = static_cast<char*>(h->smem);
@@ -766,8 +762,6 @@ int setup(ivit_handle* h, const uint16_t* wb) {
   }
   if (!make_map(&h->tm_wk0, h->layers[0].wqkv + D * D, D, D, D * 2, 64, 128))
     return h->fail(IVIT_ERR_CUDA, "cuTensorMapEncodeTiled failed for the first-layer key projection");
-  h->frames_buf = sa.at<uint8_t>(o_fb);
-  h->counts_buf = sa.at<int>(o_cb);
   const int kps = ivit::attention_keys_per_split(h->N);
   const int dh = h->D / h->H, kb = ivit::attention_key_block((dh + 15) & ~15);
   for (size_t l = 0; l < L; ++l) {
@@ -1176,8 +1170,28 @@ int capture_band_bodies(ivit_handle* h, cudaStream_t s) {
   return IVIT_OK;
 }
 
-// Enqueues the whole chain for one frame per view on `s` (eagerly or under capture).
-int run_core(ivit_handle* h, const uint8_t* frames, int32_t* user_counts, bool full, cudaStream_t s) {
+// The start of a call's launch record; its first launch is patchify.
+void begin_record(ivit_handle* h) {
+  h->launches = 0;
+  h->slots_cur.clear();
+  h->stamp_used = 0;
+  next_launch(h, kFamOther, nullptr, 0);
+}
+
+// The call's first kernel, from the caller's frames (eager, also before a replayed graph).
+int run_patchify(ivit_handle* h, const uint8_t* frames, cudaStream_t s) {
+  const ivit_config& c = h->cfg;
+  if (h->timeline && h->stamps)  // CTAs that leave early write nothing: clear the last call's stamps
+    IVIT_CK(h, cudaMemsetAsync(h->stamps, 0, static_cast<size_t>(h->stamp_cap) * 2 * ivit::kStampCtas *
+                                                 sizeof(unsigned long long), s));
+  begin_record(h);
+  IVIT_CK(h, ivit::launch_patchify(frames, h->patches, h->SV, c.img_h, c.img_w, c.patch, h->KPAD, s));
+  ++h->launches;
+  return IVIT_OK;
+}
+
+// Enqueues the rest of the chain for one frame per view on `s` (eagerly or under capture).
+int run_core(ivit_handle* h, bool full, cudaStream_t s) {
   const ivit_config& c = h->cfg;
   const int N = h->N, D = h->D, SV = h->SV, M = h->M_max;
   ivit::ColdMask cm;
@@ -1186,16 +1200,7 @@ int run_core(ivit_handle* h, const uint8_t* frames, int32_t* user_counts, bool f
     if (full || h->cold[v]) cm.bits[v >> 5] |= 1u << (v & 31);
   const GemmPlan* plan = full ? h->plan_full : h->plan_inc;
   const int* total = h->cu_rows + SV;
-  h->launches = 0;
-  h->slots_cur.clear();
-  h->stamp_used = 0;
-  if (h->timeline && h->stamps)  // CTAs that leave early write nothing: clear the last call's stamps
-    IVIT_CK(h, cudaMemsetAsync(h->stamps, 0, static_cast<size_t>(h->stamp_cap) * 2 * ivit::kStampCtas *
-                                                 sizeof(unsigned long long), s));
 
-  next_launch(h, kFamOther, nullptr, 0);  // patchify
-  IVIT_CK(h, ivit::launch_patchify(frames, h->patches, SV, c.img_h, c.img_w, c.patch, h->KPAD, s));
-  ++h->launches;
   {
     ivit::GemmArgs a;
     a.n_out = D;
@@ -1237,7 +1242,7 @@ int run_core(ivit_handle* h, const uint8_t* frames, int32_t* user_counts, bool f
   const ivit::RowLists lists{h->idx, h->cu_rows, SV, N};
   next_launch(h, kFamOther, nullptr, 2);  // select
   IVIT_CK(h, ivit::launch_select(h->sims, N, SV, full ? IVIT_SEL_THRESHOLD : c.select_mode, c.threshold,
-                                 c.topk, cm, h->idx, h->counts, h->cu_rows, h->done_ctr, user_counts, s));
+                                 c.topk, cm, h->idx, h->counts, h->cu_rows, h->done_ctr, s));
   ++h->launches;
   if (c.mlp_tokens == IVIT_MLP_ALL) {
     // every token's residual stream (token-indexed), then the references of the updated
@@ -1333,7 +1338,8 @@ int capture(ivit_handle* h, bool full, cudaGraphExec_t* exec, int64_t* launches)
 
 int capture_once(ivit_handle* h, bool full, cudaGraphExec_t* exec, int64_t* launches) {
   IVIT_CK(h, cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal));
-  const int r = run_core(h, h->frames_buf, h->counts_buf, full, h->cap_stream);
+  begin_record(h);
+  const int r = run_core(h, full, h->cap_stream);
   cudaGraph_t g = nullptr;
   const cudaError_t e = cudaStreamEndCapture(h->cap_stream, &g);
   if (r != IVIT_OK) {
@@ -1352,7 +1358,6 @@ int capture_once(ivit_handle* h, bool full, cudaGraphExec_t* exec, int64_t* laun
 int run(ivit_handle* h, const uint8_t* frames, uint16_t* out, int32_t* user_counts, bool full,
         cudaStream_t s) {
   const int SV = h->SV;
-  const size_t tok_bytes = static_cast<size_t>(h->M_max) * h->D * 2;
   bool any_cold = false;
   for (int v = 0; v < SV; ++v) any_cold = any_cold || h->cold[v];
   if (h->use_graphs && (full || !any_cold)) {
@@ -1363,20 +1368,25 @@ int run(ivit_handle* h, const uint8_t* frames, uint16_t* out, int32_t* user_coun
       ivit::g_stamp = nullptr;
       if (r) return r;
     }
+    const int r = run_patchify(h, frames, s);
+    ivit::g_stamp = nullptr;
+    if (r) return r;
     h->slots_last = full ? h->slots_full : h->slots_inc;
-    const size_t fbytes = static_cast<size_t>(SV) * h->cfg.img_h * h->cfg.img_w * 3;
-    IVIT_CK(h, cudaMemcpyAsync(h->frames_buf, frames, fbytes, cudaMemcpyDeviceToDevice, s));
     IVIT_CK(h, cudaGraphLaunch(*exec, s));
-    if (out) IVIT_CK(h, cudaMemcpyAsync(out, h->tok_out, tok_bytes, cudaMemcpyDeviceToDevice, s));
-    if (user_counts)
-      IVIT_CK(h, cudaMemcpyAsync(user_counts, h->counts_buf, SV * sizeof(int), cudaMemcpyDeviceToDevice, s));
-    h->launches = *nl;
+    h->launches += *nl;
   } else {
-    const int r = run_core(h, frames, user_counts, full, s);
+    int r = run_patchify(h, frames, s);
+    if (!r) r = run_core(h, full, s);
     ivit::g_stamp = nullptr;
     if (r) return r;
     h->slots_last = h->slots_cur;
-    if (out) IVIT_CK(h, cudaMemcpyAsync(out, h->tok_out, tok_bytes, cudaMemcpyDeviceToDevice, s));
+  }
+  // every output token (updated ones recomputed, the rest from the final-token cache) and the
+  // views' counts, to the caller
+  if (out || user_counts) {
+    IVIT_CK(h, ivit::launch_outputs(h->tok_out, out, static_cast<size_t>(h->M_max) * h->D * 2, h->counts, user_counts,
+                                    SV, h->num_sms, s));
+    ++h->launches;
   }
   for (int v = 0; v < SV; ++v) h->cold[v] = 0;
 

@@ -208,7 +208,12 @@ cudaError_t launch_score(const float* e_t, float* e_ref, float* sims, int rows, 
 
 cudaError_t launch_select(const float* sims, int n_tok, int sv, int mode, float tau, int topk,
                           const ColdMask& cold, int* idx, int* counts, int* cu_rows, int* done_ctr,
-                          int* user_counts, cudaStream_t s);
+                          cudaStream_t s);
+
+// Copies the final tokens (bytes a multiple of 16) and the views' counts to the caller; either
+// destination may be null or of any alignment.
+cudaError_t launch_outputs(const bf16* tok, void* out, size_t bytes, const int* counts, int* user_counts, int sv,
+                           int num_sms, cudaStream_t s);
 
 // The selection's ascending token lists idx [sv][n_tok] and the views' packed-row offsets
 // cu_rows [sv + 1]; idx null: none.

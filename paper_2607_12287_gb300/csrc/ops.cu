@@ -118,7 +118,7 @@ __global__ void score_kernel(const float* __restrict__ e_t, float* __restrict__ 
 __global__ void select_kernel(const float* __restrict__ sims, int N, int sv, int mode, float tau,
                               int topk, const ColdMask cold, int* __restrict__ idx,
                               int* __restrict__ counts, int* __restrict__ cu_rows, int* __restrict__ done_ctr,
-                              int* __restrict__ user_counts, unsigned long long* stamp) {
+                              unsigned long long* stamp) {
   pdl_wait();
   pdl_launch_dependents();
   stamp_begin(stamp);
@@ -133,7 +133,6 @@ __global__ void select_kernel(const float* __restrict__ sims, int N, int sv, int
   if (flag) idx[static_cast<size_t>(v) * N + pos] = i;
   if (i == 0) {
     counts[v] = total;
-    if (user_counts) user_counts[v] = total;
     __threadfence();
     s_last = (atomicAdd(done_ctr, 1) == sv - 1) ? 1 : 0;
   }
@@ -455,6 +454,26 @@ __global__ void layernorm_sum_kernel(const int* __restrict__ nrows, float* __res
   stamp_end(stamp);
 }
 
+// ---------------------------------------------------------------------- outputs
+// The call's last kernel: the final tokens and the per-view counts, copied to the caller.
+// Four 128-bit loads of a thread are in flight before its first store.
+__global__ void outputs_kernel(const uint4* __restrict__ tok, uint4* __restrict__ out, size_t n,
+                               const int* __restrict__ counts, int* __restrict__ user_counts, int sv) {
+  const size_t first = blockIdx.x * static_cast<size_t>(blockDim.x) + threadIdx.x;
+  const size_t stride = static_cast<size_t>(gridDim.x) * blockDim.x;
+  if (user_counts)
+    for (size_t v = first; v < static_cast<size_t>(sv); v += stride) user_counts[v] = counts[v];
+  for (size_t i = first; i < n; i += 4 * stride) {
+    uint4 u[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (i + k * stride < n) u[k] = tok[i + k * stride];
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (i + k * stride < n) out[i + k * stride] = u[k];
+  }
+}
+
 // -------------------------------------------------------------------- attention
 // Attention of the updated queries of one view over all N keys of that view (cached
 // K/V with this call's updated rows already written), per head:
@@ -693,10 +712,10 @@ cudaError_t launch_score(const float* e_t, float* e_ref, float* sims, int rows, 
 
 cudaError_t launch_select(const float* sims, int n_tok, int sv, int mode, float tau, int topk,
                           const ColdMask& cold, int* idx, int* counts, int* cu_rows, int* done_ctr,
-                          int* user_counts, cudaStream_t s) {
+                          cudaStream_t s) {
   const int threads = (n_tok + 31) / 32 * 32;
   return launch_ex(select_kernel, dim3(sv), dim3(threads), 0, s, 1, sims, n_tok, sv, mode, tau, topk, cold, idx,
-                   counts, cu_rows, done_ctr, user_counts, g_stamp);
+                   counts, cu_rows, done_ctr, g_stamp);
 }
 
 cudaError_t launch_gather(const int* cu_rows_total, int* rowtok, const RowLists& lists, const float* e_t,
@@ -760,6 +779,29 @@ cudaError_t launch_layernorm_ex(const int* rows, float* x, const float* add, con
                   : (src_rowtok ? layernorm_kernel<false, true> : layernorm_kernel<false, false>);
   return launch_ex(kern, dim3(grid), dim3(256), 0, s, 1, rows, x, add, src_rowtok, gamma, beta, y, dst_rowtok, dim,
                    eps, g_stamp);
+}
+
+// (the copy engine's copies take over for pointers that the kernel's accesses do not fit)
+cudaError_t launch_outputs(const bf16* tok, void* out, size_t bytes, const int* counts, int* user_counts, int sv,
+                           int num_sms, cudaStream_t s) {
+  auto fits = [](const void* p, uintptr_t a) { return (reinterpret_cast<uintptr_t>(p) & (a - 1)) == 0; };
+  if (out && !fits(out, 16)) {
+    const cudaError_t e = cudaMemcpyAsync(out, tok, bytes, cudaMemcpyDeviceToDevice, s);
+    if (e != cudaSuccess) return e;
+    out = nullptr;
+  }
+  if (user_counts && !fits(user_counts, 4)) {
+    const cudaError_t e = cudaMemcpyAsync(user_counts, counts, sv * sizeof(int), cudaMemcpyDeviceToDevice, s);
+    if (e != cudaSuccess) return e;
+    user_counts = nullptr;
+  }
+  if (!out && !user_counts) return cudaSuccess;
+  const size_t n = out ? bytes / 16 : 0;
+  const size_t blocks = (n + 4 * 256 - 1) / (4 * 256), most = static_cast<size_t>(num_sms) * 8;
+  const unsigned grid = static_cast<unsigned>(blocks < 1 ? 1 : blocks < most ? blocks : most);
+  outputs_kernel<<<grid, 256, 0, s>>>(reinterpret_cast<const uint4*>(tok), static_cast<uint4*>(out), n, counts,
+                                      user_counts, sv);
+  return cudaGetLastError();
 }
 
 size_t attention_smem(int dh) {

@@ -128,3 +128,26 @@ def test_action_combine_rows_of_any_width(pkg, batch, width, bias):
     want = (want.double() + (d[5] if bias else 0.0)).float()
     # (an fp64 sum rounds once before the rounding to fp32: at most the last bit in a tie)
     assert torch.allclose(out.cpu(), want, rtol=2 ** -23, atol=2 ** -23)
+
+
+@pytest.mark.parametrize("offset", [0, 1, 8], ids=["aligned", "2bytes", "16bytes"])
+def test_outputs_at_any_alignment(pkg, offset):
+    """Tokens into a view that starts `offset` elements into its buffer: the same values, and nothing
+    written outside the view."""
+    import torch
+    from paper_2607_12287_gb300 import synth
+
+    shape = synth.EncoderShape(40, 104, 8, 192, 1, 3, 520, synth.GELU_TANH)
+    enc = pkg.IncrementalViT(shape, synth.make_weights(shape, 3), 1, 2)
+    frames = [torch.from_numpy(f).cuda() for f in synth.stream_random(shape, 2, 2, 11, change_p=0.4)]
+    n = 2 * shape.n_tokens * shape.dim
+    for call in (enc.encode_full, enc.encode_incremental):
+        frame = frames[call == enc.encode_incremental]
+        want = call(frame)
+        want = want[0] if isinstance(want, tuple) else want
+        buf = torch.full((n + 16,), 7.0, dtype=torch.bfloat16, device="cuda")
+        enc.encode_full(frames[0]) if call == enc.encode_incremental else None
+        call(frame, buf[offset:offset + n])
+        assert torch.equal(buf[offset:offset + n], want.reshape(-1))
+        assert (buf[:offset] == 7).all() and (buf[offset + n:] == 7).all()
+    enc.close()
