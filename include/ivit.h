@@ -150,7 +150,7 @@ int ivit_reset(ivit_handle* h, int stream_index);
  * them without it).  Allocates 8 MB of device memory on first use.
  * ivit_timeline_read synchronises `stream` and reads the last call: per kernel family
  * (index 0 tensor-core GEMMs, 1 attention, 2 layer norms, 3 patchify / score /
- * selection / gather) the sum over its launches of (last CTA end - first CTA start)
+ * selection / gather / output copy) the sum over its launches of (last CTA end - first CTA start)
  * in ms and the number of launches (arrays of 4, either may be NULL), the algorithmic
  * bytes of the GEMM launches (weights + input rows + outputs + bias, with this call's
  * updated-row count), and the span from the first start to the last end in ms.  Only

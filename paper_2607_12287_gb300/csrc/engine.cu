@@ -165,6 +165,10 @@ struct ivit_handle {
   bool attn_tc = true;   // tensor-core attention (IVIT_ATTN=simt selects the SIMT kernel)
 
   bf16* patches = nullptr;
+  // Where the reference is the previous frame's patch embeddings, e_t and e_ref are one buffer:
+  // the embedding GEMM's epilogue takes the scores against the content that it overwrites.
+  bool one_ref = false;
+  float4* score_parts = nullptr;  // its sums [feature tiles of 128][M_max]
   float *e_t = nullptr, *e_ref = nullptr, *sims = nullptr, *x = nullptr;
   float* key_t = nullptr;          // first-layer keys of every token (score_source KEY0)
   float* acache = nullptr;         // [L][M_max][D] attention-block outputs (mlp_tokens ALL)
@@ -704,7 +708,10 @@ int setup(ivit_handle* h, const uint16_t* wb) {
 
   // ---- state and workspaces
   Arena sa;
-  const size_t o_patch = sa.take(M * h->KPAD * 2), o_et = sa.take(M * D * 4), o_er = sa.take(M * D * 4);
+  h->one_ref = c.score_source == IVIT_SCORE_EMBED && c.ref_mode == IVIT_REF_PREV_FRAME;
+  const size_t o_patch = sa.take(M * h->KPAD * 2), o_et = sa.take(M * D * 4);
+  const size_t o_er = h->one_ref ? o_et : sa.take(M * D * 4);
+  const size_t o_sp = h->one_ref ? sa.take(M * ((D + 127) / 128) * sizeof(float4)) : 0;
   const size_t o_sims = sa.take(M * 4), o_idx = sa.take(M * 4), o_cnt = sa.take(h->SV * 4);
   const size_t o_cu = sa.take((h->SV + 1) * 4), o_rt = sa.take(M * 4), o_done = sa.take(4);
   const size_t o_x = sa.take(M * D * 4), o_xn = sa.take(M * D * 2), o_q = sa.take(M * D * 2);
@@ -733,6 +740,7 @@ int setup(ivit_handle* h, const uint16_t* wb) {
   h->patches = sa.at<bf16>(o_patch);
   h->e_t = sa.at<float>(o_et);
   h->e_ref = sa.at<float>(o_er);
+  if (h->one_ref) h->score_parts = sa.at<float4>(o_sp);
   h->sims = sa.at<float>(o_sims);
   h->idx = sa.at<int>(o_idx);
   h->counts = sa.at<int>(o_cnt);
@@ -811,7 +819,7 @@ void release(ivit_handle* h) {
 
 // Algorithmic bytes of one GEMM launch at M rows (weights, input rows, output rows, bias).
 double gemm_bytes(int n_out, int k, int kind, long long M) {
-  const double out_b = kind == ivit::kEpiF32Bias ? 4.0 : kind == ivit::kEpiResid ? 8.0 : 2.0;
+  const double out_b = kind == ivit::kEpiF32Bias ? 4.0 : kind == ivit::kEpiResid || kind == ivit::kEpiScore ? 8.0 : 2.0;
   return 2.0 * n_out * k + 2.0 * M * k + out_b * M * n_out + 4.0 * n_out;
 }
 
@@ -1206,13 +1214,15 @@ int run_core(ivit_handle* h, bool full, cudaStream_t s) {
     a.n_out = D;
     a.k = h->KPAD;
     a.m_static = M;
-    a.epi.kind = ivit::kEpiF32Bias;
+    a.epi.kind = h->one_ref && !full ? ivit::kEpiScore : ivit::kEpiF32Bias;
     a.epi.bias = h->b_pe;
     a.epi.out_f32 = h->e_t;
     a.epi.ld_out = D;
+    a.epi.score = h->score_parts;
     if (int r = gemm(h, plan[kGemmEmbed], h->tm_pe, h->w_pe, h->tm_patches, a, s)) return r;
   }
-  const float* score_vec = h->e_t;
+  const float* score_vec = h->e_t;  // what the references of updated tokens are refreshed from
+  if (h->one_ref) score_vec = nullptr;  // (they hold it already)
   if (c.score_source == IVIT_SCORE_KEY0) {
     // Eq. 3 on first-layer keys of every token: W_K LN1(e + pos) + b_K (x, xn are free
     // until the updated rows are gathered below)
@@ -1234,14 +1244,14 @@ int run_core(ivit_handle* h, bool full, cudaStream_t s) {
     if (int r = gemm(h, h->plan_keys, h->tm_wk0, nullptr, h->tm_xn, a, s)) return r;
     score_vec = h->key_t;
   }
-  if (!full) {
+  if (!full && !h->one_ref) {
     next_launch(h, kFamOther, nullptr, 1);  // score
     IVIT_CK(h, ivit::launch_score(score_vec, h->e_ref, h->sims, M, D, c.ref_mode == IVIT_REF_PREV_FRAME, s));
     ++h->launches;
   }
   const ivit::RowLists lists{h->idx, h->cu_rows, SV, N};
   next_launch(h, kFamOther, nullptr, 2);  // select
-  IVIT_CK(h, ivit::launch_select(h->sims, N, SV, full ? IVIT_SEL_THRESHOLD : c.select_mode, c.threshold,
+  IVIT_CK(h, ivit::launch_select(h->sims, h->score_parts, (D + 127) / 128, N, SV, full ? IVIT_SEL_THRESHOLD : c.select_mode, c.threshold,
                                  c.topk, cm, h->idx, h->counts, h->cu_rows, h->done_ctr, s));
   ++h->launches;
   if (c.mlp_tokens == IVIT_MLP_ALL) {
@@ -1384,8 +1394,13 @@ int run(ivit_handle* h, const uint8_t* frames, uint16_t* out, int32_t* user_coun
   // every output token (updated ones recomputed, the rest from the final-token cache) and the
   // views' counts, to the caller
   if (out || user_counts) {
+    h->slots_cur = h->slots_last;  // (a replayed graph's record, or this call's)
+    h->stamp_used = static_cast<int>(h->slots_last.size());
+    next_launch(h, kFamOther, nullptr, 4);
+    h->slots_last = h->slots_cur;
     IVIT_CK(h, ivit::launch_outputs(h->tok_out, out, static_cast<size_t>(h->M_max) * h->D * 2, h->counts, user_counts,
                                     SV, h->num_sms, s));
+    ivit::g_stamp = nullptr;
     ++h->launches;
   }
   for (int v = 0; v < SV; ++v) h->cold[v] = 0;

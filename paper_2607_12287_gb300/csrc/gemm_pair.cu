@@ -70,13 +70,29 @@ __device__ __forceinline__ float gelu_f(float x, int mode) {
   return 0.5f * x * (1.f + tanh_hw(c * (x + 0.044715f * x * x * x)));
 }
 
+// Sums over a warp of three values of four rows each (v[row]): lanes 8 k .. 8 k + 7 get row k's.
+__device__ __forceinline__ float3 sum_rows4(const float3 (&v)[4], int lane) {
+  auto fold = [&](const float3& keep, const float3& send, int o) {
+    return make_float3(keep.x + __shfl_xor_sync(0xffffffffu, send.x, o), keep.y + __shfl_xor_sync(0xffffffffu, send.y, o),
+                       keep.z + __shfl_xor_sync(0xffffffffu, send.z, o));
+  };
+  const bool hi = lane & 16, mid = lane & 8;
+  const float3 p = fold(hi ? v[2] : v[0], hi ? v[0] : v[2], 16), q = fold(hi ? v[3] : v[1], hi ? v[1] : v[3], 16);
+  float3 s = fold(mid ? q : p, mid ? p : q, 8);
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) s = fold(s, s, o);
+  return s;
+}
+
 // Drains rows [c_lo, c_hi) of the tile (columns of this CTA's accumulator) on the four
-// warps of one row half: chunks of 32 rows (16 when fp32) go from tensor memory (lane = feature) through
-// shared memory (row-major) to global memory with 16-byte accesses, 128 features of a row
-// at a time.  `release` is called once, when the accumulator has been read.
-template <int KIND, class Release>
+// warps of one row half: chunks of 32 rows (16 when fp32) go from tensor memory (lane =
+// feature) through shared memory (row-major) to global memory with 16-byte accesses, 128
+// features of a row at a time.  `ready` waits for the accumulator (false: nothing is stored),
+// `release` is called once, when it has been read.
+template <int KIND, class Ready, class Release>
 __device__ __forceinline__ void drain(const GemmArgs& a, uint32_t acc, uint8_t* stg, int bar_id, int wq, int lane,
-                                      int row0, int c_lo, int c_hi, int ft, float* slot, bool ok, Release release) {
+                                      int row0, int c_lo, int c_hi, int ft, float* slot, Ready ready,
+                                      Release release) {
   constexpr bool kBf16 = KIND == kEpiQKV || KIND == kEpiGelu;
   constexpr int CHUNK = kBf16 ? 32 : 16;
   const int f0 = ft * BM, fl = wq * 32 + lane;
@@ -87,7 +103,6 @@ __device__ __forceinline__ void drain(const GemmArgs& a, uint32_t acc, uint8_t* 
   constexpr int FPT = kBf16 ? 8 : 4, LPR = BM / FPT, RPW = 32 / LPR, ITERS = CHUNK / (4 * RPW);
   const int sub = lane % LPR, rsub = wq * RPW + lane / LPR;
   const int f = f0 + FPT * sub;
-  const bool f_ok = ok && f < a.n_out;
   bf16* dst16 = nullptr;
   float* dst32 = nullptr;
   bool by_tok = KIND == kEpiScatterF32;
@@ -105,7 +120,26 @@ __device__ __forceinline__ void drain(const GemmArgs& a, uint32_t acc, uint8_t* 
   } else {
     dst32 = a.epi.out_f32 + f;
   }
-  for (int c0 = c_lo; c0 < c_hi; c0 += CHUNK) {
+  // kEpiScore: the rows' previous content, four chunks ahead (the first ones under the main
+  // loop): one chunk at a time was bound by their latency
+  constexpr int AHEAD = 4;
+  float4 old[KIND == kEpiScore ? AHEAD : 1][ITERS];
+  auto load_old = [&](int c0) {
+    if constexpr (KIND == kEpiScore) {
+#pragma unroll
+      for (int k = 0; k < AHEAD; ++k)
+#pragma unroll
+        for (int i = 0; i < ITERS; ++i) {
+          const int c = c0 + k * CHUNK + i * 4 * RPW + rsub;
+          old[k][i] = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (c < c_hi && f < a.n_out)
+            old[k][i] = __ldcg(reinterpret_cast<const float4*>(dst32 + static_cast<size_t>(row0 + c) * ld));
+        }
+    }
+  };
+  load_old(c_lo);
+  const bool ok = ready(), f_ok = ok && f < a.n_out;
+  auto chunk = [&](int c0, const float4 (&prev)[ITERS]) {
     int rr[ITERS];  // destination rows, -1 past the tile's end
 #pragma unroll
     for (int i = 0; i < ITERS; ++i) {
@@ -138,9 +172,11 @@ __device__ __forceinline__ void drain(const GemmArgs& a, uint32_t acc, uint8_t* 
       for (int j = 0; j < CHUNK; ++j) st[j * BM] = __uint_as_float(v[j]) + bias;
     }
     named_barrier(bar_id, 128);
+    float3 sums[KIND == kEpiScore ? ITERS : 1];
 #pragma unroll
     for (int i = 0; i < ITERS; ++i) {
       const uint4 u = *reinterpret_cast<const uint4*>(stg + ((i * 4 * RPW + rsub) * LPR + sub) * 16);
+      if constexpr (KIND == kEpiScore) sums[i] = make_float3(0.f, 0.f, 0.f);
       if (rr[i] < 0) continue;
       const size_t off = static_cast<size_t>(rr[i]) * ld;
       if (kBf16)
@@ -149,7 +185,29 @@ __device__ __forceinline__ void drain(const GemmArgs& a, uint32_t acc, uint8_t* 
         red_add_f32x4(dst32 + off, *reinterpret_cast<const float4*>(&u));
       else
         *reinterpret_cast<uint4*>(dst32 + off) = u;
+      if constexpr (KIND == kEpiScore) {
+        const float4 x = *reinterpret_cast<const float4*>(&u), y = prev[i];
+        sums[i] = make_float3(x.x * y.x + x.y * y.y + x.z * y.z + x.w * y.w,
+                              x.x * x.x + x.y * x.y + x.z * x.z + x.w * x.w,
+                              y.x * y.x + y.y * y.y + y.z * y.z + y.w * y.w);
+      }
     }
+    if constexpr (KIND == kEpiScore) {  // (a warp holds 128 features of one row per iteration)
+      const float3 s = sum_rows4(sums, lane);
+      const int c = c0 + (lane >> 3) * 4 + wq;
+      if ((lane & 7) == 0 && c < c_hi && ok)
+        a.epi.score[static_cast<size_t>(ft) * a.m_static + row0 + c] = make_float4(s.x, s.y, s.z, 0.f);
+    }
+  };
+  if constexpr (KIND == kEpiScore) {
+    for (int c0 = c_lo; c0 < c_hi; c0 += AHEAD * CHUNK) {
+      if (c0 > c_lo) load_old(c0);
+#pragma unroll
+      for (int k = 0; k < AHEAD; ++k)
+        if (c0 + k * CHUNK < c_hi) chunk(c0 + k * CHUNK, old[k]);
+    }
+  } else {
+    for (int c0 = c_lo; c0 < c_hi; c0 += CHUNK) chunk(c0, old[0]);
   }
 }
 
@@ -321,17 +379,20 @@ __global__ void __launch_bounds__(THREADS, 1)
       const int ft = 2 * (tile % n_fp) + rank, tt = tile / n_fp;
       const int rows = rows_of(tt), hrows = ((rows + 63) >> 6) << 5;
       const int b = iter & 1;
-      // (after an expired wait the loop runs on without waiting or storing, so that the
-      // warps of a half still meet at their named barriers)
-      const bool aborted = *sh_abort != 0;
-      const bool done = !aborted && mbar_wait(accf + 8 * b, (iter >> 1) & 1);
-      if (!done && !aborted) {
-        atomicExch(a.err, kErrWaitAccum);
-        *sh_abort = 1;
-      }
-      tc_fence_after();
       const uint32_t acc = trow + static_cast<uint32_t>(b * BN);
       const uint32_t freed = mapa_shared(acce + 8 * b, 0);
+      // (after an expired wait the loop runs on without waiting or storing, so that the
+      // warps of a half still meet at their named barriers)
+      auto ready = [&]() {
+        const bool aborted = *sh_abort != 0;
+        const bool done = !aborted && mbar_wait(accf + 8 * b, (iter >> 1) & 1);
+        if (!done && !aborted) {
+          atomicExch(a.err, kErrWaitAccum);
+          *sh_abort = 1;
+        }
+        tc_fence_after();
+        return done;
+      };
       auto release = [&]() {
         tc_fence_before();
         __syncwarp();
@@ -341,10 +402,12 @@ __global__ void __launch_bounds__(THREADS, 1)
       float* slot = nullptr;
       if (KIND == kEpiPartial)
         slot = a.partials + (static_cast<size_t>(ft + n_ft * tt) * splits + sp) * BN * BM;
-      if (c_lo < c_hi && ft < n_ft)
-        drain<KIND>(a, acc, stg, 1 + hf, wq, lane, tt * BN, c_lo, c_hi, ft, slot, done, release);
-      else
+      if (c_lo < c_hi && ft < n_ft) {
+        drain<KIND>(a, acc, stg, 1 + hf, wq, lane, tt * BN, c_lo, c_hi, ft, slot, ready, release);
+      } else {
+        ready();
         release();
+      }
     }
   }
   tc_fence_before();
@@ -374,6 +437,7 @@ cudaError_t launch_bn(const CUtensorMap& tm_w, const CUtensorMap& tm_x, const Ge
     case kEpiResid: return launch_one<BN, kEpiResid>(tm_w, tm_x, a, n_pairs, s);
     case kEpiGelu: return launch_one<BN, kEpiGelu>(tm_w, tm_x, a, n_pairs, s);
     case kEpiScatterF32: return launch_one<BN, kEpiScatterF32>(tm_w, tm_x, a, n_pairs, s);
+    case kEpiScore: return launch_one<BN, kEpiScore>(tm_w, tm_x, a, n_pairs, s);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -389,6 +453,7 @@ cudaError_t setup_bn() {
   set(gemm_pair_kernel<BN, kEpiResid>);
   set(gemm_pair_kernel<BN, kEpiGelu>);
   set(gemm_pair_kernel<BN, kEpiScatterF32>);
+  set(gemm_pair_kernel<BN, kEpiScore>);
   set(gemm_pair_kernel<BN, kEpiPartial>);
   return e;
 }

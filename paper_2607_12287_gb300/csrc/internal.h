@@ -57,6 +57,8 @@ enum EpiKind : int {
   kEpiResid = 2,    // out_f32[r][f] += y + bias[f]  (residual stream, fp32)
   kEpiGelu = 3,     // out_bf16[r][f] = gelu(y + bias[f])
   kEpiScatterF32 = 4,  // out_f32[rowtok[r]][f] = y + bias[f]  (per-token output cache)
+  kEpiScore = 6,       // out_f32[r][f] = y + bias[f], and sums for the cosine of row r with its old
+                       // content: score[feature tile of 128 * m_static + r] (Eq. 3)
   kEpiPartial = 5,     // a K split's fp32 tile, left in the scratch (GemmArgs::defer)
 };
 
@@ -68,6 +70,7 @@ struct GemmEpilogue {
   bf16* cache_k = nullptr;       // kEpiQKV: this layer's key cache [SV*N][D]
   bf16* cache_v = nullptr;       // kEpiQKV: this layer's value cache [SV*N][D]
   const int* rowtok = nullptr;   // kEpiQKV: packed row -> token index v*N + i
+  float4* score = nullptr;       // kEpiScore: (<new, old>, |new|^2, |old|^2, 0) over 128 features
   int dim = 0;                   // kEpiQKV: D
   int gelu_mode = 0;             // kEpiGelu: 0 tanh form, 1 erf form
   int ld_out = 0;
@@ -111,7 +114,7 @@ cudaError_t launch_gemm_pair(int bn, const CUtensorMap& tm_w, const CUtensorMap&
                              int n_pairs, cudaStream_t s);
 
 // The same GEMM for a few rows: CTAs of 8 nt features (nt 1..4), rows in passes of 32, every
-// epilogue but kEpiF32Bias.  With defer set, K is split vsplit ways and the slots have 32 rows.
+// epilogue but kEpiF32Bias and kEpiScore.  With defer set, K is split vsplit ways and the slots have 32 rows.
 // k a multiple of 8.
 constexpr int GEMM_ROWS_SMEM_MAX = 160 * 1024;
 size_t gemm_rows_smem(int nt, int k, int splits);
@@ -206,7 +209,8 @@ cudaError_t launch_patchify(const uint8_t* frames, bf16* patches, int sv, int im
 cudaError_t launch_score(const float* e_t, float* e_ref, float* sims, int rows, int dim,
                          int copy_ref, cudaStream_t s);
 
-cudaError_t launch_select(const float* sims, int n_tok, int sv, int mode, float tau, int topk,
+// (scores from sims, or with parts from n_parts sums [n_parts][sv * n_tok] as the embedding GEMM leaves them)
+cudaError_t launch_select(const float* sims, const float4* parts, int n_parts, int n_tok, int sv, int mode, float tau, int topk,
                           const ColdMask& cold, int* idx, int* counts, int* cu_rows, int* done_ctr,
                           cudaStream_t s);
 

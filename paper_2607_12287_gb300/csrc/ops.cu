@@ -111,11 +111,13 @@ __global__ void score_kernel(const float* __restrict__ e_t, float* __restrict__ 
 }
 
 // ----------------------------------------------------------------------- select
-// One CTA per view (blockDim >= N).  flag(i) = cold || sim < tau (threshold mode) or sim(i)
+// One CTA per view (blockDim >= N); scores from sims, or from the partial sums that the
+// embedding GEMM left (parts).  flag(i) = cold || sim < tau (threshold mode) or sim(i)
 // among the k lowest in (sim ascending, index ascending) order (top-k mode).  Flags are
 // compacted in index order into idx[v][.] and counts[v]; the last CTA to finish turns the
 // counts into cu_rows (exclusive prefix, cu_rows[sv] = total rows).
-__global__ void select_kernel(const float* __restrict__ sims, int N, int sv, int mode, float tau,
+__global__ void select_kernel(const float* __restrict__ sims, const float4* __restrict__ parts, int n_parts, int N,
+                              int sv, int mode, float tau,
                               int topk, const ColdMask cold, int* __restrict__ idx,
                               int* __restrict__ counts, int* __restrict__ cu_rows, int* __restrict__ done_ctr,
                               unsigned long long* stamp) {
@@ -126,7 +128,23 @@ __global__ void select_kernel(const float* __restrict__ sims, int N, int sv, int
   __shared__ int s_last;
   const int v = blockIdx.x, i = threadIdx.x;
   const bool c = is_cold(cold, v);
-  const float s = (i < N) ? sims[static_cast<size_t>(v) * N + i] : 0.f;
+  float s = 0.f;
+  if (i < N && !c) {
+    const size_t t = static_cast<size_t>(v) * N + i;
+    if (parts) {  // the cosine from its sums over the feature tiles, in their order
+      float dot = 0.f, na = 0.f, nb = 0.f;
+#pragma unroll 4
+      for (int k = 0; k < n_parts; ++k) {
+        const float4 p = parts[static_cast<size_t>(k) * sv * N + t];
+        dot += p.x;
+        na += p.y;
+        nb += p.z;
+      }
+      s = dot / fmaxf(sqrtf(na) * sqrtf(nb), 1e-12f);
+    } else {
+      s = sims[t];
+    }
+  }
   const bool flag = mode == 1 && !c ? among_lowest(s, i < N, topk, hist, scratch) : i < N && (c || s < tau);
   int total;
   const int pos = block_rank(flag, scratch, total);
@@ -458,7 +476,9 @@ __global__ void layernorm_sum_kernel(const int* __restrict__ nrows, float* __res
 // The call's last kernel: the final tokens and the per-view counts, copied to the caller.
 // Four 128-bit loads of a thread are in flight before its first store.
 __global__ void outputs_kernel(const uint4* __restrict__ tok, uint4* __restrict__ out, size_t n,
-                               const int* __restrict__ counts, int* __restrict__ user_counts, int sv) {
+                               const int* __restrict__ counts, int* __restrict__ user_counts, int sv,
+                               unsigned long long* stamp) {
+  stamp_begin(stamp);
   const size_t first = blockIdx.x * static_cast<size_t>(blockDim.x) + threadIdx.x;
   const size_t stride = static_cast<size_t>(gridDim.x) * blockDim.x;
   if (user_counts)
@@ -472,6 +492,7 @@ __global__ void outputs_kernel(const uint4* __restrict__ tok, uint4* __restrict_
     for (int k = 0; k < 4; ++k)
       if (i + k * stride < n) out[i + k * stride] = u[k];
   }
+  stamp_end(stamp);
 }
 
 // -------------------------------------------------------------------- attention
@@ -710,11 +731,11 @@ cudaError_t launch_score(const float* e_t, float* e_ref, float* sims, int rows, 
   return launch_ex(score_kernel, dim3(grid), dim3(256), 0, s, 1, e_t, e_ref, sims, rows, dim, copy_ref, g_stamp);
 }
 
-cudaError_t launch_select(const float* sims, int n_tok, int sv, int mode, float tau, int topk,
+cudaError_t launch_select(const float* sims, const float4* parts, int n_parts, int n_tok, int sv, int mode, float tau, int topk,
                           const ColdMask& cold, int* idx, int* counts, int* cu_rows, int* done_ctr,
                           cudaStream_t s) {
   const int threads = (n_tok + 31) / 32 * 32;
-  return launch_ex(select_kernel, dim3(sv), dim3(threads), 0, s, 1, sims, n_tok, sv, mode, tau, topk, cold, idx,
+  return launch_ex(select_kernel, dim3(sv), dim3(threads), 0, s, 1, sims, parts, n_parts, n_tok, sv, mode, tau, topk, cold, idx,
                    counts, cu_rows, done_ctr, g_stamp);
 }
 
@@ -800,7 +821,7 @@ cudaError_t launch_outputs(const bf16* tok, void* out, size_t bytes, const int* 
   const size_t blocks = (n + 4 * 256 - 1) / (4 * 256), most = static_cast<size_t>(num_sms) * 8;
   const unsigned grid = static_cast<unsigned>(blocks < 1 ? 1 : blocks < most ? blocks : most);
   outputs_kernel<<<grid, 256, 0, s>>>(reinterpret_cast<const uint4*>(tok), static_cast<uint4*>(out), n, counts,
-                                      user_counts, sv);
+                                      user_counts, sv, g_stamp);
   return cudaGetLastError();
 }
 
