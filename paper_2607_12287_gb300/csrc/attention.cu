@@ -35,6 +35,7 @@
 //          only when a block exceeds it by more than 2^8, which keeps P in bf16's and the
 //          sums in fp32's range; the result does not depend on the reference.  At the end
 //          O / l goes to global memory.
+#include "attention.cuh"
 #include "internal.h"
 #include "ptx.cuh"
 
@@ -63,30 +64,6 @@ struct AttnCfg {
   static constexpr int OFF_CUM = OFF_BAR + 256;  // [sv + 1] items before each view
   static constexpr int BYTES = OFF_CUM + 1024;   // alignment slack
 };
-
-struct Item {
-  int v, h, r0, nq;
-};
-
-// Item g of the call: views in order, in a view the heads, in a head the query tiles, so that
-// the tiles that share keys and values run at the same time (their K and V come from L2).
-// cum[v] = items before view v.
-__device__ __forceinline__ Item item_at(int g, const int* cum, const AttnTcArgs& a) {
-  int lo = 0, hi = a.sv - 1;  // last view with cum[view] <= g
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (cum[mid] <= g) lo = mid; else hi = mid - 1;
-  }
-  Item it;
-  it.v = lo;
-  const int rb = a.cu_rows[lo], m = a.cu_rows[lo + 1] - rb;
-  const int tiles = (m + AQ - 1) / AQ, rem = g - cum[lo];
-  it.h = rem / tiles;
-  const int qt = rem - it.h * tiles;
-  it.r0 = rb + qt * AQ;
-  it.nq = min(AQ, m - qt * AQ);
-  return it;
-}
 
 __device__ __forceinline__ float ex2(float x) {
   float y;
@@ -164,21 +141,7 @@ __global__ void __launch_bounds__(THREADS, 2)
   }
   // The row offsets come from the selection kernel, at least two launches back (every kernel
   // of the library triggers its dependents only after its own wait).
-  if (warp == 0) {
-    int before = 0;
-    for (int v0 = 0; v0 < a.sv; v0 += 32) {
-      const int v = v0 + lane;
-      int n = v < a.sv ? (a.cu_rows[v + 1] - a.cu_rows[v] + AQ - 1) / AQ * a.heads : 0;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int up = __shfl_up_sync(0xffffffffu, n, o);
-        if (lane >= o) n += up;
-      }
-      if (v < a.sv) cum[v + 1] = before + n;
-      before += __shfl_sync(0xffffffffu, n, 31);
-    }
-    if (lane == 0) cum[0] = 0;
-  }
+  attention_items(a, AQ, cum);
   if (warp == 5) {
     tmem_alloc(smem_u32(tslot), C::TM_COLS);
     tmem_relinquish();
@@ -207,7 +170,7 @@ __global__ void __launch_bounds__(THREADS, 2)
     const uint64_t pol_q = l2_policy_evict_first(), pol_kv = l2_policy_evict_last();
     uint32_t t = 0;  // K / V tiles so far
     for (uint32_t n = 0; s < n_items; ++n, s += gridDim.x) {
-      const Item it = item_at(s, cum, a);
+      const AttnItem it = attention_item(s, AQ, cum, a);
       if (!__all_sync(0xffffffffu, wait(q_empty, (n & 1) ^ 1))) break;
       if (elect_one()) {
         mbar_arrive_expect_tx(q_full, C::Q1 + C::Q2);
@@ -291,7 +254,7 @@ __global__ void __launch_bounds__(THREADS, 2)
       if (lane == 0) mbar_arrive(b);
     };
     for (; ok && s < n_items; s += gridDim.x) {
-      const Item it = item_at(s, cum, a);
+      const AttnItem it = attention_item(s, AQ, cum, a);
       const bool wrow = warp * 32 < it.nq;  // warp-uniform: a warp of padding rows only keeps step
       float m_ref = -INFINITY;
       float2 l[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};

@@ -150,7 +150,8 @@ struct ivit_handle {
   int band_ub[4] = {0, 0, 0, 0};
   GemmPlan plan_band[4][kGemmSlots];
   bool capture_bands = false;  // set while the incremental graph is captured with bands
-  int known_band = -1;         // set while it is captured for a row count known in advance
+  int known_band = -1;         // set while it is captured for a row count known in advance,
+  int known_rows = 0;          // this one
   ivit::RowBands bands;        // the switch node's handle and the bands' row bounds
   cudaStream_t cap_stream2 = nullptr;  // captures the band bodies
 
@@ -163,6 +164,7 @@ struct ivit_handle {
   ActMaps tm_patches, tm_xn, tm_o, tm_h;
   ivit::AttnMaps tm_qa;  // packed queries (tcgen05 attention)
   bool attn_tc = true;   // tensor-core attention (IVIT_ATTN=simt selects the SIMT kernel)
+  int attn_forced = -1;  // which of the two (IVIT_ATTN=tc 0, rows 1), -1: attention_few decides
 
   bf16* patches = nullptr;
   // Where the reference is the previous frame's patch embeddings, e_t and e_ref are one buffer:
@@ -333,6 +335,14 @@ GemmPlan plan_gemm(int num_sms, int n_out, int k, int m_expected, int m_bound, b
     }
   }
   return best;
+}
+
+bool attention_few(const ivit_handle* h, int m_expected);
+
+// Updated rows to expect of a call in row band b: a tenth of the tokens in the first, the
+// middle of the others.
+int band_rows(const ivit_handle* h, int b) {
+  return b == 0 ? std::max(1, h->M_max / 10) : (h->band_ub[b - 1] + h->band_ub[b]) / 2;
 }
 
 // Prepares the persistent encoder (IVIT_PATH=persistent: every call runs it) when its shared
@@ -560,7 +570,11 @@ int setup(ivit_handle* h, const uint16_t* wb) {
   IVIT_CK(h, ivit::gemm_pair_setup());
   IVIT_CK(h, ivit::attention_setup());
   IVIT_CK(h, ivit::attention_tc_setup());
-  if (const char* at = std::getenv("IVIT_ATTN")) h->attn_tc = std::string(at) != "simt";
+  IVIT_CK(h, ivit::attention_rows_setup());
+  if (const char* at = std::getenv("IVIT_ATTN")) {
+    h->attn_tc = std::string(at) != "simt";
+    h->attn_forced = std::string(at) == "tc" ? 0 : std::string(at) == "rows" ? 1 : -1;
+  }
   {
     // Row bands: the first holds a tenth of the tokens (rounded up to 16, at least 64),
     // each next one twice the previous, the last all of them; at most four.
@@ -607,6 +621,8 @@ int setup(ivit_handle* h, const uint16_t* wb) {
     bool differ = false;
     for (int b = 1; b < h->n_bands; ++b)
       for (int g = 0; g < kGemmSlots; ++g) differ = differ || !same(h->plan_band[b][g], h->plan_band[0][g]);
+    for (int b = 1; b < h->n_bands; ++b)
+      differ = differ || attention_few(h, band_rows(h, b)) != attention_few(h, band_rows(h, 0));
     if (!differ) h->n_bands = 1;
     // every row's D x D projection without a residual (first-layer key scores)
     h->plan_keys = plan_gemm(h->num_sms, static_cast<int>(D), static_cast<int>(D), m_all, m_all, false, false);
@@ -934,12 +950,37 @@ void print_stream_trace(ivit_handle* h, cudaStream_t s) {
   cudaMemset(h->sk_args.trace, 0, t.size() * sizeof(unsigned long long));
 }
 
-// Attention of the updated queries over all tokens of their view for one layer.
-int attention(ivit_handle* h, const LayerW& w, const bf16* ck, const bf16* cv, bool full, cudaStream_t s) {
+// Whether the few-query attention is the faster one for about m_expected updated rows: a cost
+// model in microseconds per launch, fitted like plan_gemm's.  That kernel takes 2.0 us (1.3 for
+// heads of up to 64) + 1.5 us per 256 keys of a 72-wide head for a round of 16-query items over
+// the SMs; the other one 4.0 us + 1.0 us per key block for a round of 128-query items over two
+// CTAs per SM.  With 16 heads of 72: 26 queries x 256 keys 3.9 us against 6.1, 128 x 256 4.2
+// against 6.9, 256 x 256 7.2 against 7.3 (and 4 % of a full encode slower, for its second round
+// keeps the next kernel out), 100 x 1024 8.7 against 14.4, 32 views of 96 x 1024 171 against 38;
+// 6 views of 196 x 196 with 3 heads of 64 5.6 against 6.8.
+bool attention_few(const ivit_handle* h, int m_expected) {
+  if (h->attn_forced >= 0) return h->attn_forced == 1;
+  const int dh = h->D / h->H;
+  auto rounds = [&](int tile, int ctas) {  // a view's last tile is half full on average
+    const double tiles = std::max<double>(h->SV, static_cast<double>(m_expected) / tile + 0.5 * h->SV);
+    const double full = static_cast<double>(h->SV) * ((h->N + tile - 1) / tile);
+    return std::ceil(h->H * std::min(tiles, full) / ctas);
+  };
+  const int kb = ivit::attention_key_block((dh + 15) & ~15);
+  const double few = 0.4 + rounds(16, h->num_sms) * ((dh <= 64 ? 1.3 : 2.0) + 1.5 * dh / 72.0 * ((h->N + 255) / 256));
+  const double many = 4.0 + rounds(128, 2 * h->num_sms) * ((h->N + kb - 1) / kb);
+  return few < many;
+}
+
+// Attention of the updated queries (about m_expected) over all tokens of their view for one layer.
+int attention(ivit_handle* h, const LayerW& w, const bf16* ck, const bf16* cv, int m_expected, cudaStream_t s) {
   const int N = h->N, D = h->D, SV = h->SV;
   if (h->attn_tc) {
     ivit::AttnTcArgs at;
     at.cu_rows = h->cu_rows;
+    at.q = h->q;
+    at.k = ck;
+    at.v = cv;
     at.o = h->o;
     at.err = h->err;
     at.n_tok = N;
@@ -949,11 +990,12 @@ int attention(ivit_handle* h, const LayerW& w, const bf16* ck, const bf16* cv, b
     at.sv = SV;
     next_launch(h, kFamAttn);
     at.stamp = ivit::g_stamp;
-    IVIT_CK(h, ivit::launch_attention_tc(h->tm_qa, w.tm_ak, w.tm_av, at, h->num_sms, s));
+    IVIT_CK(h, attention_few(h, m_expected) ? ivit::launch_attention_rows(at, h->num_sms, s)
+                                            : ivit::launch_attention_tc(h->tm_qa, w.tm_ak, w.tm_av, at, h->num_sms, s));
   } else {
     next_launch(h, kFamAttn);
     IVIT_CK(h, ivit::launch_attention(w.tm_ck, w.tm_cv, h->q, ck, cv, h->cu_rows, h->rowtok, h->o, SV, N, D, h->H,
-                                      full ? (N + 31) / 32 : std::max(1, (N / 10 + 31) / 32), s));
+                                      (std::max(1, m_expected / SV) + 31) / 32, s));
   }
   ++h->launches;
   return IVIT_OK;
@@ -981,6 +1023,7 @@ int run_layers_mlp_all(ivit_handle* h, const GemmPlan* plan, bool full, cudaStre
   const ivit_config& c = h->cfg;
   const int N = h->N, D = h->D, F = h->F, SV = h->SV, M = h->M_max;
   const int* total = h->cu_rows + SV;
+  const int m_expected = full ? M : std::max(1, M / 10);
   // The down-projection's residual update of every token may still be split over the GEMM
   // scratch: the next layer's LN1 reads it for the updated tokens, its LN2 adds it to x.
   ivit::PendingSum pend;
@@ -1012,7 +1055,7 @@ int run_layers_mlp_all(ivit_handle* h, const GemmPlan* plan, bool full, cudaStre
       a.epi.dim = D;
       if (int r = gemm(h, plan[kGemmQKV], w.tm_qkv, w.wqkv, h->tm_xn, a, s)) return r;
     }
-    if (int r = attention(h, w, ck, cv, full, s)) return r;
+    if (int r = attention(h, w, ck, cv, m_expected, s)) return r;
     {
       ivit::GemmArgs a;
       a.n_out = D;
@@ -1072,8 +1115,8 @@ int run_layers_mlp_all(ivit_handle* h, const GemmPlan* plan, bool full, cudaStre
 
 // Per layer {LN1, QKV + K/V cache scatter (Eq. 4-5), attention, out-proj + residual,
 // LN2, MLP up + GELU, MLP down + residual}, then the final LN scattered into the
-// final-token cache, with the given launch plans.
-int run_layers(ivit_handle* h, const GemmPlan* plan, bool full, cudaStream_t s) {
+// final-token cache, with the given launch plans, made for about m_expected updated rows.
+int run_layers(ivit_handle* h, const GemmPlan* plan, int m_expected, cudaStream_t s) {
   const ivit_config& c = h->cfg;
   const int D = h->D, F = h->F, SV = h->SV, M = h->M_max;
   const int* total = h->cu_rows + SV;
@@ -1126,7 +1169,7 @@ int run_layers(ivit_handle* h, const GemmPlan* plan, bool full, cudaStream_t s) 
       a.epi.dim = D;
       if (int r = gemm(h, plan[kGemmQKV], w.tm_qkv, w.wqkv, h->tm_xn, a, s)) return r;
     }
-    if (int r = attention(h, w, ck, cv, full, s)) return r;
+    if (int r = attention(h, w, ck, cv, m_expected, s)) return r;
     if (int r = residual(plan[kGemmO], w.bo, w.tm_o, w.wo, h->tm_o, D)) return r;
     if (int r = layernorm(w.ln2g, w.ln2b, h->xn, nullptr)) return r;
     {
@@ -1169,7 +1212,7 @@ int capture_band_bodies(ivit_handle* h, cudaStream_t s) {
     h->launches = pre;
     IVIT_CK(h, cudaStreamBeginCaptureToGraph(h->cap_stream2, np.conditional.phGraph_out[b], nullptr, nullptr, 0,
                                              cudaStreamCaptureModeThreadLocal));
-    const int r = run_layers(h, h->plan_band[b], h->band_ub[b] >= h->M_max, h->cap_stream2);
+    const int r = run_layers(h, h->plan_band[b], band_rows(h, b), h->cap_stream2);
     cudaGraph_t body = nullptr;
     const cudaError_t e = cudaStreamEndCapture(h->cap_stream2, &body);
     if (r) return r;
@@ -1309,8 +1352,8 @@ int run_core(ivit_handle* h, bool full, cudaStream_t s) {
   }
   if (h->capture_bands) return capture_band_bodies(h, s);
   if (!full && h->known_band >= 0)  // top-k: the row count is fixed, so is its band
-    return run_layers(h, h->plan_band[h->known_band], h->band_ub[h->known_band] >= h->M_max, s);
-  return run_layers(h, plan, full, s);
+    return run_layers(h, h->plan_band[h->known_band], h->known_rows, s);
+  return run_layers(h, plan, full ? M : std::max(1, M / 10), s);
 }
 
 int capture_once(ivit_handle* h, bool full, cudaGraphExec_t* exec, int64_t* launches);
@@ -1327,6 +1370,7 @@ int capture(ivit_handle* h, bool full, cudaGraphExec_t* exec, int64_t* launches)
     int b = 0;
     while (b + 1 < h->n_bands && m > h->band_ub[b]) ++b;
     h->known_band = b;
+    h->known_rows = static_cast<int>(m);
     const int r = capture_once(h, full, exec, launches);
     h->known_band = -1;
     return r;

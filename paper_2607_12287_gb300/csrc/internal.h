@@ -284,6 +284,9 @@ cudaError_t launch_attention(const CUtensorMap& tm_k, const CUtensorMap& tm_v, c
 // ----------------------------------------------------------- attention (tcgen05)
 struct AttnTcArgs {
   const int* cu_rows = nullptr;  // [SV+1] packed-row offsets of the views' updated rows
+  const bf16* q = nullptr;       // packed queries [rows][D] and this layer's caches [SV*N][D],
+  const bf16* k = nullptr;       // for the kernel that uses no TMA maps (attention_rows)
+  const bf16* v = nullptr;
   bf16* o = nullptr;             // [rows][D] attention output, packed rows
   int* err = nullptr;            // device error word
   int n_tok = 0, dim = 0, dh = 0, heads = 0, sv = 0;
@@ -312,5 +315,10 @@ struct AttnMaps {
 // items.  At most 4096 views.
 cudaError_t launch_attention_tc(const AttnMaps& q, const AttnMaps& k, const AttnMaps& v, const AttnTcArgs& a,
                                 int num_sms, cudaStream_t s);
+
+// The same for a few queries per view, without TMA maps: CTAs walk (view, head, 16-query tile)
+// items.
+cudaError_t attention_rows_setup();
+cudaError_t launch_attention_rows(const AttnTcArgs& a, int num_sms, cudaStream_t s);
 
 }  // namespace ivit

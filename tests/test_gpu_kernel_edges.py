@@ -63,15 +63,18 @@ def test_few_row_gemm_edges(pkg, oracle_mod, grid, dim, heads, mlp, change, mlp_
 
 
 # (grid, views, dim, heads): head widths of every padded width (8 -> 16 ... 128), token counts
-# one off the key blocks of 64, 96 and 128, one and several query tiles per head
+# one off the key blocks of 64, 96 and 128 and the few-query kernel's 32 and 256, one and several
+# query tiles of 16 and 128 per head; on both kernels
 ATTN_SHAPES = [((1, 1), 2, 64, 8), ((5, 19), 2, 64, 4), ((3, 33), 1, 128, 4), ((1, 97), 2, 320, 8),
                ((8, 16), 1, 192, 3), ((3, 43), 2, 576, 8), ((1, 193), 1, 320, 4), ((1, 257), 1, 704, 8),
                ((5, 13), 3, 832, 8), ((2, 161), 1, 256, 2)]
 
 
+@pytest.mark.parametrize("kernel", ["tc", "rows"])
 @pytest.mark.parametrize("grid,views,dim,heads", ATTN_SHAPES,
                          ids=[f"n{g[0] * g[1]}x{v}_dh{d // h}" for g, v, d, h in ATTN_SHAPES])
-def test_attention_block_edges(pkg, oracle_mod, grid, views, dim, heads):
+def test_attention_block_edges(pkg, oracle_mod, monkeypatch, grid, views, dim, heads, kernel):
+    monkeypatch.setenv("IVIT_ATTN", kernel)
     _run(pkg, oracle_mod, grid, views, dim, heads, 2 * dim, 2, 0.5)
 
 
