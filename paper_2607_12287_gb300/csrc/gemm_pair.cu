@@ -35,7 +35,7 @@ constexpr int BK = 64;    // K per stage: 128-byte rows, 128-byte swizzle
 constexpr int W_BYTES = BM * BK * 2;
 constexpr int EPI_WARPS = 8;
 constexpr int THREADS = (EPI_WARPS + 2) * 32;
-constexpr int EPI_HALF = 8192;  // staging of one row half: 32 rows of 128 bf16 or 16 of fp32
+constexpr int EPI_HALF = 8192;  // a staging buffer: 32 rows of 128 bf16 or 16 of fp32
 
 // As many stages as fit for the two smaller tiles: the first ones hold weights requested before
 // the wait on the previous kernel.  64-row tiles with 2 / 3 / 4 / 5 stages: four-layer 224 px
@@ -51,7 +51,8 @@ struct PairCfg {
   static constexpr int KB_BYTES = W_BYTES + X_BYTES;
   static constexpr int STAGE_BYTES = KS * KB_BYTES;
   static constexpr int EPI_OFFSET = STAGES * STAGE_BYTES;
-  static constexpr int BAR_OFFSET = EPI_OFFSET + 2 * EPI_HALF;
+  static constexpr int BUFS = BN == 256 ? 2 : 1;  // staging buffers per row half
+  static constexpr int BAR_OFFSET = EPI_OFFSET + 2 * BUFS * EPI_HALF;
   static constexpr int TOTAL = BAR_OFFSET + 256 + 1024;  // barriers, flags, 1 KB alignment slack
   static_assert(TOTAL <= 227 * 1024, "shared memory of one CTA");
 };
@@ -88,13 +89,17 @@ __device__ __forceinline__ float3 sum_rows4(const float3 (&v)[4], int lane) {
 // warps of one row half: chunks of 32 rows (16 when fp32) go from tensor memory (lane =
 // feature) through shared memory (row-major) to global memory with 16-byte accesses, 128
 // features of a row at a time.  `ready` waits for the accumulator (false: nothing is stored),
-// `release` is called once, when it has been read.
-template <int KIND, class Ready, class Release>
+// `release` is called once, when it has been read.  The next chunk's accumulators and rows are
+// requested before this one is stored, and the staging has two buffers if there is room (`buf`:
+// the one to use, kept over the tiles of a CTA), so that a chunk costs one barrier and no round
+// trip.
+template <int KIND, int BUFS, class Ready, class Release>
 __device__ __forceinline__ void drain(const GemmArgs& a, uint32_t acc, uint8_t* stg, int bar_id, int wq, int lane,
-                                      int row0, int c_lo, int c_hi, int ft, float* slot, Ready ready,
+                                      int row0, int c_lo, int c_hi, int ft, float* slot, int& buf, Ready ready,
                                       Release release) {
   constexpr bool kBf16 = KIND == kEpiQKV || KIND == kEpiGelu;
   constexpr int CHUNK = kBf16 ? 32 : 16;
+  constexpr bool kAhead = BUFS == 2;
   const int f0 = ft * BM, fl = wq * 32 + lane;
   float bias = 0.f;
   if (KIND != kEpiPartial && f0 + fl < a.n_out) bias = __ldg(a.epi.bias + f0 + fl);
@@ -124,42 +129,59 @@ __device__ __forceinline__ void drain(const GemmArgs& a, uint32_t acc, uint8_t* 
   // loop): one chunk at a time was bound by their latency
   constexpr int AHEAD = 4;
   float4 old[KIND == kEpiScore ? AHEAD : 1][ITERS];
-  auto load_old = [&](int c0) {
-    if constexpr (KIND == kEpiScore) {
-#pragma unroll
-      for (int k = 0; k < AHEAD; ++k)
-#pragma unroll
-        for (int i = 0; i < ITERS; ++i) {
-          const int c = c0 + k * CHUNK + i * 4 * RPW + rsub;
-          old[k][i] = make_float4(0.f, 0.f, 0.f, 0.f);
-          if (c < c_hi && f < a.n_out)
-            old[k][i] = __ldcg(reinterpret_cast<const float4*>(dst32 + static_cast<size_t>(row0 + c) * ld));
-        }
-    }
-  };
-  load_old(c_lo);
-  const bool ok = ready(), f_ok = ok && f < a.n_out;
-  auto chunk = [&](int c0, const float4 (&prev)[ITERS]) {
-    int rr[ITERS];  // destination rows, -1 past the tile's end
+  auto load_old = [&](int c0, float4 (&d)[ITERS]) {
 #pragma unroll
     for (int i = 0; i < ITERS; ++i) {
       const int c = c0 + i * 4 * RPW + rsub;
-      rr[i] = -1;
-      if (c < c_hi && f_ok) rr[i] = KIND == kEpiPartial ? c : by_tok ? __ldcg(a.epi.rowtok + row0 + c) : row0 + c;
+      d[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (c < c_hi && f < a.n_out)
+        d[i] = __ldcg(reinterpret_cast<const float4*>(dst32 + static_cast<size_t>(row0 + c) * ld));
     }
-    uint32_t v[CHUNK];
-    if constexpr (kBf16) {
+  };
+  if constexpr (KIND == kEpiScore) {
+#pragma unroll
+    for (int k = 0; k < AHEAD; ++k) load_old(c_lo + k * CHUNK, old[k]);
+  }
+  int rr[ITERS];  // destination rows, -1 past the tile's end
+  auto load_rows = [&](int c0, int (&d)[ITERS]) {
+#pragma unroll
+    for (int i = 0; i < ITERS; ++i) {
+      const int c = c0 + i * 4 * RPW + rsub;
+      d[i] = -1;
+      if (c < c_hi && f < a.n_out)
+        d[i] = KIND == kEpiPartial ? c : by_tok ? __ldcg(a.epi.rowtok + row0 + c) : row0 + c;
+    }
+  };
+  if (kAhead) load_rows(c_lo, rr);
+  const bool ok = ready();
+  uint32_t v[CHUNK];
+  auto load_acc = [&](int c0) {
+    if constexpr (kBf16)
       tmem_ld32_async(acc + c0, v);
+    else
+      tmem_ld16_async(acc + c0, v);
+  };
+  if (kAhead) load_acc(c_lo);
+  auto chunk = [&](int c0, const float4 (&prev)[ITERS]) {
+    if (!kAhead) {
+      load_rows(c0, rr);
+      load_acc(c0);
+    }
+    if constexpr (kBf16) {
       tmem_ld_wait_regs(v);
     } else {
-      tmem_ld16_async(acc + c0, v);
       tmem_ld_wait();
       tmem_regs_after_wait16(v);
     }
-    if (c0 + CHUNK >= c_hi) release();
-    named_barrier(bar_id, 128);  // the previous chunk has left the staging buffer
+    const bool last = c0 + CHUNK >= c_hi;
+    if (last) release();
+    uint8_t* sb = stg + buf * EPI_HALF;
+    if (BUFS == 2)
+      buf ^= 1;
+    else
+      named_barrier(bar_id, 128);  // the previous chunk has left the staging buffer
     if (kBf16) {
-      bf16* st = reinterpret_cast<bf16*>(stg) + fl;
+      bf16* st = reinterpret_cast<bf16*>(sb) + fl;
 #pragma unroll
       for (int j = 0; j < CHUNK; ++j) {
         float y = __uint_as_float(v[j]) + bias;
@@ -167,17 +189,22 @@ __device__ __forceinline__ void drain(const GemmArgs& a, uint32_t acc, uint8_t* 
         st[j * BM] = __float2bfloat16_rn(y);
       }
     } else {
-      float* st = reinterpret_cast<float*>(stg) + fl;
+      float* st = reinterpret_cast<float*>(sb) + fl;
 #pragma unroll
       for (int j = 0; j < CHUNK; ++j) st[j * BM] = __uint_as_float(v[j]) + bias;
+    }
+    int next[ITERS];
+    if (kAhead && !last) {
+      load_acc(c0 + CHUNK);
+      load_rows(c0 + CHUNK, next);
     }
     named_barrier(bar_id, 128);
     float3 sums[KIND == kEpiScore ? ITERS : 1];
 #pragma unroll
     for (int i = 0; i < ITERS; ++i) {
-      const uint4 u = *reinterpret_cast<const uint4*>(stg + ((i * 4 * RPW + rsub) * LPR + sub) * 16);
+      const uint4 u = *reinterpret_cast<const uint4*>(sb + ((i * 4 * RPW + rsub) * LPR + sub) * 16);
       if constexpr (KIND == kEpiScore) sums[i] = make_float3(0.f, 0.f, 0.f);
-      if (rr[i] < 0) continue;
+      if (rr[i] < 0 || !ok) continue;
       const size_t off = static_cast<size_t>(rr[i]) * ld;
       if (kBf16)
         *reinterpret_cast<uint4*>(dst16 + off) = u;
@@ -198,13 +225,19 @@ __device__ __forceinline__ void drain(const GemmArgs& a, uint32_t acc, uint8_t* 
       if ((lane & 7) == 0 && c < c_hi && ok)
         a.epi.score[static_cast<size_t>(ft) * a.m_static + row0 + c] = make_float4(s.x, s.y, s.z, 0.f);
     }
+    if (kAhead && !last) {
+#pragma unroll
+      for (int i = 0; i < ITERS; ++i) rr[i] = next[i];
+    }
   };
   if constexpr (KIND == kEpiScore) {
     for (int c0 = c_lo; c0 < c_hi; c0 += AHEAD * CHUNK) {
-      if (c0 > c_lo) load_old(c0);
 #pragma unroll
-      for (int k = 0; k < AHEAD; ++k)
-        if (c0 + k * CHUNK < c_hi) chunk(c0 + k * CHUNK, old[k]);
+      for (int k = 0; k < AHEAD; ++k) {
+        if (c0 + k * CHUNK >= c_hi) break;
+        chunk(c0 + k * CHUNK, old[k]);
+        load_old(c0 + (AHEAD + k) * CHUNK, old[k]);
+      }
     }
   } else {
     for (int c0 = c_lo; c0 < c_hi; c0 += CHUNK) chunk(c0, old[0]);
@@ -372,8 +405,8 @@ __global__ void __launch_bounds__(THREADS, 1)
   } else {
     const int wq = warp & 3, hf = warp >> 2;
     const uint32_t trow = tmem + (static_cast<uint32_t>(wq * 32) << 16);
-    uint8_t* stg = smem + C::EPI_OFFSET + hf * EPI_HALF;
-    int iter = 0;
+    uint8_t* stg = smem + C::EPI_OFFSET + hf * C::BUFS * EPI_HALF;
+    int iter = 0, buf = 0;
     for (int u = pair; u < units; u += n_pairs, ++iter) {
       const int sp = u % splits, tile = u / splits;
       const int ft = 2 * (tile % n_fp) + rank, tt = tile / n_fp;
@@ -403,7 +436,7 @@ __global__ void __launch_bounds__(THREADS, 1)
       if (KIND == kEpiPartial)
         slot = a.partials + (static_cast<size_t>(ft + n_ft * tt) * splits + sp) * BN * BM;
       if (c_lo < c_hi && ft < n_ft) {
-        drain<KIND>(a, acc, stg, 1 + hf, wq, lane, tt * BN, c_lo, c_hi, ft, slot, ready, release);
+        drain<KIND, C::BUFS>(a, acc, stg, 1 + hf, wq, lane, tt * BN, c_lo, c_hi, ft, slot, buf, ready, release);
       } else {
         ready();
         release();
