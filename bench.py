@@ -499,7 +499,7 @@ def main() -> None:
                 "ms_per_step": e2e_ms / args.steps,
                 "h2d_bytes_per_step": int(frames[0].nbytes),
                 "d2h_bytes_per_step": int(out.numel() * out.element_size() + wl.sv * 4)},
-        "roofline": {"kernel": "gemm_tc_kernel (every QKV/out-proj/MLP/embed launch of a step)", "bound": "hbm",
+        "roofline": {"kernel": "gemm_rows_kernel / gemm_pair_kernel (every QKV/out-proj/MLP/embed launch of a step)", "bound": "hbm",
                      "achieved": achieved, "peak": peaks["hbm_gbs"], "unit": "GB/s",
                      "frac": (achieved / peaks["hbm_gbs"]) if achieved else None,
                      "peak_source": peaks["source"] + " (copy bandwidth, MEASURED_PEAKS.json)",

@@ -20,8 +20,8 @@
 //     epilogue that stored column by column behind a switch took 7.5 us for 64 rows x 128
 //     features, most of it on instruction fetch.  The residual is added in L2 (red.v4.f32),
 //     so it is never loaded.
-// Measured back to back, random bf16 data, before -> now: 32768 rows QKV 422 -> 159 us, up
-// 497 -> 203, out 154 -> 82, down 324 -> 211 (1540 TFLOP/s); 3080 rows QKV 65 -> 22, up
+// Measured back to back, random bf16 data, before -> now: 32768 rows QKV 422 -> 149 us
+// (1750 TFLOP/s), up 497 -> 198, out 154 -> 82, down 324 -> 211; 3080 rows QKV 65 -> 22, up
 // 60 -> 24, down 53 -> 26; 768 rows QKV 29 -> 12, up 27 -> 12; 256 rows QKV 16 -> 7.6,
 // up 16 -> 7.8.
 #include "internal.h"
