@@ -99,7 +99,7 @@ __device__ __forceinline__ void drain(const GemmArgs& a, uint32_t acc, uint8_t* 
                                       Release release) {
   constexpr bool kBf16 = KIND == kEpiQKV || KIND == kEpiGelu;
   constexpr int CHUNK = kBf16 ? 32 : 16;
-  constexpr bool kAhead = BUFS == 2;
+  constexpr bool kAhead = BUFS == 2, kByTok = KIND == kEpiQKV || KIND == kEpiScatterF32;
   const int f0 = ft * BM, fl = wq * 32 + lane;
   float bias = 0.f;
   if (KIND != kEpiPartial && f0 + fl < a.n_out) bias = __ldg(a.epi.bias + f0 + fl);
@@ -152,7 +152,9 @@ __device__ __forceinline__ void drain(const GemmArgs& a, uint32_t acc, uint8_t* 
         d[i] = KIND == kEpiPartial ? c : by_tok ? __ldcg(a.epi.rowtok + row0 + c) : row0 + c;
     }
   };
-  if (kAhead) load_rows(c_lo, rr);
+  // (the rows' tokens: a round trip under the main loop and not after it, QKV of 1176 rows x 192
+  // 3.6 -> 3.3 us)
+  if (kAhead || kByTok) load_rows(c_lo, rr);
   const bool ok = ready();
   uint32_t v[CHUNK];
   auto load_acc = [&](int c0) {
@@ -164,7 +166,7 @@ __device__ __forceinline__ void drain(const GemmArgs& a, uint32_t acc, uint8_t* 
   if (kAhead) load_acc(c_lo);
   auto chunk = [&](int c0, const float4 (&prev)[ITERS]) {
     if (!kAhead) {
-      load_rows(c0, rr);
+      if (!kByTok || c0 != c_lo) load_rows(c0, rr);
       load_acc(c0);
     }
     if constexpr (kBf16) {
