@@ -15,7 +15,9 @@
 //
 // Bound: latency at small row counts (wait, one round trip, MMAs, one exchange); mma.sync's
 // rate at larger ones, where attention.cu is the faster one (the rule is attention_few in
-// engine.cu).  16 heads of 72, 256 keys, 26 queries: 3.9 us back to back against 6.1 there, whose
+// engine.cu).  Heads of up to 64 have a form for two CTAs on an SM (128 registers; wider heads would
+// spill, 8.8 -> 11.6 us), taken when there are more items than SMs: six views of 196 x 196, 3 heads
+// of 64, 5.6 -> 4.9 us.  16 heads of 72, 256 keys, 26 queries: 3.9 us back to back against 6.1 there, whose
 // 128-query tile walks the keys in three dependent steps.
 #include "attention.cuh"
 #include "internal.h"
@@ -43,9 +45,10 @@ __device__ __forceinline__ uint32_t word(const uint4& v, int i) {
   return i == 0 ? v.x : i == 1 ? v.y : i == 2 ? v.z : v.w;
 }
 
-// NC: 32-dim chunks of a head (rounded up); NB: 64-dim blocks of V; R: 8-dim groups past them.
-template <int NC, int NB, int R>
-__global__ void __launch_bounds__(THREADS, 1) attention_rows_kernel(const AttnTcArgs a) {
+// NC: 32-dim chunks of a head (rounded up); NB: 64-dim blocks of V; R: 8-dim groups past them;
+// CTAS: CTAs per SM.
+template <int NC, int NB, int R, int CTAS>
+__global__ void __launch_bounds__(THREADS, CTAS) attention_rows_kernel(const AttnTcArgs a) {
   constexpr int NT = 8 * NB + R;             // output n-tiles
   constexpr int DW = 64 * NB + 8 * R + 4;    // floats of a partial output row
   extern __shared__ __align__(16) float sm[];
@@ -249,27 +252,32 @@ cudaError_t attention_rows_setup() {
       e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                static_cast<int>(bytes + 4 * (MAX_VIEWS + 1)));
   };
-  set(attention_rows_kernel<1, 1, 0>, smem_bytes<1, 0>());
-  set(attention_rows_kernel<2, 1, 0>, smem_bytes<1, 0>());
-  set(attention_rows_kernel<3, 1, 1>, smem_bytes<1, 1>());
-  set(attention_rows_kernel<3, 1, 2>, smem_bytes<1, 2>());
-  set(attention_rows_kernel<3, 2, 0>, smem_bytes<2, 0>());
-  set(attention_rows_kernel<4, 2, 0>, smem_bytes<2, 0>());
+  set(attention_rows_kernel<1, 1, 0, 1>, smem_bytes<1, 0>());
+  set(attention_rows_kernel<2, 1, 0, 1>, smem_bytes<1, 0>());
+  set(attention_rows_kernel<1, 1, 0, 2>, smem_bytes<1, 0>());
+  set(attention_rows_kernel<2, 1, 0, 2>, smem_bytes<1, 0>());
+  set(attention_rows_kernel<3, 1, 1, 1>, smem_bytes<1, 1>());
+  set(attention_rows_kernel<3, 1, 2, 1>, smem_bytes<1, 2>());
+  set(attention_rows_kernel<3, 2, 0, 1>, smem_bytes<2, 0>());
+  set(attention_rows_kernel<4, 2, 0, 1>, smem_bytes<2, 0>());
   return e;
 }
 
-cudaError_t launch_attention_rows(const AttnTcArgs& a, int num_sms, cudaStream_t s) {
+cudaError_t launch_attention_rows(const AttnTcArgs& a, int num_sms, int ctas, cudaStream_t s) {
   if (a.sv > MAX_VIEWS || a.dh % 8 || a.dh > 128) return cudaErrorInvalidValue;
-  const int grid = max(1, min(a.sv * a.heads * ((a.n_tok + TQ - 1) / TQ), num_sms));
+  const bool two = ctas == 2 && a.dh <= 64;
+  const int grid = max(1, min(a.sv * a.heads * ((a.n_tok + TQ - 1) / TQ), two ? 2 * num_sms : num_sms));
   auto launch = [&](auto kern, size_t bytes) {
     return launch_ex(kern, dim3(grid), dim3(THREADS), bytes + 4 * (a.sv + 1), s, 1, a);
   };
-  if (a.dh <= 32) return launch(attention_rows_kernel<1, 1, 0>, smem_bytes<1, 0>());
-  if (a.dh <= 64) return launch(attention_rows_kernel<2, 1, 0>, smem_bytes<1, 0>());
-  if (a.dh == 72) return launch(attention_rows_kernel<3, 1, 1>, smem_bytes<1, 1>());
-  if (a.dh == 80) return launch(attention_rows_kernel<3, 1, 2>, smem_bytes<1, 2>());
-  if (a.dh <= 96) return launch(attention_rows_kernel<3, 2, 0>, smem_bytes<2, 0>());
-  return launch(attention_rows_kernel<4, 2, 0>, smem_bytes<2, 0>());
+  if (two && a.dh <= 32) return launch(attention_rows_kernel<1, 1, 0, 2>, smem_bytes<1, 0>());
+  if (two && a.dh <= 64) return launch(attention_rows_kernel<2, 1, 0, 2>, smem_bytes<1, 0>());
+  if (a.dh <= 32) return launch(attention_rows_kernel<1, 1, 0, 1>, smem_bytes<1, 0>());
+  if (a.dh <= 64) return launch(attention_rows_kernel<2, 1, 0, 1>, smem_bytes<1, 0>());
+  if (a.dh == 72) return launch(attention_rows_kernel<3, 1, 1, 1>, smem_bytes<1, 1>());
+  if (a.dh == 80) return launch(attention_rows_kernel<3, 1, 2, 1>, smem_bytes<1, 2>());
+  if (a.dh <= 96) return launch(attention_rows_kernel<3, 2, 0, 1>, smem_bytes<2, 0>());
+  return launch(attention_rows_kernel<4, 2, 0, 1>, smem_bytes<2, 0>());
 }
 
 }  // namespace ivit

@@ -337,7 +337,7 @@ GemmPlan plan_gemm(int num_sms, int n_out, int k, int m_expected, int m_bound, b
   return best;
 }
 
-bool attention_few(const ivit_handle* h, int m_expected);
+int attention_few(const ivit_handle* h, int m_expected);
 
 // Updated rows to expect of a call in row band b: a tenth of the tokens in the first, the
 // middle of the others.
@@ -950,16 +950,15 @@ void print_stream_trace(ivit_handle* h, cudaStream_t s) {
   cudaMemset(h->sk_args.trace, 0, t.size() * sizeof(unsigned long long));
 }
 
-// Whether the few-query attention is the faster one for about m_expected updated rows: a cost
-// model in microseconds per launch, fitted like plan_gemm's.  That kernel takes 2.0 us (1.3 for
+// CTAs per SM (1, 2) of the few-query attention where it is the faster one for about m_expected
+// updated rows, else 0: a cost model in microseconds per launch, fitted like plan_gemm's.  That kernel takes 2.0 us (1.3 for
 // heads of up to 64) + 1.5 us per 256 keys of a 72-wide head for a round of 16-query items over
-// the SMs; the other one 4.0 us + 1.0 us per key block for a round of 128-query items over two
+// the SMs, two rounds of heads of up to 64 on twice the CTAs 0.85 times that; the other one 4.0 us + 1.0 us per key block for a round of 128-query items over two
 // CTAs per SM.  With 16 heads of 72: 26 queries x 256 keys 3.9 us against 6.1, 128 x 256 4.2
 // against 6.9, 256 x 256 7.2 against 7.3 (and 4 % of a full encode slower, for its second round
 // keeps the next kernel out), 100 x 1024 8.7 against 14.4, 32 views of 96 x 1024 171 against 38;
-// 6 views of 196 x 196 with 3 heads of 64 5.6 against 6.8.
-bool attention_few(const ivit_handle* h, int m_expected) {
-  if (h->attn_forced >= 0) return h->attn_forced == 1;
+// 6 views of 196 x 196 with 3 heads of 64 5.6 (4.9 with two CTAs per SM) against 6.8.
+int attention_few(const ivit_handle* h, int m_expected) {
   const int dh = h->D / h->H;
   auto rounds = [&](int tile, int ctas) {  // a view's last tile is half full on average
     const double tiles = std::max<double>(h->SV, static_cast<double>(m_expected) / tile + 0.5 * h->SV);
@@ -967,9 +966,11 @@ bool attention_few(const ivit_handle* h, int m_expected) {
     return std::ceil(h->H * std::min(tiles, full) / ctas);
   };
   const int kb = ivit::attention_key_block((dh + 15) & ~15);
-  const double few = 0.4 + rounds(16, h->num_sms) * ((dh <= 64 ? 1.3 : 2.0) + 1.5 * dh / 72.0 * ((h->N + 255) / 256));
+  const double round = (dh <= 64 ? 1.3 : 2.0) + 1.5 * dh / 72.0 * ((h->N + 255) / 256);
+  const bool two = dh <= 64 && rounds(16, h->num_sms) > 1;
+  const double few = 0.4 + round * (two ? 0.85 * 2 * rounds(16, 2 * h->num_sms) : rounds(16, h->num_sms));
   const double many = 4.0 + rounds(128, 2 * h->num_sms) * ((h->N + kb - 1) / kb);
-  return few < many;
+  return h->attn_forced == 0 || (h->attn_forced < 0 && few >= many) ? 0 : two ? 2 : 1;
 }
 
 // Attention of the updated queries (about m_expected) over all tokens of their view for one layer.
@@ -990,8 +991,9 @@ int attention(ivit_handle* h, const LayerW& w, const bf16* ck, const bf16* cv, i
     at.sv = SV;
     next_launch(h, kFamAttn);
     at.stamp = ivit::g_stamp;
-    IVIT_CK(h, attention_few(h, m_expected) ? ivit::launch_attention_rows(at, h->num_sms, s)
-                                            : ivit::launch_attention_tc(h->tm_qa, w.tm_ak, w.tm_av, at, h->num_sms, s));
+    const int few = attention_few(h, m_expected);
+    IVIT_CK(h, few ? ivit::launch_attention_rows(at, h->num_sms, few, s)
+                   : ivit::launch_attention_tc(h->tm_qa, w.tm_ak, w.tm_av, at, h->num_sms, s));
   } else {
     next_launch(h, kFamAttn);
     IVIT_CK(h, ivit::launch_attention(w.tm_ck, w.tm_cv, h->q, ck, cv, h->cu_rows, h->rowtok, h->o, SV, N, D, h->H,

@@ -317,8 +317,8 @@ cudaError_t launch_attention_tc(const AttnMaps& q, const AttnMaps& k, const Attn
                                 int num_sms, cudaStream_t s);
 
 // The same for a few queries per view, without TMA maps: CTAs walk (view, head, 16-query tile)
-// items.
+// items, `ctas` (1, or 2 for heads of up to 64) per SM.
 cudaError_t attention_rows_setup();
-cudaError_t launch_attention_rows(const AttnTcArgs& a, int num_sms, cudaStream_t s);
+cudaError_t launch_attention_rows(const AttnTcArgs& a, int num_sms, int ctas, cudaStream_t s);
 
 }  // namespace ivit

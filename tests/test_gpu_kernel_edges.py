@@ -67,7 +67,9 @@ def test_few_row_gemm_edges(pkg, oracle_mod, grid, dim, heads, mlp, change, mlp_
 # query tiles of 16 and 128 per head; on both kernels
 ATTN_SHAPES = [((1, 1), 2, 64, 8), ((5, 19), 2, 64, 4), ((3, 33), 1, 128, 4), ((1, 97), 2, 320, 8),
                ((8, 16), 1, 192, 3), ((3, 43), 2, 576, 8), ((1, 193), 1, 320, 4), ((1, 257), 1, 704, 8),
-               ((5, 13), 3, 832, 8), ((2, 161), 1, 256, 2)]
+               ((5, 13), 3, 832, 8), ((2, 161), 1, 256, 2),
+               # few-query kernel: more 16-query items than SMs, and than twice that
+               ((14, 14), 6, 192, 3), ((9, 11), 8, 256, 8)]
 
 
 @pytest.mark.parametrize("kernel", ["tc", "rows"])
