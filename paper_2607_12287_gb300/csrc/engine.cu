@@ -349,7 +349,7 @@ int band_rows(const ivit_handle* h, int b) {
 // memory fits (attention keeps a whole view's keys and values of one head resident, so
 // N * head_dim is bounded).  It is not the default anywhere: its SIMT attention phase and
 // 64-row GEMM tiles lose to the kernel chain also on the full encodes of small encoders
-// (six 196-token views of ViT-Tiny 1.40 ms against 0.40 ms for the chain).
+// (six 196-token views of ViT-Tiny 1.40 ms against 0.38 ms for the chain).
 int setup_persistent(ivit_handle* h) {
   const char* path = std::getenv("IVIT_PATH");
   if (!path || std::strcmp(path, "persistent") != 0) return IVIT_OK;
