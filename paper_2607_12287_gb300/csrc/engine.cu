@@ -147,6 +147,7 @@ struct ivit_handle {
   // most band_ub[b] updated rows; a switch node picks the band of each call's device-resident
   // row count.
   int n_bands = 1;
+  int row_groups = 1;  // of the few-row GEMM
   int band_ub[4] = {0, 0, 0, 0};
   GemmPlan plan_band[4][kGemmSlots];
   bool capture_bands = false;  // set while the incremental graph is captured with bands
@@ -624,6 +625,9 @@ int setup(ivit_handle* h, const uint16_t* wb) {
     for (int b = 1; b < h->n_bands; ++b)
       differ = differ || attention_few(h, band_rows(h, b)) != attention_few(h, band_rows(h, 0));
     if (!differ) h->n_bands = 1;
+    // a second row group (gemm.cu) where the band of the row count is not known at launch
+    const bool one_plan = c.mlp_tokens == IVIT_MLP_ALL || c.select_mode != IVIT_SEL_TOPK;
+    h->row_groups = one_plan && m_all > 64 && (c.mlp_tokens == IVIT_MLP_ALL || m_all / 10 <= 32) ? 2 : 1;
     // every row's D x D projection without a residual (first-layer key scores)
     h->plan_keys = plan_gemm(h->num_sms, static_cast<int>(D), static_cast<int>(D), m_all, m_all, false, false);
     if (std::getenv("IVIT_DEBUG")) {
@@ -864,6 +868,8 @@ int gemm(ivit_handle* h, const GemmPlan& plan, const CUtensorMap& tw, const bf16
   a.vsplit = plan.defer ? plan.splits : 0;
   a.w = w;
   a.x = x.base;
+  // (one plan for every row count: more rows than expected go to two CTAs)
+  a.row_groups = h->row_groups;
   next_launch(h, kFamGemm, &a);
   IVIT_CK(h, plan.nt ? ivit::launch_gemm_rows(plan.nt, a, s)
                      : ivit::launch_gemm_pair(plan.bn, tw, x.of(plan), a, plan.n_pairs, s));

@@ -10,7 +10,11 @@
 // taken in the same order on both sides these are the fragments of two mma.m16n8k16 (a dot
 // product does not care which k is called which).  So no operand is staged, and the rows cost
 // one round trip to L2.  The warps' sums meet in shared memory, in warp order.  Rows beyond
-// 32 run as further passes over the resident weights.
+// 32 run as further passes over the resident weights; where one plan serves every row count, a
+// second group of CTAs (blockIdx.y) takes every other pass and leaves at once when there is none:
+// two groups of all updates of a 256-token So400m view (four layers, two calls) 1058 -> 696 us, of
+// 30 % 451 -> 371, while a single pass costs no more (26 rows on average: 1499 -> 1419 us for 27
+// layers, for its calls of 33 rows and more).
 //
 // Bound: latency (wait, rows from L2, MMAs, sum over the warps, store).  mma.sync and not
 // tcgen05 because a tcgen05.mma takes at least about 46 cycles however few rows it has, and a
@@ -76,6 +80,10 @@ __global__ void __launch_bounds__(THREADS, 2) gemm_rows_kernel(const GemmArgs a)
   __shared__ __align__(8) uint64_t bar;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
   const int K = a.k, splits = KIND == kEpiPartial ? a.vsplit : 1;
+  // The CTAs of the second row group take every other pass; without one they have nothing to do.
+  // (The row count comes from the selection kernel, at least two launches back.)
+  const int first = blockIdx.y * ROWS;
+  if (first > 0 && (a.d_rows ? *a.d_rows : a.m_static) <= first) return;
   const int ft = blockIdx.x / splits, sp = blockIdx.x - ft * splits;
   int c_lo, c_hi;
   split_range((K + CK - 1) / CK, splits, sp, c_lo, c_hi);
@@ -99,7 +107,6 @@ __global__ void __launch_bounds__(THREADS, 2) gemm_rows_kernel(const GemmArgs a)
   float4 bias = make_float4(0.f, 0.f, 0.f, 0.f);
   if (KIND != kEpiPartial && e_ok) bias = __ldg(reinterpret_cast<const float4*>(a.epi.bias + f4));
   __syncthreads();  // the barrier exists before anyone waits on it
-  // The row count comes from the selection kernel, at least two launches back.
   const int M = a.d_rows ? *a.d_rows : a.m_static;
   pdl_wait();
   pdl_launch_dependents();
@@ -107,7 +114,8 @@ __global__ void __launch_bounds__(THREADS, 2) gemm_rows_kernel(const GemmArgs a)
 
   bool ok = true;
   const int n = max(0, (c_hi - c_lo - warp + WARPS - 1) / WARPS);  // this warp's chunks
-  for (int row0 = 0; row0 < M; row0 += ROWS) {
+  const int stride = gridDim.y * ROWS;
+  for (int row0 = first; row0 < M; row0 += stride) {
     const int rows = min(ROWS, M - row0);
     const bool two = rows > 16;  // second m16 tile in use
     uint4 x[DEPTH][4];
@@ -133,7 +141,7 @@ __global__ void __launch_bounds__(THREADS, 2) gemm_rows_kernel(const GemmArgs a)
       for (int j = 0; j < NT; ++j)
 #pragma unroll
         for (int e = 0; e < 4; ++e) acc[m][j][e] = 0.f;
-    if (row0 == 0 && !mbar_wait(bar_a, 0)) ok = false;  // the weights have landed
+    if (row0 == first && !mbar_wait(bar_a, 0)) ok = false;  // the weights have landed
     for (int i0 = 0; i0 < n; i0 += DEPTH) {
 #pragma unroll
       for (int d = 0; d < DEPTH; ++d) {
@@ -209,7 +217,7 @@ __global__ void __launch_bounds__(THREADS, 2) gemm_rows_kernel(const GemmArgs a)
         *reinterpret_cast<float4*>(a.epi.out_f32 + static_cast<size_t>(tok) * a.epi.ld_out + f4) = y;
       }
     }
-    if (row0 + ROWS < M) __syncthreads();  // the sums are read before the next pass writes
+    if (row0 + stride < M) __syncthreads();  // the sums are read before the next pass writes
   }
   if (M <= 0 && !mbar_wait(bar_a, 0)) ok = false;  // no copy in flight at exit
   if (!ok && tid == 0) atomicExch(a.err, kErrWaitTmaFull);
@@ -224,7 +232,7 @@ size_t smem_bytes(int nt, int k, int splits) {
 template <int NT>
 cudaError_t launch_nt(const GemmArgs& a, cudaStream_t s) {
   const int splits = a.defer ? a.vsplit : 1;
-  const dim3 grid((a.n_out + 8 * NT - 1) / (8 * NT) * splits);
+  const dim3 grid((a.n_out + 8 * NT - 1) / (8 * NT) * splits, a.row_groups);
   const size_t smem = smem_bytes(NT, a.k, splits);
   auto launch = [&](auto kern) { return launch_ex(kern, grid, dim3(THREADS), smem, s, 1, a); };
   if (a.defer) return launch(gemm_rows_kernel<NT, kEpiPartial>);

@@ -90,6 +90,7 @@ struct GemmArgs {
   // residual epilogue).
   int defer = 0;
   int vsplit = 0;
+  int row_groups = 1;            // few-row GEMM: CTAs per feature tile and split, 1 or 2
   unsigned long long* stamp = nullptr;  // timeline stamps of this launch (or null)
   const bf16* w = nullptr;       // W and X themselves, for the kernel that uses no TMA maps
   const bf16* x = nullptr;       // (gemm_rows)
@@ -114,7 +115,7 @@ cudaError_t launch_gemm_pair(int bn, const CUtensorMap& tm_w, const CUtensorMap&
                              int n_pairs, cudaStream_t s);
 
 // The same GEMM for a few rows: CTAs of 8 nt features (nt 1..4), rows in passes of 32, every
-// epilogue but kEpiF32Bias and kEpiScore.  With defer set, K is split vsplit ways and the slots have 32 rows.
+// epilogue but kEpiF32Bias and kEpiScore, row_groups CTAs side by side for the passes.  With defer set, K is split vsplit ways and the slots have 32 rows.
 // k a multiple of 8.
 constexpr int GEMM_ROWS_SMEM_MAX = 160 * 1024;
 size_t gemm_rows_smem(int nt, int k, int splits);
