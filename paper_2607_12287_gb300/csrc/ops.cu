@@ -397,15 +397,18 @@ __global__ void __launch_bounds__(256) layernorm_kernel(const int* __restrict__ 
 }
 
 // Layer norm after a deferred split-K GEMM with the residual epilogue: per row, x +=
-// bias + sum_s partial_s (the splits in order, the same fp32 sum the GEMM's own
-// reduction forms), x written back, then y = LN(x).  One CTA per row and one float4 of
-// the row per thread, so every split's partial of every element is in flight at once
+// bias + sum_s partial_s (the splits in order, in fp32), x written back, then y = LN(x).
+// One CTA per row and one float4 of the row per thread (at most LN_SUM_THREADS, a width of
+// 2048), so every split's partial of every element is in flight at once
 // (a row's partials are spread over the csize slots of its feature tiles).  kGather: the row
 // is src_rowtok[r], and x is not written; kAdd: a row of `add` is added as well.  MAXS: the
-// most splits, 4, 8 or 16, whose partials a thread holds: with room for 16 (135 registers) one CTA
-// fits on an SM, and 256 rows of the So400m width ran in two waves, 4.1 us against 2.0.
+// most splits, 4, 8 or 16, whose partials a thread holds: with room for 16 (128 registers, the most
+// that leaves an SM room for the widest row) one CTA fits on an SM, and 256 rows of the So400m
+// width ran in two waves, 4.1 us against 2.0.
+constexpr int LN_SUM_THREADS = 512;
+
 template <int MAXS, bool kGather, bool kAdd>
-__global__ void layernorm_sum_kernel(const int* __restrict__ nrows, float* __restrict__ x, const PendingSum ps,
+__global__ void __launch_bounds__(LN_SUM_THREADS) layernorm_sum_kernel(const int* __restrict__ nrows, float* __restrict__ x, const PendingSum ps,
                                      const float* __restrict__ add, const int* __restrict__ src_rowtok,
                                      const float* __restrict__ gamma, const float* __restrict__ beta,
                                      bf16* __restrict__ y, const int* __restrict__ dst_rowtok, int dim, float eps,
@@ -782,7 +785,7 @@ cudaError_t launch_layernorm(const int* rows, const float* x, const float* gamma
 cudaError_t launch_layernorm_sum(const int* rows, float* x, const PendingSum& ps, const float* add,
                                  const int* src_rowtok, const float* gamma, const float* beta, bf16* y,
                                  const int* dst_rowtok, int dim, float eps, int max_rows, int grid, cudaStream_t s) {
-  if (dim % 4 != 0 || dim > 4096 || ps.csize < 2 || ps.csize > 16 || ps.bn < 1 || !ps.partials || !ps.bias ||
+  if (dim % 4 != 0 || dim > 4 * LN_SUM_THREADS || ps.csize < 2 || ps.csize > 16 || ps.bn < 1 || !ps.partials || !ps.bias ||
       (add && src_rowtok))
     return cudaErrorInvalidValue;
   const int threads = (dim / 4 + 31) / 32 * 32;

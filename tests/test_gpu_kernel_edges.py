@@ -1,6 +1,8 @@
 """Kernels at the edges of their tiles, through the C ABI against the fp32 oracle: an encoder of
 one or two layers encodes a stream in full and incrementally (updated lists bit-exact, tokens
 within the parity bars of gpu_util)."""
+import re
+
 import numpy as np
 import pytest
 
@@ -60,6 +62,17 @@ ROW_SHAPES = [((6, 10), 64, 1, 264, 0.05), ((6, 10), 320, 5, 840, 0.25), ((6, 10
                          ids=[f"d{d}_f{f}_p{int(100 * c)}" for _, d, _, f, c in ROW_SHAPES])
 def test_few_row_gemm_edges(pkg, oracle_mod, grid, dim, heads, mlp, change, mlp_tokens):
     _run(pkg, oracle_mod, grid, 1, dim, heads, mlp, 2, change, n_frames=4, mlp_tokens=mlp_tokens)
+
+
+# wide encoders whose residual GEMMs leave more than 8 splits to the next layer norm, which then
+# holds 16 partials per thread of its widest blocks (416 and 512 threads)
+@pytest.mark.parametrize("grid,dim,heads", [((16, 16), 1664, 26), ((8, 8), 1664, 13), ((16, 16), 2048, 16), ((8, 8), 2048, 32)],
+                         ids=["d1664_n256", "d1664_n64", "d2048_n256", "d2048_n64"])
+def test_many_splits_of_wide_rows(pkg, oracle_mod, monkeypatch, capfd, grid, dim, heads):
+    monkeypatch.setenv("IVIT_DEBUG", "1")
+    _run(pkg, oracle_mod, grid, 1, dim, heads, 8192, 1, 0.05, n_frames=2)
+    plans = re.findall(r"^ivit gemm (?:full|inc)\s.*splits=(\d+)$", capfd.readouterr().err, flags=re.M)
+    assert len(plans) == 10 and max(map(int, plans)) > 8, plans
 
 
 # (grid, views, dim, heads): head widths of every padded width (8 -> 16 ... 128), token counts
