@@ -278,8 +278,8 @@ size_t defer_slots(const GemmPlan& pl, int n_out, int m_bound) {
   return static_cast<size_t>((n_out + 127) / 128) * ((m_bound + pl.bn - 1) / pl.bn) * pl.splits;
 }
 
-// Launch shape of a GEMM expected to see m_expected rows (and at most m_bound): the
-// cheapest candidate of a cost model in microseconds per launch, fitted to back-to-back
+// Launch shape of a GEMM expected to see m_expected rows, as wide as m_bound rows can use (any
+// count up to m_most runs): the cheapest candidate of a cost model in microseconds per launch, fitted to back-to-back
 // launches on GB300 of the SigLIP-So400m and ViT-Tiny shapes at 16 to 32768 rows.
 //   CTA pairs: a fixed part (prologue, first loads, last tile's epilogue) plus a k-block
 //     (64 wide) rate per round of units over the 76 pairs; 64-, 128- and 256-row tiles
@@ -291,13 +291,13 @@ size_t defer_slots(const GemmPlan& pl, int n_out, int m_bound) {
 //     against 7.2, of 128 rows 11.1 against 7.2.
 //   Deferred (residual GEMMs, `defer`): the next layer norm sums the partial tiles: no
 //     epilogue, but every split's fp32 tile is written and read once (about 10 TB/s, in L2).
-GemmPlan plan_gemm(int num_sms, int n_out, int k, int m_expected, int m_bound, bool few, bool defer) {
+GemmPlan plan_gemm(int num_sms, int n_out, int k, int m_expected, int m_bound, int m_most, bool few, bool defer) {
   GemmPlan best;
   double best_cost = 1e30;
   defer = defer && !std::getenv("IVIT_NO_DEFER");
   auto consider = [&](const GemmPlan& pl, double cost) {
     if (pl.defer) {
-      if (defer_slots(pl, n_out, m_bound) * pl.bn * 128 * 4 > (64ull << 20)) return;
+      if (defer_slots(pl, n_out, m_most) * pl.bn * 128 * 4 > (64ull << 20)) return;
       cost += pl.splits * (8.0 * n_out) * m_expected / 1.0e7;
     }
     if (cost < best_cost - 1e-9) {
@@ -551,6 +551,84 @@ int setup_stream(ivit_handle* h) {
   return IVIT_OK;
 }
 
+// The bands of the row count and the launch plans of every GEMM, from the configuration and the
+// number of SMs alone.
+void make_plans(ivit_handle* h) {
+  const ivit_config& c = h->cfg;
+  const int D = h->D, F = h->F, m_all = h->M_max, m_inc = std::max(1, m_all / 10);
+  // Row bands: the first holds a tenth of the tokens (rounded up to 16, at least 64),
+  // each next one twice the previous, the last all of them; at most four.
+  int ub = std::max(64, (m_all / 10 + 15) / 16 * 16);
+  h->n_bands = 0;
+  while (h->n_bands < 4) {
+    const bool last = ub >= m_all || h->n_bands == 3;
+    h->band_ub[h->n_bands++] = last ? m_all : ub;
+    if (last) break;
+    ub *= 2;
+  }
+  if (std::getenv("IVIT_NO_BANDS")) h->n_bands = 1;
+  // Full encodes know M = SV*N.  Incremental calls are planned for a tenth of the
+  // tokens updated (any count still runs correctly, with more or fewer tile rounds).
+  const int shapes[kGemmSlots][2] = {{D, h->KPAD}, {3 * D, D}, {D, D}, {F, D}, {D, F}};
+  for (int g = 0; g < kGemmSlots; ++g) {
+    // (under the MLP-on-all-tokens reading the out-projection goes to a cache, not to a layer norm)
+    const bool defer = g == kGemmDown || (g == kGemmO && c.mlp_tokens == IVIT_MLP_UPDATED);
+    auto plan = [&](int m_expected, int m_bound) {
+      return plan_gemm(h->num_sms, shapes[g][0], shapes[g][1], m_expected, m_bound, m_all, g != kGemmEmbed, defer);
+    };
+    h->plan_full[g] = plan(m_all, m_all);
+    h->plan_inc[g] = g == kGemmEmbed ? h->plan_full[g] : plan(m_inc, m_all);
+    h->plan_band[0][g] = h->plan_inc[g];
+    // (the band of all rows runs the full encode's plans)
+    for (int b = 1; b < h->n_bands; ++b)
+      h->plan_band[b][g] = g == kGemmEmbed || h->band_ub[b] >= m_all ? h->plan_full[g]
+                                                                     : plan(h->band_ub[b], h->band_ub[b]);
+  }
+  // (a switch between equal plans would only cost its dispatch, about 10 us)
+  auto same = [](const GemmPlan& a, const GemmPlan& b) {
+    return a.nt == b.nt && a.bn == b.bn && a.splits == b.splits && a.n_pairs == b.n_pairs;
+  };
+  bool differ = false;
+  for (int b = 1; b < h->n_bands; ++b)
+    for (int g = 0; g < kGemmSlots; ++g) differ = differ || !same(h->plan_band[b][g], h->plan_band[0][g]);
+  for (int b = 1; b < h->n_bands; ++b)
+    differ = differ || attention_few(h, band_rows(h, b)) != attention_few(h, band_rows(h, 0));
+  if (!differ) h->n_bands = 1;
+  // a second row group (gemm.cu) where the band of the row count is not known at launch
+  const bool one_plan = c.mlp_tokens == IVIT_MLP_ALL || c.select_mode != IVIT_SEL_TOPK;
+  h->row_groups = one_plan && m_all > 64 && (c.mlp_tokens == IVIT_MLP_ALL || m_all / 10 <= 32) ? 2 : 1;
+  // every row's D x D projection without a residual (first-layer key scores)
+  h->plan_keys = plan_gemm(h->num_sms, D, D, m_all, m_all, m_all, false, false);
+  if (std::getenv("IVIT_DEBUG")) {
+    static const char* names[kGemmSlots] = {"embed", "qkv", "out", "up", "down"};
+    auto show = [&](const char* when, const char* name, const GemmPlan& pl) {
+      std::fprintf(stderr, "ivit gemm %-6s %-5s %s bn=%d nt=%d splits=%d\n", when, name, pl.nt ? "rows" : "pair", pl.bn,
+                   pl.nt, pl.splits);
+    };
+    for (int g = 0; g < kGemmSlots; ++g) {
+      show("full", names[g], h->plan_full[g]);
+      show("inc", names[g], h->plan_inc[g]);
+      for (int b = 1; b < h->n_bands; ++b) show(b == 1 ? "band 1" : b == 2 ? "band 2" : "band 3", names[g], h->plan_band[b][g]);
+    }
+  }
+}
+
+// Floats of the split-K scratch: slots [rows of a tile][128 features] of every plan, for every
+// row of every view.  A band's bound would not do: top-k selects NaN scores beside the k lowest,
+// so a call whose plans were picked for k rows a view can bring more.
+size_t scratch_floats(const ivit_handle* h) {
+  size_t most = 64;
+  auto need = [&](const GemmPlan& pl) {
+    if (pl.defer) most = std::max(most, defer_slots(pl, h->D, h->M_max) * pl.bn * 128);
+  };
+  for (int g = 0; g < kGemmSlots; ++g) {
+    need(h->plan_full[g]);
+    need(h->plan_inc[g]);
+    for (int b = 0; b < h->n_bands; ++b) need(h->plan_band[b][g]);
+  }
+  return most;
+}
+
 int setup(ivit_handle* h, const uint16_t* wb) {
   const ivit_config& c = h->cfg;
   h->N = (c.img_h / c.patch) * (c.img_w / c.patch);
@@ -576,73 +654,12 @@ int setup(ivit_handle* h, const uint16_t* wb) {
     h->attn_tc = std::string(at) != "simt";
     h->attn_forced = std::string(at) == "tc" ? 0 : std::string(at) == "rows" ? 1 : -1;
   }
-  {
-    // Row bands: the first holds a tenth of the tokens (rounded up to 16, at least 64),
-    // each next one twice the previous, the last all of them; at most four.
-    int ub = std::max(64, (static_cast<int>(M / 10) + 15) / 16 * 16);
-    h->n_bands = 0;
-    while (h->n_bands < 4) {
-      const bool last = ub >= static_cast<int>(M) || h->n_bands == 3;
-      h->band_ub[h->n_bands++] = last ? static_cast<int>(M) : ub;
-      if (last) break;
-      ub *= 2;
-    }
-    if (std::getenv("IVIT_NO_BANDS")) h->n_bands = 1;
-  }
   if (std::getenv("IVIT_NO_PDL")) ivit::g_use_pdl = false;
   if (std::getenv("IVIT_NO_GRAPH")) h->use_graphs = false;
   IVIT_CK(h, cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking));
   IVIT_CK(h, cudaStreamCreateWithFlags(&h->cap_stream2, cudaStreamNonBlocking));
   h->row_grid = h->num_sms * 4;
-  {
-    // Full encodes know M = SV*N.  Incremental calls are planned for a tenth of the
-    // tokens updated (any count still runs correctly, with more or fewer tile rounds).
-    const int m_all = static_cast<int>(M), m_inc = std::max(1, m_all / 10);
-    const int shapes[kGemmSlots][2] = {{static_cast<int>(D), h->KPAD}, {3 * static_cast<int>(D), static_cast<int>(D)},
-                                       {static_cast<int>(D), static_cast<int>(D)}, {static_cast<int>(F), static_cast<int>(D)},
-                                       {static_cast<int>(D), static_cast<int>(F)}};
-    for (int g = 0; g < kGemmSlots; ++g) {
-      // (under the MLP-on-all-tokens reading the out-projection goes to a cache, not to a layer norm)
-      const bool defer = g == kGemmDown || (g == kGemmO && c.mlp_tokens == IVIT_MLP_UPDATED);
-      auto plan = [&](int m_expected, int m_bound) {
-        return plan_gemm(h->num_sms, shapes[g][0], shapes[g][1], m_expected, m_bound, g != kGemmEmbed, defer);
-      };
-      h->plan_full[g] = plan(m_all, m_all);
-      h->plan_inc[g] = g == kGemmEmbed ? h->plan_full[g] : plan(m_inc, m_all);
-      h->plan_band[0][g] = h->plan_inc[g];
-      // (the band of all rows runs the full encode's plans)
-      for (int b = 1; b < h->n_bands; ++b)
-        h->plan_band[b][g] = g == kGemmEmbed || h->band_ub[b] >= m_all ? h->plan_full[g]
-                                                                       : plan(h->band_ub[b], h->band_ub[b]);
-    }
-    // (a switch between equal plans would only cost its dispatch, about 10 us)
-    auto same = [](const GemmPlan& a, const GemmPlan& b) {
-      return a.nt == b.nt && a.bn == b.bn && a.splits == b.splits && a.n_pairs == b.n_pairs;
-    };
-    bool differ = false;
-    for (int b = 1; b < h->n_bands; ++b)
-      for (int g = 0; g < kGemmSlots; ++g) differ = differ || !same(h->plan_band[b][g], h->plan_band[0][g]);
-    for (int b = 1; b < h->n_bands; ++b)
-      differ = differ || attention_few(h, band_rows(h, b)) != attention_few(h, band_rows(h, 0));
-    if (!differ) h->n_bands = 1;
-    // a second row group (gemm.cu) where the band of the row count is not known at launch
-    const bool one_plan = c.mlp_tokens == IVIT_MLP_ALL || c.select_mode != IVIT_SEL_TOPK;
-    h->row_groups = one_plan && m_all > 64 && (c.mlp_tokens == IVIT_MLP_ALL || m_all / 10 <= 32) ? 2 : 1;
-    // every row's D x D projection without a residual (first-layer key scores)
-    h->plan_keys = plan_gemm(h->num_sms, static_cast<int>(D), static_cast<int>(D), m_all, m_all, false, false);
-    if (std::getenv("IVIT_DEBUG")) {
-      static const char* names[kGemmSlots] = {"embed", "qkv", "out", "up", "down"};
-      auto show = [&](const char* when, const char* name, const GemmPlan& pl) {
-        std::fprintf(stderr, "ivit gemm %-6s %-5s %s bn=%d nt=%d splits=%d\n", when, name, pl.nt ? "rows" : "pair", pl.bn,
-                     pl.nt, pl.splits);
-      };
-      for (int g = 0; g < kGemmSlots; ++g) {
-        show("full", names[g], h->plan_full[g]);
-        show("inc", names[g], h->plan_inc[g]);
-        for (int b = 1; b < h->n_bands; ++b) show(b == 1 ? "band 1" : b == 2 ? "band 2" : "band 3", names[g], h->plan_band[b][g]);
-      }
-    }
-  }
+  make_plans(h);
 
   // ---- weights: bf16 matrices (W_pe padded to KPAD columns), fp32 vectors
   Arena wa;
@@ -740,19 +757,7 @@ int setup(ivit_handle* h, const uint16_t* wb) {
   const size_t o_err = sa.take(4);
   const size_t o_key = c.score_source == IVIT_SCORE_KEY0 ? sa.take(M * D * 4) : 0;
   const size_t o_acache = c.mlp_tokens == IVIT_MLP_ALL ? sa.take(L * M * D * 4) : 0;
-  // slots for every plan that splits K, fp32 [row tile][128 features] each
-  size_t part_floats = 64;
-  for (int g = 0; g < kGemmSlots; ++g)
-  {
-    auto need = [&](const GemmPlan& pl, int m_bound) -> size_t {
-      return pl.defer ? defer_slots(pl, static_cast<int>(D), m_bound) * pl.bn * 128 : 0;
-    };
-    part_floats = std::max(part_floats, need(h->plan_full[g], static_cast<int>(M)));
-    part_floats = std::max(part_floats, need(h->plan_inc[g], static_cast<int>(M)));
-    for (int b = 0; b < h->n_bands; ++b)
-      part_floats = std::max(part_floats, need(h->plan_band[b][g], b == 0 ? static_cast<int>(M) : h->band_ub[b]));
-  }
-  const size_t o_gpart = sa.take(part_floats * 4);
+  const size_t o_gpart = sa.take(scratch_floats(h) * 4);
   const size_t o_rta = sa.take(M * 4), o_mall = sa.take(4);
   IVIT_CK(h, cudaMalloc(&h->smem, sa.size));
   IVIT_CK(h, cudaMemset(h->smem, 0, sa.size));
