@@ -279,7 +279,7 @@ size_t defer_slots(const GemmPlan& pl, int n_out, int m_bound) {
 }
 
 // Launch shape of a GEMM expected to see m_expected rows, as wide as m_bound rows can use (any
-// count up to m_most runs): the cheapest candidate of a cost model in microseconds per launch, fitted to back-to-back
+// count runs): the cheapest candidate of a cost model in microseconds per launch, fitted to back-to-back
 // launches on GB300 of the SigLIP-So400m and ViT-Tiny shapes at 16 to 32768 rows.
 //   CTA pairs: a fixed part (prologue, first loads, last tile's epilogue) plus a k-block
 //     (64 wide) rate per round of units over the 76 pairs; 64-, 128- and 256-row tiles
@@ -290,14 +290,15 @@ size_t defer_slots(const GemmPlan& pl, int n_out, int m_bound) {
 //     to 32 features per CTA.  QKV of 26 rows 4.0 us against 7.2 in pairs, of 64 rows 6.6
 //     against 7.2, of 128 rows 11.1 against 7.2.
 //   Deferred (residual GEMMs, `defer`): the next layer norm sums the partial tiles: no
-//     epilogue, but every split's fp32 tile is written and read once (about 10 TB/s, in L2).
-GemmPlan plan_gemm(int num_sms, int n_out, int k, int m_expected, int m_bound, int m_most, bool few, bool defer) {
+//     epilogue, but every split's fp32 tile is written and read once (about 10 TB/s, in L2, hence
+//     at most 64 MB of them for m_bound rows; the scratch itself has room for every row).
+GemmPlan plan_gemm(int num_sms, int n_out, int k, int m_expected, int m_bound, bool few, bool defer) {
   GemmPlan best;
   double best_cost = 1e30;
   defer = defer && !std::getenv("IVIT_NO_DEFER");
   auto consider = [&](const GemmPlan& pl, double cost) {
     if (pl.defer) {
-      if (defer_slots(pl, n_out, m_most) * pl.bn * 128 * 4 > (64ull << 20)) return;
+      if (defer_slots(pl, n_out, m_bound) * pl.bn * 128 * 4 > (64ull << 20)) return;
       cost += pl.splits * (8.0 * n_out) * m_expected / 1.0e7;
     }
     if (cost < best_cost - 1e-9) {
@@ -574,7 +575,7 @@ void make_plans(ivit_handle* h) {
     // (under the MLP-on-all-tokens reading the out-projection goes to a cache, not to a layer norm)
     const bool defer = g == kGemmDown || (g == kGemmO && c.mlp_tokens == IVIT_MLP_UPDATED);
     auto plan = [&](int m_expected, int m_bound) {
-      return plan_gemm(h->num_sms, shapes[g][0], shapes[g][1], m_expected, m_bound, m_all, g != kGemmEmbed, defer);
+      return plan_gemm(h->num_sms, shapes[g][0], shapes[g][1], m_expected, m_bound, g != kGemmEmbed, defer);
     };
     h->plan_full[g] = plan(m_all, m_all);
     h->plan_inc[g] = g == kGemmEmbed ? h->plan_full[g] : plan(m_inc, m_all);
@@ -598,7 +599,7 @@ void make_plans(ivit_handle* h) {
   const bool one_plan = c.mlp_tokens == IVIT_MLP_ALL || c.select_mode != IVIT_SEL_TOPK;
   h->row_groups = one_plan && m_all > 64 && (c.mlp_tokens == IVIT_MLP_ALL || m_all / 10 <= 32) ? 2 : 1;
   // every row's D x D projection without a residual (first-layer key scores)
-  h->plan_keys = plan_gemm(h->num_sms, D, D, m_all, m_all, m_all, false, false);
+  h->plan_keys = plan_gemm(h->num_sms, D, D, m_all, m_all, false, false);
   if (std::getenv("IVIT_DEBUG")) {
     static const char* names[kGemmSlots] = {"embed", "qkv", "out", "up", "down"};
     auto show = [&](const char* when, const char* name, const GemmPlan& pl) {

@@ -42,5 +42,5 @@ def test_split_scratch_holds_every_row(probe, tokens, dim, heads, mlp, views, se
     rows = tokens * views
     plans = [pl for name, group in p.items() if name.startswith(("full", "inc", "band")) and name != "bands" for pl in group]
     need = max(scratch_of(pl, dim, rows) for pl in plans)
-    assert need <= p["scratch"] <= max(64, (64 << 20) // 4)
+    assert need <= p["scratch"]
     assert p["bands"][-1] == rows or len(p["bands"]) == 1
