@@ -102,8 +102,10 @@ int ivit_create(const ivit_config* cfg, const uint16_t* weights_bf16_host,
                 ivit_handle** out);
 
 /* Full encode of one frame per view (the paper's full forward that seeds the
- * reference, Sec. III-B).  frames_dev: uint8 [SV][img_h][img_w][3], any byte address
- * (an odd address makes the patchify kernel use byte loads).
+ * reference, Sec. III-B).  frames_dev: uint8 [SV][img_h][img_w][3], any byte address.
+ * The kernels read frames and write tokens and counts at the caller's addresses; frames
+ * at an odd address, a misaligned output (tokens 16 bytes, counts 4) and memory that is
+ * not the handle's GPU's go through one more copy on `stream`.
  * tokens_out_dev: bf16 [SV][N][D] final tokens (after the final LN), or NULL.
  * Re-seeds every cache and reference and marks every view warm. */
 int ivit_encode_full(ivit_handle* h, const uint8_t* frames_dev, uint16_t* tokens_out_dev,

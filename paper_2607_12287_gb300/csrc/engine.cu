@@ -208,6 +208,7 @@ struct ivit_handle {
   // caller's pointers (patchify before it, the output copy after it) are launched outside the
   // graph, so its kernel parameters never change.
   bool use_graphs = true;
+  uint8_t* frames_buf = nullptr;  // frames that patchify cannot read where they are
   cudaStream_t cap_stream = nullptr;
   cudaGraphExec_t graph_full = nullptr, graph_inc = nullptr;
   int64_t graph_full_launches = 0, graph_inc_launches = 0;
@@ -760,6 +761,7 @@ int setup(ivit_handle* h, const uint16_t* wb) {
   const size_t o_acache = c.mlp_tokens == IVIT_MLP_ALL ? sa.take(L * M * D * 4) : 0;
   const size_t o_gpart = sa.take(scratch_floats(h) * 4);
   const size_t o_rta = sa.take(M * 4), o_mall = sa.take(4);
+  const size_t o_fb = sa.take(static_cast<size_t>(h->SV) * c.img_h * c.img_w * 3);
   IVIT_CK(h, cudaMalloc(&h->smem, sa.size));
   IVIT_CK(h, cudaMemset(h->smem, 0, sa.size));
   sa.base = static_cast<char*>(h->smem);
@@ -787,6 +789,7 @@ int setup(ivit_handle* h, const uint16_t* wb) {
   h->gemm_partials = sa.at<float>(o_gpart);
   h->rowtok_all = sa.at<int>(o_rta);
   h->m_all = sa.at<int>(o_mall);
+  h->frames_buf = sa.at<uint8_t>(o_fb);
   {
     std::vector<int> ident(M);
     for (size_t i = 0; i < M; ++i) ident[i] = static_cast<int>(i);
@@ -1243,9 +1246,28 @@ void begin_record(ivit_handle* h) {
   next_launch(h, kFamOther, nullptr, 0);
 }
 
+// Whether the library's kernels may use a caller's pointer where it points: memory of the handle's
+// own GPU, aligned to `align`.  The copy engine carries everything else that it can reach, another
+// GPU's memory or pinned host memory, where a kernel would fault or run at the link's latency.
+bool in_place(const ivit_handle* h, const void* p, uintptr_t align) {
+  if (reinterpret_cast<uintptr_t>(p) & (align - 1)) return false;
+  cudaPointerAttributes at;
+  if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return at.type == cudaMemoryTypeDevice && at.device == h->device;
+}
+
 // The call's first kernel, from the caller's frames (eager, also before a replayed graph).
 int run_patchify(ivit_handle* h, const uint8_t* frames, cudaStream_t s) {
   const ivit_config& c = h->cfg;
+  // (patch rows of an even number of bytes are read two at a time)
+  if (!in_place(h, frames, c.patch % 2 ? 1 : 2)) {
+    const size_t bytes = static_cast<size_t>(h->SV) * c.img_h * c.img_w * 3;
+    IVIT_CK(h, cudaMemcpyAsync(h->frames_buf, frames, bytes, cudaMemcpyDefault, s));
+    frames = h->frames_buf;
+  }
   if (h->timeline && h->stamps)  // CTAs that leave early write nothing: clear the last call's stamps
     IVIT_CK(h, cudaMemsetAsync(h->stamps, 0, static_cast<size_t>(h->stamp_cap) * 2 * ivit::kStampCtas *
                                                  sizeof(unsigned long long), s));
@@ -1451,13 +1473,21 @@ int run(ivit_handle* h, const uint8_t* frames, uint16_t* out, int32_t* user_coun
   }
   // every output token (updated ones recomputed, the rest from the final-token cache) and the
   // views' counts, to the caller
+  const size_t tok_bytes = static_cast<size_t>(h->M_max) * h->D * 2;
+  if (out && !in_place(h, out, 16)) {
+    IVIT_CK(h, cudaMemcpyAsync(out, h->tok_out, tok_bytes, cudaMemcpyDefault, s));
+    out = nullptr;
+  }
+  if (user_counts && !in_place(h, user_counts, 4)) {
+    IVIT_CK(h, cudaMemcpyAsync(user_counts, h->counts, SV * sizeof(int), cudaMemcpyDefault, s));
+    user_counts = nullptr;
+  }
   if (out || user_counts) {
     h->slots_cur = h->slots_last;  // (a replayed graph's record, or this call's)
     h->stamp_used = static_cast<int>(h->slots_last.size());
     next_launch(h, kFamOther, nullptr, 4);
     h->slots_last = h->slots_cur;
-    IVIT_CK(h, ivit::launch_outputs(h->tok_out, out, static_cast<size_t>(h->M_max) * h->D * 2, h->counts, user_counts,
-                                    SV, h->num_sms, s));
+    IVIT_CK(h, ivit::launch_outputs(h->tok_out, out, tok_bytes, h->counts, user_counts, SV, h->num_sms, s));
     ivit::g_stamp = nullptr;
     ++h->launches;
   }

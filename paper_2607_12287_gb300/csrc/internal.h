@@ -215,8 +215,8 @@ cudaError_t launch_select(const float* sims, const float4* parts, int n_parts, i
                           const ColdMask& cold, int* idx, int* counts, int* cu_rows, int* done_ctr,
                           cudaStream_t s);
 
-// Copies the final tokens (bytes a multiple of 16) and the views' counts to the caller; either
-// destination may be null or of any alignment.
+// Copies the final tokens (bytes a multiple of 16, out aligned to 16) and the views' counts to the
+// caller, both in this GPU's memory; either destination may be null.
 cudaError_t launch_outputs(const bf16* tok, void* out, size_t bytes, const int* counts, int* user_counts, int sv,
                            int num_sms, cudaStream_t s);
 

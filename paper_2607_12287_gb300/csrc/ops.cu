@@ -823,21 +823,8 @@ cudaError_t launch_layernorm_ex(const int* rows, float* x, const float* add, con
                 layernorm_kernel<16, true, false>, layernorm_kernel<16, true, true>);
 }
 
-// (the copy engine's copies take over for pointers that the kernel's accesses do not fit)
 cudaError_t launch_outputs(const bf16* tok, void* out, size_t bytes, const int* counts, int* user_counts, int sv,
                            int num_sms, cudaStream_t s) {
-  auto fits = [](const void* p, uintptr_t a) { return (reinterpret_cast<uintptr_t>(p) & (a - 1)) == 0; };
-  if (out && !fits(out, 16)) {
-    const cudaError_t e = cudaMemcpyAsync(out, tok, bytes, cudaMemcpyDeviceToDevice, s);
-    if (e != cudaSuccess) return e;
-    out = nullptr;
-  }
-  if (user_counts && !fits(user_counts, 4)) {
-    const cudaError_t e = cudaMemcpyAsync(user_counts, counts, sv * sizeof(int), cudaMemcpyDeviceToDevice, s);
-    if (e != cudaSuccess) return e;
-    user_counts = nullptr;
-  }
-  if (!out && !user_counts) return cudaSuccess;
   const size_t n = out ? bytes / 16 : 0;
   const size_t blocks = (n + 4 * 256 - 1) / (4 * 256), most = static_cast<size_t>(num_sms) * 8;
   const unsigned grid = static_cast<unsigned>(blocks < 1 ? 1 : blocks < most ? blocks : most);

@@ -169,3 +169,44 @@ def test_outputs_at_any_alignment(pkg, offset):
         assert torch.equal(buf[offset:offset + n], want.reshape(-1))
         assert (buf[:offset] == 7).all() and (buf[offset + n:] == 7).all()
     enc.close()
+
+
+def test_pointers_outside_the_gpu_take_the_copy_engine(pkg):
+    """Frames, tokens and counts in pinned host memory (which, like another GPU's, the copy engine
+    reaches), and frames at an odd address: the results of buffers on the GPU, without the library's
+    output copy among the launches."""
+    import torch
+    from paper_2607_12287_gb300 import synth
+
+    shape = synth.EncoderShape(40, 104, 8, 192, 1, 3, 520, synth.GELU_TANH)
+    frames = list(synth.stream_random(shape, 2, 2, 11, change_p=0.4))
+    weights = synth.make_weights(shape, 3)
+
+    def encode(where):
+        enc = pkg.IncrementalViT(shape, weights, 1, 2)
+        host = where == "host"
+        out = torch.zeros(2, shape.n_tokens, shape.dim, dtype=torch.bfloat16, device="cpu" if host else "cuda", pin_memory=host)
+        cnt = torch.zeros(2, dtype=torch.int32, device=out.device, pin_memory=host)
+        got = []
+        for call, frame in enumerate(frames):
+            f = torch.from_numpy(frame).reshape(-1)
+            buf = torch.empty(f.numel() + 1, dtype=torch.uint8, device=out.device, pin_memory=host)
+            at = buf[1:] if where == "odd" else buf[:-1]
+            at.copy_(f)
+            torch.cuda.synchronize()
+            if call == 0:
+                pkg.ivit_encode_full(enc.h, at.data_ptr(), out.data_ptr())
+            else:
+                pkg.ivit_encode_incremental(enc.h, at.data_ptr(), out.data_ptr(), cnt.data_ptr())
+            torch.cuda.synchronize()
+            got.append((out.cpu().clone(), cnt.cpu().clone(), pkg.ivit_last_launch_count(enc.h)))
+        assert enc.device_status() == 0
+        enc.close()
+        return got
+
+    gpu = encode("gpu")
+    assert gpu[1][1].sum() > 0
+    for where, fewer in (("host", 1), ("odd", 0)):
+        for (tok, cnt, n), (tok0, cnt0, n0) in zip(encode(where), gpu):
+            assert torch.equal(tok, tok0) and torch.equal(cnt, cnt0), where
+            assert n == n0 - fewer, where
