@@ -17,7 +17,7 @@ OUT_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT_DIR, "libivit.so")
 SOURCES = ["gemm.cu", "gemm_pair.cu", "ops.cu", "attention.cu", "attention_rows.cu", "persistent.cu", "stream.cu", "engine.cu", "noalloc.cu",
            "action.cu"]
-HEADERS = ["ptx.cuh", "internal.h", "select.cuh", "attention.cuh"]
+HEADERS = ["ptx.cuh", "internal.h", "select.cuh", "attention.cuh", "gelu.cuh"]
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-I", os.path.join(ROOT, "include")]

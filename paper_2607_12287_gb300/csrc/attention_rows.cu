@@ -11,13 +11,15 @@
 //     dims 8 g .. 8 g + 7 of the keys 2 t, 2 t + 1, 2 t + 8, 2 t + 9 and interleaves them: the
 //     eight MMAs of a 64-dim block then each cover every eighth dim.  One or two 8-dim groups
 //     past a block (heads of 72 and 80) come in single elements.
-// Each warp keeps its own running maximum, sum and output; they meet once in shared memory.
+// Each warp keeps its own running maximum, sum and output; they meet once in shared memory.  In
+// the exact form a probability is three bf16 terms that together hold all 24 bits of its fp32
+// value, multiplied by V in turn.
 //
 // Bound: latency at small row counts (wait, one round trip, MMAs, one exchange); mma.sync's
 // rate at larger ones, where attention.cu is the faster one (the rule is attention_few in
 // engine.cu).  Heads of up to 64 have a form for two CTAs on an SM (128 registers; wider heads would
 // spill, 8.8 -> 11.6 us), taken when there are more items than SMs: six views of 196 x 196, 3 heads
-// of 64, 5.6 -> 4.9 us.  16 heads of 72, 256 keys, 26 queries: 3.9 us back to back against 6.1 there, whose
+// of 64, 5.6 -> 4.9 us (a full encode of them in the exact form: 384 us, 392 with one CTA).  16 heads of 72, 256 keys, 26 queries: 3.9 us back to back against 6.1 there, whose
 // 128-query tile walks the keys in three dependent steps.
 #include "attention.cuh"
 #include "internal.h"
@@ -45,9 +47,20 @@ __device__ __forceinline__ uint32_t word(const uint4& v, int i) {
   return i == 0 ? v.x : i == 1 ? v.y : i == 2 ? v.z : v.w;
 }
 
+__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
+  const __nv_bfloat162 b = __floats2bfloat162_rn(lo, hi);
+  return *reinterpret_cast<const uint32_t*>(&b);
+}
+
+// (bf16 widens to fp32 by its bits)
+__device__ __forceinline__ float2 unpack_bf16(uint32_t w) {
+  return make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
+}
+
 // NC: 32-dim chunks of a head (rounded up); NB: 64-dim blocks of V; R: 8-dim groups past them;
-// CTAS: CTAs per SM.
-template <int NC, int NB, int R, int CTAS>
+// CTAS: CTAs per SM; TERMS: bf16 terms of a probability in P V, 1 (rounded, and the normaliser
+// sums the rounded values) or 3 (all 24 bits of the fp32 value).
+template <int NC, int NB, int R, int CTAS, int TERMS>
 __global__ void __launch_bounds__(THREADS, CTAS) attention_rows_kernel(const AttnTcArgs a) {
   constexpr int NT = 8 * NB + R;             // output n-tiles
   constexpr int DW = 64 * NB + 8 * R + 4;    // floats of a partial output row
@@ -141,11 +154,15 @@ __global__ void __launch_bounds__(THREADS, CTAS) attention_rows_kernel(const Att
         float sum = 0.f;
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-          const __nv_bfloat162 b = __floats2bfloat162_rn(ex2(fmaf(sv[j][2 * r], sc, -mo)),
-                                                         ex2(fmaf(sv[j][2 * r + 1], sc, -mo)));
-          const float2 f = __bfloat1622float2(b);
+          float2 f = make_float2(ex2(fmaf(sv[j][2 * r], sc, -mo)), ex2(fmaf(sv[j][2 * r + 1], sc, -mo)));
+          if (TERMS == 1) {
+            p[j][r] = pack_bf16(f.x, f.y);
+            f = unpack_bf16(p[j][r]);
+          } else {
+            sv[j][2 * r] = f.x;
+            sv[j][2 * r + 1] = f.y;
+          }
           sum += f.x + f.y;  // the normaliser sums the values the MMA multiplies
-          p[j][r] = *reinterpret_cast<const uint32_t*>(&b);
         }
         l[r] = l[r] * alpha + sum;
         if (k0 >= WARPS * KW) {
@@ -158,20 +175,37 @@ __global__ void __launch_bounds__(THREADS, CTAS) attention_rows_kernel(const Att
       }
 #pragma unroll
       for (int u = 0; u < 2; ++u) {
-        const uint32_t a0 = p[2 * u][0], a1 = p[2 * u][1], a2 = p[2 * u + 1][0], a3 = p[2 * u + 1][1];
+        uint32_t pa[TERMS][4];
+#pragma unroll
+        for (int x = 0; x < TERMS; ++x)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const int j = 2 * u + (e >> 1), r = e & 1;
+            if (TERMS == 1) {
+              pa[x][e] = p[j][r];
+            } else {  // the next 8 bits of both probabilities
+              pa[x][e] = pack_bf16(sv[j][2 * r], sv[j][2 * r + 1]);
+              const float2 f = unpack_bf16(pa[x][e]);
+              sv[j][2 * r] -= f.x;
+              sv[j][2 * r + 1] -= f.y;
+            }
+          }
 #pragma unroll
         for (int b = 0; b < NB; ++b)
 #pragma unroll
           for (int j = 0; j < 8; ++j) {
             const uint32_t sel = (j & 1) ? 0x7632u : 0x5410u;
-            mma_bf16_16816(o[8 * b + j], a0, a1, a2, a3,
-                           __byte_perm(word(vf[u][0][b], j >> 1), word(vf[u][1][b], j >> 1), sel),
-                           __byte_perm(word(vf[u][2][b], j >> 1), word(vf[u][3][b], j >> 1), sel));
+            const uint32_t b0 = __byte_perm(word(vf[u][0][b], j >> 1), word(vf[u][1][b], j >> 1), sel),
+                           b1 = __byte_perm(word(vf[u][2][b], j >> 1), word(vf[u][3][b], j >> 1), sel);
+#pragma unroll
+            for (int x = 0; x < TERMS; ++x) mma_bf16_16816(o[8 * b + j], pa[x][0], pa[x][1], pa[x][2], pa[x][3], b0, b1);
           }
 #pragma unroll
-        for (int x = 0; x < R; ++x)
-          mma_bf16_16816(o[8 * NB + x], a0, a1, a2, a3, vr[u][0][x] | (vr[u][1][x] << 16),
-                         vr[u][2][x] | (vr[u][3][x] << 16));
+        for (int y = 0; y < R; ++y)
+#pragma unroll
+          for (int x = 0; x < TERMS; ++x)
+            mma_bf16_16816(o[8 * NB + y], pa[x][0], pa[x][1], pa[x][2], pa[x][3], vr[u][0][y] | (vr[u][1][y] << 16),
+                           vr[u][2][y] | (vr[u][3][y] << 16));
       }
     }
 
@@ -252,32 +286,44 @@ cudaError_t attention_rows_setup() {
       e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                static_cast<int>(bytes + 4 * (MAX_VIEWS + 1)));
   };
-  set(attention_rows_kernel<1, 1, 0, 1>, smem_bytes<1, 0>());
-  set(attention_rows_kernel<2, 1, 0, 1>, smem_bytes<1, 0>());
-  set(attention_rows_kernel<1, 1, 0, 2>, smem_bytes<1, 0>());
-  set(attention_rows_kernel<2, 1, 0, 2>, smem_bytes<1, 0>());
-  set(attention_rows_kernel<3, 1, 1, 1>, smem_bytes<1, 1>());
-  set(attention_rows_kernel<3, 1, 2, 1>, smem_bytes<1, 2>());
-  set(attention_rows_kernel<3, 2, 0, 1>, smem_bytes<2, 0>());
-  set(attention_rows_kernel<4, 2, 0, 1>, smem_bytes<2, 0>());
+  auto both = [&](auto rounded, auto exact, size_t bytes) {
+    set(rounded, bytes);
+    set(exact, bytes);
+  };
+  both(attention_rows_kernel<1, 1, 0, 1, 1>, attention_rows_kernel<1, 1, 0, 1, 3>, smem_bytes<1, 0>());
+  both(attention_rows_kernel<2, 1, 0, 1, 1>, attention_rows_kernel<2, 1, 0, 1, 3>, smem_bytes<1, 0>());
+  both(attention_rows_kernel<1, 1, 0, 2, 1>, attention_rows_kernel<1, 1, 0, 2, 3>, smem_bytes<1, 0>());
+  both(attention_rows_kernel<2, 1, 0, 2, 1>, attention_rows_kernel<2, 1, 0, 2, 3>, smem_bytes<1, 0>());
+  set(attention_rows_kernel<3, 1, 1, 1, 1>, smem_bytes<1, 1>());
+  both(attention_rows_kernel<3, 1, 2, 1, 1>, attention_rows_kernel<3, 1, 2, 1, 3>, smem_bytes<1, 2>());
+  both(attention_rows_kernel<3, 2, 0, 1, 1>, attention_rows_kernel<3, 2, 0, 1, 3>, smem_bytes<2, 0>());
+  both(attention_rows_kernel<4, 2, 0, 1, 1>, attention_rows_kernel<4, 2, 0, 1, 3>, smem_bytes<2, 0>());
   return e;
 }
 
-cudaError_t launch_attention_rows(const AttnTcArgs& a, int num_sms, int ctas, cudaStream_t s) {
+cudaError_t launch_attention_rows(const AttnTcArgs& a, int num_sms, int ctas, bool exact, cudaStream_t s) {
   if (a.sv > MAX_VIEWS || a.dh % 8 || a.dh > 128) return cudaErrorInvalidValue;
   const bool two = ctas == 2 && a.dh <= 64;
   const int grid = max(1, min(a.sv * a.heads * ((a.n_tok + TQ - 1) / TQ), two ? 2 * num_sms : num_sms));
-  auto launch = [&](auto kern, size_t bytes) {
-    return launch_ex(kern, dim3(grid), dim3(THREADS), bytes + 4 * (a.sv + 1), s, 1, a);
+  auto launch = [&](auto rounded, auto full, size_t bytes) {
+    return launch_ex(exact ? full : rounded, dim3(grid), dim3(THREADS), bytes + 4 * (a.sv + 1), s, 1, a);
   };
-  if (two && a.dh <= 32) return launch(attention_rows_kernel<1, 1, 0, 2>, smem_bytes<1, 0>());
-  if (two && a.dh <= 64) return launch(attention_rows_kernel<2, 1, 0, 2>, smem_bytes<1, 0>());
-  if (a.dh <= 32) return launch(attention_rows_kernel<1, 1, 0, 1>, smem_bytes<1, 0>());
-  if (a.dh <= 64) return launch(attention_rows_kernel<2, 1, 0, 1>, smem_bytes<1, 0>());
-  if (a.dh == 72) return launch(attention_rows_kernel<3, 1, 1, 1>, smem_bytes<1, 1>());
-  if (a.dh == 80) return launch(attention_rows_kernel<3, 1, 2, 1>, smem_bytes<1, 2>());
-  if (a.dh <= 96) return launch(attention_rows_kernel<3, 2, 0, 1>, smem_bytes<2, 0>());
-  return launch(attention_rows_kernel<4, 2, 0, 1>, smem_bytes<2, 0>());
+  if (two && a.dh <= 32)
+    return launch(attention_rows_kernel<1, 1, 0, 2, 1>, attention_rows_kernel<1, 1, 0, 2, 3>, smem_bytes<1, 0>());
+  if (two) return launch(attention_rows_kernel<2, 1, 0, 2, 1>, attention_rows_kernel<2, 1, 0, 2, 3>, smem_bytes<1, 0>());
+  if (a.dh <= 32)
+    return launch(attention_rows_kernel<1, 1, 0, 1, 1>, attention_rows_kernel<1, 1, 0, 1, 3>, smem_bytes<1, 0>());
+  if (a.dh <= 64)
+    return launch(attention_rows_kernel<2, 1, 0, 1, 1>, attention_rows_kernel<2, 1, 0, 1, 3>, smem_bytes<1, 0>());
+  if (a.dh == 72) {  // (an encoder with such heads is at least 576 wide: no exact form)
+    if (exact) return cudaErrorInvalidValue;
+    return launch(attention_rows_kernel<3, 1, 1, 1, 1>, attention_rows_kernel<3, 1, 1, 1, 1>, smem_bytes<1, 1>());
+  }
+  if (a.dh == 80)
+    return launch(attention_rows_kernel<3, 1, 2, 1, 1>, attention_rows_kernel<3, 1, 2, 1, 3>, smem_bytes<1, 2>());
+  if (a.dh <= 96)
+    return launch(attention_rows_kernel<3, 2, 0, 1, 1>, attention_rows_kernel<3, 2, 0, 1, 3>, smem_bytes<2, 0>());
+  return launch(attention_rows_kernel<4, 2, 0, 1, 1>, attention_rows_kernel<4, 2, 0, 1, 3>, smem_bytes<2, 0>());
 }
 
 }  // namespace ivit

@@ -25,6 +25,7 @@
 // 5.3 -> 3.9; a further 32 rows cost 2.3 to 2.8 us, so the CTA-pair kernel takes over past
 // about 64.  Fetching a next pass's rows early made one pass 0.7 us slower (the loop's code
 // is on the critical path) and was left out.
+#include "gelu.cuh"
 #include "internal.h"
 #include "ptx.cuh"
 
@@ -45,20 +46,6 @@ __device__ __forceinline__ int red_at(int r, int f) {
 // Bytes from one feature's weights to the next in shared memory: 64 bytes past a multiple of
 // 128, so that the 16-byte loads of two features by 8 lanes cover all banks.
 __host__ __device__ __forceinline__ int w_pitch(int k) { return (k * 2 + 127) / 128 * 128 + 64; }
-
-// Hardware tanh (one MUFU instruction, relative error about 2^-11: below the bf16
-// rounding the GELU output gets).
-__device__ __forceinline__ float tanh_hw(float x) {
-  float y;
-  asm("tanh.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-
-__device__ __forceinline__ float gelu_f(float x, int mode) {
-  if (mode == 1) return 0.5f * x * (1.f + erff(x * 0.70710678118654752f));
-  const float c = 0.79788456080286536f;  // sqrt(2/pi)
-  return 0.5f * x * (1.f + tanh_hw(c * (x + 0.044715f * x * x * x)));
-}
 
 __device__ __forceinline__ uint2 pack4(float4 v) {
   const __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);
@@ -207,9 +194,9 @@ __global__ void __launch_bounds__(THREADS, 2) gemm_rows_kernel(const GemmArgs a)
                            : (f4 < 2 * D ? a.epi.cache_k + static_cast<size_t>(tok) * D + (f4 - D)
                                          : a.epi.cache_v + static_cast<size_t>(tok) * D + (f4 - 2 * D));
         *reinterpret_cast<uint2*>(dst) = pack4(y);
-      } else if (KIND == kEpiGelu) {
-        y = make_float4(gelu_f(y.x, a.epi.gelu_mode), gelu_f(y.y, a.epi.gelu_mode), gelu_f(y.z, a.epi.gelu_mode),
-                        gelu_f(y.w, a.epi.gelu_mode));
+      } else if (KIND == kEpiGelu || KIND == kEpiGeluTanhf) {
+        const int mode = a.epi.gelu_mode;
+        y = make_float4(gelu_f<KIND>(y.x, mode), gelu_f<KIND>(y.y, mode), gelu_f<KIND>(y.z, mode), gelu_f<KIND>(y.w, mode));
         *reinterpret_cast<uint2*>(a.epi.out_bf16 + static_cast<size_t>(r) * a.epi.ld_out + f4) = pack4(y);
       } else if (KIND == kEpiResid) {
         red_add_f32x4(a.epi.out_f32 + static_cast<size_t>(r) * a.epi.ld_out + f4, y);
@@ -240,6 +227,7 @@ cudaError_t launch_nt(const GemmArgs& a, cudaStream_t s) {
     case kEpiQKV: return launch(gemm_rows_kernel<NT, kEpiQKV>);
     case kEpiResid: return launch(gemm_rows_kernel<NT, kEpiResid>);
     case kEpiGelu: return launch(gemm_rows_kernel<NT, kEpiGelu>);
+    case kEpiGeluTanhf: return launch(gemm_rows_kernel<NT, kEpiGeluTanhf>);
     case kEpiScatterF32: return launch(gemm_rows_kernel<NT, kEpiScatterF32>);
     default: return cudaErrorInvalidValue;
   }
@@ -256,6 +244,7 @@ cudaError_t setup_nt() {
   set(gemm_rows_kernel<NT, kEpiQKV>);
   set(gemm_rows_kernel<NT, kEpiResid>);
   set(gemm_rows_kernel<NT, kEpiGelu>);
+  set(gemm_rows_kernel<NT, kEpiGeluTanhf>);
   set(gemm_rows_kernel<NT, kEpiScatterF32>);
   return e;
 }

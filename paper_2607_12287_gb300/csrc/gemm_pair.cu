@@ -24,6 +24,7 @@
 // (1750 TFLOP/s), up 497 -> 198, out 154 -> 82, down 324 -> 211; 3080 rows QKV 65 -> 22, up
 // 60 -> 24, down 53 -> 26; 768 rows QKV 29 -> 12, up 27 -> 12; 256 rows QKV 16 -> 7.6,
 // up 16 -> 7.8.
+#include "gelu.cuh"
 #include "internal.h"
 #include "ptx.cuh"
 
@@ -57,20 +58,6 @@ struct PairCfg {
   static_assert(TOTAL <= 227 * 1024, "shared memory of one CTA");
 };
 
-// Hardware tanh (one MUFU instruction, relative error about 2^-11: below the bf16
-// rounding the GELU output gets).
-__device__ __forceinline__ float tanh_hw(float x) {
-  float y;
-  asm("tanh.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-
-__device__ __forceinline__ float gelu_f(float x, int mode) {
-  if (mode == 1) return 0.5f * x * (1.f + erff(x * 0.70710678118654752f));
-  const float c = 0.79788456080286536f;  // sqrt(2/pi)
-  return 0.5f * x * (1.f + tanh_hw(c * (x + 0.044715f * x * x * x)));
-}
-
 // Sums over a warp of three values of four rows each (v[row]): lanes 8 k .. 8 k + 7 get row k's.
 __device__ __forceinline__ float3 sum_rows4(const float3 (&v)[4], int lane) {
   auto fold = [&](const float3& keep, const float3& send, int o) {
@@ -97,7 +84,7 @@ template <int KIND, int BUFS, class Ready, class Release>
 __device__ __forceinline__ void drain(const GemmArgs& a, uint32_t acc, uint8_t* stg, int bar_id, int wq, int lane,
                                       int row0, int c_lo, int c_hi, int ft, float* slot, int& buf, Ready ready,
                                       Release release) {
-  constexpr bool kBf16 = KIND == kEpiQKV || KIND == kEpiGelu;
+  constexpr bool kGelu = KIND == kEpiGelu || KIND == kEpiGeluTanhf, kBf16 = KIND == kEpiQKV || kGelu;
   constexpr int CHUNK = kBf16 ? 32 : 16;
   constexpr bool kAhead = BUFS == 2, kByTok = KIND == kEpiQKV || KIND == kEpiScatterF32;
   const int f0 = ft * BM, fl = wq * 32 + lane;
@@ -117,7 +104,7 @@ __device__ __forceinline__ void drain(const GemmArgs& a, uint32_t acc, uint8_t* 
     dst16 = f < D ? a.epi.out_bf16 + f : f < 2 * D ? a.epi.cache_k + (f - D) : a.epi.cache_v + (f - 2 * D);
     by_tok = f >= D;
     ld = D;
-  } else if (KIND == kEpiGelu) {
+  } else if (kGelu) {
     dst16 = a.epi.out_bf16 + f;
   } else if (KIND == kEpiPartial) {
     dst32 = slot + FPT * sub;
@@ -187,7 +174,7 @@ __device__ __forceinline__ void drain(const GemmArgs& a, uint32_t acc, uint8_t* 
 #pragma unroll
       for (int j = 0; j < CHUNK; ++j) {
         float y = __uint_as_float(v[j]) + bias;
-        if (KIND == kEpiGelu) y = gelu_f(y, a.epi.gelu_mode);
+        if (kGelu) y = gelu_f<KIND>(y, a.epi.gelu_mode);
         st[j * BM] = __float2bfloat16_rn(y);
       }
     } else {
@@ -532,6 +519,7 @@ cudaError_t launch_bn(const CUtensorMap& tm_w, const CUtensorMap& tm_x, const Ge
     case kEpiQKV: return launch_one<BN, kEpiQKV>(tm_w, tm_x, a, n_pairs, s);
     case kEpiResid: return launch_one<BN, kEpiResid>(tm_w, tm_x, a, n_pairs, s);
     case kEpiGelu: return launch_one<BN, kEpiGelu>(tm_w, tm_x, a, n_pairs, s);
+    case kEpiGeluTanhf: return launch_one<BN, kEpiGeluTanhf>(tm_w, tm_x, a, n_pairs, s);
     case kEpiScatterF32: return launch_one<BN, kEpiScatterF32>(tm_w, tm_x, a, n_pairs, s);
     case kEpiScore: return launch_one<BN, kEpiScore>(tm_w, tm_x, a, n_pairs, s);
     default: return cudaErrorInvalidValue;
@@ -548,6 +536,7 @@ cudaError_t setup_bn() {
   set(gemm_pair_kernel<BN, kEpiQKV>);
   set(gemm_pair_kernel<BN, kEpiResid>);
   set(gemm_pair_kernel<BN, kEpiGelu>);
+  set(gemm_pair_kernel<BN, kEpiGeluTanhf>);
   set(gemm_pair_kernel<BN, kEpiScatterF32>);
   set(gemm_pair_kernel<BN, kEpiScore>);
   set(gemm_pair_kernel<BN, kEpiPartial>);

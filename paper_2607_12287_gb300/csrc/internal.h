@@ -59,6 +59,7 @@ enum EpiKind : int {
   kEpiScatterF32 = 4,  // out_f32[rowtok[r]][f] = y + bias[f]  (per-token output cache)
   kEpiScore = 6,       // out_f32[r][f] = y + bias[f], and sums for the cosine of row r with its old
                        // content: score[feature tile of 128 * m_static + r] (Eq. 3)
+  kEpiGeluTanhf = 7,   // as kEpiGelu, tanh form, with tanhf in place of the hardware's tanh
   kEpiPartial = 5,     // a K split's fp32 tile, left in the scratch (GemmArgs::defer)
 };
 
@@ -318,8 +319,9 @@ cudaError_t launch_attention_tc(const AttnMaps& q, const AttnMaps& k, const Attn
                                 int num_sms, cudaStream_t s);
 
 // The same for a few queries per view, without TMA maps: CTAs walk (view, head, 16-query tile)
-// items, `ctas` (1, or 2 for heads of up to 64) per SM.
+// items, `ctas` (1, or 2 for heads of up to 64) per SM; with `exact` the probabilities are not
+// rounded to bf16.
 cudaError_t attention_rows_setup();
-cudaError_t launch_attention_rows(const AttnTcArgs& a, int num_sms, int ctas, cudaStream_t s);
+cudaError_t launch_attention_rows(const AttnTcArgs& a, int num_sms, int ctas, bool exact, cudaStream_t s);
 
 }  // namespace ivit

@@ -1,0 +1,99 @@
+"""Full encodes of small encoders (dim up to 384, at most 256 tokens per view) keep the softmax's
+probabilities and GELU's tanh in fp32: inputs that cancel what would hide a bf16 probability or the
+hardware's tanh, against a float64 restatement of the same bf16 operands."""
+import numpy as np
+import pytest
+
+from paper_2607_12287_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def pkg():
+    import paper_2607_12287_gb300 as p
+    p.load()
+    return p
+
+
+def _bf16(x):
+    return synth.bf16_bits_to_f32(synth.f32_to_bf16_bits(np.asarray(x, np.float32))).astype(np.float64)
+
+
+def _ln(x):
+    c = x - x.mean(-1, keepdims=True)
+    return c / np.sqrt((c * c).mean(-1, keepdims=True) + 1e-6)
+
+
+def _encode(pkg, grid, dim, heads, mlp, **tensors):
+    """One layer on one view whose patches embed to zero, so that the residual stream starts as `pos`:
+    the tokens, and the layer's keys and values."""
+    import torch
+    shape = synth.EncoderShape(grid[0], grid[1], 1, dim, 1, heads, mlp, synth.GELU_TANH)
+    flat = np.zeros(synth.weight_count(shape), np.uint16)
+    w = synth.split_weights(shape, flat)
+    for name, t in w.items():
+        if name.endswith("_g"):
+            t[...] = synth.f32_to_bf16_bits(np.float32([1.0]))[0]
+        for key, value in tensors.items():
+            if name.split(".")[-1] == key:
+                t[...] = synth.f32_to_bf16_bits(np.asarray(value, np.float32).reshape(-1)).reshape(t.shape)
+    enc = pkg.IncrementalViT(shape, flat, 1, 1)
+    out = enc.encode_full(torch.zeros(1, grid[0], grid[1], 3, dtype=torch.uint8, device="cuda"))
+    got = [t.float().cpu().numpy().astype(np.float64)[0] for t in (out, enc.cache("K", 0), enc.cache("V", 0))]
+    assert enc.device_status() == 0
+    enc.close()
+    return got
+
+
+@pytest.mark.parametrize("path", ["kernels", "persistent"])
+@pytest.mark.parametrize("grid,dim,heads", [((14, 14), 192, 3), ((16, 16), 256, 8), ((12, 17), 320, 4), ((7, 10), 192, 2),
+                                            ((16, 16), 384, 3), ((1, 6), 64, 4)],
+                         ids=["dh64", "dh32", "dh80", "dh96", "dh128", "dh16"])
+def test_probabilities_in_fp32(pkg, monkeypatch, path, grid, dim, heads):
+    """Tokens come in pairs with opposite values and keys that are nearly the same, so that O is a sum of
+    differences of probabilities, 1 % of them: rounding those to bf16 leaves an error of 2 to 4 % of it, the
+    roundings of O and of the tokens to bf16 one of 2^-9."""
+    monkeypatch.setenv("IVIT_PATH", path)
+    rng = np.random.default_rng(dim)
+    n, dh, half = grid[0] * grid[1], dim // heads, dim // 2
+    even = rng.standard_normal((n // 2, half))
+    odd = rng.standard_normal((n // 2, half // 2))
+    odd = np.concatenate([odd, -odd], 1)  # (sums to zero: the pair has one mean and variance)
+    pos = np.empty((n, dim))
+    pos[0::2] = np.concatenate([even, odd], 1)
+    pos[1::2] = np.concatenate([even, -odd], 1)
+    pos = _bf16(pos)
+    w_qkv = np.zeros((3 * dim, dim))
+    w_qkv[:2 * dim, :half] = rng.standard_normal((2 * dim, half)) / np.sqrt(half)
+    w_qkv[dim:2 * dim, half:] = 0.005 * rng.standard_normal((dim, half)) / np.sqrt(half)
+    w_qkv[2 * dim:, half:] = rng.standard_normal((dim, half)) / np.sqrt(half)
+    w_qkv = _bf16(w_qkv)
+    gain = 2.0 ** 12
+    out, k, v = _encode(pkg, grid, dim, heads, 64, pos=pos, W_qkv=w_qkv, W_o=gain * np.eye(dim))
+    q = _bf16(_bf16(_ln(pos)) @ w_qkv[:dim].T).reshape(n, heads, dh)
+    k, v = k.reshape(n, heads, dh), v.reshape(n, heads, dh)
+    s = np.einsum("qhd,khd->hqk", q, k) / np.sqrt(dh)
+    p = np.exp(s - s.max(-1, keepdims=True))
+    o = np.einsum("hqk,khd->qhd", p / p.sum(-1, keepdims=True), v).reshape(n, dim)
+    want = _ln(pos + gain * o)
+    err = np.linalg.norm(out - want) / np.linalg.norm(want)
+    assert err < 0.01, err
+
+
+@pytest.mark.parametrize("path", ["kernels", "persistent"])
+@pytest.mark.parametrize("grid,dim", [((14, 14), 384), ((4, 5), 384)], ids=["n196", "n20"])
+def test_gelu_tanh_in_fp32(pkg, monkeypatch, path, grid, dim):
+    """The MLP is h = GELU(LN(x)) added to x with a large gain, so that a hidden value rounded to another
+    bf16 shows in the tokens: the hardware's tanh (2^-11) moves 0.7 % of them, fp32's one in 10^5."""
+    monkeypatch.setenv("IVIT_PATH", path)
+    rng = np.random.default_rng(dim)
+    n = grid[0] * grid[1]
+    pos = _bf16(rng.uniform(-1, 1, (n, dim)))
+    gain = 2.0 ** 12
+    out, _, _ = _encode(pkg, grid, dim, dim // 64, dim, pos=pos, W_1=np.eye(dim), W_2=gain * np.eye(dim))
+    y = _bf16(_ln(pos))
+    h = _bf16(0.5 * y * (1 + np.tanh(np.sqrt(2 / np.pi) * (y + 0.044715 * y ** 3))))
+    want = _bf16(_ln(pos + gain * h))
+    moved = np.mean(out != want)
+    assert moved < 0.001, moved
