@@ -289,7 +289,7 @@ __global__ void __launch_bounds__(THREADS, 2)
           alpha = ex2((m_ref - m_blk) * sc);
           m_ref = m_blk;
         }
-        const float mo = m_ref * sc;
+        const float mo = m_ref == -INFINITY ? 0.f : m_ref * sc;  // (scores of -inf alone so far: P = 0)
         const bool rescale = __any_sync(0xffffffffu, grow);
         if (rescale) {
 #pragma unroll

@@ -149,7 +149,8 @@ __global__ void __launch_bounds__(THREADS, CTAS) attention_rows_kernel(const Att
         for (int j = 0; j < 4; ++j) mx = fmaxf(mx, fmaxf(sv[j][2 * r], sv[j][2 * r + 1]));
         mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
         mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-        const float m_new = fmaxf(m[r], mx), alpha = ex2((m[r] - m_new) * sc), mo = m_new * sc;
+        const float m_new = fmaxf(m[r], mx), m_fin = m_new == -INFINITY ? 0.f : m_new;  // (scores of -inf alone so far:
+        const float alpha = ex2((m[r] - m_fin) * sc), mo = m_fin * sc;                  // P = 0, nothing to rescale)
         m[r] = m_new;
         float sum = 0.f;
 #pragma unroll

@@ -1,6 +1,6 @@
-"""Full encodes of small encoders (dim up to 384, at most 256 tokens per view) keep the softmax's
-probabilities and GELU's tanh in fp32: inputs that cancel what would hide a bf16 probability or the
-hardware's tanh, against a float64 restatement of the same bf16 operands."""
+"""Numerics that weights of the usual scale do not show, on one layer against a float64 restatement
+of the same bf16 operands: full encodes of small encoders (dim up to 384, at most 256 tokens per
+view) keep the softmax's probabilities and GELU's tanh in fp32; large and infinite scores."""
 import numpy as np
 import pytest
 
@@ -97,3 +97,34 @@ def test_gelu_tanh_in_fp32(pkg, monkeypatch, path, grid, dim):
     want = _bf16(_ln(pos + gain * h))
     moved = np.mean(out != want)
     assert moved < 0.001, moved
+
+
+@pytest.mark.parametrize("kernel", ["tc", "rows", "exact"])
+@pytest.mark.parametrize("dim,heads", [(192, 3), (576, 8), (256, 2), (320, 10)], ids=["dh64", "dh72", "dh128", "dh32"])
+def test_scores_of_minus_infinity(pkg, monkeypatch, dim, heads, kernel):
+    """The first 140 keys' scores overflow to -inf, a whole key block and several warps' shares of the keys:
+    they take no part, as in a softmax over all keys."""
+    if kernel == "exact" and dim > 384:
+        pytest.skip("full encodes of small encoders only")
+    if kernel != "exact":
+        monkeypatch.setenv("IVIT_ATTN", kernel)
+    grid = (14, 14) if kernel == "exact" else (16, 17)
+    rng = np.random.default_rng(dim)
+    n, dh, masked = grid[0] * grid[1], dim // heads, 140
+    half = rng.choice([-1.0, 1.0], (n, dim // 2 - 1)) * rng.choice([0.5, 1.0, 2.0], (n, dim // 2 - 1))
+    pos = np.concatenate([np.zeros((n, 1)), half, np.zeros((n, 1)), -half], 1)  # (rows sum to zero exactly)
+    pos[:masked, 0], pos[:masked, dim // 2] = -2.0, 2.0
+    w_qkv, b_qkv = np.zeros((3 * dim, dim)), np.zeros(3 * dim)
+    b_qkv[:dim] = 1e15                                                # q k = -1e40 for the masked keys,
+    w_qkv[dim:2 * dim] = 1e-15 * rng.standard_normal((dim, dim)) / np.sqrt(dim)  # of order one for the others
+    w_qkv[dim:2 * dim, 0] = 1e25
+    w_qkv[2 * dim:] = rng.standard_normal((dim, dim)) / np.sqrt(dim)
+    out, k, v = _encode(pkg, grid, dim, heads, 64, pos=pos, W_qkv=w_qkv, b_qkv=b_qkv, W_o=2.0 ** 6 * np.eye(dim))
+    q = _bf16(b_qkv[:dim]).reshape(1, heads, dh)
+    s = np.einsum("qhd,khd->hqk", q, k.reshape(n, heads, dh)[masked:]) / np.sqrt(dh)
+    p = np.exp(s - s.max(-1, keepdims=True))
+    o = np.einsum("hqk,khd->qhd", p / p.sum(-1, keepdims=True), v.reshape(n, heads, dh)[masked:]).reshape(1, dim)
+    want = _ln(pos + 2.0 ** 6 * o)
+    assert np.isfinite(out).all()
+    err = np.linalg.norm(out - want) / np.linalg.norm(want)
+    assert err < 0.01, err  # roundings of P, O and the tokens to bf16, 2^-9 each
