@@ -128,3 +128,27 @@ def test_scores_of_minus_infinity(pkg, monkeypatch, dim, heads, kernel):
     assert np.isfinite(out).all()
     err = np.linalg.norm(out - want) / np.linalg.norm(want)
     assert err < 0.01, err  # roundings of P, O and the tokens to bf16, 2^-9 each
+
+
+@pytest.mark.parametrize("kernel", ["tc", "rows"])
+@pytest.mark.parametrize("dim,heads", [(64, 4), (64, 2), (192, 4), (64, 1), (320, 4), (192, 2), (448, 4), (128, 1)],
+                         ids=lambda x: str(x))
+def test_scores_that_grow_from_block_to_block(pkg, monkeypatch, dim, heads, kernel):
+    """Scores of standard deviation 12: the running maximum moves by more than 2^8 in many rows, so that sums
+    and outputs of earlier key blocks are rescaled, in every padded head width."""
+    monkeypatch.setenv("IVIT_ATTN", kernel)
+    rng = np.random.default_rng(dim + heads)
+    grid, n, dh = (20, 20), 400, dim // heads
+    pos = _bf16(rng.standard_normal((n, dim)))
+    w_qkv = _bf16(rng.standard_normal((3 * dim, dim)) * np.sqrt(12.0 / dim))
+    out, k, v = _encode(pkg, grid, dim, heads, 64, pos=pos, W_qkv=w_qkv, W_o=2.0 ** 6 * np.eye(dim))
+    q = _bf16(_bf16(_ln(pos)) @ w_qkv[:dim].T).reshape(n, heads, dh)
+    s = np.einsum("qhd,khd->hqk", q, k.reshape(n, heads, dh)) / np.sqrt(dh)
+    for kb in (64, 96, 128, 256):  # (the tensor-core kernel's key blocks, and one step of the few-query kernel)
+        blocks = np.stack([s[..., i:i + kb].max(-1) for i in range(0, n, kb)], -1) * np.log2(np.e)
+        assert ((blocks[..., 1:] - np.maximum.accumulate(blocks, -1)[..., :-1]).max(-1) > 8).mean() > 0.01
+    p = np.exp(s - s.max(-1, keepdims=True))
+    o = np.einsum("hqk,khd->qhd", p / p.sum(-1, keepdims=True), v.reshape(n, heads, dh)).reshape(n, dim)
+    want = _ln(pos + 2.0 ** 6 * o)
+    err = np.linalg.norm(out - want) / np.linalg.norm(want)
+    assert err < 0.01, err  # roundings of P, O and the tokens to bf16, 2^-9 each
