@@ -151,8 +151,6 @@ struct ivit_handle {
   int band_ub[4] = {0, 0, 0, 0};
   GemmPlan plan_band[4][kGemmSlots];
   bool capture_bands = false;  // set while the incremental graph is captured with bands
-  int known_band = -1;         // set while it is captured for a row count known in advance,
-  int known_rows = 0;          // this one
   ivit::RowBands bands;        // the switch node's handle and the bands' row bounds
   cudaStream_t cap_stream2 = nullptr;  // captures the band bodies
 
@@ -1039,11 +1037,10 @@ ivit::PendingSum pending_sum(ivit_handle* h, const GemmPlan& pl, const float* bi
 // tokens and the output projection, whose result replaces their rows of the layer's
 // attention-output cache; then every token adds its cached attention output to its
 // stream (fused into LN2) and runs the MLP; the final LN writes every output token.
-int run_layers_mlp_all(ivit_handle* h, const GemmPlan* plan, bool full, cudaStream_t s) {
+int run_layers_mlp_all(ivit_handle* h, const GemmPlan* plan, int m_expected, cudaStream_t s) {
   const ivit_config& c = h->cfg;
   const int N = h->N, D = h->D, F = h->F, SV = h->SV, M = h->M_max;
   const int* total = h->cu_rows + SV;
-  const int m_expected = full ? M : std::max(1, M / 10);
   // The down-projection's residual update of every token may still be split over the GEMM
   // scratch: the next layer's LN1 reads it for the updated tokens, its LN2 adds it to x.
   ivit::PendingSum pend;
@@ -1281,6 +1278,25 @@ int run_patchify(ivit_handle* h, const uint8_t* frames, cudaStream_t s) {
   return IVIT_OK;
 }
 
+// Launch plans of a call, and the updated rows that it expects.  A cold view updates every token,
+// a warm one k of them under top-k, so those calls take the band of that count: a cold 256-token
+// So400m view, four layers, takes 194 us, and 535 (top-k) or 354 (threshold) with the plans of a
+// tenth of its tokens.  Other calls' counts are known only on the device; a tenth is assumed.  (Any
+// count runs correctly: top-k selects NaN scores beside its k.)
+const GemmPlan* plan_of_call(const ivit_handle* h, bool full, int& m_expected) {
+  m_expected = h->M_max;
+  if (full) return h->plan_full;
+  const bool topk = h->cfg.select_mode == IVIT_SEL_TOPK;
+  const int n_cold = static_cast<int>(std::count_if(h->cold.begin(), h->cold.end(), [](uint8_t c) { return c != 0; }));
+  m_expected = std::max(1, h->M_max / 10);
+  if (!n_cold && (!topk || h->cfg.mlp_tokens == IVIT_MLP_ALL)) return h->plan_inc;
+  const int warm = h->SV - n_cold;
+  m_expected = std::max(1, n_cold * h->N + (topk ? warm * std::min(h->cfg.topk, h->N) : warm * h->N / 10));
+  int b = 0;
+  while (b + 1 < h->n_bands && m_expected > h->band_ub[b]) ++b;
+  return h->plan_band[b];
+}
+
 // Enqueues the rest of the chain for one frame per view on `s` (eagerly or under capture).
 int run_core(ivit_handle* h, bool full, cudaStream_t s) {
   const ivit_config& c = h->cfg;
@@ -1289,7 +1305,8 @@ int run_core(ivit_handle* h, bool full, cudaStream_t s) {
   std::memset(&cm, 0, sizeof cm);
   for (int v = 0; v < SV; ++v)
     if (full || h->cold[v]) cm.bits[v >> 5] |= 1u << (v & 31);
-  const GemmPlan* plan = full ? h->plan_full : h->plan_inc;
+  int m_expected = 0;
+  const GemmPlan* plan = plan_of_call(h, full, m_expected);
   const int* total = h->cu_rows + SV;
 
   {
@@ -1347,7 +1364,7 @@ int run_core(ivit_handle* h, bool full, cudaStream_t s) {
     IVIT_CK(h, ivit::launch_gather(total, h->rowtok, lists, h->e_t, h->pos, nullptr, score_vec, h->e_ref, N, D,
                                    c.ref_mode == IVIT_REF_LAST_REFRESH, cm, M, h->row_grid, s));
     h->launches += 2;
-    return run_layers_mlp_all(h, plan, full, s);
+    return run_layers_mlp_all(h, plan, m_expected, s);
   }
   ivit::RowBands bands;  // (no switch node: handle 0)
   if (h->capture_bands) {
@@ -1391,13 +1408,11 @@ int run_core(ivit_handle* h, bool full, cudaStream_t s) {
     return IVIT_OK;
   }
   if (h->capture_bands) return capture_band_bodies(h, s);
-  if (!full && h->known_band >= 0)  // top-k: the row count is fixed, so is its band
-    return run_layers(h, h->plan_band[h->known_band], h->known_rows, false, s);
   // The full encodes of small encoders have their probabilities and tanh in fp32, where every other
   // call has bf16 and the hardware's tanh (what the persistent kernel, which these encodes once
   // took, computes): six 196-token views of ViT-Tiny 384 us, 379 with rounded probabilities.
   const bool exact = full && D <= 384 && N <= 256;
-  return run_layers(h, plan, full ? M : std::max(1, M / 10), exact, s);
+  return run_layers(h, plan, m_expected, exact, s);
 }
 
 int capture_once(ivit_handle* h, bool full, cudaGraphExec_t* exec, int64_t* launches);
@@ -1407,22 +1422,10 @@ int capture_once(ivit_handle* h, bool full, cudaGraphExec_t* exec, int64_t* laun
 // for every row count) is captured instead.
 int capture(ivit_handle* h, bool full, cudaGraphExec_t* exec, int64_t* launches) {
   const bool chain = h->cfg.mlp_tokens == IVIT_MLP_UPDATED && !h->stream_ok && !h->persistent;
-  if (!full && chain && h->n_bands > 1 && h->cfg.select_mode == IVIT_SEL_TOPK) {
-    // top-k (no cold view in a captured call): exactly k rows per view, so the band is
-    // known when the graph is captured and no switch is needed
-    const long long m = std::min<long long>(static_cast<long long>(h->cfg.topk), h->N) * h->SV;
-    int b = 0;
-    while (b + 1 < h->n_bands && m > h->band_ub[b]) ++b;
-    h->known_band = b;
-    h->known_rows = static_cast<int>(m);
-    const int r = capture_once(h, full, exec, launches);
-    h->known_band = -1;
-    return r;
-  }
   // threshold selection: the row count is known only on the device; the switch pays its
   // fixed cost (no programmatic overlap across the node) when a tenth of the tokens
   // already exceeds 32 rows, so that row counts commonly cross bands
-  if (!full && chain && h->n_bands > 1 && h->M_max / 10 > 32) {
+  if (!full && chain && h->n_bands > 1 && h->cfg.select_mode != IVIT_SEL_TOPK && h->M_max / 10 > 32) {
     h->capture_bands = true;
     const int r = capture_once(h, full, exec, launches);
     h->capture_bands = false;

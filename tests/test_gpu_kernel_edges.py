@@ -210,3 +210,24 @@ def test_pointers_outside_the_gpu_take_the_copy_engine(pkg):
         for (tok, cnt, n), (tok0, cnt0, n0) in zip(encode(where), gpu):
             assert torch.equal(tok, tok0) and torch.equal(cnt, cnt0), where
             assert n == n0 - fewer, where
+
+
+@pytest.mark.parametrize("mlp_tokens", [0, 1], ids=["updated", "all"])
+@pytest.mark.parametrize("select,topk", [(0, 0), (1, 20)], ids=["threshold", "top20"])
+def test_cold_calls_take_the_plans_of_their_rows(pkg, select, topk, mlp_tokens):
+    """An incremental call whose views are all cold updates every token, in the launch shapes of a full
+    encode and so with its rounding: bit for bit its tokens.  (Those of a tenth of the rows split K
+    elsewhere.)"""
+    import torch
+    from paper_2607_12287_gb300 import synth
+
+    shape = synth.EncoderShape(128, 128, 8, 576, 2, 8, 2328, synth.GELU_TANH)
+    weights = synth.make_weights(shape, 3)
+    frames = [torch.from_numpy(f).cuda() for f in synth.stream_random(shape, 1, 2, 11, change_p=0.3)]
+    enc = pkg.IncrementalViT(shape, weights, 1, 1, select, 0.98, topk, mlp_tokens=mlp_tokens)
+    for frame in frames:
+        want = enc.encode_full(frame)
+        enc.reset()
+        got, count = enc.encode_incremental(frame)
+        assert int(count[0]) == shape.n_tokens and torch.equal(got, want)
+    enc.close()
