@@ -1,7 +1,9 @@
 """Kernels at the edges of their tiles, through the C ABI against the fp32 oracle: an encoder of
 one or two layers encodes a stream in full and incrementally (updated lists bit-exact, tokens
 within the parity bars of gpu_util)."""
+import os
 import re
+import subprocess
 
 import numpy as np
 import pytest
@@ -231,3 +233,11 @@ def test_cold_calls_take_the_plans_of_their_rows(pkg, select, topk, mlp_tokens):
         got, count = enc.encode_incremental(frame)
         assert int(count[0]) == shape.n_tokens and torch.equal(got, want)
     enc.close()
+
+
+def test_every_cta_of_a_grid_has_its_own_stamp(tmp_path):
+    """Timeline stamps of a grid of more than one dimension (the few-row GEMM's second row group)."""
+    from paper_2607_12287_gb300 import build as b
+    exe = str(tmp_path / "stamp_probe")
+    subprocess.run([b.NVCC, *b.ARCH, "-std=c++17", os.path.join(b.ROOT, "tests", "stamp_probe.cu"), "-o", exe], check=True)
+    assert subprocess.run([exe], check=True, capture_output=True, text=True).stdout.split() == ["30", "0"]
