@@ -149,7 +149,7 @@ int ivit_reset(ivit_handle* h, int stream_index);
  * launches, the global time at which each CTA started its work (after the wait on the
  * previous kernel) and finished; the captured CUDA graphs are rebuilt with the
  * recording in them, so the calls still run as replayed graphs (enable = 0 rebuilds
- * them without it).  Allocates 8 MB of device memory on first use.
+ * them without it).  Allocates 16 KB of device memory per launch of a call on first use.
  * ivit_timeline_read synchronises `stream` and reads the last call: per kernel family
  * (index 0 tensor-core GEMMs, 1 attention, 2 layer norms, 3 patchify / score /
  * selection / gather / output copy) the sum over its launches of (last CTA end - first CTA start)

@@ -1226,8 +1226,12 @@ int capture_band_bodies(ivit_handle* h, cudaStream_t s) {
   IVIT_CK(h, cudaGraphAddNode(&node, graph, deps, nullptr, ndeps, &np));
   IVIT_CK(h, cudaStreamUpdateCaptureDependencies(s, &node, nullptr, 1, cudaStreamSetCaptureDependencies));
   const int64_t pre = h->launches;
-  for (int b = 0; b < h->n_bands; ++b) {
+  const int pre_stamps = h->stamp_used;
+  const size_t pre_slots = h->slots_cur.size();
+  for (int b = 0; b < h->n_bands; ++b) {  // (the same sequence of launches, of which one runs per call: one set of stamps)
     h->launches = pre;
+    h->stamp_used = pre_stamps;
+    h->slots_cur.resize(pre_slots);
     IVIT_CK(h, cudaStreamBeginCaptureToGraph(h->cap_stream2, np.conditional.phGraph_out[b], nullptr, nullptr, 0,
                                              cudaStreamCaptureModeThreadLocal));
     const int r = run_layers(h, h->plan_band[b], band_rows(h, b), false, h->cap_stream2);
@@ -1612,7 +1616,7 @@ int ivit_timeline(ivit_handle* h, int enable) {
   if (!h) return IVIT_ERR_ARG;
   const bool on = enable != 0;
   if (on && !h->stamps) {
-    h->stamp_cap = 512;
+    h->stamp_cap = 7 * h->L + 12;  // the launches of the longest call
     IVIT_CK(h, cudaMalloc(&h->stamps, static_cast<size_t>(h->stamp_cap) * 2 * ivit::kStampCtas *
                                           sizeof(unsigned long long)));
     IVIT_CK(h, cudaMemset(h->stamps, 0, static_cast<size_t>(h->stamp_cap) * 2 * ivit::kStampCtas *
@@ -1652,7 +1656,7 @@ int ivit_timeline_read(ivit_handle* h, void* stream, double* family_ms, int64_t*
       if (se) e = std::max(e, se);
     }
     const TimelineSlot& sl = h->slots_last[i];
-    if (b == ~0ull) continue;  // not run (another row band's body of the graph)
+    if (b == ~0ull) continue;  // left without a stamp (no rows)
     ++cnt[sl.family];
     if (e > b) {
       ms[sl.family] += 1e-6 * static_cast<double>(e - b);

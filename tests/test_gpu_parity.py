@@ -324,6 +324,36 @@ def test_timeline_records_every_launch(pkg):
         assert torch.equal(a, b)
 
 
+@pytest.mark.parametrize("score", [synth.SCORE_EMBED, synth.SCORE_KEY0], ids=["embed", "key0"])
+def test_timeline_of_a_deep_encoder_in_every_row_band(pkg, score):
+    # 30 layers and a switch over four row bands: whichever body of the graph a call takes, every
+    # launch of it has its stamps, the output copy's after the graph included
+    import torch
+    shape = synth.EncoderShape(160, 160, 8, 192, 30, 3, 768, synth.GELU_TANH)
+    enc = pkg.IncrementalViT(shape, synth.make_weights(shape, 163), 1, 1, score_source=score)
+    pkg.ivit_timeline(enc.h, True)
+    base = next(synth.stream_random(shape, 1, 1, 164))
+    enc.encode_full(torch.from_numpy(base).cuda())
+    seen = []
+    for changed in (8, 100, 200, 400):  # of 400 patches; bands of up to 64, 128, 256 and 400 rows
+        base = base.copy()
+        rows = base[0].reshape(20, 8, 20, 8, 3).transpose(0, 2, 1, 3, 4).copy().reshape(400, -1)
+        rows[:changed] = 255 - rows[:changed]
+        base[0] = rows.reshape(20, 20, 8, 8, 3).transpose(0, 2, 1, 3, 4).reshape(160, 160, 3)
+        _, cnt = enc.encode_incremental(torch.from_numpy(base).cuda())
+        r = pkg.ivit_timeline_read(enc.h)
+        L = shape.depth
+        extra = 1 if score == synth.SCORE_KEY0 else 0  # the keys' gather, layer norm and GEMM; their score kernel
+        assert r["launches"] == {"gemm": 1 + extra + 4 * L, "attention": L, "layernorm": 2 * L + 1 + extra,
+                                 "other": 4 + 2 * extra}, changed
+        assert sum(r["launches"].values()) == pkg.ivit_last_launch_count(enc.h)
+        assert 0 < sum(r["ms"].values()) <= r["span_ms"] * 1.02
+        seen.append(int(cnt[0]))
+    assert [sum(c > ub for ub in (64, 128, 256)) for c in seen] == [0, 1, 2, 3], seen
+    assert enc.device_status() == 0
+    enc.close()
+
+
 def test_maximum_view_count(pkg, oracle_mod):
     # 4096 views, the most a handle takes (1024 streams x 4 views of a 4-token encoder):
     # one selection CTA per view, the cold-view mask and the packed-row offsets at their
