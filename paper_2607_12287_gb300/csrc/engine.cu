@@ -551,6 +551,11 @@ int setup_stream(ivit_handle* h) {
   return IVIT_OK;
 }
 
+// Whether the row counts of threshold calls commonly cross bands, so that a switch over them pays
+// its fixed cost (about 10 us: no programmatic overlap across the node).  Below, one plan serves
+// every count, with a second row group in the few-row GEMM.
+bool rows_cross_bands(const ivit_handle* h) { return h->M_max / 10 > 32; }
+
 // The bands of the row count and the launch plans of every GEMM, from the configuration and the
 // number of SMs alone.
 void make_plans(ivit_handle* h) {
@@ -596,7 +601,7 @@ void make_plans(ivit_handle* h) {
   if (!differ) h->n_bands = 1;
   // a second row group (gemm.cu) where the band of the row count is not known at launch
   const bool one_plan = c.mlp_tokens == IVIT_MLP_ALL || c.select_mode != IVIT_SEL_TOPK;
-  h->row_groups = one_plan && m_all > 64 && (c.mlp_tokens == IVIT_MLP_ALL || m_all / 10 <= 32) ? 2 : 1;
+  h->row_groups = one_plan && m_all > 64 && (c.mlp_tokens == IVIT_MLP_ALL || !rows_cross_bands(h)) ? 2 : 1;
   // every row's D x D projection without a residual (first-layer key scores)
   h->plan_keys = plan_gemm(h->num_sms, D, D, m_all, m_all, false, false);
   if (std::getenv("IVIT_DEBUG")) {
@@ -1426,10 +1431,8 @@ int capture_once(ivit_handle* h, bool full, cudaGraphExec_t* exec, int64_t* laun
 // for every row count) is captured instead.
 int capture(ivit_handle* h, bool full, cudaGraphExec_t* exec, int64_t* launches) {
   const bool chain = h->cfg.mlp_tokens == IVIT_MLP_UPDATED && !h->stream_ok && !h->persistent;
-  // threshold selection: the row count is known only on the device; the switch pays its
-  // fixed cost (no programmatic overlap across the node) when a tenth of the tokens
-  // already exceeds 32 rows, so that row counts commonly cross bands
-  if (!full && chain && h->n_bands > 1 && h->cfg.select_mode != IVIT_SEL_TOPK && h->M_max / 10 > 32) {
+  // threshold selection: the row count is known only on the device
+  if (!full && chain && h->n_bands > 1 && h->cfg.select_mode != IVIT_SEL_TOPK && rows_cross_bands(h)) {
     h->capture_bands = true;
     const int r = capture_once(h, full, exec, launches);
     h->capture_bands = false;
