@@ -44,7 +44,6 @@ namespace {
 
 constexpr int AQ = 128;             // queries per item (MMA M)
 constexpr int THREADS = 192;
-constexpr int MAX_VIEWS = 4096;
 constexpr int SMEM_HALF = 113 * 1024;  // two CTAs share an SM
 constexpr float RESCALE = 8.f;      // log2 of the growth that moves the reference maximum
 
@@ -64,12 +63,6 @@ struct AttnCfg {
   static constexpr int OFF_CUM = OFF_BAR + 256;  // [sv + 1] items before each view
   static constexpr int BYTES = OFF_CUM + 1024;   // alignment slack
 };
-
-__device__ __forceinline__ float ex2(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
 
 // 32 columns of S (bits) -> 16 packed bf16 pairs of P; l gets the rounded values.
 __device__ __forceinline__ void exp_chunk(const uint32_t* s, float sc, float mo, uint32_t* pk, float2 (&l)[2]) {

@@ -6,9 +6,17 @@
 
 namespace ivit {
 
+constexpr int MAX_VIEWS = 4096;
+
 struct AttnItem {
   int v, h, r0, nq;  // view, head, first packed row, rows
 };
+
+__device__ __forceinline__ float ex2(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
 
 // cum[v] = items before view v (cum[sv]: all of them), for query tiles of `tile` rows; by the
 // first warp of the block.

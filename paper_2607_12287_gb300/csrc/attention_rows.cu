@@ -31,13 +31,6 @@ namespace {
 constexpr int WARPS = 8, THREADS = WARPS * 32;
 constexpr int TQ = 16;       // queries per item
 constexpr int KW = 32;       // keys per warp and step
-constexpr int MAX_VIEWS = 4096;
-
-__device__ __forceinline__ float ex2(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
 
 __device__ __forceinline__ uint4 load16(const bf16* p, bool ok) {
   return ok ? __ldcg(reinterpret_cast<const uint4*>(p)) : make_uint4(0, 0, 0, 0);

@@ -26,7 +26,7 @@ struct LayerW {
   bf16 *wqkv, *wo, *w1, *w2;
   float *bqkv, *bo, *b1, *b2, *ln1g, *ln1b, *ln2g, *ln2b;
   CUtensorMap tm_qkv, tm_o, tm_1, tm_2;
-  CUtensorMap tm_ck, tm_cv;  // this layer's key / value cache, SIMT attention key-split tiles
+  CUtensorMap tm_ck, tm_cv;  // this layer's key / value cache, SIMT attention key-split tiles (if selected)
   ivit::AttnMaps tm_ak, tm_av;  // the same caches for the tcgen05 attention
 };
 
@@ -806,8 +806,8 @@ int setup(ivit_handle* h, const uint16_t* wb) {
   const int dh = h->D / h->H, kb = ivit::attention_key_block((dh + 15) & ~15);
   for (size_t l = 0; l < L; ++l) {
     const size_t off = l * M * D;
-    if (!make_map(&h->layers[l].tm_ck, h->cacheK + off, D, M, D * 2, D / h->H, kps, false) ||
-        !make_map(&h->layers[l].tm_cv, h->cacheV + off, D, M, D * 2, D / h->H, kps, false) ||
+    if ((!h->attn_tc && (!make_map(&h->layers[l].tm_ck, h->cacheK + off, D, M, D * 2, D / h->H, kps, false) ||
+                         !make_map(&h->layers[l].tm_cv, h->cacheV + off, D, M, D * 2, D / h->H, kps, false))) ||
         !make_attn_maps(&h->layers[l].tm_ak, h->cacheK + off, dh, h->H, M, kb) ||
         !make_attn_maps(&h->layers[l].tm_av, h->cacheV + off, dh, h->H, M, kb))
       return h->fail(IVIT_ERR_CUDA, "cuTensorMapEncodeTiled failed for a cache tile");

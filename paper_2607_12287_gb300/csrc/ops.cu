@@ -808,19 +808,19 @@ cudaError_t launch_layernorm_ex(const int* rows, float* x, const float* add, con
                                 const float* gamma, const float* beta, bf16* y, const int* dst_rowtok, int dim,
                                 float eps, int max_rows, int grid, cudaStream_t s) {
   grid = max(1, min(grid, (max_rows + 7) / 8));
-  if (dim % 4 != 0 || dim > 2048) return cudaErrorInvalidValue;
-  auto launch = [&](auto plain, auto gather, auto with_add, auto both) {
-    return launch_ex(add ? (src_rowtok ? both : with_add) : (src_rowtok ? gather : plain), dim3(grid), dim3(256), 0, s,
+  if (dim % 4 != 0 || dim > 2048 || (add && src_rowtok)) return cudaErrorInvalidValue;
+  auto launch = [&](auto plain, auto gather, auto with_add) {
+    return launch_ex(add ? with_add : (src_rowtok ? gather : plain), dim3(grid), dim3(256), 0, s,
                      1, rows, x, add, src_rowtok, gamma, beta, y, dst_rowtok, dim, eps, g_stamp);
   };
   if (dim <= 128 * 4)
     return launch(layernorm_kernel<4, false, false>, layernorm_kernel<4, false, true>,
-                  layernorm_kernel<4, true, false>, layernorm_kernel<4, true, true>);
+                  layernorm_kernel<4, true, false>);
   if (dim <= 128 * 10)
     return launch(layernorm_kernel<10, false, false>, layernorm_kernel<10, false, true>,
-                  layernorm_kernel<10, true, false>, layernorm_kernel<10, true, true>);
+                  layernorm_kernel<10, true, false>);
   return launch(layernorm_kernel<16, false, false>, layernorm_kernel<16, false, true>,
-                layernorm_kernel<16, true, false>, layernorm_kernel<16, true, true>);
+                layernorm_kernel<16, true, false>);
 }
 
 cudaError_t launch_outputs(const bf16* tok, void* out, size_t bytes, const int* counts, int* user_counts, int sv,
