@@ -97,7 +97,7 @@ __global__ void __launch_bounds__(THREADS, 2) gemm_rows_kernel(const GemmArgs a)
   const int M = a.d_rows ? *a.d_rows : a.m_static;
   pdl_wait();
   pdl_launch_dependents();
-  stamp_begin(a.stamp);
+  stamp_begin(a.stamp, blockIdx.x + gridDim.x * blockIdx.y);
 
   bool ok = true;
   const int n = max(0, (c_hi - c_lo - warp + WARPS - 1) / WARPS);  // this warp's chunks
@@ -208,7 +208,7 @@ __global__ void __launch_bounds__(THREADS, 2) gemm_rows_kernel(const GemmArgs a)
   }
   if (M <= 0 && !mbar_wait(bar_a, 0)) ok = false;  // no copy in flight at exit
   if (!ok && tid == 0) atomicExch(a.err, kErrWaitTmaFull);
-  stamp_end(a.stamp);
+  stamp_end(a.stamp, blockIdx.x + gridDim.x * blockIdx.y);
 }
 
 size_t smem_bytes(int nt, int k, int splits) {

@@ -473,19 +473,22 @@ __device__ __forceinline__ void fence_proxy_async_global() {
 }
 
 // ------------------------------------------------------------- kernel timeline
-// Optional per-launch stamps (the library's timeline mode): thread 0 of CTA b (counted over the
-// whole grid) writes the global time after the kernel's wait on the previous kernel to s[2b] and
-// the time it finishes to s[2b+1]; only the first kStampCtas CTAs of a launch record.
+// Optional per-launch stamps (the library's timeline mode): thread 0 of CTA b writes
+// the global time after the kernel's wait on the previous kernel to s[2b] and the time
+// it finishes to s[2b+1]; only the first kStampCtas CTAs of a launch record.  (Grids of one
+// dimension take the form without b: the general index in every kernel cost 1 %.)
 constexpr int kStampCtas = 1024;
 
-__device__ __forceinline__ void write_stamp(unsigned long long* s, int end) {
-  if (!s || threadIdx.x != 0) return;
-  const unsigned b = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
-  if (b < kStampCtas) s[2 * b + end] = globaltimer_ns();
+__device__ __forceinline__ void stamp_begin(unsigned long long* s, unsigned b) {
+  if (s && threadIdx.x == 0 && b < kStampCtas) s[2 * b] = globaltimer_ns();
 }
 
-__device__ __forceinline__ void stamp_begin(unsigned long long* s) { write_stamp(s, 0); }
-__device__ __forceinline__ void stamp_end(unsigned long long* s) { write_stamp(s, 1); }
+__device__ __forceinline__ void stamp_end(unsigned long long* s, unsigned b) {
+  if (s && threadIdx.x == 0 && b < kStampCtas) s[2 * b + 1] = globaltimer_ns();
+}
+
+__device__ __forceinline__ void stamp_begin(unsigned long long* s) { stamp_begin(s, blockIdx.x); }
+__device__ __forceinline__ void stamp_end(unsigned long long* s) { stamp_end(s, blockIdx.x); }
 
 // ------------------------------------------------------ programmatic dependent launch
 // Every tcgen05 kernel allocates its TMEM columns before pdl_wait and calls

@@ -235,9 +235,10 @@ def test_cold_calls_take_the_plans_of_their_rows(pkg, select, topk, mlp_tokens):
     enc.close()
 
 
-def test_every_cta_of_a_grid_has_its_own_stamp(tmp_path):
-    """Timeline stamps of a grid of more than one dimension (the few-row GEMM's second row group)."""
+def test_every_cta_of_both_row_groups_has_its_own_stamp(pkg, tmp_path):
+    """Timeline stamps of the few-row GEMM with more rows than one group's pass (stamp_probe.cu)."""
     from paper_2607_12287_gb300 import build as b
     exe = str(tmp_path / "stamp_probe")
-    subprocess.run([b.NVCC, *b.ARCH, "-std=c++17", os.path.join(b.ROOT, "tests", "stamp_probe.cu"), "-o", exe], check=True)
-    assert subprocess.run([exe], check=True, capture_output=True, text=True).stdout.split() == ["30", "0"]
+    subprocess.run([b.NVCC, *b.ARCH, "-std=c++17", os.path.join(b.ROOT, "tests", "stamp_probe.cu"), b.LIB, "-Xlinker",
+                    "-rpath=" + os.path.dirname(b.LIB), "-o", exe], check=True)
+    assert subprocess.run([exe], check=True, capture_output=True, text=True).stdout.split() == ["24", "24", "0"]
