@@ -11,10 +11,10 @@
 // product does not care which k is called which).  So no operand is staged, and the rows cost
 // one round trip to L2.  The warps' sums meet in shared memory, in warp order.  Rows beyond
 // 32 run as further passes over the resident weights; where one plan serves every row count, a
-// second group of CTAs (blockIdx.y) takes every other pass and leaves at once when there is none:
-// two groups of all updates of a 256-token So400m view (four layers, two calls) 1058 -> 696 us, of
-// 30 % 451 -> 371, while a single pass costs no more (26 rows on average: 1499 -> 1419 us for 27
-// layers, for its calls of 33 rows and more).
+// second group of CTAs (blockIdx.y) takes every other pass and leaves at once when there is none.
+// Two calls of four So400m layers took 1058 us with one group and take 696 with two when all 256
+// tokens of a view change, 451 and 371 when 30 % do.  A call of one pass costs no more: two calls
+// of 27 layers with 26 rows on average went from 1499 to 1419 us, by those of 33 rows and more.
 //
 // Bound: latency (wait, rows from L2, MMAs, sum over the warps, store).  mma.sync and not
 // tcgen05 because a tcgen05.mma takes at least about 46 cycles however few rows it has, and a

@@ -20,10 +20,10 @@
 //     epilogue that stored column by column behind a switch took 7.5 us for 64 rows x 128
 //     features, most of it on instruction fetch.  The residual is added in L2 (red.v4.f32),
 //     so it is never loaded.
-// Measured back to back, random bf16 data, before -> now: 32768 rows QKV 422 -> 149 us
-// (1750 TFLOP/s), up 497 -> 198, out 154 -> 82, down 324 -> 211; 3080 rows QKV 65 -> 22, up
-// 60 -> 24, down 53 -> 26; 768 rows QKV 29 -> 12, up 27 -> 12; 256 rows QKV 16 -> 7.6,
-// up 16 -> 7.8.
+// Measured back to back (whole launches, prologue included), random bf16 data, before -> now:
+// 32768 rows QKV 422 -> 149 us (1750 TFLOP/s), up 497 -> 195, out 154 -> 78, down 324 -> 218; 3080
+// rows QKV 65 -> 23, up 60 -> 27, down 53 -> 29; 768 rows QKV 29 -> 12, up 27 -> 13; 256 rows QKV
+// 16 -> 6.9, up 16 -> 7.6.
 #include "gelu.cuh"
 #include "internal.h"
 #include "ptx.cuh"
@@ -235,8 +235,10 @@ __device__ __forceinline__ void drain(const GemmArgs& a, uint32_t acc, uint8_t* 
 
 // The same for a half of a 64-row tile, where it is faster: at most 32 rows of this warp's 32
 // features straight from the registers, 64 or 128 bytes per access, without the exchange through
-// shared memory and its barriers.  256 rows of the So400m shapes, staged -> direct: out and down
-// 5.9 -> 5.7 us, QKV 5.4 -> 5.3, but up with GELU 6.2 -> 7.1 and the embedding 4.5 -> 4.7.
+// shared memory and its barriers.  256 rows of the So400m shapes in the replayed graph, from a
+// launch's wait on the kernel before to its last store (without the prologue of the figures above),
+// staged -> direct: out and down 5.9 -> 5.7 us, QKV 5.4 -> 5.3, but up with GELU 6.2 -> 7.1 and the
+// embedding 4.5 -> 4.7.
 template <int KIND>
 constexpr bool kDirect = KIND == kEpiResid || KIND == kEpiPartial || KIND == kEpiQKV || KIND == kEpiScatterF32;
 
