@@ -19,7 +19,7 @@
 // rate at larger ones, where attention.cu is the faster one (the rule is attention_few in
 // engine.cu).  Heads of up to 64 have a form for two CTAs on an SM (128 registers; wider heads would
 // spill, 8.8 -> 11.6 us), taken when there are more items than SMs: six views of 196 x 196, 3 heads
-// of 64, 5.6 -> 4.9 us (a full encode of them in the exact form: 384 us, 392 with one CTA).  16 heads of 72, 256 keys, 26 queries: 3.9 us back to back against 6.1 there, whose
+// of 64, 5.6 -> 4.9 us (a full encode of 12 layers in the exact form: 8 us less than with one CTA).  16 heads of 72, 256 keys, 26 queries: 3.9 us back to back against 6.1 there, whose
 // 128-query tile walks the keys in three dependent steps.
 #include "attention.cuh"
 #include "internal.h"

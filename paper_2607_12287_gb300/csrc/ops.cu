@@ -328,7 +328,7 @@ __global__ void gather_bulk_kernel(const int* __restrict__ total_rows, int* __re
 // now 4.9 (10: 64 registers, four CTAs of an SM in flight; 8-byte stores).  Rows are taken
 // from the last to the first: the residual rows that the GEMM before wrote last are still
 // in L2, and the next GEMM finds the rows it begins with there.  32768 rows of 1152: 50.4 us,
-// 46.9 by width, 41.5 in this order (5.5 TB/s).
+// 46.9 by width, 40 in this order (5.7 TB/s).
 // Optionally the input row is gathered (row src_rowtok[r] of x) and, with kAdd, a
 // second fp32 array is added to it first and the sum written back to x (the residual
 // addition fused into the LN).
